@@ -1,6 +1,5 @@
 // Dense FP64 building blocks for the rank truncation and the solvers: batched GEMM (Gram matrices and
-// core contractions), a cyclic two-sided Jacobi eigensolver for the small symmetric Gram matrices,
-// and reductions.
+// core contractions) and reductions.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -363,247 +362,6 @@ void gemm_nosplit(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, do
   else
     launch_dgemm<64, double>(ctx, transA, transB, grid, flops, bytes, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C,
                              ldc, sC, 1, kchunk, nullptr, 1, nullptr, 1, nullptr, nullptr);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Symmetric eigensolver, two stages:
-//  1. cyclic two-sided Jacobi with the round-robin (circle) ordering, so that each round applies m'/2
-//     disjoint rotations in parallel (Golub & Van Loan, "Matrix Computations", 4th ed., Sec. 8.5: the
-//     2x2 symmetric Schur step and parallel orderings).  One block per matrix, working matrices in
-//     shared memory when they fit, else in a global scratch slice.  The working precision T is FP32
-//     for speed (GB300 issues FP32 at ~58x its FP64 rate) or FP64.
-//  2. (FP32 start) refinement to FP64 accuracy by the iteration of Ogita & Aishima, "Iterative
-//     refinement for symmetric eigenvalue decomposition", Japan J. Indust. Appl. Math. 35 (2018):
-//        R = I - X^T X,  S = X^T A X,  lam_i = S_ii / (1 - R_ii),
-//        E_ij = (S_ij + lam_j R_ij) / (lam_j - lam_i)  if |lam_i - lam_j| > delta,  R_ij / 2 otherwise,
-//        X <- X + X E,   delta = 2 (||S - diag(lam)|| + ||A|| ||R||),
-//     which converges quadratically; eigenvalues closer than delta are treated as a cluster whose
-//     invariant subspace (not its individual vectors) is refined.  All of it is GEMM work in FP64.
-// ------------------------------------------------------------------------------------------------
-constexpr int kJacobiMaxSweeps = 30;
-constexpr int kJacobiThreads = 512;
-
-__device__ __forceinline__ void rr_pair(int round, int i, int mp, int* p, int* q) {
-  // circle method: player mp-1 fixed, the others rotate
-  const int n1 = mp - 1;
-  if (i == 0) { *p = round % n1; *q = n1; return; }
-  *p = (round + i) % n1;
-  *q = (round - i + n1) % n1;
-}
-
-template <typename T>
-__device__ __forceinline__ T block_sum(T v, T* red) {
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffff, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  T s = 0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-  return s;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double* __restrict__ Ag, double* w,
-                                                               double* Vout, int m, T* scratch, int use_smem,
-                                                               T eps) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int mp = m + (m & 1);
-  const int npair = mp / 2;
-  T* cs = (T*)smraw;                                   // 2 npair (c, s)
-  int* pq = (int*)(cs + 2 * npair);                    // 2 npair
-  T* red = (T*)(pq + 2 * npair);                       // 32 partial sums
-  int* rank = (int*)(red + 32);                        // m (+1) ints
-  T* A;
-  T* V;
-  if (use_smem == 2) {         // A and V in shared memory
-    A = (T*)(rank + m + (m & 1));
-    V = A + (size_t)m * m;
-  } else if (use_smem == 1) {  // A in shared memory, V in a global scratch slice
-    A = (T*)(rank + m + (m & 1));
-    V = scratch + (size_t)blockIdx.x * m * m;
-  } else {
-    A = scratch + (size_t)blockIdx.x * 2 * m * m;
-    V = A + (size_t)m * m;
-  }
-  const double* Ain = Ag + (size_t)blockIdx.x * m * m;
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    A[t] = (T)Ain[t];
-    V[t] = ((t / m) == (t % m)) ? T(1) : T(0);
-  }
-  __syncthreads();
-  T loc = 0;
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) loc += A[t] * A[t];
-  const T fro2 = block_sum(loc, red);
-  const T tol2 = T(16) * eps * eps * fro2;
-  T prev_off = fro2;
-  if (m > 1 && fro2 > T(0)) {
-    for (int sweep = 0; sweep < kJacobiMaxSweeps; ++sweep) {
-      for (int round = 0; round < mp - 1; ++round) {
-        for (int i = threadIdx.x; i < npair; i += blockDim.x) {
-          int p, q;
-          rr_pair(round, i, mp, &p, &q);
-          if (p > q) { int t = p; p = q; q = t; }
-          T c = 1, s = 0;
-          if (q < m) {
-            T apq = A[(size_t)p * m + q];
-            T app = A[(size_t)p * m + p], aqq = A[(size_t)q * m + q];
-            if (apq != T(0) && fabs(apq) > T(0.01) * eps * sqrt(fabs(app * aqq))) {
-              T tau = (aqq - app) / (T(2) * apq);
-              T t = (tau >= T(0) ? T(1) : T(-1)) / (fabs(tau) + sqrt(T(1) + tau * tau));
-              c = T(1) / sqrt(T(1) + t * t);
-              s = t * c;
-            }
-          } else {
-            q = -1;
-          }
-          cs[2 * i] = c;
-          cs[2 * i + 1] = s;
-          pq[2 * i] = p;
-          pq[2 * i + 1] = (s == T(0)) ? -1 : q;
-        }
-        __syncthreads();
-        // rows: A <- J^T A
-        for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {
-          int i = t / m, j = t - (t / m) * m;
-          int q = pq[2 * i + 1];
-          if (q < 0) continue;
-          int p = pq[2 * i];
-          T c = cs[2 * i], s = cs[2 * i + 1];
-          T ap = A[(size_t)p * m + j], aq = A[(size_t)q * m + j];
-          A[(size_t)p * m + j] = c * ap - s * aq;
-          A[(size_t)q * m + j] = s * ap + c * aq;
-        }
-        __syncthreads();
-        // columns: A <- A J, V <- V J
-        for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {
-          int i = t / m, j = t - (t / m) * m;
-          int q = pq[2 * i + 1];
-          if (q < 0) continue;
-          int p = pq[2 * i];
-          T c = cs[2 * i], s = cs[2 * i + 1];
-          T ap = A[(size_t)j * m + p], aq = A[(size_t)j * m + q];
-          A[(size_t)j * m + p] = c * ap - s * aq;
-          A[(size_t)j * m + q] = s * ap + c * aq;
-          T vp = V[(size_t)j * m + p], vq = V[(size_t)j * m + q];
-          V[(size_t)j * m + p] = c * vp - s * vq;
-          V[(size_t)j * m + q] = s * vp + c * vq;
-        }
-        __syncthreads();
-      }
-      T off = 0;
-      for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-        int i = t / m, j = t - (t / m) * m;
-        if (i != j) off += A[t] * A[t];
-      }
-      off = block_sum(off, red);
-      // converged, or rounding has stopped the decrease (off-diagonal mass at the precision floor)
-      if (off <= tol2 || (off > T(0.25) * prev_off && off <= T(4096) * eps * eps * fro2)) break;
-      prev_off = off;
-    }
-  }
-  // sort descending: rank[j] = position of eigenvalue j (ties by index)
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    T lj = A[(size_t)j * m + j];
-    int pos = 0;
-    for (int i = 0; i < m; ++i) {
-      T li = A[(size_t)i * m + i];
-      if (li > lj || (li == lj && i < j)) ++pos;
-    }
-    rank[j] = pos;
-  }
-  __syncthreads();
-  double* wb = w + (size_t)blockIdx.x * m;
-  double* Vb = Vout + (size_t)blockIdx.x * m * m;
-  for (int j = threadIdx.x; j < m; j += blockDim.x) wb[rank[j]] = (double)A[(size_t)j * m + j];
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t / m, j = t - (t / m) * m;
-    Vb[(size_t)i * m + rank[j]] = (double)V[t];
-  }
-}
-
-template <typename T>
-static void jacobi_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch) {
-  const int mp = m + (m & 1);
-  const int npair = mp / 2;
-  size_t head = sizeof(T) * 2 * npair + sizeof(int) * 2 * npair + sizeof(T) * 32 + sizeof(int) * (m + (m & 1));
-  head = (head + 15) / 16 * 16;
-  const size_t limit = (size_t)std::min(ctx->max_smem_optin, 220 * 1024);
-  const size_t one = head + sizeof(T) * (size_t)m * m, two = one + sizeof(T) * (size_t)m * m;
-  int use_smem = two <= limit ? 2 : (one <= limit ? 1 : 0);
-  size_t smem = use_smem == 2 ? two : (use_smem == 1 ? one : head);
-  DBuf<T> scratch;
-  if (use_smem == 1) scratch = DBuf<T>(ctx->pool, (size_t)m * m * batch);
-  if (use_smem == 0) scratch = DBuf<T>(ctx->pool, (size_t)2 * m * m * batch);
-  LRFG_CUDA(raise_smem_limit((const void*)jacobi_kernel<T>, smem));
-  const T eps = sizeof(T) == 4 ? (T)1.1920929e-07 : (T)2.220446049250313e-16;
-  // one sweep of the two-sided cyclic Jacobi costs about 9 m^3 flops (rows, columns and V)
-  LRFG_LAUNCH(ctx, KC_EIGEN, 9.0 * (double)m * m * m * batch, 3.0 * sizeof(double) * (double)m * m * batch,
-              jacobi_kernel<T><<<batch, kJacobiThreads, smem, ctx->stream>>>(A, w, V, m, scratch.get(), use_smem,
-                                                                              eps));
-}
-
-// Ogita–Aishima correction from G = X^T X and S = X^T A X (one block per matrix): writes lam and E.
-__global__ void __launch_bounds__(512) oa_correction_kernel(const double* __restrict__ Ag, const double* __restrict__ Gg,
-                                                            const double* __restrict__ Sg, double* lamg, double* Eg,
-                                                            int m) {
-  __shared__ double red[32];
-  const size_t off = (size_t)blockIdx.x * m * m;
-  const double* A = Ag + off;
-  const double* G = Gg + off;
-  const double* S = Sg + off;
-  double* E = Eg + off;
-  double* lam = lamg + (size_t)blockIdx.x * m;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) lam[i] = S[(size_t)i * m + i] / G[(size_t)i * m + i];
-  __syncthreads();
-  double a2 = 0.0, r2 = 0.0, s2 = 0.0;
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t / m, j = t - (t / m) * m;
-    double r = (i == j ? 1.0 : 0.0) - G[t];
-    double sd = (i == j) ? S[t] - lam[i] : S[t];
-    a2 += A[t] * A[t];
-    r2 += r * r;
-    s2 += sd * sd;
-  }
-  a2 = block_sum(a2, red);
-  r2 = block_sum(r2, red);
-  s2 = block_sum(s2, red);
-  const double delta = 2.0 * (sqrt(s2) + sqrt(a2) * sqrt(r2));
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t / m, j = t - (t / m) * m;
-    double r = (i == j ? 1.0 : 0.0) - G[t];
-    double e;
-    if (i == j) {
-      e = 0.5 * r;
-    } else {
-      double gap = lam[j] - lam[i];
-      e = (fabs(gap) > delta) ? (S[t] + lam[j] * r) / gap : 0.5 * r;
-    }
-    E[t] = e;
-  }
-}
-
-void syevj_mixed(lrfg_ctx* ctx, double* A, double* w, double* V, int m, int batch) {
-  if (m <= 0 || batch <= 0) return;
-  jacobi_launch<float>(ctx, A, w, V, m, batch);
-  if (m == 1) return;
-  const long long mm = (long long)m * m;
-  DBuf<double> G(ctx->pool, mm * batch), AV(ctx->pool, mm * batch), S(ctx->pool, mm * batch),
-      E(ctx->pool, mm * batch), Vn(ctx->pool, mm * batch);
-  for (int it = 0; it < 3; ++it) {
-    gemm(ctx, 1, 0, m, m, m, 1.0, V, m, mm, V, m, mm, 0.0, G.get(), m, mm, batch);
-    gemm(ctx, 0, 0, m, m, m, 1.0, A, m, mm, V, m, mm, 0.0, AV.get(), m, mm, batch);
-    gemm(ctx, 1, 0, m, m, m, 1.0, V, m, mm, AV.get(), m, mm, 0.0, S.get(), m, mm, batch);
-    LRFG_LAUNCH(ctx, KC_EIGEN, 8.0 * (double)mm * batch, 4.0 * sizeof(double) * mm * batch,
-                oa_correction_kernel<<<batch, 512, 0, ctx->stream>>>(A, G.get(), S.get(), w, E.get(), m));
-    LRFG_CUDA(cudaMemcpyAsync(Vn.get(), V, sizeof(double) * mm * batch, cudaMemcpyDeviceToDevice, ctx->stream));
-    gemm(ctx, 0, 0, m, m, m, 1.0, V, m, mm, E.get(), m, mm, 1.0, Vn.get(), m, mm, batch);
-    LRFG_CUDA(cudaMemcpyAsync(V, Vn.get(), sizeof(double) * mm * batch, cudaMemcpyDeviceToDevice, ctx->stream));
-  }
-}
-
-void syevj(lrfg_ctx* ctx, double* A, double* w, double* V, int m, int batch) {
-  if (m <= 0 || batch <= 0) return;
-  jacobi_launch<double>(ctx, A, w, V, m, batch);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -74,16 +74,11 @@ void to_f64(lrfg_ctx* ctx, const float* in, double* out, long long n);
 void gemm_nosplit(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const double* A, int lda,
                   long long sA, const double* B, int ldb, long long sB, double beta, double* C, int ldc, long long sC,
                   int batch = 1);
-// symmetric eigen-decomposition of `batch` m x m matrices (row-major, stride m*m): eigenvalues in
-// descending order into w (stride m), eigenvectors as the COLUMNS of V (row-major m x m, stride m*m).
-// A is left unchanged.  syevj: FP64 Jacobi (absolute accuracy eps64 ||A||).  syevj_mixed: FP32 Jacobi +
-// three FP64 Ogita–Aishima refinement steps; its eigenvectors are accurate only for eigenvalues that
-// FP32 separates (gaps above ~1e-6 ||A||), so it serves the mixed-precision path, not the FP64 one.
-void syevj(lrfg_ctx* ctx, double* A, double* w, double* V, int m, int batch = 1);
-void syevj_mixed(lrfg_ctx* ctx, double* A, double* w, double* V, int m, int batch = 1);
 // FP64 k largest eigenpairs by tridiagonalisation, bisection and inverse iteration: w[0..k) descending,
 // eigenvectors in the first k columns of V (n x n row-major per batch item).  A is left unchanged.
 void syevx(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch = 1);
+// the same with kv >= k eigenvalues in w
+void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int kv, int batch);
 // Top-k left singular pairs of B (n x n per item, nonzero block nA[b] x nB[b]) from BBt = B B^T and
 // BtB = B^T B: the smaller of the two nonzero blocks is decomposed (w = sigma^2); left vectors in the
 // first k columns of V, completed to min(k, nA) orthonormal columns.

@@ -168,9 +168,9 @@ __device__ void trid_solve(int n, const double* dl, const double* dd, const doub
 }
 
 // Gershgorin interval of the tridiagonal (d, e) and the largest e_i^2, by warp 0 (lanes over the rows), left in
-// red[35] (lower end), red[36] (upper end), red[37]; e2 <- e^2 (e2[n-1] = 0).  All threads of the block call it.
-__device__ void trid_gershgorin(const double* d, const double* e, double* e2, int n, double* red) {
-  const int tid = threadIdx.x, nthr = blockDim.x;
+// red[35] (lower end), red[36] (upper end), red[37].  All threads of the block call it.
+__device__ void trid_gershgorin(const double* d, const double* e, int n, double* red) {
+  const int tid = threadIdx.x;
   if (tid < 32) {
     double l0 = INFINITY, h0 = -INFINITY, em = 0.0;
     for (int i = tid; i < n; i += 32) {
@@ -191,8 +191,6 @@ __device__ void trid_gershgorin(const double* d, const double* e, double* e2, in
     }
   }
   __syncthreads();
-  for (int i = tid; i < n; i += nthr) e2[i] = (i < n - 1) ? e[i] * e[i] : 0.0;
-  __syncthreads();
 }
 
 // ---- the decomposition in three launches -----------------------------------------------------------------
@@ -202,12 +200,12 @@ __device__ void trid_gershgorin(const double* d, const double* e, double* e2, in
 // point; inside one block the k eigenvalues shared one SM's FP64 pipe (2 FMA/clk), one warp each they get one
 // SM each, so every lane can take its own point (33-way multisection, about 5 bits per count instead of 2).
 // Per-item global scratch (doubles): a header (active size, Gershgorin interval, largest e_i^2, reduced-problem
-// flag and nA), d, e, beta (nl each), lam (kl), the reflectors W (n x n, leading dimension n), the vectors Y
+// flag and nA), d, e, beta, lam (nl each), the reflectors W (n x n, leading dimension n), the vectors Y
 // (kl x nl, vector-major) and the inverse-iteration LU factors (kl x 5 nl).
 constexpr int kHdr = 8;
 
 static size_t syevx_scratch_per(int nl, int kl) {
-  return kHdr + 3 * (size_t)nl + kl + (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl;
+  return kHdr + 4 * (size_t)nl + (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl;
 }
 
 struct SyevxScratch {
@@ -216,13 +214,12 @@ struct SyevxScratch {
 
 __device__ __forceinline__ SyevxScratch syevx_scratch(double* scratch, int nl, int kl, int item) {
   SyevxScratch g;
-  g.hdr = scratch + (size_t)item * (kHdr + 3 * (size_t)nl + kl + (size_t)nl * nl + (size_t)kl * nl +
-                                    (size_t)kl * 5 * nl);
+  g.hdr = scratch + (size_t)item * (kHdr + 4 * (size_t)nl + (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl);
   g.d = g.hdr + kHdr;
   g.e = g.d + nl;
   g.beta = g.e + nl;
   g.lam = g.beta + nl;
-  g.W = g.lam + kl;
+  g.W = g.lam + nl;
   g.Y = g.W + (size_t)nl * nl;
   g.lu = g.Y + (size_t)kl * nl;
   return g;
@@ -241,15 +238,12 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
                                                                   const double* __restrict__ Bg, double* work) {
   extern __shared__ __align__(16) double sm[];
   double* red = sm;            // 33 (32 partials + the result) + padding
-  double* d = red + 40;        // nl
-  double* e = d + nl;          // nl
-  double* beta = e + nl;       // nl
-  double* pv = beta + nl;      // nl: p / w of the current reflector
+  double* pv = red + 40;       // nl: p / w of the current reflector
   double* vv = pv + nl;        // nl: current reflector v
-  double* e2 = vv + nl;        // nl
   const size_t nnl = (size_t)nl * nl;
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
-  double* W = use_smem ? (e2 + nl) : g.W;
+  double *d = g.d, *e = g.e, *beta = g.beta;  // written once per step by thread 0
+  double* W = use_smem ? (vv + nl) : g.W;
   const int tid = threadIdx.x, nthr = blockDim.x;
   double* wout = wg + (size_t)blockIdx.x * nl;
   double* Vout = Vg + (size_t)blockIdx.x * (size_t)nl * ldv;
@@ -358,16 +352,11 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
   }
   __syncthreads();
 
-  trid_gershgorin(d, e, e2, n, red);
+  trid_gershgorin(d, e, n, red);
   if (tid == 0) {
     g.hdr[1] = red[35];
     g.hdr[2] = red[36];
     g.hdr[3] = red[37];
-  }
-  for (int i = tid; i < n; i += nthr) {
-    g.d[i] = d[i];
-    g.e[i] = e[i];
-    g.beta[i] = beta[i];
   }
   if (use_smem)
     for (size_t t = tid; t < (size_t)n * n; t += nthr) g.W[t] = W[t];
@@ -379,12 +368,12 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
 // scaled by a power of two to |T| in [0.5, 1) (the counts' range window) down to the absolute resolution
 // eps ||T||: the eigenvalues of an FP64 Gram core carry errors of that size, and inverse iteration only needs
 // the shift to that accuracy.
-__global__ void __launch_bounds__(32) syevx_bisect_kernel(int nl, int kl, double* scratch) {
+__global__ void __launch_bounds__(32) syevx_bisect_kernel(int nl, int kl, int kv, double* scratch) {
   extern __shared__ __align__(16) double sm[];
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.y);
   const int n = (int)g.hdr[0];
   const int t = blockIdx.x, lane = threadIdx.x;
-  if (t >= min(kl, n)) return;
+  if (t >= min(kv, n)) return;
   const double lo = g.hdr[1], hi = g.hdr[2], emax2 = g.hdr[3];
   const double tnorm = fmax(fabs(lo), fabs(hi));
   if (tnorm == 0.0) {
@@ -452,15 +441,15 @@ __global__ void __launch_bounds__(32) syevx_bisect_kernel(int nl, int kl, double
 
 // K3.  Eigenvectors of T by inverse iteration (three passes; vectors of eigenvalues closer than 1e-3 ||T||
 // re-orthogonalised after each pass), the back-transformation and the outputs.
-__global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl, double* wg, double* Vg, int ldv,
+__global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl, int kv, double* wg, double* Vg, int ldv,
                                                                   double* scratch, int smem_flags,
                                                                   const double* __restrict__ Bg) {
   extern __shared__ __align__(16) double sm[];
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
   const int n = (int)g.hdr[0];
   if (n == 0) return;
-  double* red = sm;            // 40
-  double* d = red + 40;        // nl
+  // flag 8: the tridiagonal, the reflector scalars and the eigenvalues in shared memory too
+  double* d = sm;              // nl
   double* e = d + nl;          // nl
   double* beta = e + nl;       // nl
   double* lam = beta + nl;     // kl
@@ -469,7 +458,15 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   // strides in shared memory are odd numbers of doubles, so that the lanes of a warp walking different vectors
   // (inverse iteration: one lane per vector) or different rows (the warp sums) hit different banks
   const int npad = nl | 1;
-  double* next = lam + kl;
+  double* next = sm;
+  if (smem_flags & 8) {
+    next = lam + kl;
+  } else {
+    d = g.d;
+    e = g.e;
+    beta = g.beta;
+    lam = g.lam;
+  }
   double* Y = g.Y;
   double* lu = g.lu;
   double* W = g.W;
@@ -487,12 +484,14 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   const int wld = (smem_flags & 4) ? npad : n;       // leading dimension of the reflectors
   double* wout = wg + (size_t)blockIdx.x * nl;
   double* Vout = Vg + (size_t)blockIdx.x * (size_t)nl * ldv;
-  for (int i = tid; i < n; i += nthr) {
-    d[i] = g.d[i];
-    e[i] = g.e[i];
-    beta[i] = g.beta[i];
+  if (smem_flags & 8) {
+    for (int i = tid; i < n; i += nthr) {
+      d[i] = g.d[i];
+      e[i] = g.e[i];
+      beta[i] = g.beta[i];
+    }
+    for (int t = tid; t < k; t += nthr) lam[t] = g.lam[t];
   }
-  for (int t = tid; t < k; t += nthr) lam[t] = g.lam[t];
   if (smem_flags & 4)
     for (size_t t = tid; t < (size_t)n * n; t += nthr) W[(t / n) * wld + t % n] = g.W[t];
   __syncthreads();
@@ -592,7 +591,7 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   __syncthreads();
 
   // outputs: eigenvalues descending, eigenvectors as the first k columns of V (leading dimension ldv)
-  for (int t = tid; t < k; t += nthr) wout[t] = lam[t];
+  for (int t = tid; t < min(kv, n); t += nthr) wout[t] = t < k ? lam[t] : g.lam[t];
   if (!viaB) {
     for (size_t q = tid; q < (size_t)k * n; q += nthr) {
       int t = (int)(q / n), i = (int)(q - (q / n) * n);
@@ -657,16 +656,18 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
 }
 
 
+// k eigenvectors and kv >= k eigenvalues of every item
 static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch,
-                         const int* nA, const int* nB, const double* A2, const double* B) {
+                         const int* nA, const int* nB, const double* A2, const double* B, int kv = 0) {
   if (n <= 0 || batch <= 0 || k <= 0) return;
   k = std::min(k, n);
-  LRFG_REQUIRE(k < 65536 && batch < 65536, "eigensolver grid too large (k = %d, batch = %d)", k, batch);
+  kv = std::min(n, std::max(k, kv));
+  LRFG_REQUIRE(kv < 65536 && batch < 65536, "eigensolver grid too large (k = %d, batch = %d)", k, batch);
   DBuf<double> scratch(ctx->pool, syevx_scratch_per(n, k) * batch);
   const size_t lim = (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
   const size_t wbytes = sizeof(double) * (size_t)n * n;
   // K1: the reflectors in shared memory when they fit
-  const size_t head1 = sizeof(double) * (40 + 6 * (size_t)n);
+  const size_t head1 = sizeof(double) * (40 + 2 * (size_t)n);
   const int smem_w1 = head1 + wbytes <= lim ? 1 : 0;
   const size_t smem1 = head1 + (smem_w1 ? wbytes : 0);
   LRFG_CUDA(raise_smem_limit((const void*)syevx_tri_kernel, smem1));
@@ -679,11 +680,12 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
   const size_t smem2 = sizeof(double) * 3 * (size_t)n;
   LRFG_CUDA(raise_smem_limit((const void*)syevx_bisect_kernel, smem2));
   LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
-              syevx_bisect_kernel<<<dim3((unsigned)k, (unsigned)batch), 32, smem2, ctx->stream>>>(n, k,
-                                                                                                scratch.get()));
+              syevx_bisect_kernel<<<dim3((unsigned)kv, (unsigned)batch), 32, smem2, ctx->stream>>>(n, k, kv,
+                                                                                                 scratch.get()));
   // K3: the vectors, then their LU factors, then the reflectors in shared memory while they fit
-  size_t smem3 = sizeof(double) * (40 + 3 * (size_t)n + (size_t)k);
-  int flags3 = 0;
+  const size_t head3 = sizeof(double) * (3 * (size_t)n + (size_t)k);
+  int flags3 = head3 <= lim ? 8 : 0;
+  size_t smem3 = flags3 ? head3 : 0;
   const size_t npad = (size_t)(n | 1);  // K3's odd shared-memory strides
   const size_t parts[3] = {sizeof(double) * (size_t)k * npad, sizeof(double) * (size_t)k * 5 * npad,
                            sizeof(double) * (size_t)n * npad};
@@ -694,12 +696,16 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
     }
   LRFG_CUDA(raise_smem_limit((const void*)syevx_vec_kernel, smem3));
   LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
-              syevx_vec_kernel<<<batch, kSyevxThreads, smem3, ctx->stream>>>(n, k, w, V, n, scratch.get(), flags3,
-                                                                             B));
+              syevx_vec_kernel<<<batch, kSyevxThreads, smem3, ctx->stream>>>(n, k, kv, w, V, n, scratch.get(),
+                                                                             flags3, B));
 }
 
 void syevx(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch) {
   syevx_launch(ctx, A, w, V, n, k, batch, nullptr, nullptr, nullptr, nullptr);
+}
+
+void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int kv, int batch) {
+  syevx_launch(ctx, A, w, V, n, k, batch, nullptr, nullptr, nullptr, nullptr, kv);
 }
 
 void syevx_sized(lrfg_ctx* ctx, const double* A, const int* n_eff, double* w, double* V, int n, int k, int batch) {
