@@ -381,17 +381,45 @@ static bool fft2_try(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N,
   }
 }
 
+// Rows of a transform tile when the largest tile (tf_max rows) leaves the SMs unevenly filled.  The passes are bound by
+// the FP64 pipe, which an SM's blocks share and which a warp instruction holds however many of its lanes work, so a
+// launch takes as long as its busiest SM: blocks per SM x warps of butterflies per pass.  The tile with the smallest
+// such count is taken, the larger one on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid in 32-row tiles ran
+// on one or two SMs (46 us per fibre pass and 88 us per fused row pass under event timing; spread over 11 to 32 SMs 20
+// and 34 us), 63^3 with its Ga double grid 125^3 gained 19%; from six blocks per SM on the rounding up costs less than the shorter memory segments of a smaller tile, and tf_max stays.
+int balanced_tile(lrfg_ctx* ctx, const FftPlan& pl, int tf_max, long long nrows) {
+  const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
+  if ((nrows + tf_max - 1) / tf_max >= 6 * nsm) return tf_max;
+  int best = tf_max;
+  double best_cost = 0.0;
+  for (int tf = tf_max; tf >= 1; --tf) {
+    const long long blocks = (nrows + tf - 1) / tf;
+    double warps = 0.0;
+    for (int s = 0; s < pl.nst; ++s) {
+      const int p = pl.radix[s];
+      warps += (double)((tf * (long long)(pl.N / p) + 31) / 32) * p * std::log2((double)p + 1.0);
+    }
+    const double cost = (double)((blocks + nsm - 1) / nsm) * warps;
+    if (tf == tf_max || cost < 0.98 * best_cost) {
+      best_cost = cost;
+      best = tf;
+    }
+  }
+  return best;
+}
+
 // Tile for the complex fibre FFT: whole 128-byte segments along the contiguous index (TF * sizeof(V) >=
 // 128) and at most 72 KB of shared memory, so that three blocks share an SM and one block's transform
-// overlaps the others' loads and stores.
-static int tile_complex(lrfg_ctx* ctx, int N, size_t elem, size_t* smem_out) {
-  const long long row = (long long)N * (long long)elem;
+// overlaps the others' loads and stores; fewer fibres where that fills the SMs more evenly.
+static int tile_complex(lrfg_ctx* ctx, const FftPlan& pl, size_t elem, long long nfib, size_t* smem_out) {
+  const long long row = (long long)pl.N * (long long)elem;
   long long limit = 72 * 1024;
   const long long tf_min = std::max<long long>(1, 128 / (long long)elem);
   if (2 * row + 2 * tf_min * row > limit) limit = std::min<long long>(ctx->max_smem_optin, 200 * 1024);
   long long tf = (limit - 2 * row) / (2 * row);
   tf = std::max<long long>(1, std::min<long long>(tf, 32));
   if (tf > tf_min) tf = (tf / tf_min) * tf_min;
+  tf = balanced_tile(ctx, pl, (int)tf, nfib);
   *smem_out = (size_t)(2 * row + 2 * tf * row);
   return (int)tf;
 }
@@ -405,8 +433,8 @@ void fft_fibres(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N, long
   FftPlan pl = make_plan(N, plan_radix<V>());
   const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
-  int TF = tile_complex(ctx, N, sizeof(V), &smem);
   long long nfib = outer * inner;
+  int TF = tile_complex(ctx, pl, sizeof(V), nfib, &smem);
   long long blocks = (nfib + TF - 1) / TF;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   const double flops = 5.0 * N * std::log2((double)N) * (double)nfib;   // radix-2-equivalent count
@@ -443,7 +471,7 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, int N0, long long inner,
   FftPlan pl = make_plan(N0, plan_radix<V>());
   const V* W = twiddle_table<R>(ctx, N0);
   size_t smem;
-  int TF = tile_complex(ctx, N0, sizeof(V), &smem);
+  int TF = tile_complex(ctx, pl, sizeof(V), inner, &smem);
   long long blocks = (inner + TF - 1) / TF;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   const double n_el = (double)N0 * (double)inner;
