@@ -850,56 +850,100 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x) {
   s = t;
 }
 
+// weighted partial inner products of one thread (weight w = 1 or 2), see above
+template <typename V>
+struct DotAcc;
+template <>
+struct DotAcc<double2> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double2 a, double2 b, int kl) {
+    s += (kl == 0 ? 1.0 : 2.0) * (a.x * b.x + a.y * b.y);
+  }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct DotAcc<float2> {
+  float fs = 0.0f, fc = 0.0f;
+  __device__ __forceinline__ void add(float2 a, float2 b, int kl) {
+    const float w = kl == 0 ? 1.0f : 2.0f;
+    const float p1 = a.x * b.x, e1 = fmaf(a.x, b.x, -p1);
+    const float p2 = a.y * b.y, e2 = fmaf(a.y, b.y, -p2);
+    two_sum_acc(fs, fc, w * p1);
+    two_sum_acc(fs, fc, w * p2);
+    fc += w * (e1 + e2);
+  }
+  __device__ __forceinline__ double value() const { return (double)fs + (double)fc; }
+};
+
+__device__ __forceinline__ double block_sum256(double s, double* red) {
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double v = 0.0;
+  for (int i = 0; i < 8; ++i) v += red[i];
+  return v;
+}
+
+// Stores this block's NV partial sums and returns true in the last block of the launch to arrive, whose every thread
+// then holds the totals, summed in block order: the same bits whichever block arrives last.  The counter is zero
+// between launches.  It replaces a second launch for the partials (8 us under event timing, three a CG step).
+template <int NV>
+__device__ bool last_block_sum(const double* mine, double* partial, unsigned int* counter, double* red, double* total) {
+  __shared__ unsigned int s_last;
+  if (threadIdx.x == 0) {
+    for (int v = 0; v < NV; ++v) partial[(size_t)v * gridDim.x + blockIdx.x] = mine[v];
+    __threadfence();
+    s_last = atomicAdd(counter, 1u) == gridDim.x - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  for (int v = 0; v < NV; ++v) {
+    double s = 0.0;
+    for (unsigned int t = threadIdx.x; t < gridDim.x; t += 256) s += __ldcg(partial + (size_t)v * gridDim.x + t);
+    total[v] = block_sum256(s, red);
+  }
+  if (threadIdx.x == 0) *counter = 0u;
+  return true;
+}
+
+// *out = <x, y>; then, if ratio: mode 1 -> *ratio = *aux / *out, mode 2 -> *out / *aux (0 when the divisor is 0): the
+// PCG step lengths, formed once on the device
 template <typename V>
 __global__ void __launch_bounds__(256) half_dot_kernel(const V* __restrict__ x, const V* __restrict__ y, long long n,
-                                                       int H, double* partial) {
+                                                       int H, double* partial, unsigned int* counter, double* out,
+                                                       const double* aux, double* ratio, int mode) {
   __shared__ double red[8];
-  double s = 0.0;
+  constexpr int kU = 4;  // elements' loads in flight before any is used
+  DotAcc<V> acc;
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   int kl = (int)(t % H);
   const int kstep = (int)(stride % H);
-  if constexpr (sizeof(V) == sizeof(float2)) {
-    // four elements' loads in flight before any is used
-    constexpr int kU = 4;
-    float fs = 0.0f, fc = 0.0f;
-    for (; t < n; t += kU * stride) {
-      V a[kU], b[kU];
+  for (; t < n; t += kU * stride) {
+    V a[kU], b[kU];
 #pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const long long tu = t + u * stride;
-        a[u] = tu < n ? x[tu] : mkc<V>(0.0f, 0.0f);
-        b[u] = tu < n ? y[tu] : mkc<V>(0.0f, 0.0f);
-      }
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const float w = kl == 0 ? 1.0f : 2.0f;
-        const float p1 = a[u].x * b[u].x, e1 = fmaf(a[u].x, b[u].x, -p1);
-        const float p2 = a[u].y * b[u].y, e2 = fmaf(a[u].y, b[u].y, -p2);
-        two_sum_acc(fs, fc, w * p1);
-        two_sum_acc(fs, fc, w * p2);
-        fc += w * (e1 + e2);
-        kl += kstep;
-        if (kl >= H) kl -= H;
-      }
+    for (int u = 0; u < kU; ++u) {
+      const long long tu = t + u * stride;
+      a[u] = tu < n ? x[tu] : mkc<V>(0, 0);
+      b[u] = tu < n ? y[tu] : mkc<V>(0, 0);
     }
-    s = (double)fs + (double)fc;
-  } else {
-    for (; t < n; t += stride) {
-      const V a = x[t], b = y[t];
-      const double w = kl == 0 ? 1.0 : 2.0;
-      s += w * ((double)a.x * (double)b.x + (double)a.y * (double)b.y);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      acc.add(a[u], b[u], kl);
       kl += kstep;
       if (kl >= H) kl -= H;
     }
   }
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
+  double mine[1] = {block_sum256(acc.value(), red)}, total[1];
+  if (!last_block_sum<1>(mine, partial, counter, red, total)) return;
   if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int i = 0; i < 8; ++i) v += red[i];
-    partial[blockIdx.x] = v;
+    *out = total[0];
+    if (ratio) {
+      const double num = mode == 1 ? *aux : total[0], den = mode == 1 ? total[0] : *aux;
+      *ratio = den != 0.0 ? num / den : 0.0;
+    }
   }
 }
 
@@ -955,36 +999,26 @@ __global__ void __launch_bounds__(256) aniso_energy_kernel(const double2* __rest
   }
 }
 
-// *out (+)= sum of partials; then, if ratio: mode 1 -> *ratio = *aux / *out, mode 2 -> *out / *aux
-// (0 when the divisor is 0): the PCG step lengths, formed once on the device
-__global__ void finish_sum_kernel(const double* __restrict__ partial, int n, double* out, int accumulate,
-                                  const double* aux, double* ratio, int mode) {
+// *out (+)= sum of partials
+__global__ void finish_sum_kernel(const double* __restrict__ partial, int n, double* out, int accumulate) {
   __shared__ double red[8];
   double s = 0.0;
   for (int t = threadIdx.x; t < n; t += blockDim.x) s += partial[t];
-  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int i = 0; i < 8; ++i) v += red[i];
-    v = accumulate ? *out + v : v;
-    *out = v;
-    if (ratio) {
-      const double num = mode == 1 ? *aux : v, den = mode == 1 ? v : *aux;
-      *ratio = den != 0.0 ? num / den : 0.0;
-    }
-  }
+  const double v = block_sum256(s, red);
+  if (threadIdx.x == 0) *out = accumulate ? *out + v : v;
 }
+
+// blocks of a reduction over n elements: four elements a thread, at most eight blocks per SM
+static int red_blocks(long long n) { return (int)std::max(1LL, std::min<long long>(kRedBlocks, (n + 1023) / 1024)); }
 
 template <typename V>
 void half_dot(lrfg_ctx* ctx, const FullGrid& g, const V* x, const V* y, double* out_dev, const double* aux,
               double* ratio, int mode) {
+  const int blocks = red_blocks(g.n_half);
   DBuf<double> partial(ctx->pool, kRedBlocks);
   LRFG_LAUNCH(ctx, KC_REDUCE, 4.0 * g.n_half, 2.0 * sizeof(V) * g.n_half,
-              half_dot_kernel<V><<<kRedBlocks, 256, 0, ctx->stream>>>(x, y, g.n_half, g.H, partial.get()));
-  LRFG_LAUNCH(ctx, KC_REDUCE, kRedBlocks, kRedBlocks * sizeof(double),
-              finish_sum_kernel<<<1, 256, 0, ctx->stream>>>(partial.get(), kRedBlocks, out_dev, 0, aux, ratio, mode));
+              half_dot_kernel<V><<<blocks, 256, 0, ctx->stream>>>(x, y, g.n_half, g.H, partial.get(), ctx->splitk_cnt,
+                                                                 out_dev, aux, ratio, mode));
 }
 
 void aniso_energy_sum(lrfg_ctx* ctx, const FullGrid& g, const double2* v, const double* B, double* out_dev,
@@ -996,8 +1030,7 @@ void aniso_energy_sum(lrfg_ctx* ctx, const FullGrid& g, const double2* v, const 
                                                                          g.d == 3 ? g.N[1] : 1, sym_b<double>(B, c),
                                                                          partial.get()));
   LRFG_LAUNCH(ctx, KC_REDUCE, kRedBlocks, kRedBlocks * sizeof(double),
-              finish_sum_kernel<<<1, 256, 0, ctx->stream>>>(partial.get(), kRedBlocks, out_dev, accumulate, nullptr,
-                                                            nullptr, 0));
+              finish_sum_kernel<<<1, 256, 0, ctx->stream>>>(partial.get(), kRedBlocks, out_dev, accumulate));
 }
 
 template <typename R>
@@ -1006,57 +1039,155 @@ void energy_sum(lrfg_ctx* ctx, const FullGrid& g, const R* e, const R* a, double
   LRFG_LAUNCH(ctx, KC_REDUCE, 4.0 * g.n_real, 2.0 * sizeof(R) * g.n_real,
               energy_kernel<R><<<kRedBlocks, 256, 0, ctx->stream>>>(e, a, E, g.n_real, partial.get()));
   LRFG_LAUNCH(ctx, KC_REDUCE, kRedBlocks, kRedBlocks * sizeof(double),
-              finish_sum_kernel<<<1, 256, 0, ctx->stream>>>(partial.get(), kRedBlocks, out_dev, accumulate, nullptr,
-                                                            nullptr, 0));
+              finish_sum_kernel<<<1, 256, 0, ctx->stream>>>(partial.get(), kRedBlocks, out_dev, accumulate));
 }
 
 // ------------------------------------------------------------------------------------------------
-// PCG vector updates with a device FP64 step length (rounded once to R)
+// PCG vector updates with device FP64 step lengths (rounded once to R).  Two passes a step, both bound by memory:
+//   residual   r -= alpha q, and the inner products <z, z> and <r, z> of z = P^-1 r, which is not stored (its multiplier
+//              costs one reciprocal per element); the last block forms beta;
+//   direction  u += alpha p and p = P^-1 r + beta p.
+// 10 vector transfers a step with the product <p, q> (2 + 3 + 5) where separate updates, products and directions took
+// 15; on 243^3 in FP32 the vector part of a step went from 0.186 to 0.133 ms (the products' error-free sums bound the rest).
 // ------------------------------------------------------------------------------------------------
+// 1/(k.k): FP32 forms the correctly rounded reciprocal (the value of the table) without the table's scattered gather
+__device__ __forceinline__ float inv_kk_of(const float*, int kk) { return kk ? __frcp_rn((float)kk) : 0.f; }
+__device__ __forceinline__ double inv_kk_of(const double* t, int kk) { return t[kk]; }
+
+// frequencies of consecutive elements of a strided walk over the half spectrum, without a division per element
+struct FreqWalk {
+  int kl, i0, i1, H, N0, N1, dkl, d0, d1, d;
+  __device__ FreqWalk(const RowMap& m, long long t, long long stride) : H(m.H), N0(m.N0), N1(m.N1), d(m.d) {
+    long long row = t / H;
+    kl = (int)(t - row * H);
+    i0 = (int)(row / N1);
+    i1 = (int)(row - (long long)i0 * N1);
+    row = stride / H;
+    dkl = (int)(stride - row * H);
+    d0 = (int)(row / N1);
+    d1 = (int)(row - (long long)d0 * N1);
+  }
+  __device__ __forceinline__ int kk() const {
+    const int k0 = freq_of(i0, N0), k1 = d == 3 ? freq_of(i1, N1) : 0;
+    return k0 * k0 + k1 * k1 + kl * kl;
+  }
+  __device__ __forceinline__ void next() {
+    kl += dkl;
+    i1 += d1;
+    i0 += d0;
+    if (kl >= H) { kl -= H; ++i1; }
+    if (i1 >= N1) { i1 -= N1; ++i0; }
+  }
+};
+
 template <typename V>
-__global__ void pcg_update_kernel(V* u, V* r, const V* __restrict__ p, const V* __restrict__ q, V* z, RowMap m,
-                                  const double* __restrict__ alpha_dev,
-                                  const typename RealOf<V>::T* __restrict__ inv_kk) {
+__global__ void __launch_bounds__(256) pcg_residual_kernel(V* r, const V* __restrict__ q, long long n, RowMap m,
+                                                           const double* __restrict__ alpha_dev,
+                                                           const typename RealOf<V>::T* __restrict__ inv_kk,
+                                                           double* partial, unsigned int* counter, double* rz,
+                                                           double* zz, double* beta) {
   using R = typename RealOf<V>::T;
-  int k[3];
-  size_t t;
-  if (!row_k(m, k[0], k[1], k[2], t)) return;
+  __shared__ double red[8];
+  constexpr int kU = 4;
   const R alpha = (R)(*alpha_dev);
-  V pv = p[t], qv = q[t], uv = u[t], rv = r[t];
-  uv.x += alpha * pv.x;
-  uv.y += alpha * pv.y;
-  rv.x -= alpha * qv.x;
-  rv.y -= alpha * qv.y;
-  u[t] = uv;
-  r[t] = rv;
-  const R s = inv_kk[k[0] * k[0] + k[1] * k[1] + k[2] * k[2]];
-  z[t] = mkc<V>(rv.x * s, rv.y * s);
+  DotAcc<V> azz, arz;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  FreqWalk w(m, t, stride);
+  for (; t < n; t += kU * stride) {
+    V rv[kU], qv[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const long long tu = t + u * stride;
+      rv[u] = tu < n ? r[tu] : mkc<V>(0, 0);
+      qv[u] = tu < n ? q[tu] : mkc<V>(0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const long long tu = t + u * stride;
+      if (tu < n) {
+        rv[u].x -= alpha * qv[u].x;
+        rv[u].y -= alpha * qv[u].y;
+        r[tu] = rv[u];
+        const R s = inv_kk_of(inv_kk, w.kk());
+        const V z = mkc<V>(rv[u].x * s, rv[u].y * s);
+        azz.add(z, z, w.kl);
+        arz.add(rv[u], z, w.kl);
+      }
+      w.next();
+    }
+  }
+  double mine[2], total[2];
+  mine[0] = block_sum256(azz.value(), red);
+  mine[1] = block_sum256(arz.value(), red);
+  if (!last_block_sum<2>(mine, partial, counter, red, total)) return;
+  if (threadIdx.x == 0) {
+    *zz = total[0];
+    *beta = *rz != 0.0 ? total[1] / *rz : 0.0;
+    *rz = total[1];
+  }
 }
 
-// p = z + beta p
+// u += alpha p, then (unless `last`) p = P^-1 r + beta p
 template <typename V>
-__global__ void pcg_direction_kernel(V* p, const V* __restrict__ z, long long n, const double* __restrict__ beta_dev) {
+__global__ void __launch_bounds__(256) pcg_direction_kernel(V* u, V* p, const V* __restrict__ r, long long n, RowMap m,
+                                                            const double* __restrict__ alpha_dev,
+                                                            const double* __restrict__ beta_dev,
+                                                            const typename RealOf<V>::T* __restrict__ inv_kk, int last) {
   using R = typename RealOf<V>::T;
-  const R beta = (R)(*beta_dev);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    V pv = p[t], zv = z[t];
-    p[t] = mkc<V>(zv.x + beta * pv.x, zv.y + beta * pv.y);
+  constexpr int kU = 2;
+  const R alpha = (R)(*alpha_dev), beta = last ? R(0) : (R)(*beta_dev);
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  FreqWalk w(m, t, stride);
+  for (; t < n; t += kU * stride) {
+    V uv[kU], pv[kU], rv[kU];
+#pragma unroll
+    for (int v = 0; v < kU; ++v) {
+      const long long tu = t + v * stride;
+      uv[v] = tu < n ? u[tu] : mkc<V>(0, 0);
+      pv[v] = tu < n ? p[tu] : mkc<V>(0, 0);
+      rv[v] = tu < n && !last ? r[tu] : mkc<V>(0, 0);
+    }
+#pragma unroll
+    for (int v = 0; v < kU; ++v) {
+      const long long tu = t + v * stride;
+      if (tu < n) {
+        uv[v].x += alpha * pv[v].x;
+        uv[v].y += alpha * pv[v].y;
+        u[tu] = uv[v];
+        if (!last) {
+          const R s = inv_kk_of(inv_kk, w.kk());
+          p[tu] = mkc<V>(rv[v].x * s + beta * pv[v].x, rv[v].y * s + beta * pv[v].y);
+        }
+      }
+      w.next();
+    }
   }
 }
 
 template <typename V>
-void pcg_update(lrfg_ctx* ctx, const FullGrid& g, V* u, V* r, const V* p, const V* q, V* z, const double* alpha) {
+void pcg_residual(lrfg_ctx* ctx, const FullGrid& g, V* r, const V* q, const double* alpha, double* rz, double* zz,
+                  double* beta) {
   using R = typename RealOf<V>::T;
   LRFG_REQUIRE(inv_table<R>(g), "reciprocal table missing");
-  LRFG_LAUNCH(ctx, KC_POINTWISE, 10.0 * g.n_half, 7.0 * sizeof(V) * g.n_half,
-              pcg_update_kernel<V><<<row_grid(g), row_block(g), 0, ctx->stream>>>(u, r, p, q, z, rowmap(g), alpha,
-                                                                                  inv_table<R>(g)));
+  const int blocks = red_blocks(g.n_half);
+  DBuf<double> partial(ctx->pool, 2 * kRedBlocks);
+  LRFG_LAUNCH(ctx, KC_POINTWISE, 14.0 * g.n_half, 3.0 * sizeof(V) * g.n_half,
+              pcg_residual_kernel<V><<<blocks, 256, 0, ctx->stream>>>(r, q, g.n_half, rowmap(g), alpha, inv_table<R>(g),
+                                                                     partial.get(), ctx->splitk_cnt, rz, zz, beta));
 }
 
 template <typename V>
-void pcg_direction(lrfg_ctx* ctx, const FullGrid& g, V* p, const V* z, const double* beta) {
-  LRFG_LAUNCH(ctx, KC_POINTWISE, 4.0 * g.n_half, 3.0 * sizeof(V) * g.n_half,
-              pcg_direction_kernel<V><<<grid1d(ctx, g.n_half), 256, 0, ctx->stream>>>(p, z, g.n_half, beta));
+void pcg_direction(lrfg_ctx* ctx, const FullGrid& g, V* u, V* p, const V* r, const double* alpha, const double* beta,
+                   bool last) {
+  using R = typename RealOf<V>::T;
+  LRFG_REQUIRE(inv_table<R>(g), "reciprocal table missing");
+  const long long cap = 16LL * (ctx->num_sms > 0 ? ctx->num_sms : 152);
+  const unsigned blocks = (unsigned)std::max(1LL, std::min<long long>(cap, (g.n_half + 511) / 512));
+  LRFG_LAUNCH(ctx, KC_POINTWISE, (last ? 4.0 : 10.0) * g.n_half, (last ? 3.0 : 5.0) * sizeof(V) * g.n_half,
+              pcg_direction_kernel<V><<<blocks, 256, 0, ctx->stream>>>(u, p, r, g.n_half, rowmap(g), alpha, beta,
+                                                                      inv_table<R>(g), last ? 1 : 0));
 }
 
 // element-wise conversions between storage precisions (round to nearest)
@@ -1085,8 +1216,8 @@ void convert(lrfg_ctx* ctx, const A* in, B* out, long long n) {
   template void half_acc_aniso<V>(lrfg_ctx*, const FullGrid&, const V*, V*, const double*, int);          \
   template void half_dot<V>(lrfg_ctx*, const FullGrid&, const V*, const V*, double*, const double*, double*, int); \
   template void energy_sum<R>(lrfg_ctx*, const FullGrid&, const R*, const R*, double, double*, int);      \
-  template void pcg_update<V>(lrfg_ctx*, const FullGrid&, V*, V*, const V*, const V*, V*, const double*);  \
-  template void pcg_direction<V>(lrfg_ctx*, const FullGrid&, V*, const V*, const double*);
+  template void pcg_residual<V>(lrfg_ctx*, const FullGrid&, V*, const V*, const double*, double*, double*, double*); \
+  template void pcg_direction<V>(lrfg_ctx*, const FullGrid&, V*, V*, const V*, const double*, const double*, bool);
 LRFG_FULL_INSTANTIATE(double2, double)
 LRFG_FULL_INSTANTIATE(float2, float)
 template void convert<double, float>(lrfg_ctx*, const double*, float*, long long);

@@ -64,12 +64,14 @@ void half_dot(lrfg_ctx* ctx, const FullGrid& g, const V* x, const V* y, double* 
 // out_dev (+)= sum_k a_k (E + e_k)^2 (FP64 accumulation)
 template <typename R>
 void energy_sum(lrfg_ctx* ctx, const FullGrid& g, const R* e, const R* a, double E, double* out_dev, int accumulate);
-// u += alpha p, r -= alpha q, z = P^-1 r (alpha a device scalar)
+// r -= alpha q; *zz = <z, z>, *beta = <r, z> / *rz, *rz = <r, z> for z = P^-1 r (device scalars)
 template <typename V>
-void pcg_update(lrfg_ctx* ctx, const FullGrid& g, V* u, V* r, const V* p, const V* q, V* z, const double* alpha);
-// p = z + beta p (beta a device scalar)
+void pcg_residual(lrfg_ctx* ctx, const FullGrid& g, V* r, const V* q, const double* alpha, double* rz, double* zz,
+                  double* beta);
+// u += alpha p, then (unless last) p = P^-1 r + beta p (device scalars)
 template <typename V>
-void pcg_direction(lrfg_ctx* ctx, const FullGrid& g, V* p, const V* z, const double* beta);
+void pcg_direction(lrfg_ctx* ctx, const FullGrid& g, V* u, V* p, const V* r, const double* alpha, const double* beta,
+                   bool last);
 template <typename A, typename B>
 void convert(lrfg_ctx* ctx, const A* in, B* out, long long n);
 // Ga (exact integration on the double grid gM, M = 2N - 1 per axis): zero padding I of a half spectrum of
