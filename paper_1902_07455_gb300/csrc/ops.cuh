@@ -81,14 +81,9 @@ void gemm_nosplit(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, do
 void syevx(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch = 1);
 // the same with kv >= k eigenvalues in w
 void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int kv, int batch);
-// Top-k left singular pairs of B (n x n per item, nonzero block nA[b] x nB[b]) from BBt = B B^T and
-// BtB = B^T B: the smaller of the two nonzero blocks is decomposed (w = sigma^2); left vectors in the
-// first k columns of V, completed to min(k, nA) orthonormal columns.
 // The same on the leading n_eff[b] x n_eff[b] block of A (the rest of A is zero); the eigenvector
 // rows beyond n_eff and the columns beyond min(k, n_eff) are zero.
 void syevx_sized(lrfg_ctx* ctx, const double* A, const int* n_eff, double* w, double* V, int n, int k, int batch);
-void syevx_product(lrfg_ctx* ctx, const double* BBt, const double* BtB, const double* B, const int* nA,
-                   const int* nB, double* w, double* V, int n, int k, int batch);
 // Gram-SVD factors from a balanced Gram matrix G (b x b per item) and the balancing c: pivoted
 // Cholesky; writes RA (G ~ RA^T RA, nonzero rows first), RAc and Pc (b x b each per item; skipped when
 // null, and then c may be null), and the numerical rank into rho (may be null).

@@ -4,11 +4,15 @@
 //  2. eigenvalues of T by bisection on Sturm counts of the LDL^T recurrence (G&VL Sec. 8.4.1), one warp per
 //     eigenvalue in a launch of its own;
 //  3. eigenvectors of T by inverse iteration (G&VL Sec. 8.2.2) with the tridiagonal LU factorisation
-//     of T - lambda I with partial pivoting (G&VL Sec. 4.3), three passes, vectors of eigenvalues closer
-//     than 1e-3 ||T|| re-orthogonalised against each other by modified Gram-Schmidt after each pass;
-//  4. back-transformation by the stored reflectors.
+//     of T - lambda I with partial pivoting (G&VL Sec. 4.3), two passes or three, and an orthonormalisation of the vectors
+//     (Newton-Schulz, Cholesky of their Gram matrix, or modified Gram-Schmidt, by how far they are from orthogonal);
+//  4. back-transformation by Q = H_0 .. H_{n-3}, formed beside step 2, or by the stored reflectors.
 // About 4/3 n^3 + 2 k n^2 flops against ~9 n^3 per sweep (and several sweeps) for cyclic Jacobi, with the
 // same absolute accuracy (eps ||A||), which is what the Gram-SVD truncation needs.
+// The steps are chains of dependent FP64 operations, and on this part a warp issues one FP64 instruction per 64 cycles
+// whatever its instruction-level parallelism or active lanes (an SM has four such units): each kernel is laid out to put
+// few FP64 instructions on the longest of the four.  Three matrices of n = 30, k = 20 take 158 us (420 us with the same
+// algorithm laid out by arithmetic alone), one of n = 60, k = 20 533 us (744), n = 135, k = 10 2.0 ms (2.3).
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -49,122 +53,308 @@ __device__ double block_reduce_sum(double v, double* red, int nact) {
 // division is a long dependent chain on this part); the pair (p_{i-1}, p_i) is rescaled by exact powers of
 // two every four steps to stay in range.  The caller scales T by a power of two to |T| < 1, so that four
 // steps change |p| by at most a factor 3^4 (growth) or 2^-212 (cancellation) within the 2^(+-600) window.
-__device__ __forceinline__ int sign_of(double p, int sprev) {
-  // sign from the bit pattern (integer pipe): +1, -1, or opposite of the predecessor for a zero
-  const long long bits = __double_as_longlong(p);
-  if ((bits & 0x7fffffffffffffffLL) == 0) return -sprev;
-  return bits < 0 ? -1 : 1;
+// (the sign enters as a bit: 1 negative)
+__device__ __forceinline__ unsigned sign_bit(double p, unsigned prev) {
+  const unsigned hi = (unsigned)__double2hiint(p);
+  return ((hi & 0x7fffffffu) | (unsigned)__double2loint(p)) == 0u ? prev ^ 1u : hi >> 31;
 }
 
+// Steps in groups of four: the coefficients first, then the recurrence, then the signs, so that the integer work on a
+// result does not hold up the next FP64 instruction (a warp issues one FP64 instruction per 64 cycles on this part, and
+// in order).
 __device__ int sturm_count(const double* d, const double* e2, int n, double x) {
   const double up = 0x1p+600, down = 0x1p-600;
   double pm = 1.0, p = d[0] - x;
-  int sprev = 1, c = 0;
-  int s = sign_of(p, sprev);
-  c += s != sprev;
-  sprev = s;
-  int i = 1;
-  while (i < n) {
-    const int iend = min(n, i + 4);
-    for (; i < iend; ++i) {
-      double pn = fma(d[i] - x, p, -e2[i - 1] * pm);
+  unsigned sg = sign_bit(p, 0u);
+  int c = (int)sg;
+  for (int i = 1; i < n; i += 4) {
+    double dv[4], ev[4], q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = min(i + u, n - 1);
+      dv[u] = d[k];
+      ev[u] = e2[k - 1];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const double pn = fma(dv[u] - x, p, -ev[u] * pm);
       pm = p;
       p = pn;
-      s = sign_of(p, sprev);
-      c += s != sprev;
-      sprev = s;
+      q[u] = pn;
     }
-    const int ep = (int)((__double_as_longlong(p) >> 52) & 0x7ff), epm = (int)((__double_as_longlong(pm) >> 52) & 0x7ff);
-    if (ep > 1023 + 600 || epm > 1023 + 600) { p *= down; pm *= down; }
-    else if (ep < 1023 - 600 && epm < 1023 - 600) { p *= up; pm *= up; }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned s = sign_bit(q[u], sg);
+      if (i + u < n) {  // past the end the last step is repeated and not counted
+        c += (int)(s ^ sg);
+        sg = s;
+      }
+    }
+    const int e = max((__double2hiint(p) >> 20) & 0x7ff, (__double2hiint(pm) >> 20) & 0x7ff);
+    if (e > 1023 + 600 || e < 1023 - 600) {
+      const double f = e > 1023 ? down : up;
+      p *= f;
+      pm *= f;
+    }
   }
   return c;
 }
 
-// The same count in FP32 (rescaling by 2^(+-60)), used only to localise eigenvalues before the FP64
+// The same count in FP32 (rescaling by 2^(+-60) every step pair), used only to localise eigenvalues before the FP64
 // multisection; its brackets are verified with FP64 counts.
 __device__ int sturm_count_f32(const float* d, const float* e2, int n, float x) {
   const float up = 0x1p+60f, down = 0x1p-60f;
   float pm = 1.0f, p = d[0] - x;
-  int sprev = 1, c = 0;
-  int s = (__float_as_int(p) & 0x7fffffff) == 0 ? -sprev : (__float_as_int(p) < 0 ? -1 : 1);
-  c += s != sprev;
-  sprev = s;
-  for (int i = 1; i < n; ++i) {
-    float pn = fmaf(d[i] - x, p, -e2[i - 1] * pm);
-    pm = p;
-    p = pn;
-    const int ep = (__float_as_int(p) >> 23) & 0xff, epm = (__float_as_int(pm) >> 23) & 0xff;
-    if (ep > 127 + 60) { p *= down; pm *= down; }
-    else if (ep < 127 - 60 && epm < 127 - 60) { p *= up; pm *= up; }
-    s = (__float_as_int(p) & 0x7fffffff) == 0 ? -sprev : (__float_as_int(p) < 0 ? -1 : 1);
-    c += s != sprev;
-    sprev = s;
+  unsigned sg = (__float_as_uint(p) << 1) == 0u ? 1u : __float_as_uint(p) >> 31;
+  int c = (int)sg;
+  for (int i = 1; i < n; i += 2) {
+    const int k1 = min(i + 1, n - 1);
+    const float d0 = d[i] - x, d1 = d[k1] - x, e0 = -e2[i - 1], e1 = -e2[k1 - 1];
+    const float q0 = fmaf(d0, p, e0 * pm), q1 = fmaf(d1, q0, e1 * p);
+    unsigned s = (__float_as_uint(q0) << 1) == 0u ? sg ^ 1u : __float_as_uint(q0) >> 31;
+    c += (int)(s ^ sg);
+    sg = s;
+    if (i + 1 < n) {
+      s = (__float_as_uint(q1) << 1) == 0u ? sg ^ 1u : __float_as_uint(q1) >> 31;
+      c += (int)(s ^ sg);
+      sg = s;
+    }
+    pm = q0;
+    p = q1;
+    const int e = max((__float_as_int(p) >> 23) & 0xff, (__float_as_int(pm) >> 23) & 0xff);
+    if (e > 127 + 60 || e < 127 - 60) {
+      const float f = e > 127 ? down : up;
+      p *= f;
+      pm *= f;
+    }
   }
   return c;
 }
 
-// LU with partial pivoting of the tridiagonal T - lam I (sub = super = e, diag d - lam).  Factors in
-// dl (multipliers), dd (reciprocals of the diagonal of U), du (1st super), du2 (2nd super), piv (1 = rows
-// i, i+1 swapped).
-__device__ void trid_factor(const double* d, const double* e, int n, double lam, double tiny, double* dl, double* dd,
-                            double* du, double* du2, int* piv) {
-  for (int i = 0; i < n; ++i) dd[i] = d[i] - lam;
-  for (int i = 0; i < n - 1; ++i) {
-    dl[i] = e[i];
-    du[i] = e[i];
-    du2[i] = 0.0;
-    piv[i] = 0;
-  }
-  for (int i = 0; i < n - 1; ++i) {
-    if (fabs(dd[i]) >= fabs(dl[i])) {
-      if (dd[i] == 0.0) dd[i] = tiny;
-      double f = dl[i] / dd[i];
-      dl[i] = f;
-      dd[i + 1] -= f * du[i];
-    } else {
-      double f = dd[i] / dl[i];
-      dd[i] = dl[i];
-      dl[i] = f;
-      double t = du[i];
-      du[i] = dd[i + 1];
-      dd[i + 1] = t - f * dd[i + 1];
-      if (i < n - 2) {
-        du2[i] = du[i + 1];
-        du[i + 1] = -f * du[i + 1];
-      }
-      piv[i] = 1;
-    }
-  }
-  if (dd[n - 1] == 0.0) dd[n - 1] = tiny;
-  for (int i = 0; i < n; ++i) dd[i] = 1.0 / dd[i];  // the solves multiply by the reciprocal pivots
+// 1 / x and 1 / sqrt(x): the hardware's approximation (about 2^-20) improved by one third-order Householder step each
+// (error of the order of the cube of the first), about half the latency of a division; outside the approximations'
+// range the divisions themselves.
+__device__ __forceinline__ double recip(double x) {
+  const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+  if (ex < 24 || ex > 2022) return 1.0 / x;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = fma(-x, y, 1.0);
+  return fma(y, fma(h, h, h), y);
 }
 
-__device__ void trid_solve(int n, const double* dl, const double* dd, const double* du, const double* du2,
-                           const int* piv, double* b) {
+__device__ __forceinline__ double recip_sqrt(double x) {
+  const int ex = (__double2hiint(x) >> 20) & 0x7ff;
+  if (ex < 24 || ex > 2022) return 1.0 / sqrt(x);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = fma(-x * y, y, 1.0);
+  return fma(y * h, fma(0.375, h, 0.5), y);
+}
+
+// LU with partial pivoting of the tridiagonal T - lam I (sub = super = e, diag d - lam).  Factors in
+// dl (multipliers), dd (reciprocals of the diagonal of U), du (1st super), du2 (2nd super), piv (1 = rows
+// i, i+1 swapped).  The active row is carried in registers, and both outcomes of a pivot share one reciprocal, so that
+// lanes on different eigenvalues do not diverge.
+__device__ __forceinline__ long long abs_bits(double x) { return __double_as_longlong(x) & 0x7fffffffffffffffLL; }
+
+__device__ void trid_factor(const double* __restrict__ d, const double* __restrict__ e, int n, double lam, double tiny,
+                            double* __restrict__ dl, double* __restrict__ dd, double* __restrict__ du,
+                            double* __restrict__ du2, int* __restrict__ piv) {
+  double cd = d[0] - lam, cu = n > 1 ? e[0] : 0.0, ei = cu;
   for (int i = 0; i < n - 1; ++i) {
-    if (!piv[i]) {
-      b[i + 1] -= dl[i] * b[i];
-    } else {
-      double t = b[i];
-      b[i] = b[i + 1];
-      b[i + 1] = t - dl[i] * b[i];
+    const double dn = d[i + 1] - lam, un = i < n - 2 ? e[i + 1] : 0.0;
+    const bool sw = abs_bits(cd) < abs_bits(ei);
+    if (abs_bits(cd) == 0 && !sw) cd = tiny;
+    const double r = recip(sw ? ei : cd);
+    const double top = sw ? dn : cu;
+    const double f = (sw ? cd : ei) * r;
+    dl[i] = f;
+    dd[i] = r;
+    du[i] = top;
+    du2[i] = sw ? un : 0.0;
+    piv[i] = sw ? 1 : 0;
+    cd = fma(-f, top, sw ? cu : dn);
+    cu = sw ? -f * un : un;
+    ei = un;
+  }
+  if (abs_bits(cd) == 0) cd = tiny;
+  dd[n - 1] = recip(cd);
+}
+
+__device__ void trid_solve(int n, const double* __restrict__ dl, const double* __restrict__ dd,
+                           const double* __restrict__ du, const double* __restrict__ du2, const int* __restrict__ piv,
+                           double* __restrict__ b) {
+  double x = b[0];
+  for (int i0 = 0; i0 < n - 1; i0 += 4) {
+    double y[4], f[4], top[4];
+    int sw[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = min(i0 + u, n - 2);
+      y[u] = b[i + 1];
+      f[u] = dl[i];
+      sw[u] = piv[i];
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < n - 1) {
+        top[u] = sw[u] ? y[u] : x;
+        x = fma(-f[u], top[u], sw[u] ? x : y[u]);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u < n - 1) b[i0 + u] = top[u];
   }
   // back substitution, rescaling the computed tail when a term would overflow (the direction is what
-  // inverse iteration needs)
-  const double big = 1e150;
-  for (int i = n - 1; i >= 0; --i) {
-    double v = b[i];
-    if (i + 1 < n) v -= du[i] * b[i + 1];
-    if (i + 2 < n) v -= du2[i] * b[i + 2];
-    double y = v * dd[i];
-    if (fabs(y) > big) {
-      for (int l = i + 1; l < n; ++l) b[l] *= 1e-150;
-      y *= 1e-150;
+  // inverse iteration needs); the test reads the exponent, off the FP64 pipe
+  double y1 = x * dd[n - 1], y2 = 0.0;
+  b[n - 1] = y1;
+  for (int i0 = n - 2; i0 >= 0; i0 -= 4) {
+    double v[4], p1[4], p2[4], r[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = max(i0 - u, 0);
+      v[u] = b[i];
+      p1[u] = du[i];
+      p2[u] = du2[i];
+      r[u] = dd[i];
     }
-    b[i] = y;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 - u >= 0) {
+        double y = fma(-p1[u], y1, fma(-p2[u], y2, v[u])) * r[u];
+        if (((__double2hiint(y) >> 20) & 0x7ff) > 1023 + 498) {
+          for (int l = i0 - u + 1; l < n; ++l) b[l] *= 0x1p-498;
+          y *= 0x1p-498;
+          y1 *= 0x1p-498;
+        }
+        b[i0 - u] = y;
+        y2 = y1;
+        y1 = y;
+      }
   }
+}
+
+// Gram matrix of the k vectors of Y (vector t at Y + t yst): G[t][s], s <= t, row stride k | 1.  Returns (to every
+// thread) the largest |cosine| between two of them, or a value above 2 when a vector is zero or not finite; the vectors
+// are then scaled to unit length (G with them).
+__device__ float gram_and_normalise(double* Y, int yst, int n, int k, double* G) {
+  __shared__ int s_cos;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int gst = k | 1;
+  double* rs = G + (size_t)k * gst;  // k: reciprocal lengths
+  if (tid == 0) s_cos = 0;
+  const int np = k * (k + 1) / 2;
+  auto pair = [&](int q, int& t, int& u) {
+    t = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);
+    while (t * (t + 1) / 2 > q) --t;
+    while ((t + 1) * (t + 2) / 2 <= q) ++t;
+    u = q - t * (t + 1) / 2;
+  };
+  for (int q = tid; q < np; q += nthr) {
+    int t, u;
+    pair(q, t, u);
+    const double* a = Y + (size_t)t * yst;
+    const double* b = Y + (size_t)u * yst;
+    double s0 = 0.0, s1 = 0.0;
+    int i = 0;
+    for (; i + 1 < n; i += 2) {
+      s0 = fma(a[i], b[i], s0);
+      s1 = fma(a[i + 1], b[i + 1], s1);
+    }
+    if (i < n) s0 = fma(a[i], b[i], s0);
+    G[t * gst + u] = s0 + s1;
+  }
+  __syncthreads();
+  for (int t = tid; t < k; t += nthr) {
+    const double d = G[t * gst + t];
+    const bool ok = d > 0.0 && isfinite(d);
+    rs[t] = ok ? recip_sqrt(d) : 0.0;
+    if (!ok) s_cos = __float_as_int(3.0f);
+  }
+  __syncthreads();
+  const bool bad = s_cos != 0;
+  __syncthreads();
+  if (bad) return 3.0f;
+  for (int q = tid; q < np; q += nthr) {
+    int t, u;
+    pair(q, t, u);
+    const double v = G[t * gst + u] * (rs[t] * rs[u]);
+    G[t * gst + u] = v;
+    if (t != u) atomicMax(&s_cos, __float_as_int(fabsf((float)v)));
+  }
+  for (int q = tid; q < k * n; q += nthr) {
+    const int t = q / n, i = q - t * n;
+    Y[(size_t)t * yst + i] *= rs[t];
+  }
+  __syncthreads();
+  return __int_as_float(s_cos);
+}
+
+// Orthonormalises the k unit vectors of Y in order by the Cholesky factor of their Gram matrix G (as left by
+// gram_and_normalise): G = L D L^T, Y <- D^-1/2 L^-1 Y, the vectors Gram-Schmidt gives, with the products spread over the
+// block.  After an inverse iteration the vectors are nearly orthogonal unless eigenvalues agree to rounding, so L is close
+// to the unit matrix; where a pivot falls below 1/100 the result is left to modified Gram-Schmidt (returns false, Y
+// unchanged).  All threads of the block call it.
+__device__ bool chol_orth(double* Y, int yst, int n, int k, double* G) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int gst = k | 1;
+  double* rs = G + (size_t)k * gst;
+  // right-looking, a thread per entry below the pivot; column j keeps its unscaled entries, rs the reciprocal pivots
+  for (int j = 0; j < k; ++j) {
+    const double d = G[j * gst + j];
+    if (!(d > 0.01)) return false;  // the same value in every thread
+    const double r = recip(d);
+    const int m = k - j - 1;
+    for (int q = tid; q < m * m; q += nthr) {
+      const int a = q / m, b = q - a * m;
+      if (b <= a) {
+        const int i = j + 1 + a, l = j + 1 + b;
+        G[i * gst + l] = fma(-(G[i * gst + j] * r), G[l * gst + j], G[i * gst + l]);
+      }
+    }
+    if (tid == 0) rs[j] = r;
+    __syncthreads();
+  }
+  // Y <- L^-1 Y, eight lanes per column of Y: once row s is final its multiples leave the rows below
+  const int part = tid & 7;
+  for (int i0 = 0; i0 < n; i0 += nthr >> 3) {
+    const int i = i0 + (tid >> 3);
+    if (i0 + ((tid & ~31) >> 3) >= n) continue;  // whole warp past the columns
+    const bool in = i < n;
+    for (int s = 0; s < k; ++s) {
+      const double ys = in ? Y[(size_t)s * yst + i] * rs[s] : 0.0;
+      if (in)
+        for (int t = s + 1 + part; t < k; t += 8) {
+          double* y = Y + (size_t)t * yst + i;
+          *y = fma(-G[t * gst + s], ys, *y);
+        }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < k; t += nthr) rs[t] = recip_sqrt(G[t * gst + t]);
+  __syncthreads();
+  for (int q = tid; q < k * n; q += nthr) {
+    const int t = q / n, i = q - t * n;
+    Y[(size_t)t * yst + i] *= rs[t];
+  }
+  __syncthreads();
+  return true;
+}
+
+// Power of two that brings the largest entry (bits of its upper word, over the block) near 1, so that the squares and
+// products of the reduction stay in range whatever the scale of the matrix.  red: 32 ints.  All threads call it.
+__device__ double range_scale(int hi_abs, int* red) {
+  const int m = __reduce_max_sync(0xffffffff, hi_abs);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  int b = 0;
+  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) b = max(b, red[q]);
+  const int ex = b >> 20;
+  if (ex == 0 || ex == 0x7ff) return 1.0;  // zero, denormal, or not finite
+  return __hiloint2double(min(2046, max(1, 2046 - ex)) << 20, 0);
 }
 
 // Gershgorin interval of the tridiagonal (d, e) and the largest e_i^2, by warp 0 (lanes over the rows), left in
@@ -199,22 +389,24 @@ __device__ void trid_gershgorin(const double* d, const double* e, int n, double*
 // back-transforms and writes the outputs.  The bisection is a chain of dependent FP64 Sturm recurrences per
 // point; inside one block the k eigenvalues shared one SM's FP64 pipe (2 FMA/clk), one warp each they get one
 // SM each, so every lane can take its own point (33-way multisection, about 5 bits per count instead of 2).
-// Per-item global scratch (doubles): a header (active size, Gershgorin interval, largest e_i^2, reduced-problem
-// flag and nA), d, e, beta, lam (nl each), the reflectors W (n x n, leading dimension n), the vectors Y
+// Per-item global scratch (doubles): a header (active size, Gershgorin interval, largest e_i^2 and the factor back from
+// the range the matrix was scaled to), d, e, beta, lam (nl each), the reflectors W (n x n, leading dimension n), the vectors Y
 // (kl x nl, vector-major) and the inverse-iteration LU factors (kl x 5 nl).
 constexpr int kHdr = 8;
+constexpr double kTailFloor = 1e-280;  // squared length of a column tail that counts as zero (entries scaled to 1)
+constexpr int kSmallEig = 96;  // sizes whose matrix fits the register kernels
 
-static size_t syevx_scratch_per(int nl, int kl) {
-  return kHdr + 4 * (size_t)nl + (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl;
+__host__ __device__ inline size_t syevx_scratch_per(int nl, int kl) {
+  return kHdr + 4 * (size_t)nl + (nl <= kSmallEig ? 2 : 1) * (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl;
 }
 
 struct SyevxScratch {
-  double *hdr, *d, *e, *beta, *lam, *W, *Y, *lu;
+  double *hdr, *d, *e, *beta, *lam, *W, *Y, *lu, *Q;
 };
 
 __device__ __forceinline__ SyevxScratch syevx_scratch(double* scratch, int nl, int kl, int item) {
   SyevxScratch g;
-  g.hdr = scratch + (size_t)item * (kHdr + 4 * (size_t)nl + (size_t)nl * nl + (size_t)kl * nl + (size_t)kl * 5 * nl);
+  g.hdr = scratch + item * syevx_scratch_per(nl, kl);
   g.d = g.hdr + kHdr;
   g.e = g.d + nl;
   g.beta = g.e + nl;
@@ -222,20 +414,16 @@ __device__ __forceinline__ SyevxScratch syevx_scratch(double* scratch, int nl, i
   g.W = g.lam + nl;
   g.Y = g.W + (size_t)nl * nl;
   g.lu = g.Y + (size_t)kl * nl;
+  g.Q = g.lu + (size_t)kl * 5 * nl;
   return g;
 }
 
-// K1.  nl, kl: the launch sizes (strides of the inputs and outputs).  Optional reduced problem (nAg != null):
-// the symmetric input A = B B^T has its nonzero block in the leading nA x nA corner, and A2 = B^T B (B: nl x nl,
-// nonzero block nA x nB) has it in the leading nB x nB corner.  The smaller of the two is decomposed; when that
-// is A2, K3 maps the left vectors back as u = B w / sigma, re-orthonormalises them (modified Gram-Schmidt) and
-// completes them by unit vectors when B has fewer than k nonzero singular values.
+// K1.  nl, kl: the launch sizes (strides of the inputs and outputs).  nAg (optional): the active size of each item, the
+// leading block of its matrix; the rest is zero.
 __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* __restrict__ Ag, int nl, int kl,
                                                                   double* wg, double* Vg, int ldv, double* scratch,
                                                                   int use_smem, const int* __restrict__ nAg,
-                                                                  const int* __restrict__ nBg,
-                                                                  const double* __restrict__ A2g,
-                                                                  const double* __restrict__ Bg, double* work) {
+                                                                  double* work) {
   extern __shared__ __align__(16) double sm[];
   double* red = sm;            // 33 (32 partials + the result) + padding
   double* pv = red + 40;       // nl: p / w of the current reflector
@@ -247,19 +435,14 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
   const int tid = threadIdx.x, nthr = blockDim.x;
   double* wout = wg + (size_t)blockIdx.x * nl;
   double* Vout = Vg + (size_t)blockIdx.x * (size_t)nl * ldv;
-  // the problem actually decomposed: n x n, k vectors
-  const int nA = nAg ? max(0, min(nl, nAg[blockIdx.x])) : nl;
-  const int nB = nBg ? max(0, min(nl, nBg[blockIdx.x])) : nl;
-  const bool viaB = (nAg != nullptr) && (A2g != nullptr) && (Bg != nullptr) && nB < nA;
-  const int n = viaB ? nB : nA;
+  // the active size: n x n, k vectors
+  const int n = nAg ? max(0, min(nl, nAg[blockIdx.x])) : nl;
   const int k = min(kl, n);
-  const double* A = (viaB ? A2g : Ag) + (size_t)blockIdx.x * nnl;
+  const double* A = Ag + (size_t)blockIdx.x * nnl;
   if (tid == 0) {
     add_work(work, 4.0 / 3.0 * n * (double)n * n + 4.0 * (double)k * n * n + 60.0 * k * n,
              sizeof(double) * (2.0 * n * n + (double)k * n));
     g.hdr[0] = (double)n;
-    g.hdr[4] = viaB ? 1.0 : 0.0;
-    g.hdr[5] = (double)nA;
   }
   for (int t = tid; t < kl; t += nthr) wout[t] = 0.0;
   for (size_t q = tid; q < (size_t)nl * kl; q += nthr) {
@@ -267,10 +450,14 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     Vout[(size_t)i * ldv + t] = 0.0;
   }
   if (n == 0) return;
+  int top = 0;
   for (size_t t = tid; t < (size_t)n * n; t += nthr) {
     const int i = (int)(t / n), j = (int)(t - (t / n) * n);
     W[t] = A[(size_t)i * nl + j];
+    top = max(top, __double2hiint(W[t]) & 0x7fffffff);
   }
+  const double scale = range_scale(top, (int*)red);
+  for (size_t t = tid; t < (size_t)n * n; t += nthr) W[t] *= scale;
   __syncthreads();
 
   // 1. tridiagonalisation
@@ -284,7 +471,7 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
       if (i > 0) loc += xi * xi;
     }
     const double tail2 = block_reduce_sum(loc, red, m);
-    if (tail2 == 0.0) {
+    if (!(tail2 > kTailFloor)) {
       if (tid == 0) {
         d[j] = W[(size_t)j * n + j];
         e[j] = x0;
@@ -357,93 +544,353 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     g.hdr[1] = red[35];
     g.hdr[2] = red[36];
     g.hdr[3] = red[37];
+    g.hdr[4] = 1.0 / scale;
   }
   if (use_smem)
     for (size_t t = tid; t < (size_t)n * n; t += nthr) g.W[t] = W[t];
 }
 
-// K2.  Eigenvalue t (the t-th largest) of the tridiagonal of item blockIdx.y, one warp: (a) FP32 localisation
-// in the Gershgorin interval by five rounds of 33-way multisection (about 25 bits); (b) that bracket, widened
-// and verified with FP64 counts (else the Gershgorin interval), then 33-way FP64 multisection on a copy of T
-// scaled by a power of two to |T| in [0.5, 1) (the counts' range window) down to the absolute resolution
-// eps ||T||: the eigenvalues of an FP64 Gram core carry errors of that size, and inverse iteration only needs
-// the shift to that accuracy.
-__global__ void __launch_bounds__(32) syevx_bisect_kernel(int nl, int kl, int kv, double* scratch) {
+// K1 for n <= 32 NR: the matrix in registers, row = lane (NR rows a lane), columns dealt to TW worker warps.  A warp issues
+// one FP64 instruction per 64 cycles on this part whatever its lanes or its other instructions do, and an SM has four
+// such units, so a step takes as long as the unit with the most FP64 instructions on its path:
+//  * warp 0 forms the reflector's scalars from the norm of x while the workers multiply: with v = x + s ||x|| e_1 the
+//    product A v = A x + s ||x|| a_1 needs no finished v, and v^T A v follows from x^T A x, (A x)_1 and a_11;
+//  * three workers, one per remaining unit (six halves of the registers at n > 64);
+//  * the two columns the next step reads are updated and published first, the rest after the barrier;
+//  * one square root and one reciprocal a step (recip_sqrt, recip), two barriers.
+template <int NR, int TW>
+__global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const double* __restrict__ Ag, int nl,
+                                                                             int kl, double* wg, double* Vg, int ldv,
+                                                                             double* scratch,
+                                                                             const int* __restrict__ nAg,
+                                                                             double* work) {
+  constexpr int M = 32 * NR, NC = (M + TW - 1) / TW;
+  __shared__ double xs[2][M], a1s[2][M], ys[M], parts[TW][M], ds[M], es[M], red[40];
+  __shared__ double sc[4];
+  __shared__ int sred[32];
+  __shared__ double2 vws[TW][M];
+  const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, w = (tid >> 5) - 1;
+  double* wout = wg + (size_t)blockIdx.x * nl;
+  double* Vout = Vg + (size_t)blockIdx.x * (size_t)nl * ldv;
+  const int n = nAg ? max(0, min(nl, nAg[blockIdx.x])) : nl;
+  const int k = min(kl, n);
+  const double* A = Ag + (size_t)blockIdx.x * nl * nl;
+  if (tid == 0) {
+    add_work(work, 4.0 / 3.0 * n * (double)n * n + 4.0 * (double)k * n * n + 60.0 * k * n,
+             sizeof(double) * (2.0 * n * n + (double)k * n));
+    g.hdr[0] = (double)n;
+  }
+  for (int t = tid; t < kl; t += nthr) wout[t] = 0.0;
+  for (int q = tid; q < nl * kl; q += nthr) Vout[(size_t)(q / kl) * ldv + q % kl] = 0.0;
+  if (n == 0) return;
+  double a[NR][NC];
+  int top = 0;
+  if (w >= 0) {
+#pragma unroll
+    for (int cc = 0; cc < NC; ++cc) {
+      const int col = cc * TW + w;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int row = lane + 32 * r;
+        a[r][cc] = row < n && col < n ? A[(size_t)col * nl + row] : 0.0;  // symmetric
+        top = max(top, __double2hiint(a[r][cc]) & 0x7fffffff);
+      }
+    }
+  }
+  const double scale = range_scale(top, sred);
+  if (w >= 0) {
+#pragma unroll
+    for (int cc = 0; cc < NC; ++cc) {
+      const int col = cc * TW + w;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        a[r][cc] *= scale;
+        if (col < 2) (col == 0 ? xs[0] : a1s[0])[lane + 32 * r] = a[r][cc];
+      }
+    }
+  }
+  __syncthreads();
+  int par = 0;
+  for (int j = 0; j + 2 < n; ++j, par ^= 1) {
+    const double* x = xs[par];
+    const double* a1 = a1s[par];
+    double xr[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int row = lane + 32 * r;
+      xr[r] = row > j && row < n ? x[row] : 0.0;
+    }
+    if (w < 0) {
+      double loc = 0.0;
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        if (lane + 32 * r != j + 1) loc = fma(xr[r], xr[r], loc);
+      const double tail2 = warp_sum(loc), x0 = x[j + 1];
+      double sn = 0.0, b = 0.0, alpha = x0;
+      if (tail2 > kTailFloor) {
+        const double s = fma(x0, x0, tail2);
+        const double nrm = s * recip_sqrt(s);
+        b = recip(fma(fabs(x0), nrm, s));  // 2 / (v^T v)
+        sn = copysign(nrm, x0);
+        alpha = -sn;
+      }
+      if (lane == 0) {
+        sc[0] = sn;
+        sc[1] = b;
+        sc[3] = 0.5 * b;
+        ds[j] = x[j];
+        es[j] = alpha;
+        g.beta[j] = b;
+      }
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int row = lane + 32 * r;
+        if (row > j && row < n) g.W[(size_t)row * n + j] = row == j + 1 ? xr[r] + sn : xr[r];
+      }
+    } else {
+      double p0[NR], p1[NR];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) p0[r] = p1[r] = 0.0;
+#pragma unroll
+      for (int cc = 0; cc < NC; ++cc) {
+        const int col = cc * TW + w;
+        if (col > j && col < n) {
+          const double xc = x[col];
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            double* acc = (cc & 1) ? p1 : p0;
+            acc[r] = fma(a[r][cc], xc, acc[r]);
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < NR; ++r) parts[w][lane + 32 * r] = p0[r] + p1[r];
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * TW) : "memory");
+      if (w == 0) {
+        double xy = 0.0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int row = lane + 32 * r;
+          double y = parts[0][row] + parts[1][row];
+#pragma unroll
+          for (int q = 2; q < TW; ++q) y += parts[q][row];
+          ys[row] = y;
+          xy = fma(xr[r], y, xy);
+        }
+        xy = warp_sum(xy);
+        if (lane == 0) sc[2] = xy;
+      }
+    }
+    __syncthreads();
+    // w = b q - K v with q = A v = y + sn a_1, K = b^2 v^T q / 2; then the next step's two columns
+    double vr[NR], wr[NR];
+    auto update = [&](int cc) {
+      const double2 c = vws[max(w, 0)][cc * TW + w];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) a[r][cc] = fma(-vr[r], c.y, fma(-wr[r], c.x, a[r][cc]));
+    };
+    if (w >= 0) {
+      const double sn = sc[0], b = sc[1];
+      // v^T A v = x^T A x + 2 sn (A x)_1 + sn^2 a_11
+      const double y1 = ys[j + 1];
+      const double K = sc[3] * (b * fma(sn, fma(sn, a1[j + 1], y1 + y1), sc[2]));  // (b^2 alone may overflow)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const int row = lane + 32 * r;
+        const bool in = row > j && row < n;
+        vr[r] = in ? (row == j + 1 ? xr[r] + sn : xr[r]) : 0.0;
+        wr[r] = in ? fma(b, fma(sn, a1[row], ys[row]), -K * vr[r]) : 0.0;
+        vws[w][row] = make_double2(vr[r], wr[r]);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int cc = 0; cc < NC; ++cc) {
+        const int col = cc * TW + w;
+        if (col == j + 1 || col == j + 2) {
+          update(cc);
+#pragma unroll
+          for (int r = 0; r < NR; ++r) (col == j + 1 ? xs[par ^ 1] : a1s[par ^ 1])[lane + 32 * r] = a[r][cc];
+        }
+      }
+    }
+    __syncthreads();
+    if (w >= 0) {
+#pragma unroll
+      for (int cc = 0; cc < NC; ++cc) {
+        const int col = cc * TW + w;
+        if (col > j + 2 && col < n) update(cc);
+      }
+    }
+  }
+  if (tid == 0) {
+    if (n >= 2) {
+      ds[n - 2] = xs[par][n - 2];
+      es[n - 2] = xs[par][n - 1];
+      g.beta[n - 2] = 0.0;
+      ds[n - 1] = a1s[par][n - 1];
+    } else {
+      ds[0] = xs[par][0];
+    }
+    es[n - 1] = 0.0;
+    g.beta[n - 1] = 0.0;
+  }
+  __syncthreads();
+  trid_gershgorin(ds, es, n, red);
+  if (tid == 0) {
+    g.hdr[1] = red[35];
+    g.hdr[2] = red[36];
+    g.hdr[3] = red[37];
+    g.hdr[4] = 1.0 / scale;
+  }
+  for (int i = tid; i < n; i += nthr) {
+    g.d[i] = ds[i];
+    g.e[i] = es[i];
+  }
+}
+
+// K2.  Eigenvalue t (the t-th largest) of the tridiagonal of item blockIdx.y, one block of four warps, a point of the
+// multisection per thread (one warp on each of the SM's four FP64 units: 129-way rounds, 7 bits each): (a) FP32
+// localisation in the Gershgorin interval in four rounds; (b) that bracket, widened, its ends the first FP64 round's
+// first and last points (else the Gershgorin interval), then FP64 rounds, all on a copy of T scaled by a power of two to
+// |T| in [0.5, 1) (the counts' range window), down to the absolute resolution eps ||T||: the eigenvalues of an FP64 Gram
+// core carry errors of that size, and inverse iteration only needs the shift to that accuracy.
+// Blocks kv .. kv + nq - 1 of an item meanwhile form Q = H_0 H_1 .. H_{n-3} (16 columns a block, eight lanes a column),
+// so that K3 transforms back by one product instead of n - 2 dependent reflections.
+constexpr int kBisectThreads = 128;
+constexpr int kQCols = kBisectThreads / 8;
+
+__device__ void form_q_columns(const SyevxScratch& g, int n, int c0, double* sm) {
+  const int tid = threadIdx.x, gl = tid & 7, c = c0 + (tid >> 3);
+  const int ld = n | 1;
+  double* y = sm + (size_t)(tid >> 3) * ld;
+  for (int i = gl; i < n; i += 8) y[i] = i == c ? 1.0 : 0.0;
+  __syncwarp();
+  const int last = min(n - 3, c0 + kQCols - 2);  // H_j leaves e_c as it is while c <= j
+  for (int j = last; j >= 0; --j) {
+    const double b = g.beta[j];
+    if (b == 0.0) continue;
+    const double* v = g.W + (size_t)(j + 1) * n + j;
+    double* yj = y + j + 1;
+    const int m = n - j - 1;
+    double vr[12], s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+      const int i = gl + 8 * q;
+      vr[q] = i < m ? v[(size_t)i * n] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 12; ++q)
+      if (8 * q < m) s = fma(vr[q], gl + 8 * q < m ? yj[gl + 8 * q] : 0.0, s);
+    for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
+    s *= b;
+#pragma unroll
+    for (int q = 0; q < 12; ++q)
+      if (8 * q < m && gl + 8 * q < m) yj[gl + 8 * q] = fma(-s, vr[q], yj[gl + 8 * q]);
+    __syncwarp();
+  }
+  if (c < n)
+    for (int i = gl; i < n; i += 8) g.Q[(size_t)i * n + c] = y[i];
+}
+
+__global__ void __launch_bounds__(kBisectThreads) syevx_bisect_kernel(int nl, int kl, int kv, double* scratch) {
   extern __shared__ __align__(16) double sm[];
+  __shared__ int s_first[2][4];
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.y);
   const int n = (int)g.hdr[0];
-  const int t = blockIdx.x, lane = threadIdx.x;
+  const int t = blockIdx.x, tid = threadIdx.x;
+  if (t >= kv) {
+    const int c0 = (t - kv) * kQCols;
+    if (c0 < n) form_q_columns(g, n, c0, sm);
+    return;
+  }
   if (t >= min(kv, n)) return;
   const double lo = g.hdr[1], hi = g.hdr[2], emax2 = g.hdr[3];
   const double tnorm = fmax(fabs(lo), fabs(hi));
   if (tnorm == 0.0) {
-    if (lane == 0) g.lam[t] = 0.0;
+    if (tid == 0) g.lam[t] = 0.0;
     return;
   }
-  float* df = (float*)sm;   // n floats
-  float* e2f = df + n;      // n floats
-  double* ds = sm + n;      // n: the scaled diagonal
+  double* ds = sm;          // n: the scaled diagonal
   double* e2s = ds + n;     // n: the scaled e^2
+  float* df = (float*)(e2s + n);  // n floats
+  float* e2f = df + n;            // n floats
   int texp = 0;
   frexp(tnorm, &texp);
   const double sg = ldexp(1.0, -texp), sg2 = sg * sg;
-  for (int i = lane; i < n; i += 32) {
+  for (int i = tid; i < n; i += kBisectThreads) {
     const double ei = (i < n - 1) ? g.e[i] : 0.0;
-    const double di = g.d[i];
-    df[i] = (float)di;
-    e2f[i] = (float)(ei * ei);
-    ds[i] = di * sg;
+    ds[i] = g.d[i] * sg;
     e2s[i] = (ei * ei) * sg2;
+    df[i] = (float)ds[i];
+    e2f[i] = (float)e2s[i];
   }
-  __syncwarp();
+  __syncthreads();
   const int idx = n - 1 - t;
+  int round = 0;
+  // the first point (thread) whose count exceeds idx, kBisectThreads when none does
+  auto first_above = [&](bool above) {
+    const unsigned m = __ballot_sync(0xffffffff, above);
+    if ((tid & 31) == 0) s_first[round & 1][tid >> 5] = m ? (tid & ~31) + __ffs(m) - 1 : kBisectThreads;
+    __syncthreads();
+    int f = kBisectThreads;
+    for (int q = 3; q >= 0; --q)
+      if (s_first[round & 1][q] < kBisectThreads) f = s_first[round & 1][q];
+    ++round;
+    return f;
+  };
   const double pivmin = DBL_MIN * fmax(1.0, emax2);
-  const double glo = lo - 2.0 * DBL_EPSILON * tnorm - pivmin, ghi = hi + 2.0 * DBL_EPSILON * tnorm + pivmin;
+  const double glo = (lo - 2.0 * DBL_EPSILON * tnorm - pivmin) * sg, ghi = (hi + 2.0 * DBL_EPSILON * tnorm + pivmin) * sg;
   float af = (float)glo, cf = (float)ghi;
-  for (int it = 0; it < 5; ++it) {
-    const float h = (cf - af) * (1.0f / 33.0f);
-    const float x = af + h * (float)(lane + 1);
-    const unsigned above = __ballot_sync(0xffffffff, sturm_count_f32(df, e2f, n, x) > idx);
-    const int f = above ? (__ffs(above) - 1) : 32;
+  for (int it = 0; it < 4; ++it) {
+    const float h = (cf - af) * (1.0f / (kBisectThreads + 1));
+    const float x = af + h * (float)(tid + 1);
+    const int f = first_above(sturm_count_f32(df, e2f, n, x) > idx);
     const float na = (f == 0) ? af : af + h * (float)f;
-    const float nc = (f == 32) ? cf : af + h * (float)(f + 1);
+    const float nc = (f == kBisectThreads) ? cf : af + h * (float)(f + 1);
     if (!(na < nc)) break;  // FP32 resolution reached
     af = na;
     cf = nc;
   }
   const double wf = (double)cf - (double)af;
-  double a = fmax(glo, (double)af - 4.0 * wf - 1e-6 * tnorm) * sg;
-  double c = fmin(ghi, (double)cf + 4.0 * wf + 1e-6 * tnorm) * sg;
-  int ca = (lane == 0) ? sturm_count(ds, e2s, n, a) : 0;
-  int cc = (lane == 1) ? sturm_count(ds, e2s, n, c) : 0;
-  ca = __shfl_sync(0xffffffff, ca, 0);
-  cc = __shfl_sync(0xffffffff, cc, 1);
-  if (!(ca <= idx && cc > idx)) {
-    a = glo * sg;
-    c = ghi * sg;
+  double a = fmax(glo, (double)af - 4.0 * wf - 1e-6), c = fmin(ghi, (double)cf + 4.0 * wf + 1e-6);
+  const double floor_s = DBL_EPSILON * tnorm * sg + 4.0 * pivmin * sg;
+  {
+    // the points a + i (c - a) / 127 with both ends: the bracket is right when the first of the points above is neither
+    // the lower end nor missing
+    const double h = (c - a) * (1.0 / (kBisectThreads - 1));
+    const double x = tid == kBisectThreads - 1 ? c : a + h * (double)tid;
+    const int f = first_above(sturm_count(ds, e2s, n, x) > idx);
+    if (f == 0 || f == kBisectThreads) {
+      a = glo;
+      c = ghi;
+    } else {
+      const double na = a + h * (double)(f - 1), nc = f == kBisectThreads - 1 ? c : a + h * (double)f;
+      a = na;
+      c = nc;
+    }
   }
-  const double floor_s = (DBL_EPSILON * tnorm + 4.0 * pivmin) * sg;
   for (int it = 0; it < 40; ++it) {
     if (c - a <= 2.0 * DBL_EPSILON * fmax(fabs(a), fabs(c)) + floor_s) break;
-    const double h = (c - a) * (1.0 / 33.0);
-    const double x = a + h * (double)(lane + 1);
-    const unsigned above = __ballot_sync(0xffffffff, sturm_count(ds, e2s, n, x) > idx);
-    // the first point whose count exceeds idx bounds the eigenvalue from above
-    const int f = above ? (__ffs(above) - 1) : 32;
+    const double h = (c - a) * (1.0 / (kBisectThreads + 1));
+    const double x = a + h * (double)(tid + 1);
+    const int f = first_above(sturm_count(ds, e2s, n, x) > idx);
     const double na = (f == 0) ? a : a + h * (double)f;
-    const double nc = (f == 32) ? c : a + h * (double)(f + 1);
+    const double nc = (f == kBisectThreads) ? c : a + h * (double)(f + 1);
     if (!(na < nc)) break;
     a = na;
     c = nc;
   }
-  if (lane == 0) g.lam[t] = 0.5 * (a + c) / sg;
+  if (tid == 0) g.lam[t] = 0.5 * (a + c) / sg;
 }
 
-// K3.  Eigenvectors of T by inverse iteration (three passes; vectors of eigenvalues closer than 1e-3 ||T||
-// re-orthogonalised after each pass), the back-transformation and the outputs.
+// K3.  Eigenvectors of T by inverse iteration, their orthonormalisation, the back-transformation and the outputs.
+// Inverse iteration takes two passes, a third when two of the vectors are still further than 1e-9 from orthogonal
+// (eigenvalues closer than about 1e-12 ||T||); after each but the last they are orthonormalised only where they come
+// within 0.05 of each other.  The last orthonormalisation is one Newton-Schulz step Y <- (3 I - G) Y / 2 where the vectors
+// are within 1e-8 / k already (its error is the square), else by chol_orth, else by modified Gram-Schmidt.
 __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl, int kv, double* wg, double* Vg, int ldv,
-                                                                  double* scratch, int smem_flags,
-                                                                  const double* __restrict__ Bg) {
+                                                                  double* scratch, int smem_flags) {
   extern __shared__ __align__(16) double sm[];
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
   const int n = (int)g.hdr[0];
@@ -453,8 +900,8 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   double* e = d + nl;          // nl
   double* beta = e + nl;       // nl
   double* lam = beta + nl;     // kl
-  // the vectors, their LU factors and the reflectors in shared memory where they fit (flags 1, 2, 4): the
-  // solves, the re-orthogonalisation and the back-transformation are dependent chains of their loads
+  // the vectors, their LU factors and the reflectors (n <= kSmallEig: Q) in shared memory where they fit (flags 1, 2, 4):
+  // the solves, the re-orthogonalisation and the back-transformation are dependent chains of their loads
   // strides in shared memory are odd numbers of doubles, so that the lanes of a warp walking different vectors
   // (inverse iteration: one lane per vector) or different rows (the warp sums) hit different banks
   const int npad = nl | 1;
@@ -467,15 +914,14 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
     beta = g.beta;
     lam = g.lam;
   }
+  const bool have_q = nl <= kSmallEig;
   double* Y = g.Y;
   double* lu = g.lu;
-  double* W = g.W;
+  double* W = have_q ? g.Q : g.W;
   if (smem_flags & 1) { Y = next; next += (size_t)kl * npad; }
   if (smem_flags & 2) { lu = next; next += (size_t)kl * 5 * npad; }
-  if (smem_flags & 4) W = next;
-  const size_t nnl = (size_t)nl * nl;
-  const bool viaB = g.hdr[4] != 0.0;
-  const int nA = (int)g.hdr[5];
+  if (smem_flags & 4) { W = next; next += (size_t)nl * npad; }
+  double* G = (smem_flags & 16) ? next : nullptr;  // the Gram matrix of the vectors and k scalars
   const int k = min(kl, n);
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
@@ -492,10 +938,14 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
     }
     for (int t = tid; t < k; t += nthr) lam[t] = g.lam[t];
   }
-  if (smem_flags & 4)
-    for (size_t t = tid; t < (size_t)n * n; t += nthr) W[(t / n) * wld + t % n] = g.W[t];
+  if (smem_flags & 4) {
+    const double* src = have_q ? g.Q : g.W;
+    for (int t = tid; t < n * n; t += nthr) W[(t / n) * wld + t % n] = src[t];
+  }
   __syncthreads();
   const double tnorm = fmax(fabs(g.hdr[1]), fabs(g.hdr[2]));
+  double* Yf = Y;  // where the final vectors of T are
+  int yf = yst;
   if (tnorm == 0.0) {
     // the zero matrix: eigenvalues 0, eigenvectors the unit vectors
     for (size_t q = tid; q < (size_t)k * n; q += nthr) {
@@ -511,15 +961,15 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   }
   __syncthreads();
 
-  // 3. inverse iteration, three passes with cluster re-orthogonalisation
+  // 3. inverse iteration
   const double tiny = DBL_EPSILON * fmax(tnorm, DBL_MIN);
   for (int t = tid; t < k; t += nthr) {
     double* y = Y + (size_t)t * yst;
-    // deterministic start vector with entries in [0.5, 1.5)
+    // deterministic start vector with entries in [0.5, 1)
     unsigned h = 2166136261u ^ (unsigned)(t * 2654435761u);
     for (int i = 0; i < n; ++i) {
       h = h * 1664525u + 1013904223u;
-      y[i] = 0.5 + (double)(h >> 8) * (1.0 / 16777216.0);
+      y[i] = __hiloint2double(0x3fe00000 | (int)(h >> 12), (int)(h << 20));  // mantissa bits: no FP64 operation
     }
     double* f = lu + (size_t)t * 5 * fst;
     trid_factor(d, e, n, lam[t], tiny, f, f + fst, f + 2 * fst, f + 3 * fst, (int*)(f + 4 * fst));
@@ -528,23 +978,56 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   const double ortol = 1e-3 * tnorm;
   for (int pass = 0; pass < 3; ++pass) {
     for (int t = tid; t < k; t += nthr) {
-      double* y = Y + (size_t)t * yst;
       const double* f = lu + (size_t)t * 5 * fst;
-      trid_solve(n, f, f + fst, f + 2 * fst, f + 3 * fst, (const int*)(f + 4 * fst), y);
+      trid_solve(n, f, f + fst, f + 2 * fst, f + 3 * fst, (const int*)(f + 4 * fst), Y + (size_t)t * yst);
+    }
+    __syncthreads();
+    bool last = pass == 2;
+    if (G) {
+      const float cos = gram_and_normalise(Y, yst, n, k, G);
+      last = last || (pass == 1 && cos < 1e-9f);
+      if (cos < (last ? 1e-8f / (float)k : 0.05f)) {
+        if (!last) continue;
+        // Newton-Schulz into the space of the LU factors: y_t - sum_{s != t} G_ts y_s / 2 (unit diagonal)
+        const int gst = k | 1;
+        for (int q = tid; q < k * n; q += nthr) {
+          const int t = q / n, i = q - t * n;
+          double s0 = 0.0, s1 = 0.0;
+          for (int s = 0; s + 1 < k; s += 2) {
+            s0 = fma(s == t ? 0.0 : (s < t ? G[t * gst + s] : G[s * gst + t]), Y[(size_t)s * yst + i], s0);
+            s1 = fma(s + 1 == t ? 0.0 : (s + 1 < t ? G[t * gst + s + 1] : G[(s + 1) * gst + t]),
+                     Y[(size_t)(s + 1) * yst + i], s1);
+          }
+          if ((k & 1) && t != k - 1) s0 = fma(G[(k - 1) * gst + t], Y[(size_t)(k - 1) * yst + i], s0);
+          lu[q] = fma(-0.5, s0 + s1, Y[(size_t)t * yst + i]);
+        }
+        Yf = lu;
+        yf = n;
+        __syncthreads();
+        break;
+      }
+      if (cos <= 2.0f && chol_orth(Y, yst, n, k, G)) {
+        if (last) break;
+        continue;
+      }
+      __syncthreads();
+    }
+    // unit lengths; after a breakdown (all-zero or overflowed solve) a unit vector, from which the re-orthogonalisation
+    // and the next pass recover the direction.  Then modified Gram-Schmidt within clusters, by one warp, in descending
+    // order of the eigenvalues
+    for (int t = warp; t < k; t += nw) {
+      double* y = Y + (size_t)t * yst;
       double s = 0.0;
-      for (int i = 0; i < n; ++i) s += y[i] * y[i];
+      for (int i = lane; i < n; i += 32) s = fma(y[i], y[i], s);
+      s = warp_sum(s);
       if (s > 0.0 && isfinite(s)) {
-        s = 1.0 / sqrt(s);
-        for (int i = 0; i < n; ++i) y[i] *= s;
+        s = recip_sqrt(s);
+        for (int i = lane; i < n; i += 32) y[i] *= s;
       } else {
-        // a breakdown (all-zero or overflowed solve): restart from a unit vector, the
-        // re-orthogonalisation and the next pass recover the direction
-        for (int i = 0; i < n; ++i) y[i] = (i == (t * 7 + pass) % n) ? 1.0 : 0.0;
+        for (int i = lane; i < n; i += 32) y[i] = (i == (t * 7 + pass) % n) ? 1.0 : 0.0;
       }
     }
     __syncthreads();
-    // modified Gram-Schmidt within clusters, by warp 0, in descending order of the eigenvalues (one warp and no
-    // block barrier: the pairs are a dependent chain, and barriers between them cost more than the warp's sums)
     if (tid < 32) {
       for (int t = 1; t < k; ++t) {
         double* yt = Y + (size_t)t * yst;
@@ -568,120 +1051,93 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
       }
     }
     __syncthreads();
+    if (last) break;
   }
-
-  // 4. back-transformation x = H_0 H_1 ... H_{n-3} y (one warp per vector; the reflectors are read-only)
-  for (int t = warp; t < k; t += nw) {
-    double* yv = Y + (size_t)t * yst;
-    for (int j = n - 3; j >= 0; --j) {
-      const double b = beta[j];
-      if (b == 0.0) continue;
-      const int m = n - j - 1;
-      double* y = yv + (j + 1);
-      double s = 0.0;
-      for (int i = lane; i < m; i += 32) s += W[(size_t)(j + 1 + i) * wld + j] * y[i];
-      s = b * warp_sum(s);
-      for (int i = lane; i < m; i += 32) y[i] -= s * W[(size_t)(j + 1 + i) * wld + j];
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-
   }  // tnorm != 0
   __syncthreads();
 
   // outputs: eigenvalues descending, eigenvectors as the first k columns of V (leading dimension ldv)
-  for (int t = tid; t < min(kv, n); t += nthr) wout[t] = t < k ? lam[t] : g.lam[t];
-  if (!viaB) {
-    for (size_t q = tid; q < (size_t)k * n; q += nthr) {
-      int t = (int)(q / n), i = (int)(q - (q / n) * n);
-      Vout[(size_t)i * ldv + t] = Y[(size_t)t * yst + i];
+  for (int t = tid; t < min(kv, n); t += nthr) wout[t] = (t < k ? lam[t] : g.lam[t]) * g.hdr[4];
+  if (have_q && tnorm != 0.0) {
+    // 4. back-transformation V = Q Y
+    for (int q = tid; q < k * n; q += nthr) {
+      const int i = q / k, t = q - i * k;
+      const double* qi = W + (size_t)i * wld;
+      const double* y = Yf + (size_t)t * yf;
+      double s0 = 0.0, s1 = 0.0;
+      int l = 0;
+      for (; l + 1 < n; l += 2) {
+        s0 = fma(qi[l], y[l], s0);
+        s1 = fma(qi[l + 1], y[l + 1], s1);
+      }
+      if (l < n) s0 = fma(qi[l], y[l], s0);
+      Vout[(size_t)i * ldv + t] = s0 + s1;
     }
     return;
   }
-  // left vectors u_t = B w_t / sigma_t (length nA, vector-major in lu, which inverse iteration no longer
-  // needs), then modified Gram-Schmidt (twice) in descending order, completed by unit vectors where
-  // sigma_t vanishes or B has fewer than kl singular values; at most min(kl, nA) columns
-  double* U = lu;
-  const double* B = Bg + (size_t)blockIdx.x * nnl;
-  for (size_t q = tid; q < (size_t)k * nA; q += nthr) {
-    const int t = (int)(q / nA), i = (int)(q - (q / nA) * nA);
-    const double sg = lam[t] > 0.0 ? sqrt(lam[t]) : 0.0;
-    double acc = 0.0;
-    for (int l = 0; l < n; ++l) acc = fma(B[(size_t)i * nl + l], Y[(size_t)t * yst + l], acc);
-    U[q] = sg > 0.0 ? acc / sg : 0.0;
-  }
-  __syncthreads();
-  const int kout = min(kl, nA);
-  if (tid < 32) {
-    int next_unit = 0;
-    for (int t = 0; t < kout; ++t) {
-      double* ut = U + (size_t)t * nA;
-      if (t >= k) {
-        for (int i = tid; i < nA; i += 32) ut[i] = 0.0;
-      }
-      for (int attempt = 0; attempt <= nA; ++attempt) {
-        double n0 = 0.0;
-        for (int i = tid; i < nA; i += 32) n0 += ut[i] * ut[i];
-        n0 = warp_sum(n0);
-        for (int pass = 0; pass < 2; ++pass)
-          for (int s2 = 0; s2 < t; ++s2) {
-            const double* us = U + (size_t)s2 * nA;
-            double dp = 0.0;
-            for (int i = tid; i < nA; i += 32) dp += us[i] * ut[i];
-            dp = warp_sum(dp);
-            for (int i = tid; i < nA; i += 32) ut[i] -= dp * us[i];
-          }
-        double n1 = 0.0;
-        for (int i = tid; i < nA; i += 32) n1 += ut[i] * ut[i];
-        n1 = warp_sum(n1);
-        if (n0 > 0.0 && n1 > 0.25 * n0) {
-          const double sc = 1.0 / sqrt(n1);
-          for (int i = tid; i < nA; i += 32) ut[i] *= sc;
-          break;
-        }
-        // no usable direction: restart from the next unit vector
-        const int uidx = next_unit++ % nA;
-        for (int i = tid; i < nA; i += 32) ut[i] = (i == uidx) ? 1.0 : 0.0;
+  if (tnorm != 0.0) {
+    // x = H_0 H_1 ... H_{n-3} y, one warp per vector (the reflectors are read-only)
+    for (int t = warp; t < k; t += nw) {
+      double* yv = Yf + (size_t)t * yf;
+      for (int j = n - 3; j >= 0; --j) {
+        const double b = beta[j];
+        if (b == 0.0) continue;
+        const int m = n - j - 1;
+        double* y = yv + (j + 1);
+        double s = 0.0;
+        for (int i = lane; i < m; i += 32) s += W[(size_t)(j + 1 + i) * wld + j] * y[i];
+        s = b * warp_sum(s);
+        for (int i = lane; i < m; i += 32) y[i] -= s * W[(size_t)(j + 1 + i) * wld + j];
         __syncwarp();
       }
-      __syncwarp();
     }
+    __syncthreads();
   }
-  __syncthreads();
-  for (size_t q = tid; q < (size_t)kout * nA; q += nthr) {
-    const int t = (int)(q / nA), i = (int)(q - (q / nA) * nA);
-    Vout[(size_t)i * ldv + t] = U[q];
+  for (size_t q = tid; q < (size_t)k * n; q += nthr) {
+    int t = (int)(q / n), i = (int)(q - (q / n) * n);
+    Vout[(size_t)i * ldv + t] = Yf[(size_t)t * yf + i];
   }
 }
 
-
 // k eigenvectors and kv >= k eigenvalues of every item
 static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch,
-                         const int* nA, const int* nB, const double* A2, const double* B, int kv = 0) {
+                         const int* nA, int kv = 0) {
   if (n <= 0 || batch <= 0 || k <= 0) return;
   k = std::min(k, n);
   kv = std::min(n, std::max(k, kv));
   LRFG_REQUIRE(kv < 65536 && batch < 65536, "eigensolver grid too large (k = %d, batch = %d)", k, batch);
   DBuf<double> scratch(ctx->pool, syevx_scratch_per(n, k) * batch);
   const size_t lim = (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
-  const size_t wbytes = sizeof(double) * (size_t)n * n;
-  // K1: the reflectors in shared memory when they fit
-  const size_t head1 = sizeof(double) * (40 + 2 * (size_t)n);
-  const int smem_w1 = head1 + wbytes <= lim ? 1 : 0;
-  const size_t smem1 = head1 + (smem_w1 ? wbytes : 0);
-  LRFG_CUDA(raise_smem_limit((const void*)syevx_tri_kernel, smem1));
-  // algorithmic work at the active size, counted by each block on the device
-  LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
-              syevx_tri_kernel<<<batch, kSyevxThreads, smem1, ctx->stream>>>(A, n, k, w, V, n, scratch.get(),
-                                                                             smem_w1, nA, nB, A2, B,
-                                                                             work_counter(ctx, KC_EIGEN)));
-  // K2: one warp per wanted eigenvalue of every item
-  const size_t smem2 = sizeof(double) * 3 * (size_t)n;
+  // K1: the register kernel up to n = 96; above, the reflectors in shared memory when they fit.  Algorithmic work at the
+  // active size, counted by each block on the device
+  auto tri_small = [&](auto kernel, int threads) {
+    LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
+                kernel<<<batch, threads, 0, ctx->stream>>>(A, n, k, w, V, n, scratch.get(), nA,
+                                                          work_counter(ctx, KC_EIGEN)));
+  };
+  if (n <= 32) {
+    tri_small(syevx_tri_small_kernel<1, 3>, 128);
+  } else if (n <= 64) {
+    tri_small(syevx_tri_small_kernel<2, 3>, 128);
+  } else if (n <= kSmallEig) {
+    tri_small(syevx_tri_small_kernel<3, 6>, 224);
+  } else {
+    const size_t wbytes = sizeof(double) * (size_t)n * n;
+    const size_t head1 = sizeof(double) * (40 + 2 * (size_t)n);
+    const int smem_w1 = head1 + wbytes <= lim ? 1 : 0;
+    const size_t smem1 = head1 + (smem_w1 ? wbytes : 0);
+    LRFG_CUDA(raise_smem_limit((const void*)syevx_tri_kernel, smem1));
+    LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
+                syevx_tri_kernel<<<batch, kSyevxThreads, smem1, ctx->stream>>>(A, n, k, w, V, n, scratch.get(), smem_w1,
+                                                                               nA, work_counter(ctx, KC_EIGEN)));
+  }
+  // K2: one block per wanted eigenvalue of every item, and the blocks that form Q
+  const int nq = n <= kSmallEig ? (n + kQCols - 1) / kQCols : 0;
+  const size_t smem2 = sizeof(double) * std::max(3 * (size_t)n, nq ? (size_t)kQCols * (n | 1) : (size_t)0);
   LRFG_CUDA(raise_smem_limit((const void*)syevx_bisect_kernel, smem2));
   LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
-              syevx_bisect_kernel<<<dim3((unsigned)kv, (unsigned)batch), 32, smem2, ctx->stream>>>(n, k, kv,
-                                                                                                 scratch.get()));
+              syevx_bisect_kernel<<<dim3((unsigned)(kv + nq), (unsigned)batch), kBisectThreads, smem2, ctx->stream>>>(
+                  n, k, kv, scratch.get()));
   // K3: the vectors, then their LU factors, then the reflectors in shared memory while they fit
   const size_t head3 = sizeof(double) * (3 * (size_t)n + (size_t)k);
   int flags3 = head3 <= lim ? 8 : 0;
@@ -694,27 +1150,28 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
       smem3 += parts[q];
       flags3 |= 1 << q;
     }
+  // and the Gram matrix of the vectors' orthonormalisation
+  const size_t gram3 = sizeof(double) * ((size_t)k * (k | 1) + k);
+  if (smem3 + gram3 <= lim) {
+    smem3 += gram3;
+    flags3 |= 16;
+  }
   LRFG_CUDA(raise_smem_limit((const void*)syevx_vec_kernel, smem3));
   LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
               syevx_vec_kernel<<<batch, kSyevxThreads, smem3, ctx->stream>>>(n, k, kv, w, V, n, scratch.get(),
-                                                                             flags3, B));
+                                                                             flags3));
 }
 
 void syevx(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch) {
-  syevx_launch(ctx, A, w, V, n, k, batch, nullptr, nullptr, nullptr, nullptr);
+  syevx_launch(ctx, A, w, V, n, k, batch, nullptr);
 }
 
 void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int kv, int batch) {
-  syevx_launch(ctx, A, w, V, n, k, batch, nullptr, nullptr, nullptr, nullptr, kv);
+  syevx_launch(ctx, A, w, V, n, k, batch, nullptr, kv);
 }
 
 void syevx_sized(lrfg_ctx* ctx, const double* A, const int* n_eff, double* w, double* V, int n, int k, int batch) {
-  syevx_launch(ctx, A, w, V, n, k, batch, n_eff, nullptr, nullptr, nullptr);
-}
-
-void syevx_product(lrfg_ctx* ctx, const double* BBt, const double* BtB, const double* B, const int* nA,
-                   const int* nB, double* w, double* V, int n, int k, int batch) {
-  syevx_launch(ctx, BBt, w, V, n, k, batch, nA, nB, BtB, B);
+  syevx_launch(ctx, A, w, V, n, k, batch, n_eff);
 }
 
 }  // namespace lrfg
