@@ -934,8 +934,8 @@ void solve_full(lrfg_problem* P, const double* E, lrfg_result* res, lrfg_field**
   int it = 0;
   double rel = nb > 0.0 ? 1.0 : 0.0;
   // Small grids queue the next step before the residual of this one is read on the host, so that the device does not
-  // wait for the host's answer (with the fused passes 8.0 -> 5.7 ms for the 62 steps of a 63 x 63 solve); the step queued
-  // past the last one changes p and q only and is dropped.  From 2^20 elements on a step takes over 100 us and the spare one would cost
+  // wait for the host's answer (about 15 us a step); the step queued past the last one touches neither u nor r's
+  // predecessors' results and is dropped.  From 2^20 elements on a step takes over 100 us and the spare one would cost
   // more than the waits.
   const bool ahead = n < (1LL << 20);
   auto step_product = [&]() {
