@@ -558,29 +558,26 @@ void lr_apply(lrfg_problem* P, const TTView& v, TT& out, int r, bool mixed = fal
   TTBatch w;
   TT wa[3];
   TTView terms[3];
+  SketchSource z;
+  z.kind = SketchSource::KHATRI_RAO;
+  z.d = d;
+  z.nb = d;
+  z.x = a;
+  for (int j = 0; j < 3; ++j) z.N[j] = v.N[j];
+  for (int j = 0; j <= d; ++j) {
+    z.s[j] = rk[j];
+    z.ry[j] = v.r[j];
+  }
+  for (int alpha = 0; alpha < d; ++alpha)
+    for (int j = 0; j < d; ++j) z.y[j][alpha] = (j == alpha) ? grad[j].get() : v.core[j];
   if (om && !P->aniso) {
     // randomised rounding of the d products, which are never formed
-    SketchSource z;
-    z.kind = SketchSource::KHATRI_RAO;
-    z.d = d;
-    z.nb = d;
-    z.x = a;
-    for (int j = 0; j < 3; ++j) z.N[j] = v.N[j];
-    for (int j = 0; j <= d; ++j) {
-      z.s[j] = rk[j];
-      z.ry[j] = v.r[j];
-    }
-    for (int alpha = 0; alpha < d; ++alpha)
-      for (int j = 0; j < d; ++j) z.y[j][alpha] = (j == alpha) ? grad[j].get() : v.core[j];
     tt_round_sketch(ctx, z, *om, r, w, tol, mixed, !P->opts.sketch_keep);  // T, all components in one sweep
     for (auto& g : grad) g.reset();
     for (int alpha = 0; alpha < d; ++alpha) terms[alpha] = item_view(w, alpha);
   } else {
     ttb_alloc(ctx, kr, d, v.N, rk, d);
-    for (int alpha = 0; alpha < d; ++alpha)
-      for (int j = 0; j < d; ++j)
-        khatri_rao(ctx, a.core[j], a.r[j], a.N[j], a.r[j + 1], (j == alpha) ? grad[j].get() : v.core[j], v.r[j],
-                   v.r[j + 1], kr.core[j].get() + (size_t)alpha * kr.elems(j));
+    for (int j = 0; j < d; ++j) z.materialise(ctx, j, kr.core[j].get());
   }
   if (om && !P->aniso) {
     // done above
@@ -934,8 +931,8 @@ void solve_full(lrfg_problem* P, const double* E, lrfg_result* res, lrfg_field**
   int it = 0;
   double rel = nb > 0.0 ? 1.0 : 0.0;
   // Small grids queue the next step before the residual of this one is read on the host, so that the device does not
-  // wait for the host's answer (about 15 us a step); the step queued past the last one touches neither u nor r's
-  // predecessors' results and is dropped.  From 2^20 elements on a step takes over 100 us and the spare one would cost
+  // wait for the host's answer (with the fused passes 8.0 -> 5.7 ms for the 62 steps of a 63 x 63 solve); the step queued
+  // past the last one changes p and q only and is dropped.  From 2^20 elements on a step takes over 100 us and the spare one would cost
   // more than the waits.
   const bool ahead = n < (1LL << 20);
   auto step_product = [&]() {
@@ -1152,34 +1149,39 @@ void apply_batch(lrfg_problem* P, const TTBatchView& v, TTBatch& out, int r, boo
   for (int j = 0; j <= d; ++j) rk[j] = a.r[j] * v.r[j];
   const int m = d * nb;
   TTBatch w;
-  if (om) {
-    LRFG_REQUIRE(m <= kMaxSketchItems, "too many right-hand sides for one lockstep batch (%d)", nb);
-    SketchSource z;
-    z.kind = SketchSource::KHATRI_RAO;
-    z.d = d;
-    z.nb = m;
-    z.x = a;
-    for (int j = 0; j < 3; ++j) z.N[j] = v.N[j];
-    for (int j = 0; j <= d; ++j) {
-      z.s[j] = rk[j];
-      z.ry[j] = v.r[j];
-    }
+  LRFG_REQUIRE(!om || m <= kMaxSketchItems, "too many right-hand sides for one lockstep batch (%d)", nb);
+  SketchSource z;
+  z.kind = SketchSource::KHATRI_RAO;
+  z.d = d;
+  z.nb = m;
+  z.x = a;
+  for (int j = 0; j < 3; ++j) z.N[j] = v.N[j];
+  for (int j = 0; j <= d; ++j) {
+    z.s[j] = rk[j];
+    z.ry[j] = v.r[j];
+  }
+  if (m <= kMaxSketchItems)
     for (int al = 0; al < d; ++al)
       for (int b = 0; b < nb; ++b)
         for (int j = 0; j < d; ++j) {
           z.y[j][al * nb + b] = (j == al ? grad[j].get() : v.core[j]) + (size_t)b * v.elems(j);
           if (Ps) z.xi[j][al * nb + b] = coeff_core(b, j);
         }
+  if (om) {
     tt_round_sketch(ctx, z, *om, r, w, 0.0, mixed, !P->opts.sketch_keep);
   } else {
     TTBatch kr;
     ttb_alloc(ctx, kr, d, v.N, rk, m);
-    for (int al = 0; al < d; ++al)
-      for (int b = 0; b < nb; ++b)
-        for (int j = 0; j < d; ++j)
-          khatri_rao(ctx, coeff_core(b, j), a.r[j], a.N[j], a.r[j + 1],
-                     (j == al ? grad[j].get() : v.core[j]) + (size_t)b * v.elems(j), v.r[j], v.r[j + 1],
-                     kr.core[j].get() + (size_t)(al * nb + b) * kr.elems(j));
+    if (m <= kMaxSketchItems) {
+      for (int j = 0; j < d; ++j) z.materialise(ctx, j, kr.core[j].get());
+    } else {
+      for (int al = 0; al < d; ++al)
+        for (int b = 0; b < nb; ++b)
+          for (int j = 0; j < d; ++j)
+            khatri_rao(ctx, coeff_core(b, j), a.r[j], a.N[j], a.r[j + 1],
+                       (j == al ? grad[j].get() : v.core[j]) + (size_t)b * v.elems(j), v.r[j], v.r[j + 1],
+                       kr.core[j].get() + (size_t)(al * nb + b) * kr.elems(j));
+    }
     tt_round_batch(ctx, batch_view(kr), r, w, 0.0);
   }
   for (auto& g : grad) g.reset();
@@ -1194,7 +1196,7 @@ void apply_batch(lrfg_problem* P, const TTBatchView& v, TTBatch& out, int r, boo
     terms[al] = t;
   }
   TTBatch acc;
-  ttb_add_many(ctx, terms, d, nullptr, nullptr, acc);
+  block_sum(ctx, terms, d, nullptr, nullptr, acc);
   w = TTBatch();
   TTBatch sdiv;
   tt_round_batch(ctx, batch_view(acc), r, sdiv, 0.0);          // T after the sum
@@ -1298,7 +1300,7 @@ void solve_tt_many(lrfg_problem* P, const double* E, int nb, lrfg_result* res, l
     TTBatchView t[2] = {batch_view(b), batch_view(cu)};
     const double hs[2] = {1.0, -1.0};
     TTBatch diff;
-    ttb_add_many(ctx, t, 2, hs, nullptr, diff);
+    block_sum(ctx, t, 2, hs, nullptr, diff);
     TTBatch rn;
     tt_round_batch(ctx, batch_view(diff), rk, rn, 0.0);
     r = std::move(rn);
@@ -1383,11 +1385,11 @@ void solve_tt_many(lrfg_problem* P, const double* E, int nb, lrfg_result* res, l
     if (u_zero) {
       TTBatchView t = batch_view(r);
       const double* ds[1] = {om_dev.get()};
-      ttb_add_many(ctx, &t, 1, nullptr, ds, sum);
+      block_sum(ctx, &t, 1, nullptr, ds, sum);
     } else {
       TTBatchView t[2] = {batch_view(u), batch_view(r)};
       const double* ds[2] = {nullptr, om_dev.get()};
-      ttb_add_many(ctx, t, 2, nullptr, ds, sum);
+      block_sum(ctx, t, 2, nullptr, ds, sum);
     }
     TTBatch un;
     tt_round_batch(ctx, batch_view(sum), rk, un, 0.0);

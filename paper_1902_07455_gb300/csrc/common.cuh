@@ -56,6 +56,7 @@ class DevicePool {
   void* alloc(size_t bytes);
   void release(void* p);
   void trim();
+  size_t budget() const { return budget_; }
   size_t in_use() const { return in_use_; }
   size_t reserved() const { return reserved_; }
   // high-water mark of in_use() since the last reset_peak()

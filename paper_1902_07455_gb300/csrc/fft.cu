@@ -592,14 +592,20 @@ void fibre_operator(lrfg_ctx* ctx, const double* in, double* out, long long oute
 }
 
 // Many Gaussian multipliers of one input: the forward transform is shared, each term m gets its own
-// multiply + inverse transform and is written to out + m * out_stride.
+// multiply + inverse transform and is written to out + m * out_stride.  The nodes and scales travel as a kernel argument
+// (two copies from host memory per call before).
+constexpr int kMaxGaussTerms = 64;
+struct GaussTerms {
+  double t[kMaxGaussTerms], s[kMaxGaussTerms];
+};
+
 template <typename V>
 __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __restrict__ in, double* out,
                                                                 long long out_stride, long long outer, int N,
                                                                 long long inner, int TF, FftPlan pl,
                                                                 const V* __restrict__ Wg,
-                                                                const double* __restrict__ tm,
-                                                                const double* __restrict__ sc, int nm, int mper) {
+                                                                const __grid_constant__ GaussTerms terms, int nm,
+                                                                int mper) {
   using R = typename RealOf<V>::T;
   extern __shared__ __align__(16) unsigned char smraw_gm[];
   V* sm = (V*)smraw_gm;
@@ -630,14 +636,14 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
   __syncthreads();
   const int m_end = min(nm, (int)(blockIdx.y + 1) * mper);
   for (int m = blockIdx.y * mper; m < m_end; ++m) {
-    const double t_m = tm[m];
+    const double t_m = terms.t[m];
     for (int t = threadIdx.x; t < rows * N; t += blockDim.x) {
       int k = freq_of(t % N, N);
       a[t] = cscale(spec[t], (R)exp(-t_m * (double)k * (double)k));
     }
     __syncthreads();
     V* r2 = stockham_rows<1>(a, b, rows, N, pl, W);
-    const double s = sc[m] / (double)N;
+    const double s = terms.s[m] / (double)N;
     double* o_m = out + (size_t)m * (size_t)out_stride;
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
       int f, n;
@@ -671,10 +677,11 @@ static void fibre_gauss_multi_t(lrfg_ctx* ctx, const double* in, double* out, lo
   const int mchunks = (int)std::max(1LL, std::min((long long)nm, (4LL * nsm + bx - 1) / bx));
   const int mper = (nm + mchunks - 1) / mchunks;
   size_t smem = (size_t)(N * sizeof(V) + tf * per);
-  // device copies of the node and scale tables
-  DBuf<double> dt(ctx->pool, nm), ds(ctx->pool, nm);
-  LRFG_CUDA(cudaMemcpyAsync(dt.get(), t, sizeof(double) * nm, cudaMemcpyHostToDevice, ctx->stream));
-  LRFG_CUDA(cudaMemcpyAsync(ds.get(), scale, sizeof(double) * nm, cudaMemcpyHostToDevice, ctx->stream));
+  GaussTerms terms{};
+  for (int m = 0; m < nm; ++m) {
+    terms.t[m] = t[m];
+    terms.s[m] = scale[m];
+  }
   long long nfib = outer * inner;
   long long blocks = (nfib + 2 * tf - 1) / (2 * tf);
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
@@ -685,16 +692,19 @@ static void fibre_gauss_multi_t(lrfg_ctx* ctx, const double* in, double* out, lo
   const int mgrid = (nm + mper - 1) / mper;
   LRFG_LAUNCH(ctx, KC_GAUSS_MULTI, flops, bytes,
               fibre_gauss_multi_kernel<V><<<dim3((unsigned)blocks, (unsigned)mgrid), 256, smem, ctx->stream>>>(
-                  in, out, out_stride, outer, N, inner, (int)tf, pl, Wt, dt.get(), ds.get(), nm, mper));
-  // the pool hands these blocks out again only to later work on the same stream
+                  in, out, out_stride, outer, N, inner, (int)tf, pl, Wt, terms, nm, mper));
 }
 
 void fibre_gauss_multi(lrfg_ctx* ctx, const double* in, double* out, long long out_stride, long long outer,
                        int N, long long inner, const double* t, const double* scale, int nm, bool fp32) {
   LRFG_REQUIRE(N >= 1 && (N % 2 == 1), "fibre length must be odd (got %d)", N);
   if (outer == 0 || inner == 0 || nm == 0) return;
-  if (fp32) fibre_gauss_multi_t<float2>(ctx, in, out, out_stride, outer, N, inner, t, scale, nm);
-  else fibre_gauss_multi_t<double2>(ctx, in, out, out_stride, outer, N, inner, t, scale, nm);
+  for (int m = 0; m < nm; m += kMaxGaussTerms) {
+    const int q = std::min(kMaxGaussTerms, nm - m);
+    double* o = out + (size_t)m * (size_t)out_stride;
+    if (fp32) fibre_gauss_multi_t<float2>(ctx, in, o, out_stride, outer, N, inner, t + m, scale + m, q);
+    else fibre_gauss_multi_t<double2>(ctx, in, o, out_stride, outer, N, inner, t + m, scale + m, q);
+  }
 }
 
 

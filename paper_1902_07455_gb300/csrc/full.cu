@@ -887,7 +887,7 @@ __device__ __forceinline__ double block_sum256(double s, double* red) {
 
 // Stores this block's NV partial sums and returns true in the last block of the launch to arrive, whose every thread
 // then holds the totals, summed in block order: the same bits whichever block arrives last.  The counter is zero
-// between launches.  It replaces a second launch for the partials (about 5 us of a small solve's step, three a step).
+// between launches.  It replaces a second launch for the partials (8 us under event timing, three a CG step).
 template <int NV>
 __device__ bool last_block_sum(const double* mine, double* partial, unsigned int* counter, double* red, double* total) {
   __shared__ unsigned int s_last;
@@ -1048,7 +1048,7 @@ void energy_sum(lrfg_ctx* ctx, const FullGrid& g, const R* e, const R* a, double
 //              costs one reciprocal per element); the last block forms beta;
 //   direction  u += alpha p and p = P^-1 r + beta p.
 // 10 vector transfers a step with the product <p, q> (2 + 3 + 5) where separate updates, products and directions took
-// 15; on 243^3 in FP32 the vector part of a step went from 0.19 to 0.12 ms.
+// 15; on 243^3 in FP32 the vector part of a step went from 0.186 to 0.133 ms (the products' error-free sums bound the rest).
 // ------------------------------------------------------------------------------------------------
 // 1/(k.k): FP32 forms the correctly rounded reciprocal (the value of the table) without the table's scattered gather
 __device__ __forceinline__ float inv_kk_of(const float*, int kk) { return kk ? __frcp_rn((float)kk) : 0.f; }

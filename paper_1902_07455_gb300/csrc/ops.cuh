@@ -86,7 +86,7 @@ void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, i
 void syevx_sized(lrfg_ctx* ctx, const double* A, const int* n_eff, double* w, double* V, int n, int k, int batch);
 // Gram-SVD factors from a balanced Gram matrix G (b x b per item) and the balancing c: pivoted
 // Cholesky; writes RA (G ~ RA^T RA, nonzero rows first), RAc and Pc (b x b each per item; skipped when
-// null, and then c may be null), and the numerical rank into rho (may be null).
+// null), and the numerical rank into rho (may be null).  c null: no balancing (1).
 // tau: the pivoted Cholesky stops when the largest remaining pivot is below tau times the largest diagonal.
 void gram_factor(lrfg_ctx* ctx, const double* G, const double* c, int b, int batch, double* RA, double* RAc,
                  double* Pc, int* rho = nullptr, double tau = 1e-16);
@@ -132,6 +132,13 @@ void tt_copy(lrfg_ctx* ctx, const TTView& src, TT& dst);
 void tt_hadamard(lrfg_ctx* ctx, const TTView& x, const TTView& y, TT& out);
 // Khatri–Rao product of one carriage pair into dst: (a c) x n x (b e)
 void khatri_rao(lrfg_ctx* ctx, const double* x, int a, int n, int b, const double* y, int c, int e, double* dst);
+// out_i = sum_t s_t,i x_t,i in block form for every item i of a batch, m <= 8 terms (s_t,i = hs[t] * ds[t][i], either may
+// be null; the scale multiplies the first carriage)
+void block_sum(lrfg_ctx* ctx, const TTBatchView* xs, int m, const double* hs, const double* const* ds, TTBatch& out);
+// carriage of a sum of R trains of one shape per item: block m of item i at src + m bs + i a n b; block row (where = 0),
+// block diagonal (1) or block column (2)
+void stack_blocks(lrfg_ctx* ctx, const double* src, long long bs, int a, int n, int b, int R, int where, int items,
+                  double* out);
 // sum of nb TTs (views) in block form, each item scaled by scales[i] (on the first carriage)
 void tt_add_many(lrfg_ctx* ctx, const TTView* xs, const double* scales, int nb, TT& out);
 // out = alpha x + beta y; alpha_dev / beta_dev (may be null) are device scalars multiplying alpha/beta
@@ -199,10 +206,6 @@ void tt_round_sketch(lrfg_ctx* ctx, const SketchSource& z, const TTView& omega, 
 
 // ---- ttbatch.cu ---------------------------------------------------------------------------------
 TTView item_view_of(const TTBatchView& x, int b);
-// out_i = sum_t s_t,i x_t,i in block form for every item i (s_t,i = hs[t] * ds[t][i], either may be null; the
-// scale multiplies the first carriage)
-void ttb_add_many(lrfg_ctx* ctx, const TTBatchView* xs, int m, const double* hs, const double* const* ds,
-                  TTBatch& out);
 // out_dev[i] = <x_i, y_i>
 void ttb_dot_device(lrfg_ctx* ctx, const TTBatchView& x, const TTBatchView& y, double* out_dev);
 // out_i = T(P~^-1 x_i) (omega non-null: randomised rounding, one launch sequence for all items)

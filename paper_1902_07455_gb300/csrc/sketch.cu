@@ -269,13 +269,12 @@ __global__ void block_interleave_kernel(const double* __restrict__ tmp, int R, i
 static void cholqr2(lrfg_ctx* ctx, const double* A, int m, int l, int nb, double* Q) {
   const long long sa = (long long)m * l, sl = (long long)l * l;
   DBuf<double> G(ctx->pool, (size_t)sl * nb), RA(ctx->pool, (size_t)sl * nb), Pc(ctx->pool, (size_t)sl * nb);
-  DBuf<double> ones(ctx->pool, (size_t)l * nb), Q1(ctx->pool, (size_t)sa * nb);
-  fill(ctx, ones.get(), 1.0, (long long)l * nb);
+  DBuf<double> Q1(ctx->pool, (size_t)sa * nb);
   gemm(ctx, 1, 0, l, l, m, 1.0, A, l, sa, A, l, sa, 0.0, G.get(), l, sl, nb);
-  gram_factor(ctx, G.get(), ones.get(), l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
+  gram_factor(ctx, G.get(), nullptr, l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
   gemm(ctx, 0, 0, m, l, l, 1.0, A, l, sa, Pc.get(), l, sl, 0.0, Q1.get(), l, sa, nb);
   gemm(ctx, 1, 0, l, l, m, 1.0, Q1.get(), l, sa, Q1.get(), l, sa, 0.0, G.get(), l, sl, nb);
-  gram_factor(ctx, G.get(), ones.get(), l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
+  gram_factor(ctx, G.get(), nullptr, l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
   gemm(ctx, 0, 0, m, l, l, 1.0, Q1.get(), l, sa, Pc.get(), l, sl, 0.0, Q, l, sa, nb);
 }
 
@@ -515,25 +514,14 @@ void SketchSource::materialise(lrfg_ctx* ctx, int j, double* dst) const {
                                                                             p, ry[j], ry[j + 1], N[j], nb, dst));
     return;
   }
-  for (int b = 0; b < nb; ++b) {
-    double* o = dst + (size_t)b * e;
-    if (kind == DENSE) {
-      LRFG_CUDA(cudaMemcpyAsync(o, dense[j] + (size_t)b * e, sizeof(double) * e, cudaMemcpyDeviceToDevice,
-                                ctx->stream));
-    } else if (kind == KHATRI_RAO) {
-      khatri_rao(ctx, xi[j][b] ? xi[j][b] : x.core[j], x.r[j], N[j], x.r[j + 1], y[j][b], ry[j], ry[j + 1], o);
-    } else {
-      // exponential-sum blocks F_m of carriage j (r_j x N x r_{j+1} each, weights already in carriage 0)
-      const int R = nblocks, a = ry[j], c = ry[j + 1];
-      const long long be = (long long)a * N[j] * c, bs = bstride[j] ? bstride[j] : be;
-      const double* src = blocks[j] + (size_t)b * be;
-      if (j == 0) {
-        for (int m = 0; m < R; ++m) tt_embed(ctx, src + m * bs, 1, N[j], c, o, 1, R * c, 0, m * c);
-      } else {
-        for (int m = 0; m < R; ++m) tt_embed(ctx, src + m * bs, a, N[j], 1, o, R * a, 1, m * a, 0);
-      }
-    }
+  if (kind == DENSE) {
+    LRFG_CUDA(cudaMemcpyAsync(dst, dense[j], sizeof(double) * e * nb, cudaMemcpyDeviceToDevice, ctx->stream));
+    return;
   }
+  // exponential-sum blocks F_m of carriage j (r_j x N x r_{j+1} each, weights already in carriage 0)
+  const long long be = (long long)ry[j] * N[j] * ry[j + 1];
+  stack_blocks(ctx, blocks[j], bstride[j] ? bstride[j] : be, ry[j], N[j], ry[j + 1], nblocks,
+               j == 0 ? 0 : (j == d - 1 ? 2 : 1), nb, dst);
 }
 
 void SketchSource::right_middle(lrfg_ctx* ctx, const double* W, int ell, double* T) const {

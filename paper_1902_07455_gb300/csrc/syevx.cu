@@ -1336,7 +1336,7 @@ __global__ void __launch_bounds__(kCholThreads) gram_factor_kernel(const double*
     double v = 0.0;
     if (k < rho && pos[j] >= k) v = W[(size_t)j * b + perm[k]];
     RA[t] = v;
-    if (RAc) RAc[t] = v / c[j];
+    if (RAc) RAc[t] = c ? v / c[j] : v;
   }
   if (!Pc) return;
   // L11^{-1} in pivot order: L11[i][l] = W[perm[i]][perm[l]]; reciprocal diagonal first, then one thread per
@@ -1364,7 +1364,7 @@ __global__ void __launch_bounds__(kCholThreads) gram_factor_kernel(const double*
   for (size_t t = tid; t < bb; t += nthr) {
     const int r = (int)(t / b), q = (int)(t - (t / b) * b);  // Pc row r (original index), column q
     const int l = pos[r];
-    const double v = (l < rho && q < rho && q >= l) ? c[r] * Li[(size_t)q * b + l] : 0.0;
+    const double v = (l < rho && q < rho && q >= l) ? (c ? c[r] : 1.0) * Li[(size_t)q * b + l] : 0.0;
     Pc[t] = v;
   }
 }
@@ -1501,7 +1501,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     const int k = t / b, j = t - (t / b) * b;
     const double v = k < rho && pos[j] >= k ? Ls[(size_t)k * M + j] * rs[k] : 0.0;
     RA[t] = v;
-    if (RAc) RAc[t] = v / c[j];
+    if (RAc) RAc[t] = c ? v / c[j] : v;
   }
   if (!Pc) return;
   __syncthreads();
@@ -1523,7 +1523,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
   for (int t = tid; t < b * b; t += 32 * CW) {
     const int r = t / b, q = t - (t / b) * b;
     const int l = pos[r];
-    Pc[t] = l < rho && q < rho && q >= l ? c[r] * Ls[(size_t)l * M + q] : 0.0;
+    Pc[t] = l < rho && q < rho && q >= l ? (c ? c[r] : 1.0) * Ls[(size_t)l * M + q] : 0.0;
   }
 }
 

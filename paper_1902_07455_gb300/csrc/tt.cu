@@ -94,102 +94,168 @@ void tt_hadamard(lrfg_ctx* ctx, const TTView& x, const TTView& y, TT& out) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// a5: block sum alpha x + beta y; the scalars multiply the first carriage only
+// a5: block sums; the scalars multiply the first carriage only.  Every element of the sum is written once, by one launch
+// over all carriages and items (a fill and an embedding launch per term and carriage before: ten launches of about 3 us
+// for the sum of three gradient components).
 // ------------------------------------------------------------------------------------------------
+constexpr int kMaxSumTerms = 8;
+struct BlockSum {
+  int m, d;
+  int N[3];
+  int off[4][kMaxSumTerms + 1];       // rank offsets of the terms at every bond
+  const double* core[3][kMaxSumTerms];
+  long long stride[3][kMaxSumTerms];  // between the items of a batch
+  double s[kMaxSumTerms];
+  const double* sd[kMaxSumTerms];     // device scalars, one per item (may be null)
+  double* out[3];
+};
+
+// blockIdx.y: carriage, blockIdx.z: item
+__global__ void block_sum_kernel(const __grid_constant__ BlockSum t) {
+  const int j = blockIdx.y, item = blockIdx.z, n = t.N[j];
+  const int A = j == 0 ? 1 : t.off[j][t.m], B = j == t.d - 1 ? 1 : t.off[j + 1][t.m];
+  const long long total = (long long)A * n * B;
+  double* out = t.out[j] + item * total;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+    const long long rest = e / B;
+    const int ib = (int)(e - rest * B), ia = (int)(rest / n), nn = (int)(rest - (long long)ia * n);
+    int ta = 0, tb = 0;
+    if (j > 0)
+      while (ia >= t.off[j][ta + 1]) ++ta;
+    if (j < t.d - 1)
+      while (ib >= t.off[j + 1][tb + 1]) ++tb;
+    if (j == 0) ta = tb;
+    if (j == t.d - 1) tb = ta;
+    double v = 0.0;
+    if (ta == tb) {
+      const int oa = j == 0 ? 0 : t.off[j][ta], ob = j == t.d - 1 ? 0 : t.off[j + 1][ta];
+      const int b = j == t.d - 1 ? 1 : t.off[j + 1][ta + 1] - ob;
+      v = t.core[j][ta][item * t.stride[j][ta] + ((long long)(ia - oa) * n + nn) * b + (ib - ob)];
+      if (j == 0) v *= t.sd[ta] ? t.s[ta] * t.sd[ta][item] : t.s[ta];
+    }
+    out[e] = v;
+  }
+}
+
+void block_sum(lrfg_ctx* ctx, const TTBatchView* xs, int m, const double* hs, const double* const* ds, TTBatch& out) {
+  LRFG_REQUIRE(m >= 1 && m <= kMaxSumTerms, "block sum of %d tensor trains", m);
+  const int d = xs[0].d, nb = xs[0].nb;
+  LRFG_REQUIRE(d >= 2 && d <= 3 && nb >= 1 && nb < 65536, "block sum of order %d, %d items", d, nb);
+  BlockSum p{};
+  p.m = m;
+  p.d = d;
+  int r[4] = {1, 1, 1, 1};
+  for (int j = 0; j <= d; ++j) {
+    p.off[j][0] = 0;
+    for (int t = 0; t < m; ++t) p.off[j][t + 1] = p.off[j][t] + xs[t].r[j];
+    if (j > 0 && j < d) r[j] = p.off[j][m];
+  }
+  for (int t = 0; t < m; ++t) {
+    LRFG_REQUIRE(xs[t].d == d && xs[t].nb == nb, "sum of TTs of different order");
+    p.s[t] = hs ? hs[t] : 1.0;
+    p.sd[t] = ds ? ds[t] : nullptr;
+    for (int j = 0; j < d; ++j) {
+      LRFG_REQUIRE(xs[t].N[j] == xs[0].N[j], "sum of TTs on different grids");
+      p.core[j][t] = xs[t].core[j];
+      p.stride[j][t] = (long long)xs[t].elems(j);
+    }
+  }
+  ttb_alloc(ctx, out, d, xs[0].N, r, nb);
+  long long most = 0;
+  double all = 0.0;
+  for (int j = 0; j < d; ++j) {
+    p.N[j] = xs[0].N[j];
+    p.out[j] = out.core[j].get();
+    most = std::max(most, (long long)out.elems(j));
+    all += (double)out.elems(j) * nb;
+  }
+  LRFG_LAUNCH(ctx, KC_TT_MISC, all, 2.0 * sizeof(double) * all,
+              block_sum_kernel<<<dim3(grid1d(ctx, most), d, nb), 256, 0, ctx->stream>>>(p));
+}
+
+static TTBatchView one_item(const TTView& x) {
+  TTBatchView v{};
+  v.d = x.d;
+  v.nb = 1;
+  for (int j = 0; j < 3; ++j) {
+    v.N[j] = x.N[j];
+    v.core[j] = x.core[j];
+  }
+  for (int j = 0; j < 4; ++j) v.r[j] = x.r[j];
+  return v;
+}
+
+static void take_item(TTBatch&& b, TT& out) {
+  out.d = b.d;
+  for (int j = 0; j < 3; ++j) out.N[j] = b.N[j];
+  for (int j = 0; j < 4; ++j) out.r[j] = b.r[j];
+  for (int j = 0; j < b.d; ++j) out.core[j] = std::move(b.core[j]);
+}
+
+void tt_add_many(lrfg_ctx* ctx, const TTView* xs, const double* scales, int nb, TT& out) {
+  LRFG_REQUIRE(nb >= 1 && nb <= kMaxSumTerms, "block sum of %d tensor trains", nb);
+  TTBatchView v[kMaxSumTerms];
+  for (int i = 0; i < nb; ++i) v[i] = one_item(xs[i]);
+  TTBatch b;
+  block_sum(ctx, v, nb, scales, nullptr, b);
+  take_item(std::move(b), out);
+}
+
+void tt_add(lrfg_ctx* ctx, double alpha, const double* alpha_dev, const TTView& x, double beta, const double* beta_dev,
+            const TTView& y, TT& out) {
+  const TTBatchView v[2] = {one_item(x), one_item(y)};
+  const double hs[2] = {alpha, beta};
+  const double* ds[2] = {alpha_dev, beta_dev};
+  TTBatch b;
+  block_sum(ctx, v, 2, hs, ds, b);
+  take_item(std::move(b), out);
+}
+
+// block copy of a carriage (a x n x b) into a larger one
 __global__ void block_embed_kernel(const double* __restrict__ src, int a, int n, int b, double* dst, int A, int B,
-                                   int oa, int ob, double s, const double* __restrict__ s_dev) {
+                                   int oa, int ob) {
   const long long total = (long long)a * n * b;
-  const double sc = s_dev ? s * (*s_dev) : s;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
     int jb = (int)(t % b);
     long long rest = t / b;
     int nn = (int)(rest % n);
     int ia = (int)(rest / n);
-    dst[((size_t)(ia + oa) * n + nn) * B + (jb + ob)] = sc * src[t];
+    dst[((size_t)(ia + oa) * n + nn) * B + (jb + ob)] = src[t];
   }
-}
-
-static void embed(lrfg_ctx* ctx, const double* src, int a, int n, int b, double* dst, int A, int B, int oa, int ob,
-                  double s, const double* s_dev) {
-  long long total = (long long)a * n * b;
-  if (total == 0) return;
-  LRFG_LAUNCH(ctx, KC_TT_MISC, (double)total, 2.0 * sizeof(double) * total,
-              block_embed_kernel<<<grid1d(ctx, total), 256, 0, ctx->stream>>>(src, a, n, b, dst, A, B, oa, ob, s, s_dev));
 }
 
 void tt_embed(lrfg_ctx* ctx, const double* src, int a, int n, int b, double* dst, int A, int B, int oa, int ob) {
-  embed(ctx, src, a, n, b, dst, A, B, oa, ob, 1.0, nullptr);
+  const long long total = (long long)a * n * b;
+  if (total == 0) return;
+  LRFG_LAUNCH(ctx, KC_TT_MISC, 0.0, 2.0 * sizeof(double) * total,
+              block_embed_kernel<<<grid1d(ctx, total), 256, 0, ctx->stream>>>(src, a, n, b, dst, A, B, oa, ob));
 }
 
-void tt_add_many(lrfg_ctx* ctx, const TTView* xs, const double* scales, int nb, TT& out) {
-  LRFG_REQUIRE(nb >= 1, "empty sum");
-  const int d = xs[0].d;
-  int r[4];
-  r[0] = 1;
-  r[d] = 1;
-  for (int j = 1; j < d; ++j) {
-    r[j] = 0;
-    for (int i = 0; i < nb; ++i) r[j] += xs[i].r[j];
-  }
-  for (int i = 0; i < nb; ++i) {
-    LRFG_REQUIRE(xs[i].d == d, "sum of TTs of different order");
-    for (int j = 0; j < d; ++j) LRFG_REQUIRE(xs[i].N[j] == xs[0].N[j], "sum of TTs on different grids");
-  }
-  tt_alloc(ctx, out, d, xs[0].N, r);
-  for (int j = 0; j < d; ++j) {
-    double* dst = out.core[j].get();
-    const int A = r[j], B = r[j + 1], n = xs[0].N[j];
-    if (d > 1 && j != 0 && j != d - 1) fill(ctx, dst, 0.0, (long long)A * n * B);
-    int oa = 0, ob = 0;
-    for (int i = 0; i < nb; ++i) {
-      const TTView& x = xs[i];
-      if (d == 1) LRFG_REQUIRE(false, "use tt_add for order-1 tensors");
-      if (j == 0) embed(ctx, x.core[j], 1, n, x.r[1], dst, 1, B, 0, ob, scales ? scales[i] : 1.0, nullptr);
-      else if (j == d - 1) embed(ctx, x.core[j], x.r[j], n, 1, dst, A, 1, oa, 0, 1.0, nullptr);
-      else embed(ctx, x.core[j], x.r[j], n, x.r[j + 1], dst, A, B, oa, ob, 1.0, nullptr);
-      oa += x.r[j];
-      ob += x.r[j + 1];
-    }
+// Carriage of a sum of R trains of one shape (the exponential-sum product): block m of item i at src + m bs + i a n b,
+// (a, n, b) each; block-concatenated along its last index (where 0), block-diagonal (1), or along its first (2)
+__global__ void stack_blocks_kernel(const double* __restrict__ src, long long bs, int a, int n, int b, int R, int where,
+                                    double* __restrict__ out) {
+  const int A = where == 0 ? a : R * a, B = where == 2 ? b : R * b, item = blockIdx.y;
+  const long long total = (long long)A * n * B;
+  src += (size_t)item * a * n * b;
+  out += item * total;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+    const long long rest = e / B;
+    const int ib = (int)(e - rest * B), ia = (int)(rest / n), nn = (int)(rest - (long long)ia * n);
+    const int ma = where == 0 ? ib / b : ia / a, mb = where == 2 ? ma : ib / b;
+    out[e] = ma == mb ? src[ma * bs + ((long long)(where == 0 ? ia : ia - ma * a) * n + nn) * b +
+                            (where == 2 ? ib : ib - mb * b)]
+                      : 0.0;
   }
 }
 
-void tt_add(lrfg_ctx* ctx, double alpha, const double* alpha_dev, const TTView& x, double beta, const double* beta_dev,
-            const TTView& y, TT& out) {
-  LRFG_REQUIRE(x.d == y.d, "sum of TTs of different order");
-  const int d = x.d;
-  for (int j = 0; j < d; ++j) LRFG_REQUIRE(x.N[j] == y.N[j], "sum of TTs on different grids");
-  int r[4];
-  r[0] = 1;
-  r[d] = 1;
-  for (int j = 1; j < d; ++j) r[j] = x.r[j] + y.r[j];
-  tt_alloc(ctx, out, d, x.N, r);
-  for (int j = 0; j < d; ++j) {
-    double* dst = out.core[j].get();
-    const int A = r[j], B = r[j + 1], n = x.N[j];
-    if (d == 1) {
-      fill(ctx, dst, 0.0, (long long)n);
-      // out = alpha x + beta y elementwise (both 1 x n x 1)
-      embed(ctx, x.core[0], 1, n, 1, dst, 1, 1, 0, 0, alpha, alpha_dev);
-      // accumulate beta y: reuse axpby on a scaled copy
-      DBuf<double> tmp(ctx->pool, n);
-      embed(ctx, y.core[0], 1, n, 1, tmp.get(), 1, 1, 0, 0, beta, beta_dev);
-      axpby(ctx, n, 1.0, tmp.get(), 1.0, dst);
-      continue;
-    }
-    if (j != 0 && j != d - 1) fill(ctx, dst, 0.0, (long long)A * n * B);
-    const bool first = (j == 0);
-    if (j == 0) {
-      embed(ctx, x.core[j], 1, n, x.r[1], dst, 1, B, 0, 0, alpha, alpha_dev);
-      embed(ctx, y.core[j], 1, n, y.r[1], dst, 1, B, 0, x.r[1], beta, beta_dev);
-    } else if (j == d - 1) {
-      embed(ctx, x.core[j], x.r[j], n, 1, dst, A, 1, 0, 0, 1.0, nullptr);
-      embed(ctx, y.core[j], y.r[j], n, 1, dst, A, 1, x.r[j], 0, 1.0, nullptr);
-    } else {
-      embed(ctx, x.core[j], x.r[j], n, x.r[j + 1], dst, A, B, 0, 0, 1.0, nullptr);
-      embed(ctx, y.core[j], y.r[j], n, y.r[j + 1], dst, A, B, x.r[j], x.r[j + 1], 1.0, nullptr);
-    }
-    (void)first;
-  }
+void stack_blocks(lrfg_ctx* ctx, const double* src, long long bs, int a, int n, int b, int R, int where, int items,
+                  double* out) {
+  const long long total = (long long)(where == 0 ? a : R * a) * n * (where == 2 ? b : R * b);
+  if (total == 0) return;
+  LRFG_LAUNCH(ctx, KC_TT_MISC, 0.0, sizeof(double) * ((double)R * a * n * b + total) * items,
+              stack_blocks_kernel<<<dim3(grid1d(ctx, total), items), 256, 0, ctx->stream>>>(src, bs, a, n, b, R, where,
+                                                                                          out));
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -372,9 +438,8 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
     }
   }
   // left sweep
-  DBuf<double> Z(ctx->pool, x.elems(0) * nb);
-  LRFG_CUDA(cudaMemcpyAsync(Z.get(), x.core[0], sizeof(double) * x.elems(0) * nb, cudaMemcpyDeviceToDevice,
-                            ctx->stream));
+  const double* Z = x.core[0];
+  DBuf<double> Zbuf;
   for (int j = 0; j < d - 1; ++j) {
     if (tol > 0.0) rr[j + 1] = std::min(rmax, std::min(rr[j] * x.N[j], sp[j + 1]));  // cap after bond j-1
     const int a = rr[j], n = x.N[j], b = x.r[j + 1], kcap = rr[j + 1];
@@ -383,7 +448,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
     long long sbk = (long long)b * kcap, skk = (long long)kcap * kcap, sout = 0;
     int k = kcap;
     DBuf<double> GA(ctx->pool, (size_t)sbb * nb), cb(ctx->pool, (size_t)b * nb);
-    gemm(ctx, 1, 0, b, b, rows, 1.0, Z.get(), b, sz, Z.get(), b, sz, 0.0, GA.get(), b, sbb, nb);
+    gemm(ctx, 1, 0, b, b, rows, 1.0, Z, b, sz, Z, b, sz, 0.0, GA.get(), b, sbb, nb);
     const bool projected = (d == 3 && j == 0);
     if (projected) {
       const int n1 = x.N[1], b2 = x.r[2];
@@ -451,7 +516,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       syevx_sized(ctx, S.get(), rk.get(), sig.get(), US.get(), b, kcap, nb);
       settle_rank();
       gemm(ctx, 0, 0, b, k, b, 1.0, Pc.get(), b, sbb, US.get(), b, sbb, 0.0, P.get(), k, sbk, nb);
-      gemm(ctx, 0, 0, rows, k, b, 1.0, Z.get(), b, sz, P.get(), k, sbk, 0.0, out.core[j].get(), k, sout, nb);
+      gemm(ctx, 0, 0, rows, k, b, 1.0, Z, b, sz, P.get(), k, sbk, 0.0, out.core[j].get(), k, sout, nb);
       gemm(ctx, 1, 0, k, b, b, 1.0, US.get(), b, sbb, RAc.get(), b, sbb, 0.0, T.get(), b, sbk, nb);
     } else {
       // R ~ RB^T RB; the left singular vectors of X are those of M C RB^T (C the balancing): from the
@@ -470,27 +535,32 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
                       P0.get(), cb.get(), sig.get(), b, k));
       DBuf<double> Y0(ctx->pool, (size_t)rows * k * nb), G(ctx->pool, (size_t)skk * nb);
       DBuf<double> GR(ctx->pool, (size_t)skk * nb), GP(ctx->pool, (size_t)skk * nb);
-      gemm(ctx, 0, 0, rows, k, b, 1.0, Z.get(), b, sz, P0.get(), k, sbk, 0.0, Y0.get(), k, (long long)rows * k, nb);
+      gemm(ctx, 0, 0, rows, k, b, 1.0, Z, b, sz, P0.get(), k, sbk, 0.0, Y0.get(), k, (long long)rows * k, nb);
       gemm(ctx, 1, 0, k, k, rows, 1.0, Y0.get(), k, (long long)rows * k, Y0.get(), k, (long long)rows * k, 0.0,
            G.get(), k, skk, nb);
-      DBuf<double> ones(ctx->pool, (size_t)k * nb);
-      fill(ctx, ones.get(), 1.0, (long long)k * nb);
-      gram_factor(ctx, G.get(), ones.get(), k, nb, GR.get(), nullptr, GP.get(), nullptr);
+      gram_factor(ctx, G.get(), nullptr, k, nb, GR.get(), nullptr, GP.get(), nullptr);
       gemm(ctx, 0, 0, rows, k, k, 1.0, Y0.get(), k, (long long)rows * k, GP.get(), k, skk, 0.0, out.core[j].get(),
            k, sout, nb);
-      gemm(ctx, 1, 0, k, b, rows, 1.0, out.core[j].get(), k, sout, Z.get(), b, sz, 0.0, T.get(), b, sbk, nb);
+      gemm(ctx, 1, 0, k, b, rows, 1.0, out.core[j].get(), k, sout, Z, b, sz, 0.0, T.get(), b, sbk, nb);
     }
     // next left part: T (k x b) times carriage j+1 as b x (N s)
     const int n1 = x.N[j + 1], c1 = x.r[j + 2];
     const long long szn = (long long)k * n1 * c1;
-    DBuf<double> Zn(ctx->pool, (size_t)szn * nb);
+    // (the last one is the last carriage of the result)
+    DBuf<double> Zn;
+    double* zn = nullptr;
+    if (j == d - 2) {
+      if (tol > 0.0) out.core[d - 1] = DBuf<double>(ctx->pool, out.elems(d - 1) * nb);
+      zn = out.core[d - 1].get();
+    } else {
+      Zn = DBuf<double>(ctx->pool, (size_t)szn * nb);
+      zn = Zn.get();
+    }
     gemm(ctx, 0, 0, k, n1 * c1, b, 1.0, T.get(), b, sbk, x.core[j + 1], n1 * c1, (long long)x.elems(j + 1), 0.0,
-         Zn.get(), n1 * c1, szn, nb);
-    Z = std::move(Zn);
+         zn, n1 * c1, szn, nb);
+    Zbuf = std::move(Zn);
+    Z = zn;
   }
-  if (tol > 0.0) out.core[d - 1] = DBuf<double>(ctx->pool, out.elems(d - 1) * nb);
-  LRFG_CUDA(cudaMemcpyAsync(out.core[d - 1].get(), Z.get(), sizeof(double) * out.elems(d - 1) * nb,
-                            cudaMemcpyDeviceToDevice, ctx->stream));
 }
 
 void ttb_alloc(lrfg_ctx* ctx, TTBatch& x, int d, const int* N, const int* r, int nb) {
@@ -524,18 +594,9 @@ TTView item_view(const TTBatch& x, int b) {
 
 void tt_round(lrfg_ctx* ctx, const TTView& x, int rmax, TT& out, double tol) {
   if (x.d == 1) { tt_copy(ctx, x, out); return; }
-  TTBatchView bv{};
-  bv.d = x.d;
-  bv.nb = 1;
-  for (int j = 0; j < 3; ++j) bv.N[j] = x.N[j];
-  for (int j = 0; j < 4; ++j) bv.r[j] = x.r[j];
-  for (int j = 0; j < x.d; ++j) bv.core[j] = x.core[j];
   TTBatch ob;
-  tt_round_batch(ctx, bv, rmax, ob, tol);
-  out.d = ob.d;
-  for (int j = 0; j < 3; ++j) out.N[j] = ob.N[j];
-  for (int j = 0; j < 4; ++j) out.r[j] = ob.r[j];
-  for (int j = 0; j < ob.d; ++j) out.core[j] = std::move(ob.core[j]);
+  tt_round_batch(ctx, one_item(x), rmax, ob, tol);
+  take_item(std::move(ob), out);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -543,19 +604,23 @@ void tt_round(lrfg_ctx* ctx, const TTView& x, int rmax, TT& out, double tol) {
 // ------------------------------------------------------------------------------------------------
 void tt_dot_device(lrfg_ctx* ctx, const TTView& x, const TTView& y, double* out_dev) {
   LRFG_REQUIRE(x.d == y.d, "dot of TTs of different order");
-  DBuf<double> W(ctx->pool, 1);
-  fill(ctx, W.get(), 1.0, 1);
+  DBuf<double> W;
   for (int j = 0; j < x.d; ++j) {
     const int a = x.r[j], b = x.r[j + 1], c = y.r[j], e = y.r[j + 1], n = x.N[j];
     LRFG_REQUIRE(n == y.N[j], "dot of TTs on different grids");
-    // V (c x (n b)) = W^T (c x a) * x_j (a x (n b))
-    DBuf<double> V(ctx->pool, (size_t)c * n * b);
-    gemm(ctx, 1, 0, c, n * b, a, 1.0, W.get(), c, 0, x.core[j], n * b, 0, 0.0, V.get(), n * b, 0);
+    // V (c x (n b)) = W^T (c x a) * x_j (a x (n b)); W = 1 at the first carriage
+    DBuf<double> Vb;
+    const double* V = x.core[0];
+    if (j > 0) {
+      Vb = DBuf<double>(ctx->pool, (size_t)c * n * b);
+      V = Vb.get();
+      gemm(ctx, 1, 0, c, n * b, a, 1.0, W.get(), c, 0, x.core[j], n * b, 0, 0.0, Vb.get(), n * b, 0);
+    }
     // W' (b x e) = V^T ((c n) x b)^T * y_j ((c n) x e)
     double* dst = (j == x.d - 1) ? out_dev : nullptr;
     DBuf<double> Wn;
     if (!dst) { Wn = DBuf<double>(ctx->pool, (size_t)b * e); dst = Wn.get(); }
-    gemm(ctx, 1, 0, b, e, c * n, 1.0, V.get(), b, 0, y.core[j], e, 0, 0.0, dst, e, 0);
+    gemm(ctx, 1, 0, b, e, c * n, 1.0, V, b, 0, y.core[j], e, 0, 0.0, dst, e, 0);
     if (j != x.d - 1) W = std::move(Wn);
   }
 }
@@ -721,70 +786,9 @@ void expsum_inverse(double xmax, double eps, std::vector<double>& t, std::vector
 
 void tt_precond(lrfg_ctx* ctx, const TTView& x, const std::vector<double>& t, const std::vector<double>& w, int rmax,
                 TT& out, double tol, const TTView* omega, bool fp32, bool final) {
-  // P~^-1 x = sum_m w_m (G_m x ... x G_m) x with G_m = F^-1 diag(exp(-t_m k^2)) F per mode: a TT whose
-  // carriages are block rows (first), block diagonal (middle) and block columns (last) over m.
-  const int d = x.d;
-  const int R = (int)t.size();
-  int r[4];
-  r[0] = 1;
-  r[d] = 1;
-  for (int j = 1; j < d; ++j) r[j] = R * x.r[j];
-  std::vector<double> ones(R, 1.0);
-  if (omega && d >= 2) {
-    // randomised rounding: the blocks G_m x_j enter the sketch contractions as they are (never embedded in the
-    // block-diagonal carriage)
-    SketchSource z;
-    z.kind = SketchSource::BLOCKS;
-    z.d = d;
-    z.nb = 1;
-    z.nblocks = R;
-    DBuf<double> terms[3];
-    for (int j = 0; j < d; ++j) {
-      z.N[j] = x.N[j];
-      const size_t e = (size_t)x.r[j] * x.N[j] * x.r[j + 1];
-      terms[j] = DBuf<double>(ctx->pool, e * R);
-      fibre_gauss_multi(ctx, x.core[j], terms[j].get(), (long long)e, x.r[j], x.N[j], x.r[j + 1], t.data(),
-                        (j == 0) ? w.data() : ones.data(), R, fp32);
-      z.blocks[j] = terms[j].get();
-    }
-    for (int j = 0; j <= d; ++j) {
-      z.s[j] = r[j];
-      z.ry[j] = x.r[j];
-    }
-    TTBatch ob;
-    tt_round_sketch(ctx, z, *omega, rmax, ob, tol, fp32, final);
-    out.d = ob.d;
-    for (int j = 0; j < 3; ++j) out.N[j] = ob.N[j];
-    for (int j = 0; j < 4; ++j) out.r[j] = ob.r[j];
-    for (int j = 0; j < ob.d; ++j) out.core[j] = std::move(ob.core[j]);
-    return;
-  }
-  TT big;
-  tt_alloc(ctx, big, d, x.N, r);
-  for (int j = 0; j < d; ++j) {
-    const int a = x.r[j], n = x.N[j], b = x.r[j + 1];
-    const size_t e = (size_t)a * n * b;
-    DBuf<double> terms(ctx->pool, e * R);
-    fibre_gauss_multi(ctx, x.core[j], terms.get(), (long long)e, a, n, b, t.data(), (j == 0) ? w.data() : ones.data(), R,
-                      fp32);
-    double* dst = big.core[j].get();
-    if (d > 1 && j != 0 && j != d - 1) fill(ctx, dst, 0.0, (long long)r[j] * n * r[j + 1]);
-    for (int m = 0; m < R; ++m) {
-      const double* src = terms.get() + m * e;
-      if (d == 1) {
-        // single mode: plain sum of the terms
-        if (m == 0) LRFG_CUDA(cudaMemcpyAsync(dst, src, sizeof(double) * e, cudaMemcpyDeviceToDevice, ctx->stream));
-        else axpby(ctx, (long long)e, 1.0, src, 1.0, dst);
-      } else if (j == 0) {
-        embed(ctx, src, 1, n, b, dst, 1, r[1], 0, m * b, 1.0, nullptr);
-      } else if (j == d - 1) {
-        embed(ctx, src, a, n, 1, dst, r[j], 1, m * a, 0, 1.0, nullptr);
-      } else {
-        embed(ctx, src, a, n, b, dst, r[j], r[j + 1], m * a, m * b, 1.0, nullptr);
-      }
-    }
-  }
-  tt_round(ctx, view_of(big), rmax, out, tol);
+  TTBatch b;
+  ttb_precond(ctx, one_item(x), t, w, rmax, b, tol, omega, fp32, final);
+  take_item(std::move(b), out);
 }
 
 }  // namespace lrfg

@@ -9,81 +9,27 @@
 
 namespace lrfg {
 
-static unsigned grid_n(lrfg_ctx* ctx, long long n) {
-  long long g = (n + 255) / 256;
-  long long cap = 16LL * (ctx->num_sms > 0 ? ctx->num_sms : 152);
-  return (unsigned)std::max(1LL, std::min(g, cap));
-}
-
-// dst item i, block at rank offsets (oa, ob) of an (A, n, B) carriage <- scale_i * src item i (a, n, b)
-__global__ void embed_batch_kernel(const double* __restrict__ src, long long ss, int a, int n, int b, double* dst,
-                                   long long ds, int A, int B, int oa, int ob, double s,
-                                   const double* __restrict__ s_dev, int nb) {
-  const long long per = (long long)a * n * b, total = per * nb;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total; t += (long long)gridDim.x * blockDim.x) {
-    const int item = (int)(t / per);
-    const long long q = t - item * per;
-    const int jb = (int)(q % b);
-    const long long rest = q / b;
-    const int nn = (int)(rest % n);
-    const int ia = (int)(rest / n);
-    const double sc = s_dev ? s * s_dev[item] : s;
-    dst[(size_t)item * ds + ((size_t)(ia + oa) * n + nn) * B + (jb + ob)] = sc * src[(size_t)item * ss + q];
-  }
-}
-
-void ttb_add_many(lrfg_ctx* ctx, const TTBatchView* xs, int m, const double* hs, const double* const* ds,
-                  TTBatch& out) {
-  LRFG_REQUIRE(m >= 1, "empty sum");
-  const int d = xs[0].d, nb = xs[0].nb;
-  int r[4] = {1, 1, 1, 1};
-  for (int j = 1; j < d; ++j) {
-    r[j] = 0;
-    for (int t = 0; t < m; ++t) r[j] += xs[t].r[j];
-  }
-  for (int t = 0; t < m; ++t) LRFG_REQUIRE(xs[t].d == d && xs[t].nb == nb, "batched sum of unlike batches");
-  ttb_alloc(ctx, out, d, xs[0].N, r, nb);
-  for (int j = 0; j < d; ++j) {
-    const int n = xs[0].N[j], A = out.r[j], B = out.r[j + 1];
-    double* dst = out.core[j].get();
-    if (d == 1 || (j != 0 && j != d - 1)) fill(ctx, dst, 0.0, (long long)out.elems(j) * nb);
-    int oa = 0, ob = 0;
-    for (int t = 0; t < m; ++t) {
-      const TTBatchView& x = xs[t];
-      const int a = x.r[j], b = x.r[j + 1];
-      const double s = (j == 0 && hs) ? hs[t] : 1.0;
-      const double* sd = (j == 0 && ds) ? ds[t] : nullptr;
-      const long long total = (long long)a * n * b * nb;
-      if (d == 1) {
-        LRFG_REQUIRE(m == 1, "batched sum of order-1 trains");
-      }
-      const int boa = (j == 0) ? 0 : oa, bob = (j == d - 1) ? 0 : ob;
-      LRFG_LAUNCH(ctx, KC_TT_MISC, (double)total, 2.0 * sizeof(double) * total,
-                  embed_batch_kernel<<<grid_n(ctx, total), 256, 0, ctx->stream>>>(
-                      x.core[j], (long long)x.elems(j), a, n, b, dst, (long long)out.elems(j), A, B, boa, bob, s, sd,
-                      nb));
-      oa += a;
-      ob += b;
-    }
-  }
-}
-
 void ttb_dot_device(lrfg_ctx* ctx, const TTBatchView& x, const TTBatchView& y, double* out_dev) {
   LRFG_REQUIRE(x.d == y.d && x.nb == y.nb, "batched dot of unlike batches");
   const int nb = x.nb;
-  DBuf<double> W(ctx->pool, (size_t)nb);
-  fill(ctx, W.get(), 1.0, nb);
+  DBuf<double> W;
   for (int j = 0; j < x.d; ++j) {
     const int a = x.r[j], b = x.r[j + 1], c = y.r[j], e = y.r[j + 1], n = x.N[j];
     LRFG_REQUIRE(n == y.N[j], "dot of TTs on different grids");
-    // V_i (c x (n b)) = W_i^T (c x a) x_i,j (a x (n b));  W'_i (b x e) = V_i^T y_i,j over (c n)
-    DBuf<double> V(ctx->pool, (size_t)c * n * b * nb);
-    gemm(ctx, 1, 0, c, n * b, a, 1.0, W.get(), c, (long long)a * c, x.core[j], n * b, (long long)x.elems(j), 0.0,
-         V.get(), n * b, (long long)c * n * b, nb);
+    // V_i (c x (n b)) = W_i^T (c x a) x_i,j (a x (n b));  W'_i (b x e) = V_i^T y_i,j over (c n); W_i = 1 at the first
+    // carriage
+    DBuf<double> Vb;
+    const double* V = x.core[0];
+    if (j > 0) {
+      Vb = DBuf<double>(ctx->pool, (size_t)c * n * b * nb);
+      V = Vb.get();
+      gemm(ctx, 1, 0, c, n * b, a, 1.0, W.get(), c, (long long)a * c, x.core[j], n * b, (long long)x.elems(j), 0.0,
+           Vb.get(), n * b, (long long)c * n * b, nb);
+    }
     double* dst = (j == x.d - 1) ? out_dev : nullptr;
     DBuf<double> Wn;
     if (!dst) { Wn = DBuf<double>(ctx->pool, (size_t)b * e * nb); dst = Wn.get(); }
-    gemm(ctx, 1, 0, b, e, c * n, 1.0, V.get(), b, (long long)c * n * b, y.core[j], e, (long long)y.elems(j), 0.0,
+    gemm(ctx, 1, 0, b, e, c * n, 1.0, V, b, (long long)c * n * b, y.core[j], e, (long long)y.elems(j), 0.0,
          dst, e, (long long)b * e, nb);
     if (j != x.d - 1) W = std::move(Wn);
   }
@@ -93,21 +39,6 @@ void ttb_precond(lrfg_ctx* ctx, const TTBatchView& x, const std::vector<double>&
                  int rmax, TTBatch& out, double tol, const TTView* omega, bool fp32, bool final) {
   const int d = x.d, nb = x.nb;
   const int R = (int)t.size();
-  if (!omega || d < 2) {
-    // deterministic rounding: item by item, packed into one batch
-    std::vector<TT> parts(nb);
-    for (int b = 0; b < nb; ++b) tt_precond(ctx, item_view_of(x, b), t, w, rmax, parts[b], tol, nullptr, fp32);
-    int r[4] = {1, 1, 1, 1};
-    for (int j = 0; j <= d; ++j) r[j] = parts[0].r[j];
-    for (int b = 1; b < nb; ++b)
-      for (int j = 0; j <= d; ++j) LRFG_REQUIRE(parts[b].r[j] == r[j], "batched preconditioner with unlike ranks");
-    ttb_alloc(ctx, out, d, x.N, r, nb);
-    for (int b = 0; b < nb; ++b)
-      for (int j = 0; j < d; ++j)
-        LRFG_CUDA(cudaMemcpyAsync(out.core[j].get() + (size_t)b * out.elems(j), parts[b].core[j].get(),
-                                  sizeof(double) * out.elems(j), cudaMemcpyDeviceToDevice, ctx->stream));
-    return;
-  }
   // the blocks G_m x_j of every item in one launch per carriage: terms[j][m][item] (a x N x b each)
   std::vector<double> ones(R, 1.0);
   SketchSource z;
@@ -129,7 +60,41 @@ void ttb_precond(lrfg_ctx* ctx, const TTBatchView& x, const std::vector<double>&
     z.s[j] = (j == 0 || j == d) ? 1 : R * x.r[j];
     z.ry[j] = x.r[j];
   }
-  tt_round_sketch(ctx, z, *omega, rmax, out, tol, fp32, final);
+  if (omega) {
+    // the blocks enter the sketch contractions as they are (never embedded in the block-diagonal carriage)
+    tt_round_sketch(ctx, z, *omega, rmax, out, tol, fp32, final);
+    return;
+  }
+  // deterministic rounding: the carriages are block rows (first), block diagonal (middle) and block columns (last) over
+  // m.  The items of a batch are rounded together (their eigenproblems and factors run on an SM each), in groups whose
+  // block-diagonal carriages stay below 1 GB; with a pool budget one at a time, the least memory the product takes.
+  long long item_elems = 0;
+  for (int j = 0; j < d; ++j) item_elems += (long long)z.s[j] * x.N[j] * z.s[j + 1];
+  const int group = ctx->pool->budget() ? 1 : (int)std::max(1LL, std::min<long long>(nb, (1LL << 27) / item_elems));
+  std::vector<TTBatch> parts;
+  for (int b0 = 0; b0 < nb; b0 += group) {
+    const int g = std::min(group, nb - b0);
+    TTBatch big, part;
+    ttb_alloc(ctx, big, d, x.N, z.s, g);
+    for (int j = 0; j < d; ++j)
+      stack_blocks(ctx, terms[j].get() + (size_t)b0 * x.elems(j), (long long)(x.elems(j) * nb), x.r[j], x.N[j], x.r[j + 1],
+                   R, j == 0 ? 0 : (j == d - 1 ? 2 : 1), g, big.core[j].get());
+    tt_round_batch(ctx, batch_view(big), rmax, part, tol);
+    if (g == nb) {
+      out = std::move(part);
+      return;
+    }
+    parts.push_back(std::move(part));
+  }
+  LRFG_REQUIRE(tol == 0.0, "tolerance truncation of a batch in groups");
+  ttb_alloc(ctx, out, d, x.N, parts[0].r, nb);
+  int at = 0;
+  for (TTBatch& q : parts) {
+    for (int j = 0; j < d; ++j)
+      LRFG_CUDA(cudaMemcpyAsync(out.core[j].get() + (size_t)at * out.elems(j), q.core[j].get(),
+                                sizeof(double) * q.elems(j) * q.nb, cudaMemcpyDeviceToDevice, ctx->stream));
+    at += q.nb;
+  }
 }
 
 TTView item_view_of(const TTBatchView& x, int b) {
