@@ -9,6 +9,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "../../include/lrfg.h"
@@ -108,6 +109,19 @@ struct TT {
   int max_rank() const { int m = 1; for (int j = 1; j < d; ++j) m = r[j] > m ? r[j] : m; return m; }
 };
 
+constexpr int kMaxStages = 24;
+// passes of a transform of length N
+struct FftPlan {
+  int N;
+  int nst;
+  int radix[kMaxStages];
+};
+// how a launch shape is run: its plan, rows a tile, Gaussian terms a block
+struct FftChoice {
+  FftPlan plan{};
+  int tf = 0, mper = 0;
+};
+
 // twiddle tables W[j] = exp(-2 pi i j / N), cached per N on the device
 struct Twiddles {
   double2* W = nullptr;
@@ -151,6 +165,7 @@ struct lrfg_ctx {
   cudaStream_t stream = nullptr;  // caller's stream (NULL: the legacy default stream)
   lrfg::DevicePool* pool = nullptr;
   std::map<int, lrfg::Twiddles> twiddles;
+  std::map<std::tuple<int, int, long long, int>, lrfg::FftChoice> fft_choices;  // by (N, kind, rows, tile or terms)
   std::string last_error;
   int num_sms = 0;
   int max_smem_optin = 0;

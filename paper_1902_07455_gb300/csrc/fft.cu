@@ -21,7 +21,7 @@ FftPlan make_plan(int N, int max_radix) {
   // the order of the passes does not change the transform
   const int pref[] = {27, 9, 5, 7, 3};
   for (int p : pref) {
-    if (p > max_radix) continue;
+    if (p > max_radix && p > 7) continue;  // (limits the composite radices)
     while (n % p == 0) {
       if (pl.nst >= kMaxStages) fail(LRFG_ENOTSUP, "grid size %d has too many factors", N);
       pl.radix[pl.nst++] = p;
@@ -81,25 +81,13 @@ const float2* twiddle_table<float>(lrfg_ctx* ctx, int N) {
   return t.Wf;
 }
 
-static int tile_fibres(lrfg_ctx* ctx, int N, int rows_per_fibre_pair, size_t* smem_out, size_t elem = sizeof(double2)) {
-  // shared memory: twiddles N + 2 buffers of TF rows (+ N multipliers for the operator kernels)
+// rows of a real-fibre tile that fit in shared memory: N twiddles and `fixed` further tables of N, `per` buffers of N
+// for each row
+static int tile_fibres(lrfg_ctx* ctx, int N, size_t elem, int fixed, int per) {
   size_t limit = 100 * 1024;
   if (N > 300) limit = (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
-  long long per = 2LL * N * (long long)elem;
-  long long fixed = 2LL * N * (long long)elem;
-  long long tf = ((long long)limit - fixed) / per;
-  if (tf > 64) tf = 64;
-  if (tf < 1) tf = 1;
-  (void)rows_per_fibre_pair;
-  *smem_out = (size_t)(fixed + tf * per);
-  return (int)tf;
-}
-
-// Fewer rows per tile when the fibres are few (the carriages of a low-rank tensor: r^2 fibres of one length),
-// so that the launch still spreads over about `target` blocks instead of leaving most SMs idle.
-static int spread_tf(int tf_max, long long nfib, long long target) {
-  long long tf = (nfib + 2 * target - 1) / (2 * target);
-  return (int)std::max(1LL, std::min((long long)tf_max, tf));
+  const long long row = (long long)N * (long long)elem;
+  return (int)std::max(1LL, std::min(64LL, ((long long)limit - (1 + fixed) * row) / (per * row)));
 }
 
 // ----------------------------------------------------------------------------------------------------
@@ -381,47 +369,87 @@ static bool fft2_try(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N,
   }
 }
 
-// Rows of a transform tile when the largest tile (tf_max rows) leaves the SMs unevenly filled.  The passes are bound by
-// the FP64 pipe, which an SM's blocks share and which a warp instruction holds however many of its lanes work, so a
-// launch takes as long as its busiest SM: blocks per SM x warps of butterflies per pass.  The tile with the smallest
-// such count is taken, the larger one on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid in 32-row tiles ran
-// on one or two SMs (46 us per fibre pass and 88 us per fused row pass under event timing; spread over 11 to 32 SMs 20
-// and 34 us), 63^3 with its Ga double grid 125^3 gained 19%; from six blocks per SM on the rounding up costs less than the shorter memory segments of a smaller tile, and tf_max stays.
-int balanced_tile(lrfg_ctx* ctx, const FftPlan& pl, int tf_max, long long nrows) {
+// FP64 operations of a radix-p butterfly with its twiddles
+static double butterfly_ops(int p) {
+  switch (p) {
+    case 3: return 20.0;
+    case 5: return 52.0;
+    case 7: return 90.0;
+    case 9: return 120.0;
+    default: return (double)(p - 1) * (p - 1) + 14.0 * p;
+  }
+}
+
+// Cycles of one transform of tf rows in each of `blocks` blocks on the SM with the most of them.  An SM has four FP64
+// units, a warp issues one FP64 instruction per 64 cycles on its unit (about 70 when all four are busy) however many of
+// its lanes work, so a pass takes the instructions of the warps on one unit, plus a barrier and a trip through shared
+// memory.
+double fft_cycles(lrfg_ctx* ctx, const FftPlan& pl, long long tf, long long blocks) {
   const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
-  if ((nrows + tf_max - 1) / tf_max >= 6 * nsm) return tf_max;
-  int best = tf_max;
-  double best_cost = 0.0;
-  for (int tf = tf_max; tf >= 1; --tf) {
-    const long long blocks = (nrows + tf - 1) / tf;
-    double warps = 0.0;
-    for (int s = 0; s < pl.nst; ++s) {
-      const int p = pl.radix[s];
-      warps += (double)((tf * (long long)(pl.N / p) + 31) / 32) * p * std::log2((double)p + 1.0);
-    }
-    const double cost = (double)((blocks + nsm - 1) / nsm) * warps;
-    if (tf == tf_max || cost < 0.98 * best_cost) {
-      best_cost = cost;
-      best = tf;
+  const long long per_sm = (blocks + nsm - 1) / nsm;
+  double c = 0.0;
+  for (int s = 0; s < pl.nst; ++s) {
+    const int p = pl.radix[s];
+    const long long warps = per_sm * ((tf * (pl.N / p) + 31) / 32);
+    c += (double)((warps + 3) / 4) * butterfly_ops(p) * 70.0 + 400.0;
+  }
+  return c;
+}
+
+// the context's earlier choice for a launch shape (tf = 0: none yet); the table is emptied when it has grown to 4096
+static FftChoice& fft_choice(lrfg_ctx* ctx, int N, int kind, long long nrows, int extra) {
+  auto& m = ctx->fft_choices;
+  if (m.size() >= 4096) m.clear();
+  return m[std::make_tuple(N, kind, nrows, extra)];
+}
+
+// Plan and tile for nrows FP64 rows, at most tf_max rows a tile: the cheapest by fft_cycles over the tiles and over
+// radix-9 passes or radix-3 ones (a few percent more operations in pieces a sixth as long: the shorter chain where a
+// launch has fewer butterflies than units), the larger tile on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid
+// in 32-row tiles ran on one or two SMs: 46 us per fibre pass and 88 us per fused row pass under event timing; 63^3 with
+// its Ga double grid 125^3 gained 19% from even tiles.  From six full tiles per SM on the rounding up costs less than the
+// shorter memory segments of a smaller tile, and tf_max stays.
+FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf) {
+  const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
+  FftPlan best = make_plan(N, fp64 ? plan_radix<double2>() : plan_radix<float2>());
+  *tf = tf_max;
+  if ((nrows + tf_max - 1) / tf_max >= 6 * nsm) return best;
+  FftChoice& known = fft_choice(ctx, N, fp64 ? 1 : 0, nrows, tf_max);
+  if (known.tf) {
+    *tf = known.tf;
+    return known.plan;
+  }
+  const FftPlan small = make_plan(N, 3);
+  double cost = 0.0;
+  for (int q = 0; q < (fp64 ? 2 : 1); ++q) {
+    const FftPlan pl = q ? small : best;
+    for (int t = tf_max; t >= 1; --t) {
+      const double c = fft_cycles(ctx, pl, t, (nrows + t - 1) / t);
+      if (cost == 0.0 || c < 0.97 * cost) {
+        cost = c;
+        best = pl;
+        *tf = t;
+      }
     }
   }
+  known = {best, *tf, 0};
   return best;
 }
 
-// Tile for the complex fibre FFT: whole 128-byte segments along the contiguous index (TF * sizeof(V) >=
+// Plan and tile for the complex fibre FFT: whole 128-byte segments along the contiguous index (TF * sizeof(V) >=
 // 128) and at most 72 KB of shared memory, so that three blocks share an SM and one block's transform
 // overlaps the others' loads and stores; fewer fibres where that fills the SMs more evenly.
-static int tile_complex(lrfg_ctx* ctx, const FftPlan& pl, size_t elem, long long nfib, size_t* smem_out) {
-  const long long row = (long long)pl.N * (long long)elem;
+static FftPlan tile_complex(lrfg_ctx* ctx, int N, size_t elem, long long nfib, int* tf_out, size_t* smem_out) {
+  const long long row = (long long)N * (long long)elem;
   long long limit = 72 * 1024;
   const long long tf_min = std::max<long long>(1, 128 / (long long)elem);
   if (2 * row + 2 * tf_min * row > limit) limit = std::min<long long>(ctx->max_smem_optin, 200 * 1024);
   long long tf = (limit - 2 * row) / (2 * row);
   tf = std::max<long long>(1, std::min<long long>(tf, 32));
   if (tf > tf_min) tf = (tf / tf_min) * tf_min;
-  tf = balanced_tile(ctx, pl, (int)tf, nfib);
-  *smem_out = (size_t)(2 * row + 2 * tf * row);
-  return (int)tf;
+  const FftPlan pl = choose_plan(ctx, N, elem == sizeof(double2), nfib, (int)tf, tf_out);
+  *smem_out = (size_t)(2 * row + 2 * *tf_out * row);
+  return pl;
 }
 
 template <typename V>
@@ -430,11 +458,11 @@ void fft_fibres(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N, long
   LRFG_REQUIRE(N >= 1 && (N % 2 == 1), "fft length must be odd (got %d)", N);
   LRFG_REQUIRE(outer >= 0 && inner >= 0, "negative batch");
   if (outer == 0 || inner == 0) return;
-  FftPlan pl = make_plan(N, plan_radix<V>());
   const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
+  int TF;
   long long nfib = outer * inner;
-  int TF = tile_complex(ctx, pl, sizeof(V), nfib, &smem);
+  const FftPlan pl = tile_complex(ctx, N, sizeof(V), nfib, &TF, &smem);
   long long blocks = (nfib + TF - 1) / TF;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   const double flops = 5.0 * N * std::log2((double)N) * (double)nfib;   // radix-2-equivalent count
@@ -468,10 +496,10 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, int N0, long long inner,
   LRFG_REQUIRE(fm.mode == 1 || in != out, "the accumulator cannot hold the input");
   LRFG_REQUIRE(!(fm.mode == 2 && fm.precond) || fm.inv_kk, "reciprocal table missing");
   if (inner == 0) return;
-  FftPlan pl = make_plan(N0, plan_radix<V>());
   const V* W = twiddle_table<R>(ctx, N0);
   size_t smem;
-  int TF = tile_complex(ctx, pl, sizeof(V), inner, &smem);
+  int TF;
+  const FftPlan pl = tile_complex(ctx, N0, sizeof(V), inner, &TF, &smem);
   long long blocks = (inner + TF - 1) / TF;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   const double n_el = (double)N0 * (double)inner;
@@ -496,7 +524,8 @@ template void fft_fibres_mul<double2>(lrfg_ctx*, const double2*, double2*, int, 
 template void fft_fibres_mul<float2>(lrfg_ctx*, const float2*, float2*, int, long long, const FibreMul<float>&);
 
 // ----------------------------------------------------------------------------------------------------
-// real fibres under a multiplier: rows hold fibre f (real part) and fibre f + TF (imaginary part)
+// real fibres under a multiplier: row f holds fibre 2 f (real part) and fibre 2 f + 1 (imaginary part), so a fibre's partner
+// does not depend on the tile (the FP32 transforms' rounding does depend on the partner)
 // ----------------------------------------------------------------------------------------------------
 __device__ __forceinline__ double2 multiplier(int kind, int k, double param) {
   if (kind == LRFG_MUL_DERIV) return make_double2(0.0, 6.283185307179586476925286766559 * (double)k);
@@ -526,7 +555,7 @@ __global__ void __launch_bounds__(256) fibre_op_kernel(const double* in, double*
   const long long nfib = outer * inner;
   const long long g0 = (long long)blockIdx.x * (2LL * TF);
   const int nf = (int)min(2LL * TF, nfib - g0);   // real fibres in this tile
-  const int rows = min(nf, TF);
+  const int rows = (nf + 1) / 2;
   for (int t = threadIdx.x; t < rows * N; t += blockDim.x) a[t] = mkc<V>((R)0, (R)0);
   __syncthreads();
   const int total = nf * N;
@@ -537,7 +566,8 @@ __global__ void __launch_bounds__(256) fibre_op_kernel(const double* in, double*
     long long g = g0 + f;
     long long o = g / inner, i = g - o * inner;
     const R v = (R)in[((size_t)o * N + n) * (size_t)inner + (size_t)i];
-    if (f < TF) a[(size_t)f * N + n].x = v; else a[(size_t)(f - TF) * N + n].y = v;
+    V* z = a + (size_t)(f >> 1) * N + n;
+    if (f & 1) z->y = v; else z->x = v;
   }
   __syncthreads();
   V* res = stockham_rows<-1>(a, b, rows, N, pl, W);
@@ -554,22 +584,20 @@ __global__ void __launch_bounds__(256) fibre_op_kernel(const double* in, double*
     if (across) { f = t % nf; n = t / nf; } else { f = t / N; n = t % N; }
     long long g = g0 + f;
     long long o = g / inner, i = g - o * inner;
-    V v = (f < TF) ? res[(size_t)f * N + n] : res[(size_t)(f - TF) * N + n];
-    out[((size_t)o * N + n) * (size_t)inner + (size_t)i] = s * (double)((f < TF) ? v.x : v.y);
+    const V v = res[(size_t)(f >> 1) * N + n];
+    out[((size_t)o * N + n) * (size_t)inner + (size_t)i] = s * (double)((f & 1) ? v.y : v.x);
   }
 }
 
 template <typename V>
 static void fibre_operator_t(lrfg_ctx* ctx, const double* in, double* out, long long outer, int N, long long inner,
                              int kind, double param, double scale) {
-  FftPlan pl = make_plan(N, plan_radix<V>());
   const V* W = twiddle_table<typename RealOf<V>::T>(ctx, N);
-  size_t smem;
-  int TF = tile_fibres(ctx, N, 2, &smem, sizeof(V));
-  long long nfib = outer * inner;
-  const int nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
-  TF = spread_tf(TF, nfib, 2LL * nsm);
-  smem = (size_t)(2LL * N * sizeof(V) + (long long)TF * 2LL * N * sizeof(V));
+  const long long nfib = outer * inner;
+  int TF;  // a row carries two real fibres
+  const FftPlan pl = choose_plan(ctx, N, sizeof(V) == sizeof(double2), (nfib + 1) / 2, tile_fibres(ctx, N, sizeof(V), 1, 2),
+                                 &TF);
+  const size_t smem = (size_t)(2LL * N * sizeof(V) + (long long)TF * 2LL * N * sizeof(V));
   long long blocks = (nfib + 2LL * TF - 1) / (2LL * TF);
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   LRFG_CUDA(raise_smem_limit((const void*)fibre_op_kernel<V>, smem));
@@ -595,6 +623,7 @@ void fibre_operator(lrfg_ctx* ctx, const double* in, double* out, long long oute
 // multiply + inverse transform and is written to out + m * out_stride.  The nodes and scales travel as a kernel argument
 // (two copies from host memory per call before).
 constexpr int kMaxGaussTerms = 64;
+constexpr int kMaxGaussHalf = 512;
 struct GaussTerms {
   double t[kMaxGaussTerms], s[kMaxGaussTerms];
 };
@@ -613,11 +642,12 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
   V* spec = sm + N;              // TF rows: the shared forward spectrum
   V* a = spec + (size_t)TF * N;  // TF rows
   V* b = a + (size_t)TF * N;     // TF rows
+  __shared__ R mult[kMaxGaussHalf];  // exp(-t_m k^2), k = 0..(N-1)/2: an FP64 exponential takes tens of operations
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
   const long long nfib = outer * inner;
   const long long g0 = (long long)blockIdx.x * (2LL * TF);
   const int nf = (int)min(2LL * TF, nfib - g0);
-  const int rows = min(nf, TF);
+  const int rows = (nf + 1) / 2;
   for (int t = threadIdx.x; t < rows * N; t += blockDim.x) a[t] = mkc<V>((R)0, (R)0);
   __syncthreads();
   const int total = nf * N;
@@ -628,7 +658,8 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
     long long g = g0 + f;
     long long o = g / inner, i = g - o * inner;
     const R v = (R)in[((size_t)o * N + n) * (size_t)inner + (size_t)i];
-    if (f < TF) a[(size_t)f * N + n].x = v; else a[(size_t)(f - TF) * N + n].y = v;
+    V* z = a + (size_t)(f >> 1) * N + n;
+    if (f & 1) z->y = v; else z->x = v;
   }
   __syncthreads();
   V* res = stockham_rows<-1>(a, b, rows, N, pl, W);
@@ -637,9 +668,16 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
   const int m_end = min(nm, (int)(blockIdx.y + 1) * mper);
   for (int m = blockIdx.y * mper; m < m_end; ++m) {
     const double t_m = terms.t[m];
-    for (int t = threadIdx.x; t < rows * N; t += blockDim.x) {
-      int k = freq_of(t % N, N);
-      a[t] = cscale(spec[t], (R)exp(-t_m * (double)k * (double)k));
+    const int half = (N - 1) / 2;
+    if (half < kMaxGaussHalf) {
+      for (int k = threadIdx.x; k <= half; k += blockDim.x) mult[k] = (R)exp(-t_m * (double)k * (double)k);
+      __syncthreads();
+      for (int t = threadIdx.x; t < rows * N; t += blockDim.x) a[t] = cscale(spec[t], mult[abs(freq_of(t % N, N))]);
+    } else {
+      for (int t = threadIdx.x; t < rows * N; t += blockDim.x) {
+        const int k = freq_of(t % N, N);
+        a[t] = cscale(spec[t], (R)exp(-t_m * (double)k * (double)k));
+      }
     }
     __syncthreads();
     V* r2 = stockham_rows<1>(a, b, rows, N, pl, W);
@@ -650,8 +688,8 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
       if (across) { f = t % nf; n = t / nf; } else { f = t / N; n = t % N; }
       long long g = g0 + f;
       long long o = g / inner, i = g - o * inner;
-      V v = (f < TF) ? r2[(size_t)f * N + n] : r2[(size_t)(f - TF) * N + n];
-      o_m[((size_t)o * N + n) * (size_t)inner + (size_t)i] = s * (double)((f < TF) ? v.x : v.y);
+      const V v = r2[(size_t)(f >> 1) * N + n];
+      o_m[((size_t)o * N + n) * (size_t)inner + (size_t)i] = s * (double)((f & 1) ? v.y : v.x);
     }
     __syncthreads();
   }
@@ -660,30 +698,49 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
 template <typename V>
 static void fibre_gauss_multi_t(lrfg_ctx* ctx, const double* in, double* out, long long out_stride, long long outer,
                                 int N, long long inner, const double* t, const double* scale, int nm) {
-  FftPlan pl = make_plan(N, plan_radix<V>());
   const V* Wt = twiddle_table<typename RealOf<V>::T>(ctx, N);
-  size_t limit = 100 * 1024;
-  if (N > 300) limit = (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
-  long long per = 3LL * N * (long long)sizeof(V);
-  long long tf = ((long long)limit - (long long)N * (long long)sizeof(V)) / per;
-  if (tf > 64) tf = 64;
-  if (tf < 1) tf = 1;
-  // few fibres (low-rank carriages): smaller tiles, and the terms split over grid.y (each block redoes the
-  // shared forward transform of its tile), so that the launch covers the SMs
+  // few fibres (low-rank carriages): small tiles, and the terms split over grid.y (each block redoes the shared forward
+  // transform of its tile), so that the launch covers the SMs: the cheapest of the splits by the inverse transforms a
+  // block runs plus its forward one
   const int nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
-  const long long nfib0 = outer * inner;
-  tf = spread_tf((int)tf, nfib0, 2LL * nsm);
-  const long long bx = (nfib0 + 2 * tf - 1) / (2 * tf);
-  const int mchunks = (int)std::max(1LL, std::min((long long)nm, (4LL * nsm + bx - 1) / bx));
-  const int mper = (nm + mchunks - 1) / mchunks;
+  const long long nfib = outer * inner, nrows = (nfib + 1) / 2;
+  const long long per = 3LL * N * (long long)sizeof(V);
+  const int tf_max = tile_fibres(ctx, N, sizeof(V), 0, 3);
+  int tf = 1, mper = nm;
+  FftPlan pl{};
+  double cost = 0.0;
+  FftChoice& known = fft_choice(ctx, N, sizeof(V) == sizeof(double2) ? 3 : 2, nrows, nm);
+  if (known.tf) {
+    pl = known.plan;
+    tf = known.tf;
+    mper = known.mper;
+  }
+  for (int q = 0; !known.tf && q < (sizeof(V) == sizeof(double2) ? 2 : 1); ++q) {
+    const FftPlan cand = make_plan(N, q ? 3 : plan_radix<V>());
+    for (int t = tf_max; t >= 1; --t) {
+      const long long bx = (nrows + t - 1) / t;
+      if (t < tf_max && bx > 8LL * nsm) break;
+      for (int chunks = 1; chunks <= nm; ++chunks) {
+        const int mp = (nm + chunks - 1) / chunks, mg = (nm + mp - 1) / mp;
+        if (chunks > 1 && bx * mg > 8LL * nsm) break;
+        const double c = fft_cycles(ctx, cand, t, bx * mg) * (1 + mp);
+        if (cost == 0.0 || c < 0.97 * cost) {
+          cost = c;
+          pl = cand;
+          tf = t;
+          mper = mp;
+        }
+      }
+    }
+  }
+  known = {pl, tf, mper};
   size_t smem = (size_t)(N * sizeof(V) + tf * per);
   GaussTerms terms{};
   for (int m = 0; m < nm; ++m) {
     terms.t[m] = t[m];
     terms.s[m] = scale[m];
   }
-  long long nfib = outer * inner;
-  long long blocks = (nfib + 2 * tf - 1) / (2 * tf);
+  long long blocks = (nrows + tf - 1) / tf;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
   LRFG_CUDA(raise_smem_limit((const void*)fibre_gauss_multi_kernel<V>, smem));
   // one forward and nm inverse complex transforms per pair of real fibres (algorithmic count)

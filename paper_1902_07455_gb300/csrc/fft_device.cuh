@@ -19,9 +19,10 @@
 #include <cmath>
 #include <mutex>
 
+#include "common.cuh"
+
 namespace lrfg {
 
-constexpr int kMaxStages = 24;
 constexpr int kMaxGenericRadix = 31;
 
 // roots of unity exp(-2 pi i j / p) of the register radices, concatenated (filled once per device)
@@ -53,12 +54,6 @@ static inline cudaError_t ensure_roots(int device) {
   if (e == cudaSuccess && device >= 0 && device < 64) done |= 1ULL << device;
   return e;
 }
-
-struct FftPlan {
-  int N;
-  int nst;
-  int radix[kMaxStages];
-};
 
 // complex vector type of a real type
 template <typename R> struct CplxOf;

@@ -379,18 +379,18 @@ __global__ void __launch_bounds__(32 * P2, 3) rows2_mul_kernel(const float2* in,
 }
 
 template <typename R>
-static int row_tile(lrfg_ctx* ctx, const FftPlan& pl, long long rows, size_t* smem) {
+static FftPlan row_tile(lrfg_ctx* ctx, int N, long long rows, int* tf_out, size_t* smem) {
   using V = typename CplxOf<R>::T;
-  const int N = pl.N;
   // at most 72 KB for N <= 300, so that three blocks share an SM
   size_t limit = 72 * 1024;
   if (N > 300) limit = (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
   long long per = 2LL * N * (long long)sizeof(V);
   long long tf = ((long long)limit - 2LL * N * (long long)sizeof(V)) / per;
   tf = std::max(1LL, std::min(tf, 32LL));
-  tf = balanced_tile(ctx, pl, (int)tf, (rows + 1) / 2);  // a tile row carries two real rows
-  *smem = (size_t)(2LL * N * sizeof(V) + tf * per);
-  return (int)tf;
+  // a tile row carries two real rows
+  const FftPlan pl = choose_plan(ctx, N, sizeof(R) == sizeof(double), (rows + 1) / 2, (int)tf, tf_out);
+  *smem = (size_t)(2LL * N * sizeof(V) + *tf_out * per);
+  return pl;
 }
 
 template <typename R>
@@ -398,11 +398,11 @@ void full_forward(lrfg_ctx* ctx, const FullGrid& g, const R* real_in, const R* c
                   typename CplxOf<R>::T* half_out) {
   using V = typename CplxOf<R>::T;
   const int N = g.N[g.d - 1];
-  FftPlan pl = make_plan(N, plan_radix<V>());
   LRFG_CUDA(ensure_roots(ctx->device));
   const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
-  int TF = row_tile<R>(ctx, pl, g.rows, &smem);
+  int TF;
+  const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
   long long blocks = (g.rows + 2LL * TF - 1) / (2LL * TF);
   LRFG_CUDA(raise_smem_limit((const void*)r2c_rows_kernel<R>, smem));
   LRFG_LAUNCH(ctx, KC_R2C, 2.5 * N * std::log2((double)N) * (double)g.rows,
@@ -430,11 +430,11 @@ void full_inverse(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half_
     fft_fibres(ctx, half_inout, half_inout, outer, g.N[ax], inner, 1);
   }
   const int N = g.N[g.d - 1];
-  FftPlan pl = make_plan(N, plan_radix<V>());
   LRFG_CUDA(ensure_roots(ctx->device));
   const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
-  int TF = row_tile<R>(ctx, pl, g.rows, &smem);
+  int TF;
+  const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
   long long blocks = (g.rows + 2LL * TF - 1) / (2LL * TF);
   LRFG_CUDA(raise_smem_limit((const void*)c2r_rows_kernel<R>, smem));
   LRFG_LAUNCH(ctx, KC_C2R, 2.5 * N * std::log2((double)N) * (double)g.rows,
@@ -466,11 +466,11 @@ void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half
     if (N == 243) return rows2_launch<27, 9>(ctx, g, half_inout, coef, scale);
     if (N == 81) return rows2_launch<9, 9>(ctx, g, half_inout, coef, scale);
   }
-  FftPlan pl = make_plan(N, plan_radix<V>());
   LRFG_CUDA(ensure_roots(ctx->device));
   const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
-  int TF = row_tile<R>(ctx, pl, g.rows, &smem);
+  int TF;
+  const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
   long long blocks = (g.rows + 2LL * TF - 1) / (2LL * TF);
   LRFG_CUDA(raise_smem_limit((const void*)c2r_mul_r2c_rows_kernel<R>, smem));
   LRFG_LAUNCH(ctx, KC_ROWS_FUSED, 5.0 * N * std::log2((double)N) * (double)g.rows,
