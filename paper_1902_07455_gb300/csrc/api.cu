@@ -87,6 +87,14 @@ void* DevicePool::alloc(size_t bytes) {
   return p;
 }
 
+bool DevicePool::room(int count, size_t bytes) const {
+  if (!budget_) return true;
+  const size_t sz = rounded(bytes);
+  const auto it = sized_.find(sz);
+  const size_t have = it == sized_.end() ? 0 : it->second.size();
+  return have >= (size_t)count || reserved_ + ((size_t)count - have) * sz <= budget_;
+}
+
 void DevicePool::release(void* p) {
   auto it = live_size_.find(p);
   if (it == live_size_.end()) return;
@@ -785,6 +793,15 @@ void full_apply(lrfg_problem* P, const typename CplxOf<R>::T* v, typename CplxOf
   const FullGrid& g = P->g;
   FullWork<R> w(P);
   const double inv = 1.0 / (double)g.n_real;
+  // the shared passes need two more half spectra; under a pool budget that has no room for them the components run one
+  // by one
+  using V = typename CplxOf<R>::T;
+  if (g.d == 3 && ctx->pool->room(2, sizeof(V) * g.n_half)) {
+    DBuf<V> w1(ctx->pool, g.n_half), w2(ctx->pool, g.n_half);
+    full_operator_3d<R>(ctx, g, v, out, w.a, inv, precond && !P->aniso, w.wc, w1.get(), w2.get());
+    if (P->aniso) half_acc_aniso(ctx, g, v, out, P->B, precond);
+    return;
+  }
   for (int alpha = 0; alpha < g.d; ++alpha) {
     // grad^ (with 1/|N| of Phi^-1) and F^-1 on the complex axes, then on the rows fused with A~ and F there,
     // then F on the complex axes and grad^* (P~^-1 after the last component)

@@ -58,6 +58,8 @@ class DevicePool {
   void release(void* p);
   void trim();
   size_t budget() const { return budget_; }
+  // whether `count` blocks of `bytes` fit without passing the budget (or returning cached blocks to the driver)
+  bool room(int count, size_t bytes) const;
   size_t in_use() const { return in_use_; }
   size_t reserved() const { return reserved_; }
   // high-water mark of in_use() since the last reset_peak()

@@ -93,17 +93,26 @@ static int tile_fibres(lrfg_ctx* ctx, int N, size_t elem, int fixed, int per) {
 // ----------------------------------------------------------------------------------------------------
 // complex fibres
 // ----------------------------------------------------------------------------------------------------
-// frequencies (k1, k2) of fibre i of the axis-0 pass over a d = 2 or 3 half spectrum
+// the two frequencies (ka, kb) that are constant on fibre (o, i), in the order of their axes
 template <typename R>
-__device__ __forceinline__ void fibre_freqs(const FibreMul<R>& fm, long long i, int& k1, int& k2) {
-  if (fm.d == 3) {
+__device__ __forceinline__ void fibre_freqs(const FibreMul<R>& fm, long long o, long long i, int& ka, int& kb) {
+  if (fm.axis == 1) {
+    ka = freq_of((int)o, fm.N0);
+    kb = (int)i;
+  } else if (fm.d == 3) {
     const int i1 = (int)(i / fm.H);
-    k1 = freq_of(i1, fm.N1);
-    k2 = (int)(i - (long long)i1 * fm.H);
+    ka = freq_of(i1, fm.N1);
+    kb = (int)(i - (long long)i1 * fm.H);
   } else {
-    k1 = (int)i;
-    k2 = 0;
+    ka = (int)i;
+    kb = 0;
   }
+}
+
+// frequency k_alpha of an element: kn along the fibre, (ka, kb) constant on it
+template <typename R>
+__device__ __forceinline__ int freq_alpha(const FibreMul<R>& fm, int kn, int ka, int kb) {
+  return fm.alpha == fm.axis ? kn : (fm.alpha == (fm.axis == 0 ? 1 : 0) ? ka : kb);
 }
 
 // v * (2 pi i k) * scale, f = c2 k
@@ -112,27 +121,26 @@ __device__ __forceinline__ V times_2pi_ik(V v, typename RealOf<V>::T f) {
   return mkc<V>(-v.y * f, v.x * f);
 }
 
-// mode 2 of FibreMul: the divergence term of element (k0, k1, k2) accumulated into *dst
+// mode 2 of FibreMul: the divergence term of element kn of a fibre accumulated into *dst
 template <typename V>
-__device__ __forceinline__ void acc_div_store(const FibreMul<typename RealOf<V>::T>& fm, V* dst, V x, int k0, int k1,
-                                              int k2) {
+__device__ __forceinline__ void acc_div_store(const FibreMul<typename RealOf<V>::T>& fm, V* dst, V x, int kn, int ka,
+                                              int kb) {
   using R = typename RealOf<V>::T;
-  const int ka = fm.alpha == 0 ? k0 : (fm.alpha == 1 ? k1 : k2);
-  V r = times_2pi_ik<V>(x, -fm.c2 * (R)ka);
+  V r = fm.alpha < 0 ? x : times_2pi_ik<V>(x, -fm.c2 * (R)freq_alpha(fm, kn, ka, kb));
   if (!fm.init) {
     const V o = *dst;
     r.x += o.x;
     r.y += o.y;
   }
   if (fm.precond) {
-    const R s = fm.inv_kk[k0 * k0 + k1 * k1 + k2 * k2];
+    const R s = fm.inv_kk[kn * kn + ka * ka + kb * kb];
     r.x *= s;
     r.y *= s;
   }
   *dst = r;
 }
 
-// OP 0: plain transform; OP 1 and 2: the modes of FibreMul (outer = 1)
+// OP 0: plain transform; OP 1 and 2: the modes of FibreMul
 template <int SIGN, typename V, int OP>
 __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out, long long outer, int N, long long inner,
                                                          int TF, FftPlan pl, const V* __restrict__ Wg,
@@ -173,21 +181,21 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
     if (across) {
       const int step = blockDim.x / nf;
       const int f = threadIdx.x % nf, n0 = threadIdx.x / nf;
-      int k1, k2;
-      fibre_freqs(fm, g0 + f, k1, k2);
-      const R fc = fm.c2 * (R)(fm.alpha == 1 ? k1 : k2);
+      const long long o = (g0 + f) / inner;
+      int ka, kb;
+      fibre_freqs(fm, o, g0 + f - o * inner, ka, kb);
       if (n0 < step)
         for (int n = n0; n < N; n += step) {
           V* p = a + (size_t)f * N + n;
-          *p = times_2pi_ik<V>(*p, fm.alpha == 0 ? fm.c2 * (R)freq_of(n, N) : fc);
+          *p = times_2pi_ik<V>(*p, fm.c2 * (R)freq_alpha(fm, freq_of(n, N), ka, kb));
         }
     } else {
       for (int t = threadIdx.x; t < total; t += blockDim.x) {
         const int f = small_div(t, N, 1.0f / (float)N), n = t - f * N;
-        int k1, k2;
-        fibre_freqs(fm, g0 + f, k1, k2);
-        const int ka = fm.alpha == 0 ? freq_of(n, N) : (fm.alpha == 1 ? k1 : k2);
-        a[t] = times_2pi_ik<V>(a[t], fm.c2 * (R)ka);
+        const long long o = (g0 + f) / inner;
+        int ka, kb;
+        fibre_freqs(fm, o, g0 + f - o * inner, ka, kb);
+        a[t] = times_2pi_ik<V>(a[t], fm.c2 * (R)freq_alpha(fm, freq_of(n, N), ka, kb));
       }
     }
   }
@@ -200,11 +208,11 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
     const long long o = g / inner, i = g - o * inner;
     V* dst = out + (size_t)o * N * (size_t)inner + (size_t)i;
     if constexpr (OP == 2) {
-      int k1, k2;
-      fibre_freqs(fm, i, k1, k2);
+      int ka, kb;
+      fibre_freqs(fm, o, i, ka, kb);
       if (n0 < step)
         for (int n = n0; n < N; n += step)
-          acc_div_store<V>(fm, dst + (size_t)n * inner, res[(size_t)f * N + n], freq_of(n, N), k1, k2);
+          acc_div_store<V>(fm, dst + (size_t)n * inner, res[(size_t)f * N + n], freq_of(n, N), ka, kb);
     } else {
       if (n0 < step)
         for (int n = n0; n < N; n += step) dst[(size_t)n * inner] = res[(size_t)f * N + n];
@@ -216,9 +224,9 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
       const long long o = g / inner, i = g - o * inner;
       V* dst = out + ((size_t)o * N + n) * (size_t)inner + (size_t)i;
       if constexpr (OP == 2) {
-        int k1, k2;
-        fibre_freqs(fm, i, k1, k2);
-        acc_div_store<V>(fm, dst, res[(size_t)f * N + n], freq_of(n, N), k1, k2);
+        int ka, kb;
+        fibre_freqs(fm, o, i, ka, kb);
+        acc_div_store<V>(fm, dst, res[(size_t)f * N + n], freq_of(n, N), ka, kb);
       } else {
         *dst = res[(size_t)f * N + n];
       }
@@ -260,8 +268,8 @@ __global__ void __launch_bounds__(32 * P2, fft2_min_blocks<P1, P2, OP>()) fft2_f
     o = g / inner;
     i = g - o * inner;
   }
-  int k1 = 0, k2 = 0;
-  if constexpr (OP != 0) fibre_freqs(fm, i, k1, k2);
+  int ka = 0, kb = 0;
+  if constexpr (OP != 0) fibre_freqs(fm, o, i, ka, kb);
   const size_t base = (size_t)o * N * (size_t)inner + (size_t)i;
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
 
@@ -269,9 +277,9 @@ __global__ void __launch_bounds__(32 * P2, fft2_min_blocks<P1, P2, OP>()) fft2_f
 #pragma unroll
   for (int r = 0; r < P1; ++r) x[r] = valid ? in[base + (size_t)(w + P2 * r) * (size_t)inner] : make_float2(0.f, 0.f);
   if constexpr (OP == 1) {
-    // k_0 varies along the fibre: multiply before the transform; k_1 and k_2 are constant on it and
+    // k of the fibre's own axis varies along it: multiply before the transform; the others are constant on it and
     // the product commutes with the transform, so it is taken after pass 2 (fewer live registers)
-    if (fm.alpha == 0) {
+    if (fm.alpha == fm.axis) {
 #pragma unroll
       for (int r = 0; r < P1; ++r) x[r] = times_2pi_ik<float2>(x[r], fm.c2 * (float)freq_of(w + P2 * r, N));
     }
@@ -303,23 +311,22 @@ __global__ void __launch_bounds__(32 * P2, fft2_min_blocks<P1, P2, OP>()) fft2_f
         const int n = f + P1 * q;
         float2* dst = out + base + (size_t)n * (size_t)inner;
         if constexpr (OP == 2) {
-          const int k0 = freq_of(n, N);
-          const int ka = fm.alpha == 0 ? k0 : (fm.alpha == 1 ? k1 : k2);
-          float2 r = times_2pi_ik<float2>(y[q], -fm.c2 * (float)ka);
+          const int kn = freq_of(n, N);
+          float2 r = fm.alpha < 0 ? y[q] : times_2pi_ik<float2>(y[q], -fm.c2 * (float)freq_alpha(fm, kn, ka, kb));
           if (!fm.init) {
             r.x += prev[q].x;
             r.y += prev[q].y;
           }
           if (fm.precond) {
             // the correctly rounded reciprocal, the value the table holds, without its scattered gather
-            const int kk = k0 * k0 + k1 * k1 + k2 * k2;
+            const int kk = kn * kn + ka * ka + kb * kb;
             const float sc = kk ? __frcp_rn((float)kk) : 0.f;
             r.x *= sc;
             r.y *= sc;
           }
           *dst = r;
         } else if constexpr (OP == 1) {
-          *dst = fm.alpha == 0 ? y[q] : times_2pi_ik<float2>(y[q], fm.c2 * (float)(fm.alpha == 1 ? k1 : k2));
+          *dst = fm.alpha == fm.axis ? y[q] : times_2pi_ik<float2>(y[q], fm.c2 * (float)freq_alpha(fm, 0, ka, kb));
         } else {
           *dst = y[q];
         }
@@ -487,41 +494,45 @@ template void fft_fibres<double2>(lrfg_ctx*, const double2*, double2*, long long
 template void fft_fibres<float2>(lrfg_ctx*, const float2*, float2*, long long, int, long long, int);
 
 template <typename V>
-void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, int N0, long long inner, const FibreMul<typename RealOf<V>::T>& fm) {
+void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename RealOf<V>::T>& fm) {
   using R = typename RealOf<V>::T;
-  LRFG_REQUIRE(N0 >= 1 && (N0 % 2 == 1), "fft length must be odd (got %d)", N0);
   LRFG_REQUIRE(fm.mode == 1 || fm.mode == 2, "multiplier mode %d", fm.mode);
   LRFG_REQUIRE(fm.d == 2 || fm.d == 3, "d = %d", fm.d);
-  LRFG_REQUIRE(inner == (long long)(fm.d == 3 ? fm.N1 : 1) * fm.H, "axis-0 fibres of a half spectrum expected");
+  LRFG_REQUIRE(fm.axis == 0 || (fm.axis == 1 && fm.d == 3), "axis %d of a half spectrum with d = %d", fm.axis, fm.d);
+  LRFG_REQUIRE(fm.alpha >= (fm.mode == 2 ? -1 : 0) && fm.alpha < fm.d, "component %d", fm.alpha);
+  const int N = fm.axis == 0 ? fm.N0 : fm.N1;
+  const long long outer = fm.axis == 0 ? 1 : fm.N0;
+  const long long inner = fm.axis == 0 ? (long long)(fm.d == 3 ? fm.N1 : 1) * fm.H : fm.H;
+  LRFG_REQUIRE(N >= 1 && (N % 2 == 1), "fft length must be odd (got %d)", N);
   LRFG_REQUIRE(fm.mode == 1 || in != out, "the accumulator cannot hold the input");
   LRFG_REQUIRE(!(fm.mode == 2 && fm.precond) || fm.inv_kk, "reciprocal table missing");
   if (inner == 0) return;
-  const V* W = twiddle_table<R>(ctx, N0);
+  const V* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
-  const FftPlan pl = tile_complex(ctx, N0, sizeof(V), inner, &TF, &smem);
-  long long blocks = (inner + TF - 1) / TF;
+  const FftPlan pl = tile_complex(ctx, N, sizeof(V), outer * inner, &TF, &smem);
+  long long blocks = (outer * inner + TF - 1) / TF;
   LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
-  const double n_el = (double)N0 * (double)inner;
-  const double flops = 5.0 * N0 * std::log2((double)N0) * (double)inner + (fm.mode == 1 ? 2.0 : 4.0) * n_el;
+  const double n_el = (double)N * (double)outer * (double)inner;
+  const double flops = 5.0 * std::log2((double)N) * n_el + (fm.mode == 1 ? 2.0 : 4.0) * n_el;
   const double bytes = (fm.mode == 1 || fm.init ? 2.0 : 3.0) * sizeof(V) * n_el;
-  if (fm.mode == 1 ? fft2_try<V, 1, 1>(ctx, in, out, 1, N0, inner, fm, flops, bytes)
-                   : fft2_try<V, -1, 2>(ctx, in, out, 1, N0, inner, fm, flops, bytes))
+  if (fm.mode == 1 ? fft2_try<V, 1, 1>(ctx, in, out, outer, N, inner, fm, flops, bytes)
+                   : fft2_try<V, -1, 2>(ctx, in, out, outer, N, inner, fm, flops, bytes))
     return;
   if (fm.mode == 1) {
     LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 1>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<1, V, 1><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, 1, N0, inner, TF, pl,
+                fft_fibres_kernel<1, V, 1><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
                                                                                         W, fm));
   } else {
     LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 2>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<-1, V, 2><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, 1, N0, inner, TF, pl,
+                fft_fibres_kernel<-1, V, 2><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
                                                                                          W, fm));
   }
 }
-template void fft_fibres_mul<double2>(lrfg_ctx*, const double2*, double2*, int, long long, const FibreMul<double>&);
-template void fft_fibres_mul<float2>(lrfg_ctx*, const float2*, float2*, int, long long, const FibreMul<float>&);
+template void fft_fibres_mul<double2>(lrfg_ctx*, const double2*, double2*, const FibreMul<double>&);
+template void fft_fibres_mul<float2>(lrfg_ctx*, const float2*, float2*, const FibreMul<float>&);
 
 // ----------------------------------------------------------------------------------------------------
 // real fibres under a multiplier: row f holds fibre 2 f (real part) and fibre 2 f + 1 (imaginary part), so a fibre's partner

@@ -92,87 +92,42 @@ __device__ __forceinline__ V tw(const V* W, int j) {
   return w;
 }
 
-// One radix-p butterfly: inputs Z[c + m' r][f] (row offset (c + m' r) L + f), outputs Z'[c][f + L q].
+// One butterfly of a prime radix p > 7: inputs Z[c + m' r][f] (row offset (c + m' r) L + f), outputs Z'[c][f + L q].
 template <int SIGN, typename V>
 __device__ __forceinline__ void butterfly(int p, const V* __restrict__ in, V* __restrict__ out, int c, int f, int L,
                                           int mp, int N, const V* W) {
   using R = typename RealOf<V>::T;
-  if (p == 3) {
-    V x0 = in[c * L + f];
-    V x1 = in[(c + mp) * L + f];
-    V x2 = in[(c + 2 * mp) * L + f];
+  // direct length-p DFT with table twiddles, by the symmetric halves of the inputs
+  // (see RegDFT<7>): (p - 1)^2 / 4 pairs of real-coefficient products instead of (p - 1)^2 complex ones
+  V s[kMaxGenericRadix / 2 + 1], d[kMaxGenericRadix / 2 + 1];
+  const int h = (p - 1) / 2;
+  const V x0 = in[c * L + f];
+  V sum = x0;
+  for (int r = 1; r <= h; ++r) {
+    V u = in[(c + r * mp) * L + f], v = in[(c + (p - r) * mp) * L + f];
     if (f) {
-      x1 = cmul(x1, tw<SIGN>(W, f * mp));
-      x2 = cmul(x2, tw<SIGN>(W, 2 * f * mp));
+      u = cmul(u, tw<SIGN>(W, f * r * mp));
+      v = cmul(v, tw<SIGN>(W, f * (p - r) * mp));
     }
-    const R s = (R)0.86602540378443864676;  // sin(2 pi / 3) = sqrt(3)/2
-    V t1 = cadd(x1, x2), t2 = csub(x1, x2);
-    V m = csub(x0, cscale(t1, (R)0.5));
-    V u = cimul(t2, (R)SIGN * s);
-    V* o = out + c * L * 3 + f;
-    o[0] = cadd(x0, t1);
-    o[L] = cadd(m, u);
-    o[2 * L] = csub(m, u);
-  } else if (p == 5) {
-    V x0 = in[c * L + f];
-    V x1 = in[(c + mp) * L + f];
-    V x2 = in[(c + 2 * mp) * L + f];
-    V x3 = in[(c + 3 * mp) * L + f];
-    V x4 = in[(c + 4 * mp) * L + f];
-    if (f) {
-      int j = f * mp;
-      x1 = cmul(x1, tw<SIGN>(W, j));
-      x2 = cmul(x2, tw<SIGN>(W, 2 * j));
-      x3 = cmul(x3, tw<SIGN>(W, 3 * j));
-      x4 = cmul(x4, tw<SIGN>(W, 4 * j));
-    }
-    // cos/sin of 2 pi/5 and 4 pi/5: (sqrt5-1)/4, -(sqrt5+1)/4, sqrt((5+sqrt5)/8), sqrt((5-sqrt5)/8)
-    const R c1 = (R)0.30901699437494742410, c2 = (R)-0.80901699437494742410;
-    const R s1 = (R)0.95105651629515357212, s2 = (R)0.58778525229247312917;
-    V a1 = cadd(x1, x4), b1 = csub(x1, x4), a2 = cadd(x2, x3), b2 = csub(x2, x3);
-    V m1 = cadd(x0, cadd(cscale(a1, c1), cscale(a2, c2)));
-    V m2 = cadd(x0, cadd(cscale(a1, c2), cscale(a2, c1)));
-    V n1 = cimul(cadd(cscale(b1, s1), cscale(b2, s2)), (R)SIGN);
-    V n2 = cimul(csub(cscale(b1, s2), cscale(b2, s1)), (R)SIGN);
-    V* o = out + c * L * 5 + f;
-    o[0] = cadd(x0, cadd(a1, a2));
-    o[L] = cadd(m1, n1);
-    o[2 * L] = cadd(m2, n2);
-    o[3 * L] = csub(m2, n2);
-    o[4 * L] = csub(m1, n1);
-  } else {
-    // generic prime radix (11, 13, ...): direct length-p DFT with table twiddles, by the symmetric halves of the inputs
-    // (see RegDFT<7>): (p - 1)^2 / 4 pairs of real-coefficient products instead of (p - 1)^2 complex ones
-    V s[kMaxGenericRadix / 2 + 1], d[kMaxGenericRadix / 2 + 1];
-    const int h = (p - 1) / 2;
-    const V x0 = in[c * L + f];
-    V sum = x0;
+    s[r] = cadd(u, v);
+    d[r] = csub(u, v);
+    sum = cadd(sum, s[r]);
+  }
+  const int step = N / p;
+  V* o = out + c * L * p + f;
+  o[0] = sum;
+  for (int q = 1; q <= h; ++q) {
+    V re = x0, im = mkc<V>((R)0, (R)0);
+    int j = 0;
     for (int r = 1; r <= h; ++r) {
-      V u = in[(c + r * mp) * L + f], v = in[(c + (p - r) * mp) * L + f];
-      if (f) {
-        u = cmul(u, tw<SIGN>(W, f * r * mp));
-        v = cmul(v, tw<SIGN>(W, f * (p - r) * mp));
-      }
-      s[r] = cadd(u, v);
-      d[r] = csub(u, v);
-      sum = cadd(sum, s[r]);
+      j += q;
+      if (j >= p) j -= p;
+      const V w = tw<SIGN>(W, j * step);
+      re = mkc<V>(re.x + w.x * s[r].x, re.y + w.x * s[r].y);
+      im = mkc<V>(im.x + w.y * d[r].x, im.y + w.y * d[r].y);
     }
-    const int step = N / p;
-    V* o = out + c * L * p + f;
-    o[0] = sum;
-    for (int q = 1; q <= h; ++q) {
-      V re = x0, im = mkc<V>((R)0, (R)0);
-      int j = 0;
-      for (int r = 1; r <= h; ++r) {
-        j += q;
-        if (j >= p) j -= p;
-        const V w = tw<SIGN>(W, j * step);
-        re = mkc<V>(re.x + w.x * s[r].x, re.y + w.x * s[r].y);
-        im = mkc<V>(im.x + w.y * d[r].x, im.y + w.y * d[r].y);
-      }
-      o[q * L] = mkc<V>(re.x - im.y, re.y + im.x);
-      o[(p - q) * L] = mkc<V>(re.x + im.y, re.y - im.x);
-    }
+    o[q * L] = mkc<V>(re.x - im.y, re.y + im.x);
+    o[(p - q) * L] = mkc<V>(re.x + im.y, re.y - im.x);
   }
 }
 
@@ -206,17 +161,17 @@ __device__ __forceinline__ V root(int j) {
 template <int P, int SIGN, typename V>
 struct RegDFT;
 
+// Multiplications are written as multiply-adds with the additions that follow them (12 FP64 operations at p = 3).
 template <int SIGN, typename V>
 struct RegDFT<3, SIGN, V> {
   static __device__ __forceinline__ void run(V* x) {
     using R = typename RealOf<V>::T;
-    const R s = (R)0.86602540378443864676;  // sin(2 pi / 3)
-    V t1 = cadd(x[1], x[2]), t2 = csub(x[1], x[2]);
-    V m = csub(x[0], cscale(t1, (R)0.5));
-    V u = cimul(t2, (R)SIGN * s);
+    const R s = (R)SIGN * (R)0.86602540378443864676;  // sin(2 pi / 3)
+    const V t1 = cadd(x[1], x[2]), t2 = csub(x[1], x[2]);
+    const R mx = fma(R(-0.5), t1.x, x[0].x), my = fma(R(-0.5), t1.y, x[0].y);
     x[0] = cadd(x[0], t1);
-    x[1] = cadd(m, u);
-    x[2] = csub(m, u);
+    x[1] = mkc<V>(fma(-s, t2.y, mx), fma(s, t2.x, my));
+    x[2] = mkc<V>(fma(s, t2.y, mx), fma(-s, t2.x, my));
   }
 };
 
@@ -226,16 +181,17 @@ struct RegDFT<5, SIGN, V> {
     using R = typename RealOf<V>::T;
     const R c1 = (R)0.30901699437494742410, c2 = (R)-0.80901699437494742410;
     const R s1 = (R)0.95105651629515357212, s2 = (R)0.58778525229247312917;
-    V a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]), a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
-    V m1 = cadd(x[0], cadd(cscale(a1, c1), cscale(a2, c2)));
-    V m2 = cadd(x[0], cadd(cscale(a1, c2), cscale(a2, c1)));
-    V n1 = cimul(cadd(cscale(b1, s1), cscale(b2, s2)), (R)SIGN);
-    V n2 = cimul(csub(cscale(b1, s2), cscale(b2, s1)), (R)SIGN);
+    const V a1 = cadd(x[1], x[4]), b1 = csub(x[1], x[4]), a2 = cadd(x[2], x[3]), b2 = csub(x[2], x[3]);
+    const V m1 = mkc<V>(fma(c2, a2.x, fma(c1, a1.x, x[0].x)), fma(c2, a2.y, fma(c1, a1.y, x[0].y)));
+    const V m2 = mkc<V>(fma(c1, a2.x, fma(c2, a1.x, x[0].x)), fma(c1, a2.y, fma(c2, a1.y, x[0].y)));
+    const R sa = (R)SIGN * s1, sb = (R)SIGN * s2;
+    const V n1 = mkc<V>(fma(sb, b2.x, sa * b1.x), fma(sb, b2.y, sa * b1.y));
+    const V n2 = mkc<V>(fma(-sa, b2.x, sb * b1.x), fma(-sa, b2.y, sb * b1.y));
     x[0] = cadd(x[0], cadd(a1, a2));
-    x[1] = cadd(m1, n1);
-    x[2] = cadd(m2, n2);
-    x[3] = csub(m2, n2);
-    x[4] = csub(m1, n1);
+    x[1] = mkc<V>(m1.x - n1.y, m1.y + n1.x);
+    x[2] = mkc<V>(m2.x - n2.y, m2.y + n2.x);
+    x[3] = mkc<V>(m2.x + n2.y, m2.y - n2.x);
+    x[4] = mkc<V>(m1.x + n1.y, m1.y - n1.x);
   }
 };
 

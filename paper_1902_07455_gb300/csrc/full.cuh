@@ -41,6 +41,12 @@ void half_fibres_forward_div(lrfg_ctx* ctx, const FullGrid& g, V* half, V* acc, 
 // half <- R2C(scale * coef (.) C2R(half)) along the rows (unnormalised transforms, in place)
 template <typename R>
 void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half_inout, const R* coef, R scale);
+// out = (precond: P~^-1) grad^* F coef F^-1 grad^ v on a d = 3 grid (scale: 1/|N| of the unnormalised transforms);
+// w0, w1, w2: half spectra of work space, distinct from v and out
+template <typename R>
+void full_operator_3d(lrfg_ctx* ctx, const FullGrid& g, const typename CplxOf<R>::T* v, typename CplxOf<R>::T* out,
+                      const R* coef, double scale, int precond, typename CplxOf<R>::T* w0, typename CplxOf<R>::T* w1,
+                      typename CplxOf<R>::T* w2);
 template <typename V>
 void half_mul_grad(lrfg_ctx* ctx, const FullGrid& g, const V* in, V* out, int alpha, double scale);
 template <typename V>
