@@ -755,22 +755,16 @@ template <> struct FullWork<float> {
   }
 };
 
-// Ga operator (FP64): per component, the gradient zero-padded to the double grid, multiplied there by the
-// modified coefficient, transformed back and projected on the frequencies of the grid, then grad^*
+// Ga operator (FP64): the gradient zero-padded to the double grid, multiplied there by the modified coefficient,
+// transformed back and projected on the frequencies of the grid, then grad^*
 void full_apply_ga(lrfg_problem* P, const double2* v, double2* out, int precond) {
   lrfg_ctx* ctx = P->ctx;
   const FullGrid& g = P->g;
   const FullGrid& gM = P->gM;
-  const double inv = 1.0 / (double)g.n_real;
-  for (int alpha = 0; alpha < g.d; ++alpha) {
-    half_mul_grad(ctx, g, v, P->wc.get(), alpha, inv);                           // grad^ (1/|N| of Phi^-1)
-    half_inject(ctx, g, gM, P->wc.get(), P->wcM.get());                          // I
-    full_inverse<double>(ctx, gM, P->wcM.get(), P->a_ga.get(), 1.0, P->wrM.get());  // A~ F_M^-1
-    full_forward<double>(ctx, gM, P->wrM.get(), nullptr, 1.0, P->wcM.get());     // F_M
-    half_project(ctx, g, gM, P->wcM.get(), P->wc.get());                         // I*
-    half_acc_div(ctx, g, (const double2*)P->wc.get(), out, alpha, 1.0, alpha == 0,
-                 precond && alpha == g.d - 1 && !P->aniso);                       // grad^*
-  }
+  // work space: the double grid's half spectrum, and two spectra of a quarter of it in the real double grid's buffer
+  double2* w1 = reinterpret_cast<double2*>(P->wrM.get());
+  double2* w2 = w1 + (size_t)gM.N[0] * (g.d == 3 ? g.N[1] : 1) * g.H;
+  ga_operator(ctx, g, gM, v, out, P->a_ga.get(), 1.0 / (double)g.n_real, precond && !P->aniso, P->wcM.get(), w1, w2);
   // constant anisotropic part: its exact integral is the grid's, grad^* F B F^-1 grad^ = 4 pi^2 k.B k, on the
   // scale of the double-grid product above: A~ carries the double grid's quadrature weight 1 / |M| (a constant
   // material c gives c / |M| times the GaNi operator), so B enters as B / |M|

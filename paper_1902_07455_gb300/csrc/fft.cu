@@ -7,6 +7,7 @@
 // Real fibres are packed two per complex row (x + i y): a real-symmetric multiplier maps it to
 // Mx + i My, so one complex transform pair serves two real fibres.
 #include <cmath>
+#include <type_traits>
 
 #include "ops.cuh"
 
@@ -140,11 +141,19 @@ __device__ __forceinline__ void acc_div_store(const FibreMul<typename RealOf<V>:
   *dst = r;
 }
 
-// OP 0: plain transform; OP 1 and 2: the modes of FibreMul
-template <int SIGN, typename V, int OP>
+// index in a spectrum of length m of the frequency stored at index n of one of length N, -1 where it has none
+__device__ __forceinline__ int same_freq(int n, int N, int m) {
+  const int f = freq_of(n, N);
+  return abs(f) > (m - 1) / 2 ? -1 : (f < 0 ? f + m : f);
+}
+
+// OP 0: plain transform; OP 1 and 2: the modes of FibreMul.  PAD: the input holds nin <= N frequencies of a fibre, the
+// others are zero, or the output keeps nout <= N of them (the double grid of the exact integration)
+template <int SIGN, typename V, int OP, bool PAD>
 __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out, long long outer, int N, long long inner,
                                                          int TF, FftPlan pl, const V* __restrict__ Wg,
-                                                         FibreMul<typename RealOf<V>::T> fm) {
+                                                         FibreMul<typename RealOf<V>::T> fm, int nin,
+                                                         int nout) {
   using R = typename RealOf<V>::T;
   extern __shared__ __align__(16) unsigned char smraw_fib[];
   V* sm = (V*)smraw_fib;
@@ -163,15 +172,21 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
     const int f = threadIdx.x % nf, n0 = threadIdx.x / nf;
     const long long g = g0 + f;
     const long long o = g / inner, i = g - o * inner;
-    const V* src = in + (size_t)o * N * (size_t)inner + (size_t)i;
+    const V* src = in + (size_t)o * (PAD ? nin : N) * (size_t)inner + (size_t)i;
     if (n0 < step)
-      for (int n = n0; n < N; n += step) cp_async<sizeof(V)>(a + (size_t)f * N + n, src + (size_t)n * inner);
+      for (int n = n0; n < N; n += step) {
+        const int m = PAD ? same_freq(n, N, nin) : n;
+        if (m >= 0) cp_async<sizeof(V)>(a + (size_t)f * N + n, src + (size_t)m * inner);
+        else a[(size_t)f * N + n] = mkc<V>(0, 0);
+      }
   } else {
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
       const int f = small_div(t, N, 1.0f / (float)N), n = t - f * N;
       const long long g = g0 + f;
       const long long o = g / inner, i = g - o * inner;
-      cp_async<sizeof(V)>(a + (size_t)f * N + n, in + ((size_t)o * N + n) * (size_t)inner + (size_t)i);
+      const int m = PAD ? same_freq(n, N, nin) : n;
+      if (m >= 0) cp_async<sizeof(V)>(a + t, in + ((size_t)o * (PAD ? nin : N) + m) * (size_t)inner + (size_t)i);
+      else a[t] = mkc<V>(0, 0);
     }
   }
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
@@ -206,29 +221,33 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
     const int f = threadIdx.x % nf, n0 = threadIdx.x / nf;
     const long long g = g0 + f;
     const long long o = g / inner, i = g - o * inner;
-    V* dst = out + (size_t)o * N * (size_t)inner + (size_t)i;
+    const int no = PAD ? nout : N;
+    V* dst = out + (size_t)o * no * (size_t)inner + (size_t)i;
+    const V* row = res + (size_t)f * N;
     if constexpr (OP == 2) {
       int ka, kb;
       fibre_freqs(fm, o, i, ka, kb);
       if (n0 < step)
-        for (int n = n0; n < N; n += step)
-          acc_div_store<V>(fm, dst + (size_t)n * inner, res[(size_t)f * N + n], freq_of(n, N), ka, kb);
+        for (int n = n0; n < no; n += step)
+          acc_div_store<V>(fm, dst + (size_t)n * inner, row[PAD ? same_freq(n, no, N) : n], freq_of(n, no), ka, kb);
     } else {
       if (n0 < step)
-        for (int n = n0; n < N; n += step) dst[(size_t)n * inner] = res[(size_t)f * N + n];
+        for (int n = n0; n < no; n += step) dst[(size_t)n * inner] = row[PAD ? same_freq(n, no, N) : n];
     }
   } else {
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int f = small_div(t, N, 1.0f / (float)N), n = t - f * N;
+    const int no = PAD ? nout : N;
+    for (int t = threadIdx.x; t < nf * no; t += blockDim.x) {
+      const int f = small_div(t, no, 1.0f / (float)no), n = t - f * no;
       const long long g = g0 + f;
       const long long o = g / inner, i = g - o * inner;
-      V* dst = out + ((size_t)o * N + n) * (size_t)inner + (size_t)i;
+      V* dst = out + ((size_t)o * no + n) * (size_t)inner + (size_t)i;
+      const V value = res[(size_t)f * N + (PAD ? same_freq(n, no, N) : n)];
       if constexpr (OP == 2) {
         int ka, kb;
         fibre_freqs(fm, o, i, ka, kb);
-        acc_div_store<V>(fm, dst, res[(size_t)f * N + n], freq_of(n, N), ka, kb);
+        acc_div_store<V>(fm, dst, value, freq_of(n, no), ka, kb);
       } else {
-        *dst = res[(size_t)f * N + n];
+        *dst = value;
       }
     }
   }
@@ -479,15 +498,15 @@ void fft_fibres(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N, long
                : fft2_try<V, 1, 0>(ctx, in, out, outer, N, inner, none, flops, bytes))
     return;
   if (sign < 0) {
-    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 0>, smem));
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 0, false>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<-1, V, 0><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF,
-                                                                                         pl, W, none));
+                fft_fibres_kernel<-1, V, 0, false><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF,
+                                                                                         pl, W, none, N, N));
   } else {
-    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 0>, smem));
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 0, false>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<1, V, 0><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF,
-                                                                                        pl, W, none));
+                fft_fibres_kernel<1, V, 0, false><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF,
+                                                                                        pl, W, none, N, N));
   }
 }
 template void fft_fibres<double2>(lrfg_ctx*, const double2*, double2*, long long, int, long long, int);
@@ -500,8 +519,10 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename 
   LRFG_REQUIRE(fm.d == 2 || fm.d == 3, "d = %d", fm.d);
   LRFG_REQUIRE(fm.axis == 0 || (fm.axis == 1 && fm.d == 3), "axis %d of a half spectrum with d = %d", fm.axis, fm.d);
   LRFG_REQUIRE(fm.alpha >= (fm.mode == 2 ? -1 : 0) && fm.alpha < fm.d, "component %d", fm.alpha);
-  const int N = fm.axis == 0 ? fm.N0 : fm.N1;
-  const long long outer = fm.axis == 0 ? 1 : fm.N0;
+  // the grid's length along the axis, and the transform's (the double grid's where fm.L is set)
+  const int Ng = fm.axis == 0 ? fm.N0 : fm.N1;
+  const int N = fm.L ? fm.L : Ng;
+  const long long outer = fm.axis == 0 ? 1 : (fm.L0 ? fm.L0 : fm.N0);
   const long long inner = fm.axis == 0 ? (long long)(fm.d == 3 ? fm.N1 : 1) * fm.H : fm.H;
   LRFG_REQUIRE(N >= 1 && (N % 2 == 1), "fft length must be odd (got %d)", N);
   LRFG_REQUIRE(fm.mode == 1 || in != out, "the accumulator cannot hold the input");
@@ -516,19 +537,65 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename 
   const double n_el = (double)N * (double)outer * (double)inner;
   const double flops = 5.0 * std::log2((double)N) * n_el + (fm.mode == 1 ? 2.0 : 4.0) * n_el;
   const double bytes = (fm.mode == 1 || fm.init ? 2.0 : 3.0) * sizeof(V) * n_el;
+  if (N != Ng) {
+    LRFG_REQUIRE((std::is_same<V, double2>::value) && N > Ng, "a padded transform is longer than its grid (FP64)");
+    if constexpr (std::is_same<V, double2>::value) {
+      if (fm.mode == 1) {
+        LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 1, true>, smem));
+        LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
+                    fft_fibres_kernel<1, V, 1, true><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
+                        in, out, outer, N, inner, TF, pl, W, fm, Ng, N));
+      } else {
+        LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 2, true>, smem));
+        LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
+                    fft_fibres_kernel<-1, V, 2, true><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
+                        in, out, outer, N, inner, TF, pl, W, fm, N, Ng));
+      }
+    }
+    return;
+  }
   if (fm.mode == 1 ? fft2_try<V, 1, 1>(ctx, in, out, outer, N, inner, fm, flops, bytes)
                    : fft2_try<V, -1, 2>(ctx, in, out, outer, N, inner, fm, flops, bytes))
     return;
   if (fm.mode == 1) {
-    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 1>, smem));
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, V, 1, false>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<1, V, 1><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
-                                                                                        W, fm));
+                fft_fibres_kernel<1, V, 1, false><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
+                                                                                        W, fm, N, N));
   } else {
-    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 2>, smem));
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, V, 2, false>, smem));
     LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
-                fft_fibres_kernel<-1, V, 2><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
-                                                                                         W, fm));
+                fft_fibres_kernel<-1, V, 2, false><<<(unsigned)blocks, 256, smem, ctx->stream>>>(in, out, outer, N, inner, TF, pl,
+                                                                                         W, fm, N, N));
+  }
+}
+
+// Plain transforms between n frequencies and the L > n points of the double grid along the middle axis: inverse
+// (outer, n, inner) -> (outer, L, inner) with zeros for the other frequencies, forward (outer, L, inner) -> (outer, n,
+// inner) keeping n of them.
+void fft_fibres_pad(lrfg_ctx* ctx, const double2* in, double2* out, long long outer, int n, int L, long long inner,
+                    int sign) {
+  LRFG_REQUIRE(L > n && L % 2 == 1 && n % 2 == 1 && in != out, "padded transform %d -> %d", n, L);
+  if (outer == 0 || inner == 0) return;
+  const double2* W = twiddle_table<double>(ctx, L);
+  size_t smem;
+  int TF;
+  const FftPlan pl = tile_complex(ctx, L, sizeof(double2), outer * inner, &TF, &smem);
+  const long long blocks = (outer * inner + TF - 1) / TF;
+  LRFG_REQUIRE(blocks < (1LL << 31), "too many fibres");
+  const double nfib = (double)outer * (double)inner;
+  const double flops = 5.0 * L * std::log2((double)L) * nfib, bytes = sizeof(double2) * (double)(n + L) * nfib;
+  const FibreMul<double> none{};
+  if (sign > 0) {
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<1, double2, 0, true>, smem));
+    LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
+                fft_fibres_kernel<1, double2, 0, true><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
+                    in, out, outer, L, inner, TF, pl, W, none, n, L));
+  } else {
+    LRFG_CUDA(raise_smem_limit((const void*)fft_fibres_kernel<-1, double2, 0, true>, smem));
+    LRFG_LAUNCH(ctx, KC_FFT_FIBRES, flops, bytes,
+                fft_fibres_kernel<-1, double2, 0, true><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
+                    in, out, outer, L, inner, TF, pl, W, none, L, n));
   }
 }
 template void fft_fibres_mul<double2>(lrfg_ctx*, const double2*, double2*, const FibreMul<double>&);

@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(256, 3) c2r_rows_kernel(const typename CplxOf<
 // the material product and the R2C pass of the operator fused, so the real grid never goes to memory.  Both
 // directions pair rows f and f + TF in one complex FFT (real and imaginary parts), so after the inverse
 // transform the product acts on the two parts in place and the forward transform runs on the result as is.
-// `in` and `out` may alias (a block reads all of its rows before it writes them).
+// `in` and `out` may alias (a block reads all of its rows before it writes them).  H: stored frequencies of a row, at
+// most (N + 1) / 2 (fewer on the double grid of the exact integration, where the others are zero and not wanted).
 template <typename R>
 __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename CplxOf<R>::T* in,
                                                                const R* __restrict__ coef, R scale,
@@ -189,9 +190,11 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
         x1[u] = mkc<V>(R(0), R(0));
         if (t < total) {
           const int row = small_div(t, N, invN), k = t - row * N;
-          const int kk = k < H ? k : N - k;
-          x0[u] = in[(size_t)(r0 + row) * H + kk];
-          if (row + TF < nr) x1[u] = in[(size_t)(r0 + row + TF) * H + kk];
+          const int kk = min(k, N - k);
+          if (kk < H) {
+            x0[u] = in[(size_t)(r0 + row) * H + kk];
+            if (row + TF < nr) x1[u] = in[(size_t)(r0 + row + TF) * H + kk];
+          }
         }
       }
 #pragma unroll
@@ -200,7 +203,7 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
         if (t < total) {
           const int row = small_div(t, N, invN), k = t - row * N;
           V p = x0[u], q = x1[u];
-          if (k >= H) { p.y = -p.y; q.y = -q.y; }
+          if (2 * k > N) { p.y = -p.y; q.y = -q.y; }
           a[(size_t)row * N + k] = mkc<V>(p.x - q.y, p.y + q.x);
         }
       }
@@ -479,6 +482,21 @@ void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half
                   half_inout, coef, scale, half_inout, g.rows, N, g.H, TF, pl, W));
 }
 
+void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef) {
+  LRFG_CUDA(ensure_roots(ctx->device));
+  const double2* W = twiddle_table<double>(ctx, N);
+  size_t smem;
+  int TF;
+  const FftPlan pl = row_tile<double>(ctx, N, rows, &TF, &smem);
+  const long long blocks = (rows + 2LL * TF - 1) / (2LL * TF);
+  LRFG_REQUIRE(blocks < (1LL << 31), "too many rows");
+  LRFG_CUDA(raise_smem_limit((const void*)c2r_mul_r2c_rows_kernel<double>, smem));
+  LRFG_LAUNCH(ctx, KC_ROWS_FUSED, 5.0 * N * std::log2((double)N) * (double)rows,
+              (double)rows * (2.0 * H * sizeof(double2) + N * sizeof(double)),
+              c2r_mul_r2c_rows_kernel<double><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
+                  half_inout, coef, 1.0, half_inout, rows, N, H, TF, pl, W));
+}
+
 template void full_rows_mul<double>(lrfg_ctx*, const FullGrid&, double2*, const double*, double);
 template void full_rows_mul<float>(lrfg_ctx*, const FullGrid&, float2*, const float*, float);
 
@@ -728,6 +746,44 @@ void full_operator_3d(lrfg_ctx* ctx, const FullGrid& g, const typename CplxOf<R>
     fft_fibres_mul(ctx, (const V*)h, w2, fibre_mul<R>(g, 2, 1, alpha, 1.0, alpha == 1, 0));
   }
   fft_fibres_mul(ctx, (const V*)w2, out, fibre_mul<R>(g, 2, 0, -1, 1.0, 0, precond));
+}
+
+// The Ga operator (Eq. (ls_Ga_fourier)): as above with every transform between the grid's N frequencies and the double
+// grid's M points.  A zero-padded spectrum is padded axis by axis inside the passes, so the fibres of frequencies outside
+// the grid, zero before the inverse passes and dropped after the forward ones, are never transformed: axis 0 runs on a
+// quarter of the double grid's fibres, axis 1 on half of them, and the real double grid never goes to memory.  w0: one half
+// spectrum of the double grid; w1, w2: M_0 N_1 H each (d = 3).
+void ga_operator(lrfg_ctx* ctx, const FullGrid& g, const FullGrid& gM, const double2* v, double2* out, const double* coef,
+                 double scale, int precond, double2* w0, double2* w1, double2* w2) {
+  auto fm = [&](int mode, int axis, int alpha, double sc, int init, int pc) {
+    FibreMul<double> f = fibre_mul<double>(g, mode, axis, alpha, sc, init, pc);
+    f.L = gM.N[axis];
+    f.L0 = gM.N[0];
+    return f;
+  };
+  const int last = gM.N[g.d - 1];
+  if (g.d == 2) {
+    for (int alpha = 0; alpha < 2; ++alpha) {
+      fft_fibres_mul(ctx, v, w0, fm(1, 0, alpha, scale, 0, 0));
+      half_rows_mul(ctx, gM.N[0], last, g.H, w0, coef);
+      fft_fibres_mul(ctx, (const double2*)w0, out, fm(2, 0, alpha, 1.0, alpha == 0, alpha == 1 && precond));
+    }
+    return;
+  }
+  const long long in0 = (long long)g.N[1] * g.H, rows = (long long)gM.N[0] * gM.N[1];
+  const int n1 = g.N[1], m1 = gM.N[1];
+  fft_fibres_mul(ctx, v, w1, fm(1, 0, 0, scale, 0, 0));
+  fft_fibres_pad(ctx, w1, w0, gM.N[0], n1, m1, g.H, 1);
+  half_rows_mul(ctx, rows, last, g.H, w0, coef);
+  fft_fibres_pad(ctx, w0, w1, gM.N[0], n1, m1, g.H, -1);
+  fft_fibres_mul(ctx, (const double2*)w1, out, fm(2, 0, 0, 1.0, 1, 0));
+  fft_fibres_pad(ctx, v, w1, 1, g.N[0], gM.N[0], in0, 1);
+  for (int alpha = 1; alpha <= 2; ++alpha) {
+    fft_fibres_mul(ctx, (const double2*)w1, w0, fm(1, 1, alpha, scale, 0, 0));
+    half_rows_mul(ctx, rows, last, g.H, w0, coef);
+    fft_fibres_mul(ctx, (const double2*)w0, w2, fm(2, 1, alpha, 1.0, alpha == 1, 0));
+  }
+  fft_fibres_mul(ctx, (const double2*)w2, out, fm(2, 0, -1, 1.0, 0, precond));
 }
 
 template void full_operator_3d<double>(lrfg_ctx*, const FullGrid&, const double2*, double2*, const double*, double, int,

@@ -30,11 +30,17 @@ void fft_fibres(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N, long
 template <typename R>
 struct FibreMul {
   int mode, axis, alpha, d, N0, N1, H, init, precond;
+  // transforms of length L > the grid's along the axis (the double grid of the exact integration): mode 1 takes the other
+  // frequencies as zero, mode 2 drops them; L0: points of axis 0 when axis 1 is transformed (0: N0, and L = 0: none)
+  int L, L0;
   R c2;             // 2 pi scale, rounded to R
   const R* inv_kk;  // 1/(k.k) indexed by k.k, 0 at k = 0 (mode 2 with precond)
 };
 template <typename V>
 void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename RealOf<V>::T>& fm);
+// plain transforms between n frequencies and L > n points (see fft.cu)
+void fft_fibres_pad(lrfg_ctx* ctx, const double2* in, double2* out, long long outer, int n, int L, long long inner,
+                    int sign);
 // Ga mode maps on real fibres (outer, n_in, inner) -> (outer, n_out, inner), M = 2N - 1 (Sec. 2.2.3):
 //  GA_UP      N -> M  band-limited interpolation to the double grid, F_M^-1 I F_N;
 //  GA_DOWN    M -> N  projection, F_N^-1 I* F_M;
