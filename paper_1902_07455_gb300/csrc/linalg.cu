@@ -41,7 +41,9 @@ __device__ __forceinline__ void gemm_fma_rows(T* acc, const T (*As)[TILE + 1], c
 // four times the blocks, so that a product of a few tiles still spreads over the SMs) or 16 (one per thread,
 // for products of one or a few 32-tiles with a short K, see gemm_impl).
 // T = double (the FP64 products) or float (the FP32 sketch products of the mixed-precision path).
-template <bool TA, bool TB, int TILE, typename T>
+// SYM: the product is symmetric (a Gram matrix, or F R F^T with a symmetric R); only the tiles and outputs on and below
+// the diagonal are computed, each written to both places: half the FP64 work of a product that is bound by it.
+template <bool TA, bool TB, int TILE, typename T, bool SYM>
 __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double alpha_d, const T* __restrict__ A,
                                                     int lda, long long sA, const T* __restrict__ B, int ldb,
                                                     long long sB, double beta_d, T* C, int ldc, long long sC,
@@ -63,21 +65,32 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
   if (dynM) M = min(M, dynM[batch] * mulM);
   if (dynN) N = min(N, dynN[batch] * mulN);
   if (work && bm == 0 && bn == 0 && split == 0 && threadIdx.x == 0)
-    add_work(work, 2.0 * M * N * (double)K, (double)sizeof(T) * ((double)M * K + (double)K * N + (double)M * N));
+    add_work(work, (SYM ? 1.0 * M * (M + 1.0) : 2.0 * M * N) * (double)K, (double)sizeof(T) * ((double)M * K + (double)K * N + (double)M * N));
   const int m0 = bm * TILE, n0 = bn * TILE;
   const int Mb = min(TILE, M - m0), Nb = min(TILE, N - n0);
   if (Mb <= 0 || Nb <= 0) return;
+  if (SYM && bn > bm) return;
+  const bool tri = SYM && bn == bm;
   const int kbeg = split * kchunk, kend = min(K, kbeg + kchunk);
   // this thread's outputs o = t + 256 j < Mb Nb, as (row, column) within the block
-  const int tot = Mb * Nb;
+  const int tot = tri ? Mb * (Mb + 1) / 2 : Mb * Nb;
   const int nact = tot > (int)threadIdx.x ? min(NMAX, (tot - (int)threadIdx.x + 255) / 256) : 0;
   int pk[NMAX];
   T acc[NMAX];
 #pragma unroll
   for (int j = 0; j < NMAX; ++j) {
     const int o = threadIdx.x + 256 * j;
-    const int m = o / Nb;
-    pk[j] = j < nact ? (m << 16) | (o - m * Nb) : 0;
+    int m, c0;  // row and the index of its first output
+    if (tri) {
+      m = (int)((sqrtf(8.0f * (float)o + 1.0f) - 1.0f) * 0.5f);
+      while (m * (m + 1) / 2 > o) --m;
+      while ((m + 1) * (m + 2) / 2 <= o) ++m;
+      c0 = m * (m + 1) / 2;
+    } else {
+      m = o / Nb;
+      c0 = m * Nb;
+    }
+    pk[j] = j < nact ? (m << 16) | (o - c0) : 0;
     acc[j] = (T)0;
   }
   for (int k0 = kbeg; k0 < kend; k0 += GK) {
@@ -188,7 +201,9 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
       T v = (T)0;
       for (int s = 0; s < nsum; ++s) v += __ldcg(S + s * pstride + off);
       T* cp = C + (size_t)(m0 + (pk[j] >> 16)) * ldc + n0 + (pk[j] & 0xffff);
-      *cp = (beta_d == 0.0) ? alpha * v : alpha * v + beta * (*cp);
+      v = (beta_d == 0.0) ? alpha * v : alpha * v + beta * (*cp);
+      *cp = v;
+      if (SYM) C[(size_t)(n0 + (pk[j] & 0xffff)) * ldc + m0 + (pk[j] >> 16)] = v;
     }
     if (threadIdx.x == 0) *c = 0u;  // ready for the next product
     return;
@@ -197,7 +212,9 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
   for (int j = 0; j < NMAX; ++j) {
     if (j >= nact) break;
     T* c = C + (size_t)(m0 + (pk[j] >> 16)) * ldc + n0 + (pk[j] & 0xffff);
-    *c = (beta_d == 0.0) ? alpha * acc[j] : alpha * acc[j] + beta * (*c);
+    const T v = (beta_d == 0.0) ? alpha * acc[j] : alpha * acc[j] + beta * (*c);
+    *c = v;
+    if (SYM) C[(size_t)(n0 + (pk[j] & 0xffff)) * ldc + m0 + (pk[j] >> 16)] = v;
   }
 }
 
@@ -206,23 +223,24 @@ static void launch_dgemm(lrfg_ctx* ctx, int transA, int transB, dim3 grid, doubl
                          int K, double alpha, const T* A, int lda, long long sA, const T* B, int ldb,
                          long long sB, double beta, T* C, int ldc, long long sC, int splits, int kchunk,
                          const int* dynM, int mulM, const int* dynN, int mulN, double* work, T* part,
-                         int gsize = 1 << 30) {
-  if (!transA && !transB)
-    LRFG_LAUNCH_KC(ctx, (std::is_same<T, float>::value ? KC_GEMM32 : KC_GEMM), flops, bytes, dgemm_kernel<false, false, TILE, T><<<grid, 256, 0, ctx->stream>>>(
-        M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part,
-        ctx->splitk_cnt, gsize));
-  else if (transA && !transB)
-    LRFG_LAUNCH_KC(ctx, (std::is_same<T, float>::value ? KC_GEMM32 : KC_GEMM), flops, bytes, dgemm_kernel<true, false, TILE, T><<<grid, 256, 0, ctx->stream>>>(
-        M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part,
-        ctx->splitk_cnt, gsize));
-  else if (!transA && transB)
-    LRFG_LAUNCH_KC(ctx, (std::is_same<T, float>::value ? KC_GEMM32 : KC_GEMM), flops, bytes, dgemm_kernel<false, true, TILE, T><<<grid, 256, 0, ctx->stream>>>(
-        M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part,
-        ctx->splitk_cnt, gsize));
-  else
-    LRFG_LAUNCH_KC(ctx, (std::is_same<T, float>::value ? KC_GEMM32 : KC_GEMM), flops, bytes, dgemm_kernel<true, true, TILE, T><<<grid, 256, 0, ctx->stream>>>(
-        M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part,
-        ctx->splitk_cnt, gsize));
+                         int gsize = 1 << 30, bool sym = false) {
+  auto launch = [&](auto kernel) {
+    LRFG_LAUNCH_KC(ctx, (std::is_same<T, float>::value ? KC_GEMM32 : KC_GEMM), flops, bytes,
+                   kernel<<<grid, 256, 0, ctx->stream>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, splits,
+                                                         kchunk, dynM, mulM, dynN, mulN, work, part, ctx->splitk_cnt,
+                                                         gsize));
+  };
+  if constexpr (std::is_same<T, double>::value) {
+    if (sym) {
+      if (transA && !transB) launch(dgemm_kernel<true, false, TILE, T, true>);
+      else launch(dgemm_kernel<false, true, TILE, T, true>);
+      return;
+    }
+  }
+  if (!transA && !transB) launch(dgemm_kernel<false, false, TILE, T, false>);
+  else if (transA && !transB) launch(dgemm_kernel<true, false, TILE, T, false>);
+  else if (!transA && transB) launch(dgemm_kernel<false, true, TILE, T, false>);
+  else launch(dgemm_kernel<true, true, TILE, T, false>);
 }
 
 __global__ void scale_matrix_kernel(double* C, int M, int N, int ldc, long long sC, int batch, double beta) {
@@ -246,8 +264,9 @@ void gemm(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alp
 template <typename T>
 static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const T* A, int lda,
                       long long sA, const T* B, int ldb, long long sB, double beta, T* C, int ldc, long long sC,
-                      int batch, const int* dynM, int mulM, const int* dynN, int mulN) {
+                      int batch, const int* dynM, int mulM, const int* dynN, int mulN, bool sym = false) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
+  LRFG_REQUIRE(!sym || (M == N && transA != transB && beta == 0.0), "not a symmetric product");
   if (K <= 0) {
     LRFG_REQUIRE((std::is_same<T, double>::value), "FP32 product with an empty inner dimension");
     LRFG_LAUNCH(ctx, KC_GEMM, (double)M * N * batch, 2.0 * sizeof(double) * M * N * batch,
@@ -260,7 +279,8 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // blocks expected to be active: the static count, or for data-dependent sizes a quarter of it (the
   // numerical ranks are typically well below their bounds), at least one per item
   auto active_tiles = [&](int tile) {
-    long long a = (long long)((M + tile - 1) / tile) * ((N + tile - 1) / tile) * batch;
+    const long long tm = (M + tile - 1) / tile, tn = (N + tile - 1) / tile;
+    long long a = (sym ? tm * (tm + 1) / 2 : tm * tn) * batch;
     if (dynM || dynN) a = std::max<long long>(batch, a / 4);
     return a;
   };
@@ -306,18 +326,18 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   if (splits > 1) part = DBuf<T>(ctx->pool, (size_t)(splits + ngroups) * M * N * batch);
   // products with data-dependent sizes count their work on the device
   double* work = (dynM || dynN) ? work_counter(ctx, KC_GEMM) : nullptr;
-  const double flops = work ? 0.0 : 2.0 * M * N * (double)K * batch;
+  const double flops = work ? 0.0 : (sym ? 1.0 * M * (M + 1.0) : 2.0 * M * N) * (double)K * batch;
   const double bytes = work ? 0.0 : sizeof(T) * ((double)M * K + (double)K * N + (double)M * N) * batch;
   dim3 grid(bnn, bmn * splits, batch);
   if (tile == 16)
     launch_dgemm<16, T>(ctx, transA, transB, grid, flops, bytes, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
-                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize);
+                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize, sym);
   else if (tile == 32)
     launch_dgemm<32, T>(ctx, transA, transB, grid, flops, bytes, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
-                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize);
+                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize, sym);
   else
     launch_dgemm<64, T>(ctx, transA, transB, grid, flops, bytes, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc,
-                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize);
+                     sC, splits, kchunk, dynM, mulM, dynN, mulN, work, part.get(), gsize, sym);
 }
 
 void gemm_dyn(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const double* A, int lda,
@@ -325,6 +345,11 @@ void gemm_dyn(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double
               int batch, const int* dynM, int mulM, const int* dynN, int mulN) {
   gemm_impl<double>(ctx, transA, transB, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, batch, dynM, mulM,
                     dynN, mulN);
+}
+
+void gemm_sym(lrfg_ctx* ctx, int trans, int M, int K, const double* A, int lda, long long sA, const double* B, int ldb,
+              long long sB, double* C, int ldc, long long sC, int batch, const int* dyn) {
+  gemm_impl<double>(ctx, trans, !trans, M, M, K, 1.0, A, lda, sA, B, ldb, sB, 0.0, C, ldc, sC, batch, dyn, 1, dyn, 1, true);
 }
 
 void gemm_f32(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const float* A, int lda,

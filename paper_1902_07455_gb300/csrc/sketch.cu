@@ -270,10 +270,10 @@ static void cholqr2(lrfg_ctx* ctx, const double* A, int m, int l, int nb, double
   const long long sa = (long long)m * l, sl = (long long)l * l;
   DBuf<double> G(ctx->pool, (size_t)sl * nb), RA(ctx->pool, (size_t)sl * nb), Pc(ctx->pool, (size_t)sl * nb);
   DBuf<double> Q1(ctx->pool, (size_t)sa * nb);
-  gemm(ctx, 1, 0, l, l, m, 1.0, A, l, sa, A, l, sa, 0.0, G.get(), l, sl, nb);
+  gemm_sym(ctx, 1, l, m, A, l, sa, A, l, sa, G.get(), l, sl, nb);
   gram_factor(ctx, G.get(), nullptr, l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
   gemm(ctx, 0, 0, m, l, l, 1.0, A, l, sa, Pc.get(), l, sl, 0.0, Q1.get(), l, sa, nb);
-  gemm(ctx, 1, 0, l, l, m, 1.0, Q1.get(), l, sa, Q1.get(), l, sa, 0.0, G.get(), l, sl, nb);
+  gemm_sym(ctx, 1, l, m, Q1.get(), l, sa, Q1.get(), l, sa, G.get(), l, sl, nb);
   gram_factor(ctx, G.get(), nullptr, l, nb, RA.get(), nullptr, Pc.get(), nullptr, 1e-16);
   gemm(ctx, 0, 0, m, l, l, 1.0, Q1.get(), l, sa, Pc.get(), l, sl, 0.0, Q, l, sa, nb);
 }
@@ -322,7 +322,7 @@ static void truncate_left_orth(lrfg_ctx* ctx, const TTBatch& y, int rmax, TTBatc
     const int a = y.r[j], n = y.N[j], cols = n * b, kcap = kr[j];
     const long long sc = (long long)a * cols, saa = (long long)a * a;
     DBuf<double> S(ctx->pool, (size_t)saa * nb), w(ctx->pool, (size_t)a * nb), V(ctx->pool, (size_t)saa * nb);
-    gemm(ctx, 0, 1, a, a, cols, 1.0, Cg, cols, sc, Cg, cols, sc, 0.0, S.get(), a, saa, nb);
+    gemm_sym(ctx, 0, a, cols, Cg, cols, sc, Cg, cols, sc, S.get(), a, saa, nb);
     syevx(ctx, S.get(), w.get(), V.get(), a, kcap, nb);
     int k = kcap;
     if (tol > 0.0) {

@@ -424,7 +424,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
     const int s = x.r[j], n = x.N[j];
     const long long sx = (long long)x.elems(j), ss = (long long)s * s;
     R[j] = DBuf<double>(ctx->pool, (size_t)ss * nb);
-    gemm(ctx, 0, 1, s, s, n, 1.0, x.core[j], n, sx, x.core[j], n, sx, 0.0, R[j].get(), s, ss, nb);
+    gemm_sym(ctx, 0, s, n, x.core[j], n, sx, x.core[j], n, sx, R[j].get(), s, ss, nb);
     // d = 3: bond 0 contracts carriage 1 with R[2] after projecting on its left basis (below), so the
     // Gram of carriages 1..2 (the 2 N s^3 term that dominates the rounding of rank-s products) is not
     // formed
@@ -434,7 +434,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       DBuf<double> T(ctx->pool, (size_t)sxj * nb);
       gemm(ctx, 0, 0, a * nn, b, b, 1.0, x.core[jj], b, sxj, R[jj + 1].get(), b, sb, 0.0, T.get(), b, sxj, nb);
       R[jj] = DBuf<double>(ctx->pool, (size_t)sa * nb);
-      gemm(ctx, 0, 1, a, a, nn * b, 1.0, T.get(), nn * b, sxj, x.core[jj], nn * b, sxj, 0.0, R[jj].get(), a, sa, nb);
+      gemm_sym(ctx, 0, a, nn * b, T.get(), nn * b, sxj, x.core[jj], nn * b, sxj, R[jj].get(), a, sa, nb);
     }
   }
   // left sweep
@@ -448,7 +448,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
     long long sbk = (long long)b * kcap, skk = (long long)kcap * kcap, sout = 0;
     int k = kcap;
     DBuf<double> GA(ctx->pool, (size_t)sbb * nb), cb(ctx->pool, (size_t)b * nb);
-    gemm(ctx, 1, 0, b, b, rows, 1.0, Z, b, sz, Z, b, sz, 0.0, GA.get(), b, sbb, nb);
+    gemm_sym(ctx, 1, b, rows, Z, b, sz, Z, b, sz, GA.get(), b, sbb, nb);
     const bool projected = (d == 3 && j == 0);
     if (projected) {
       const int n1 = x.N[1], b2 = x.r[2];
@@ -507,11 +507,10 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
                  Wc.get(), n1 * b2, sw, nb, rk.get(), 1, nullptr, 1);
         gemm_dyn(ctx, 0, 0, b * n1, b2, b2, 1.0, Wc.get(), b2, sw, R[2].get(), b2, sr2, 0.0, Qw.get(), b2, sw, nb,
                  rk.get(), n1, nullptr, 1);
-        gemm_dyn(ctx, 0, 1, b, b, n1 * b2, 1.0, Qw.get(), n1 * b2, sw, Wc.get(), n1 * b2, sw, 0.0, S.get(), b, sbb,
-                 nb, rk.get(), 1, rk.get(), 1);
+        gemm_sym(ctx, 0, b, n1 * b2, Qw.get(), n1 * b2, sw, Wc.get(), n1 * b2, sw, S.get(), b, sbb, nb, rk.get());
       } else {
         gemm(ctx, 0, 0, b, b, b, 1.0, F.get(), b, sbb, R[j + 1].get(), b, sbb, 0.0, F1.get(), b, sbb, nb);
-        gemm(ctx, 0, 1, b, b, b, 1.0, F1.get(), b, sbb, F.get(), b, sbb, 0.0, S.get(), b, sbb, nb);
+        gemm_sym(ctx, 0, b, b, F1.get(), b, sbb, F.get(), b, sbb, S.get(), b, sbb, nb);
       }
       syevx_sized(ctx, S.get(), rk.get(), sig.get(), US.get(), b, kcap, nb);
       settle_rank();
@@ -525,7 +524,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       // the same truncation); transfer T = Y^T M, computed explicitly
       gram_factor(ctx, R[j + 1].get(), nullptr, b, nb, F.get(), nullptr, nullptr, rk.get());
       gemm(ctx, 0, 0, b, b, b, 1.0, F.get(), b, sbb, GA.get(), b, sbb, 0.0, F1.get(), b, sbb, nb);
-      gemm(ctx, 0, 1, b, b, b, 1.0, F1.get(), b, sbb, F.get(), b, sbb, 0.0, S.get(), b, sbb, nb);
+      gemm_sym(ctx, 0, b, b, F1.get(), b, sbb, F.get(), b, sbb, S.get(), b, sbb, nb);
       syevx_sized(ctx, S.get(), rk.get(), sig.get(), US.get(), b, kcap, nb);
       settle_rank();
       DBuf<double> P0(ctx->pool, (size_t)sbk * nb);
@@ -536,8 +535,7 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       DBuf<double> Y0(ctx->pool, (size_t)rows * k * nb), G(ctx->pool, (size_t)skk * nb);
       DBuf<double> GR(ctx->pool, (size_t)skk * nb), GP(ctx->pool, (size_t)skk * nb);
       gemm(ctx, 0, 0, rows, k, b, 1.0, Z, b, sz, P0.get(), k, sbk, 0.0, Y0.get(), k, (long long)rows * k, nb);
-      gemm(ctx, 1, 0, k, k, rows, 1.0, Y0.get(), k, (long long)rows * k, Y0.get(), k, (long long)rows * k, 0.0,
-           G.get(), k, skk, nb);
+      gemm_sym(ctx, 1, k, rows, Y0.get(), k, (long long)rows * k, Y0.get(), k, (long long)rows * k, G.get(), k, skk, nb);
       gram_factor(ctx, G.get(), nullptr, k, nb, GR.get(), nullptr, GP.get(), nullptr);
       gemm(ctx, 0, 0, rows, k, k, 1.0, Y0.get(), k, (long long)rows * k, GP.get(), k, skk, 0.0, out.core[j].get(),
            k, sout, nb);
@@ -714,9 +712,9 @@ void tt_compress(lrfg_ctx* ctx, int d, const int* N, const double* values, int r
     const int m = use_rows ? rows : (int)cols;
     DBuf<double> G(ctx->pool, (size_t)m * m), lam(ctx->pool, m), V(ctx->pool, (size_t)m * m);
     if (use_rows)
-      gemm(ctx, 0, 1, m, m, (int)cols, 1.0, C.get(), (int)cols, 0, C.get(), (int)cols, 0, 0.0, G.get(), m, 0);
+      gemm_sym(ctx, 0, m, (int)cols, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0);
     else
-      gemm(ctx, 1, 0, m, m, rows, 1.0, C.get(), (int)cols, 0, C.get(), (int)cols, 0, 0.0, G.get(), m, 0);
+      gemm_sym(ctx, 1, m, rows, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0);
     // only the kept eigenpairs are decomposed (with a tolerance, every eigenvalue: the rule sums the tail): a cyclic
     // Jacobi of the whole m x m Gram matrix in one block took 46 ms per bond at m = 135, this 2.3 ms; a compression of
     // 135^3 values to rank 10 with its expansion went from 98.3 to 5.8 ms

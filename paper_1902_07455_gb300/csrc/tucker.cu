@@ -101,14 +101,14 @@ static void mode_gram(lrfg_ctx* ctx, const double* in, int d, const int* dims, i
   const int nj = dims[j];
   const int rest = (int)(tot / nj);
   if (j == 0) {
-    gemm(ctx, 0, 1, nj, nj, rest, 1.0, in, rest, 0, in, rest, 0, 0.0, S, nj, 0);
+    gemm_sym(ctx, 0, nj, rest, in, rest, 0, in, rest, 0, S, nj, 0);
   } else if (j == d - 1) {
-    gemm(ctx, 1, 0, nj, nj, rest, 1.0, in, nj, 0, in, nj, 0, 0.0, S, nj, 0);
+    gemm_sym(ctx, 1, nj, rest, in, nj, 0, in, nj, 0, S, nj, 0);
   } else {
     DBuf<double> tmp(ctx->pool, (size_t)tot);
     LRFG_LAUNCH(ctx, KC_TT_MISC, 0.0, 16.0 * tot,
                 swap01_kernel<<<grid_of(ctx, tot), 256, 0, ctx->stream>>>(in, tmp.get(), dims[0], dims[1], dims[2]));
-    gemm(ctx, 0, 1, nj, nj, rest, 1.0, tmp.get(), rest, 0, tmp.get(), rest, 0, 0.0, S, nj, 0);
+    gemm_sym(ctx, 0, nj, rest, tmp.get(), rest, 0, tmp.get(), rest, 0, S, nj, 0);
   }
 }
 
@@ -242,7 +242,7 @@ void tk_round(lrfg_ctx* ctx, const TKView& x, int rmax, TK& out, double tol) {
   for (int j = 0; j < d; ++j) {
     const int m = r[j];
     DBuf<double> G(ctx->pool, (size_t)m * m), c(ctx->pool, m), RA(ctx->pool, (size_t)m * m);
-    gemm(ctx, 1, 0, m, m, x.N[j], 1.0, x.fac[j], m, 0, x.fac[j], m, 0, 0.0, G.get(), m, 0);
+    gemm_sym(ctx, 1, m, x.N[j], x.fac[j], m, 0, x.fac[j], m, 0, G.get(), m, 0);
     LRFG_LAUNCH(ctx, KC_TT_MISC, 2.0 * m * m, 16.0 * m * m,
                 unit_balance_kernel<<<1, 256, sizeof(double) * m, ctx->stream>>>(G.get(), c.get(), m));
     RAc[j] = DBuf<double>(ctx->pool, (size_t)m * m);
