@@ -11,8 +11,8 @@
 // same absolute accuracy (eps ||A||), which is what the Gram-SVD truncation needs.
 // The steps are chains of dependent FP64 operations, and on this part a warp issues one FP64 instruction per 64 cycles
 // whatever its instruction-level parallelism or active lanes (an SM has four such units): each kernel is laid out to put
-// few FP64 instructions on the longest of the four.  Three matrices of n = 30, k = 20 take 158 us (420 us with the same
-// algorithm laid out by arithmetic alone), one of n = 60, k = 20 533 us (744), n = 135, k = 10 2.0 ms (2.3).
+// few FP64 instructions on the longest of the four.  Three matrices of n = 30, k = 20 take 155 us (420 us with the same
+// algorithm laid out by arithmetic alone), one of n = 60, k = 20 402 us (744), n = 135, k = 10 2.0 ms (2.3).
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -555,7 +555,8 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
 // such units, so a step takes as long as the unit with the most FP64 instructions on its path:
 //  * warp 0 forms the reflector's scalars from the norm of x while the workers multiply: with v = x + s ||x|| e_1 the
 //    product A v = A x + s ||x|| a_1 needs no finished v, and v^T A v follows from x^T A x, (A x)_1 and a_11;
-//  * three workers, one per remaining unit (six halves of the registers at n > 64);
+//  * three workers, one per remaining unit (four at n > 32, where their share outweighs warp 0's; six halves of the
+//    registers at n > 64); operands are loaded four columns ahead of the arithmetic they feed;
 //  * the two columns the next step reads are updated and published first, the rest after the barrier;
 //  * one square root and one reciprocal a step (recip_sqrt, recip), two barriers.
 template <int NR, int TW>
@@ -565,10 +566,10 @@ __global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const do
                                                                              const int* __restrict__ nAg,
                                                                              double* work) {
   constexpr int M = 32 * NR, NC = (M + TW - 1) / TW;
-  __shared__ double xs[2][M], a1s[2][M], ys[M], parts[TW][M], ds[M], es[M], red[40];
+  __shared__ double xs[2][M + 4 * TW], a1s[2][M + 4 * TW], ys[M], parts[TW][M], ds[M], es[M], red[40];
   __shared__ double sc[4];
   __shared__ int sred[32];
-  __shared__ double2 vws[TW][M];
+  __shared__ double2 vws[TW][M + 4 * TW];
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, w = (tid >> 5) - 1;
   double* wout = wg + (size_t)blockIdx.x * nl;
@@ -649,23 +650,27 @@ __global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const do
         if (row > j && row < n) g.W[(size_t)row * n + j] = row == j + 1 ? xr[r] + sn : xr[r];
       }
     } else {
-      double p0[NR], p1[NR];
+      double p0[NR];
 #pragma unroll
-      for (int r = 0; r < NR; ++r) p0[r] = p1[r] = 0.0;
+      for (int r = 0; r < NR; ++r) p0[r] = 0.0;
+      // (the operands of four columns are loaded before any is used; row slots above the trailing block are skipped)
 #pragma unroll
-      for (int cc = 0; cc < NC; ++cc) {
-        const int col = cc * TW + w;
-        if (col > j && col < n) {
-          const double xc = x[col];
+      for (int c0 = 0; c0 < NC; c0 += 4) {
+        if ((c0 + 3) * TW + w <= j) continue;
+        double xc[4];
 #pragma unroll
-          for (int r = 0; r < NR; ++r) {
-            double* acc = (cc & 1) ? p1 : p0;
-            acc[r] = fma(a[r][cc], xc, acc[r]);
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u < NC) xc[u] = x[(c0 + u) * TW + w];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u < NC && (c0 + u) * TW + w > j && (c0 + u) * TW + w < n) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+              if (32 * r + 31 > j) p0[r] = fma(a[r][c0 + u], xc[u], p0[r]);
           }
-        }
       }
 #pragma unroll
-      for (int r = 0; r < NR; ++r) parts[w][lane + 32 * r] = p0[r] + p1[r];
+      for (int r = 0; r < NR; ++r) parts[w][lane + 32 * r] = p0[r];
       asm volatile("bar.sync 1, %0;" ::"n"(32 * TW) : "memory");
       if (w == 0) {
         double xy = 0.0;
@@ -685,10 +690,10 @@ __global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const do
     __syncthreads();
     // w = b q - K v with q = A v = y + sn a_1, K = b^2 v^T q / 2; then the next step's two columns
     double vr[NR], wr[NR];
-    auto update = [&](int cc) {
-      const double2 c = vws[max(w, 0)][cc * TW + w];
+    auto update = [&](int cc, double2 c) {
 #pragma unroll
-      for (int r = 0; r < NR; ++r) a[r][cc] = fma(-vr[r], c.y, fma(-wr[r], c.x, a[r][cc]));
+      for (int r = 0; r < NR; ++r)
+        if (32 * r + 31 > j) a[r][cc] = fma(-vr[r], c.y, fma(-wr[r], c.x, a[r][cc]));
     };
     if (w >= 0) {
       const double sn = sc[0], b = sc[1];
@@ -708,7 +713,7 @@ __global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const do
       for (int cc = 0; cc < NC; ++cc) {
         const int col = cc * TW + w;
         if (col == j + 1 || col == j + 2) {
-          update(cc);
+          update(cc, vws[w][col]);
 #pragma unroll
           for (int r = 0; r < NR; ++r) (col == j + 1 ? xs[par ^ 1] : a1s[par ^ 1])[lane + 32 * r] = a[r][cc];
         }
@@ -717,9 +722,17 @@ __global__ void __launch_bounds__(32 * (TW + 1)) syevx_tri_small_kernel(const do
     __syncthreads();
     if (w >= 0) {
 #pragma unroll
-      for (int cc = 0; cc < NC; ++cc) {
-        const int col = cc * TW + w;
-        if (col > j + 2 && col < n) update(cc);
+      for (int c0 = 0; c0 < NC; c0 += 4) {
+        if ((c0 + 3) * TW + w <= j + 2) continue;
+        double2 c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u < NC) c[u] = vws[w][(c0 + u) * TW + w];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int col = (c0 + u) * TW + w;
+          if (c0 + u < NC && col > j + 2 && col < n) update(c0 + u, c[u]);
+        }
       }
     }
   }
@@ -763,30 +776,40 @@ constexpr int kQCols = kBisectThreads / 8;
 __device__ void form_q_columns(const SyevxScratch& g, int n, int c0, double* sm) {
   const int tid = threadIdx.x, gl = tid & 7, c = c0 + (tid >> 3);
   const int ld = n | 1;
-  double* y = sm + (size_t)(tid >> 3) * ld;
-  for (int i = gl; i < n; i += 8) y[i] = i == c ? 1.0 : 0.0;
-  __syncwarp();
+  double* v = sm;                    // reflector j at v + j ld, rows j + 1 .. n - 1; beta_j at row j
+  double* y = sm + (size_t)n * ld + (size_t)(tid >> 3) * ld;
   const int last = min(n - 3, c0 + kQCols - 2);  // H_j leaves e_c as it is while c <= j
+  for (int q = tid; q < n * n; q += kBisectThreads) {
+    const int i = q / n, j = q - i * n;
+    if (j <= last && i >= j) v[j * ld + i] = i == j ? g.beta[j] : g.W[q];
+  }
+  for (int i = gl; i < n; i += 8) y[i] = i == c ? 1.0 : 0.0;
+  __syncthreads();
   for (int j = last; j >= 0; --j) {
-    const double b = g.beta[j];
+    const double* vj = v + j * ld;
+    const double b = vj[j];
     if (b == 0.0) continue;
-    const double* v = g.W + (size_t)(j + 1) * n + j;
-    double* yj = y + j + 1;
-    const int m = n - j - 1;
-    double vr[12], s = 0.0;
+    // rows j + 1 .. n - 1 dealt to eight lanes
+    double vr[12], yr[12], s0 = 0.0;
 #pragma unroll
     for (int q = 0; q < 12; ++q) {
-      const int i = gl + 8 * q;
-      vr[q] = i < m ? v[(size_t)i * n] : 0.0;
+      const int i = j + 1 + gl + 8 * q;
+      vr[q] = i < n ? vj[i] : 0.0;
+      yr[q] = i < n ? y[i] : 0.0;
     }
 #pragma unroll
     for (int q = 0; q < 12; ++q)
-      if (8 * q < m) s = fma(vr[q], gl + 8 * q < m ? yj[gl + 8 * q] : 0.0, s);
-    for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
-    s *= b;
+      if (j + 1 + 8 * q < n) s0 = fma(vr[q], yr[q], s0);
+    for (int o = 4; o; o >>= 1) s0 += __shfl_xor_sync(0xffffffff, s0, o);
+    s0 *= b;
 #pragma unroll
-    for (int q = 0; q < 12; ++q)
-      if (8 * q < m && gl + 8 * q < m) yj[gl + 8 * q] = fma(-s, vr[q], yj[gl + 8 * q]);
+    for (int q = 0; q < 12; ++q) {
+      const int i = j + 1 + gl + 8 * q;
+      if (j + 1 + 8 * q < n) {
+        yr[q] = fma(-s0, vr[q], yr[q]);
+        if (i < n) y[i] = yr[q];
+      }
+    }
     __syncwarp();
   }
   if (c < n)
@@ -1118,7 +1141,7 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
   if (n <= 32) {
     tri_small(syevx_tri_small_kernel<1, 3>, 128);
   } else if (n <= 64) {
-    tri_small(syevx_tri_small_kernel<2, 3>, 128);
+    tri_small(syevx_tri_small_kernel<2, 4>, 160);
   } else if (n <= kSmallEig) {
     tri_small(syevx_tri_small_kernel<3, 6>, 224);
   } else {
@@ -1133,7 +1156,7 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
   }
   // K2: one block per wanted eigenvalue of every item, and the blocks that form Q
   const int nq = n <= kSmallEig ? (n + kQCols - 1) / kQCols : 0;
-  const size_t smem2 = sizeof(double) * std::max(3 * (size_t)n, nq ? (size_t)kQCols * (n | 1) : (size_t)0);
+  const size_t smem2 = sizeof(double) * std::max(3 * (size_t)n, nq ? (size_t)(n + kQCols) * (n | 1) : (size_t)0);
   LRFG_CUDA(raise_smem_limit((const void*)syevx_bisect_kernel, smem2));
   LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
               syevx_bisect_kernel<<<dim3((unsigned)(kv + nq), (unsigned)batch), kBisectThreads, smem2, ctx->stream>>>(
@@ -1375,7 +1398,7 @@ __global__ void __launch_bounds__(kCholThreads) gram_factor_kernel(const double*
 // after the owner of the pivot's column has published it, and the chain reduction - reciprocal - two multiply-adds; the
 // factor is kept as L D L^T until the end (no square root in the loop).  L11^-1 grows beside it by the same row
 // operations on the unit matrix, in the shadow of that chain, instead of forward substitutions after it.
-// One barrier and about 900 cycles a pivot against two and about 3500 in the kernel above.
+// One barrier a pivot against two, and a third of the time of the kernel above (b = 30: 105 -> 46 us).
 template <int NR, int CW>
 __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double* __restrict__ Gg,
                                                                            const double* __restrict__ cg, int b,
@@ -1411,7 +1434,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     perm[i] = i;
     pos[i] = b;
   }
-  double maxd0 = 0.0;
+  long long floor_bits = 0;
   int rho = b;
   for (int k = 0; k < b; ++k) {
     // the largest remaining diagonal (ties: the smallest row)
@@ -1427,8 +1450,9 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     const unsigned lo = hi == mh ? (unsigned)__double2loint(best) : 0u, ml = __reduce_max_sync(0xffffffff, lo);
     const int p = (int)__reduce_min_sync(0xffffffff, hi == mh && (unsigned)__double2loint(best) == ml ? (unsigned)bi : 1u << 30);
     const double piv = __hiloint2double(mh, (int)ml);
-    if (k == 0) maxd0 = piv > 0.0 ? piv : 0.0;
-    if (!(piv > tau * maxd0) || !(piv > 0.0)) {
+    // (positive doubles compare as integers: no FP64 comparison in the loop)
+    if (k == 0) floor_bits = piv > 0.0 ? __double_as_longlong(tau * piv) : 0;
+    if (mh < 0 || __double_as_longlong(piv) <= floor_bits || mh >= 0x7ff00000) {
       rho = k;
       break;
     }
@@ -1459,31 +1483,43 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
       if (is_p) rows_done |= 1u << r;
     }
     if (w == p % CW) cols_done |= 1u << pc;
+    // four columns' operands ahead of the arithmetic they feed
 #pragma unroll
-    for (int cc = 0; cc < NC; ++cc) {
-      const int col = cc * CW + w;
-      if (col < b && !(cols_done >> cc & 1u)) {
-        const double lc = col_p[col];
+    for (int c0 = 0; c0 < NC; c0 += 4) {
+      if (c0 * CW + w >= b || (~cols_done >> c0 & 15u) == 0) continue;
+      double lc[4];
 #pragma unroll
-        for (int r = 0; r < NR; ++r) a[r][cc] = fma(-t[r], lc, a[r][cc]);
-      }
+      for (int q = 0; q < 4; ++q) lc[q] = col_p[(c0 + q) * CW + w];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if ((c0 + q) * CW + w < b && !(cols_done >> (c0 + q) & 1u)) {
+#pragma unroll
+          for (int r = 0; r < NR; ++r) a[r][c0 + q] = fma(-t[r], lc[q], a[r][c0 + q]);
+        }
     }
     if (Pc) {
 #pragma unroll
-      for (int cc = 0; cc < NC; ++cc) {
-        const int q = cc * CW + w;
-        if (q <= k) {
-          double up = 0.0;
+      for (int c0 = 0; c0 < NC; c0 += 4) {
+        if (c0 * CW + w > k) continue;
+        double up[4];
 #pragma unroll
-          for (int r = 0; r < NR; ++r) {
+        for (int q = 0; q < 4; ++q) {
+          const int cc = c0 + q;
+          double v = u[0][cc];
+#pragma unroll
+          for (int r = 0; r < NR; ++r)
             if (r == pr) {
-              if (q == k && lane == pl) u[r][cc] = 1.0;
-              up = __shfl_sync(0xffffffff, u[r][cc], pl);
+              if (cc * CW + w == k && lane == pl) u[r][cc] = 1.0;
+              v = u[r][cc];
             }
-          }
-#pragma unroll
-          for (int r = 0; r < NR; ++r) u[r][cc] = fma(-t[r], up, u[r][cc]);
+          up[q] = __shfl_sync(0xffffffff, v, pl);
         }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if ((c0 + q) * CW + w <= k) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) u[r][c0 + q] = fma(-t[r], up[q], u[r][c0 + q]);
+          }
       }
     }
   }
