@@ -291,8 +291,13 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // spreads those products)
   auto fill = [&](long long blocks) { return (double)blocks / (double)(((blocks + nsm - 1) / nsm) * nsm); };
   const bool dyn = dynM || dynN;
-  int tile = (!dyn && (std::min(M, N) <= 32 || active_tiles(64) < nsm ||
-                       fill(active_tiles(32)) > fill(active_tiles(64)) + 0.05))
+  // (data-dependent sizes are judged by their static bounds: the tile's evenness costs little where they are far below)
+  auto tiles_of = [&](int tile) {
+    const long long tm = (M + tile - 1) / tile, tn = (N + tile - 1) / tile;
+    return (sym ? tm * (tm + 1) / 2 : tm * tn) * batch;
+  };
+  int tile = ((!dyn && (std::min(M, N) <= 32 || active_tiles(64) < nsm)) ||
+              fill(tiles_of(32)) > fill(tiles_of(64)) + 0.05)
                  ? 32
                  : 64;
   // 16 x 16 tiles when even the largest split of the 32-tiles leaves most SMs idle: one k-step of a 32-tile
@@ -300,17 +305,26 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // split further runs on a few SMs for that long; 16-tiles give four times the blocks at a quarter of the work
   if (tile == 32 && active_tiles(32) * std::max(1, K / GK) < nsm) tile = 16;
   const long long active = active_tiles(tile);
-  // split long K until about two blocks per SM are busy, without passing that (a second, partial round of
-  // blocks would cost as much as the first)
-  const int target = 2 * nsm;
-  int splits = 1;
-  if (active < target) {
-    splits = (int)std::min<long long>((target + active - 1) / active, std::max(1, K / GK));
-    if (active * splits > target) splits = (int)std::max<long long>(1, target / active);
+  // Split long K so that the busiest SM has the fewest k-steps: a block of c k-steps, active * ceil(steps / c) blocks, and
+  // a round of blocks costs c steps plus about one for its first loads and its partial sums.  Rounding a target of two
+  // blocks per SM to whole k-steps left 228 blocks of two steps on 152 SMs (four steps on the busiest one) where 152
+  // blocks of three do: the 60 x 60 x 14580 Gram product took 140 us.  At most four blocks per SM (the partials' sum).
+  const int steps = (K + GK - 1) / GK;
+  int per = steps;
+  if (active < 2LL * nsm) {
+    double best = 0.0;
+    for (int c = (int)std::max(1LL, std::min<long long>(steps, active * steps / (4LL * nsm))); c <= steps; ++c) {
+      const long long blocks = active * ((steps + c - 1) / c);
+      const double cost = (double)((blocks + nsm - 1) / nsm) * (c + 1.0);
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        per = c;
+      }
+      if (blocks <= nsm) break;  // longer blocks only add steps from here on
+    }
   }
-  int kchunk = (K + splits - 1) / splits;
-  kchunk = ((kchunk + GK - 1) / GK) * GK;
-  splits = (K + kchunk - 1) / kchunk;
+  const int kchunk = per * GK;
+  int splits = (steps + per - 1) / per;
   const int bmn = (M + tile - 1) / tile, bnn = (N + tile - 1) / tile;
   LRFG_REQUIRE((long long)bmn * splits < 65536, "gemm too many row blocks x splits");
   if (splits > 1)
