@@ -276,20 +276,21 @@ void stack_blocks(lrfg_ctx* ctx, const double* src, long long bs, int a, int n, 
 // right part have very different scales (e.g. after Khatri–Rao products and exponential sums).
 __global__ void balance_kernel(double* GAg, double* Rg, double* cg, int m) {
   extern __shared__ double cs[];
+  double* ci = cs + m;  // reciprocals: a division takes as long as five multiplications
   double* GA = GAg + (size_t)blockIdx.x * m * m;
   double* R = Rg + (size_t)blockIdx.x * m * m;
   double* c = cg + (size_t)blockIdx.x * m;
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     double ga = GA[(size_t)i * m + i], rb = R[(size_t)i * m + i];
     cs[i] = (ga > 0.0 && rb > 0.0) ? sqrt(sqrt(rb / ga)) : 1.0;
+    ci[i] = 1.0 / cs[i];
     c[i] = cs[i];
   }
   __syncthreads();
   for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
     int i = t / m, j = t - (t / m) * m;
-    double f = cs[i] * cs[j];
-    GA[t] *= f;
-    R[t] /= f;
+    GA[t] *= cs[i] * cs[j];
+    R[t] *= ci[i] * ci[j];
   }
 }
 
@@ -303,10 +304,15 @@ __global__ void diag_estimate_kernel(const double* __restrict__ C1g, const doubl
   const double* R2 = R2g + item * (size_t)b2 * b2;
   __shared__ double red[32];
   double s = 0.0;
-  for (int t = threadIdx.x; t < n * b2; t += blockDim.x) {
-    const int bp = t % b2;
-    const double v = C1[t];
-    s += v * v * R2[(size_t)bp * b2 + bp];
+  // a row of b2 entries per group of lanes: sum_b' (sum_i C1[i][b']^2) R2[b'][b'], one multiply-add per entry
+  const int rows = max(1, (int)blockDim.x / b2), r0 = threadIdx.x / b2;
+  for (int bp = threadIdx.x % b2; bp < b2 && r0 < rows; bp += (int)blockDim.x) {
+    double q0 = 0.0;
+    for (int i = r0; i < n; i += rows) {
+      const double v = C1[(size_t)i * b2 + bp];
+      q0 = fma(v, v, q0);
+    }
+    s = fma(q0, R2[(size_t)bp * b2 + bp], s);
   }
   for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffff, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -454,13 +460,13 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       const int n1 = x.N[1], b2 = x.r[2];
       DBuf<double> rd(ctx->pool, (size_t)b * nb);
       LRFG_LAUNCH(ctx, KC_TT_MISC, 3.0 * b * n1 * (double)b2 * nb, sizeof(double) * (double)x.elems(1) * nb,
-                  diag_estimate_kernel<<<dim3(b, nb), 256, 0, ctx->stream>>>(x.core[1], R[2].get(), b, n1, b2,
+                  diag_estimate_kernel<<<dim3(b, nb), 1024, 0, ctx->stream>>>(x.core[1], R[2].get(), b, n1, b2,
                                                                            rd.get()));
       LRFG_LAUNCH(ctx, KC_TT_MISC, 2.0 * sbb * nb, 2.0 * sizeof(double) * sbb * nb,
-                  balance_diag_kernel<<<nb, 256, sizeof(double) * b, ctx->stream>>>(GA.get(), rd.get(), cb.get(), b));
+                  balance_diag_kernel<<<nb, 1024, sizeof(double) * b, ctx->stream>>>(GA.get(), rd.get(), cb.get(), b));
     } else {
       LRFG_LAUNCH(ctx, KC_TT_MISC, 2.0 * sbb * nb, 4.0 * sizeof(double) * sbb * nb,
-                  balance_kernel<<<nb, 256, sizeof(double) * b, ctx->stream>>>(GA.get(), R[j + 1].get(), cb.get(), b));
+                  balance_kernel<<<nb, 1024, 2 * sizeof(double) * b, ctx->stream>>>(GA.get(), R[j + 1].get(), cb.get(), b));
     }
     // The unfolding X = M N (M: rows x b left part, N: b x cols right part) has the Gram matrices
     // GA = M^T M and R = N N^T.  Only the side whose numerical rank is smaller is factored (pivoted
