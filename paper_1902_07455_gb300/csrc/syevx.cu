@@ -353,7 +353,8 @@ __device__ double range_scale(int hi_abs, int* red) {
   int b = 0;
   for (int q = 0; q < (int)(blockDim.x >> 5); ++q) b = max(b, red[q]);
   const int ex = b >> 20;
-  if (ex == 0 || ex == 0x7ff) return 1.0;  // zero, denormal, or not finite
+  if (ex == 0) return 1.0;  // zero or denormal
+  if (ex == 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);  // not finite: so are all results (see K2, K3)
   return __hiloint2double(min(2046, max(1, 2046 - ex)) << 20, 0);
 }
 
@@ -827,7 +828,7 @@ __global__ void __launch_bounds__(kBisectThreads) syevx_bisect_kernel(int nl, in
     if (c0 < n) form_q_columns(g, n, c0, sm);
     return;
   }
-  if (t >= min(kv, n)) return;
+  if (t >= min(kv, n) || isnan(g.hdr[4])) return;
   const double lo = g.hdr[1], hi = g.hdr[2], emax2 = g.hdr[3];
   const double tnorm = fmax(fabs(lo), fabs(hi));
   if (tnorm == 0.0) {
@@ -918,6 +919,15 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_vec_kernel(int nl, int kl
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
   const int n = (int)g.hdr[0];
   if (n == 0) return;
+  if (isnan(g.hdr[4])) {
+    // an entry that is not finite: the vectors' fallbacks below would make finite ones of it
+    for (int t = threadIdx.x; t < min(kv, n); t += blockDim.x) wg[(size_t)blockIdx.x * nl + t] = g.hdr[4];
+    for (size_t q = threadIdx.x; q < (size_t)n * min(kl, n); q += blockDim.x) {
+      const size_t i = q / min(kl, n);
+      Vg[(size_t)blockIdx.x * (size_t)nl * ldv + i * ldv + (q - i * min(kl, n))] = g.hdr[4];
+    }
+    return;
+  }
   // flag 8: the tridiagonal, the reflector scalars and the eigenvalues in shared memory too
   double* d = sm;              // nl
   double* e = d + nl;          // nl
@@ -1436,6 +1446,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
   }
   long long floor_bits = 0;
   int rho = b;
+  bool is_nan = false;  // the same in every thread
   for (int k = 0; k < b; ++k) {
     // the largest remaining diagonal (ties: the smallest row)
     double best = dv[0];
@@ -1453,6 +1464,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     // (positive doubles compare as integers: no FP64 comparison in the loop)
     if (k == 0) floor_bits = piv > 0.0 ? __double_as_longlong(tau * piv) : 0;
     if (mh < 0 || __double_as_longlong(piv) <= floor_bits || mh >= 0x7ff00000) {
+      is_nan = mh >= 0x7ff00000 && isnan(piv);
       rho = k;
       break;
     }
@@ -1524,6 +1536,16 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     }
   }
   __syncthreads();
+  if (is_nan) {
+    // a NaN on the diagonal stays one in every result instead of a factor of rank 0
+    if (rhog && tid == 0) rhog[blockIdx.x] = b;
+    for (int t = tid; t < b * b; t += 32 * CW) {
+      RA[t] = __longlong_as_double(0x7ff8000000000000LL);
+      if (RAc) RAc[t] = RA[t];
+      if (Pc) Pc[t] = RA[t];
+    }
+    return;
+  }
   if (rhog && tid == 0) rhog[blockIdx.x] = rho;
   if (tid == 0) {
     // column q of L: (b - q - 1) rows of q multiply-adds; the triangular inverse (rho^3/6)
