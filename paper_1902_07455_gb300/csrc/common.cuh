@@ -124,9 +124,9 @@ struct FftChoice {
   int tf = 0, mper = 0;
 };
 
-// twiddle tables W[j] = exp(-2 pi i j / N), cached per N on the device
+// twiddle tables W[j] = exp(-2 pi i j / N), cached per N on the device: fixed point for FP64 data (fft_fixed.cuh), FP32
 struct Twiddles {
-  double2* W = nullptr;
+  int4* W = nullptr;
   float2* Wf = nullptr;  // the same table rounded to FP32 (made on first use)
   int N = 0;
 };

@@ -44,24 +44,19 @@ const Twiddles& twiddles_for(lrfg_ctx* ctx, int N) {
   LRFG_CUDA(ensure_roots(ctx->device));
   auto it = ctx->twiddles.find(N);
   if (it != ctx->twiddles.end()) return it->second;
-  std::vector<double2> h(N);
-  const double two_pi = 6.283185307179586476925286766559;
-  for (int j = 0; j < N; ++j) {
-    // reduce the angle to [0, pi/4]-friendly symmetric form for accuracy: exp(-2 pi i j/N)
-    double ang = two_pi * (double)j / (double)N;
-    h[j] = make_double2(std::cos(ang), -std::sin(ang));
-  }
+  std::vector<int4> h(N);
+  for (int j = 0; j < N; ++j) h[j] = fixed_root(j, N);
   Twiddles t;
   t.N = N;
-  LRFG_CUDA(cudaMalloc(&t.W, sizeof(double2) * N));
+  LRFG_CUDA(cudaMalloc(&t.W, sizeof(int4) * N));
   // on the context's stream (ordered before its kernels, also when that stream is non-blocking)
-  LRFG_CUDA(cudaMemcpyAsync(t.W, h.data(), sizeof(double2) * N, cudaMemcpyHostToDevice, ctx->stream));
+  LRFG_CUDA(cudaMemcpyAsync(t.W, h.data(), sizeof(int4) * N, cudaMemcpyHostToDevice, ctx->stream));
   LRFG_CUDA(cudaStreamSynchronize(ctx->stream));
   return ctx->twiddles.emplace(N, t).first->second;
 }
 
 template <>
-const double2* twiddle_table<double>(lrfg_ctx* ctx, int N) {
+const int4* twiddle_table<double>(lrfg_ctx* ctx, int N) {
   return twiddles_for(ctx, N).W;
 }
 
@@ -151,13 +146,13 @@ __device__ __forceinline__ int same_freq(int n, int N, int m) {
 // others are zero, or the output keeps nout <= N of them (the double grid of the exact integration)
 template <int SIGN, typename V, int OP, bool PAD>
 __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out, long long outer, int N, long long inner,
-                                                         int TF, FftPlan pl, const V* __restrict__ Wg,
+                                                         int TF, FftPlan pl, const typename TwOf<V>::T* __restrict__ Wg,
                                                          FibreMul<typename RealOf<V>::T> fm, int nin,
                                                          int nout) {
   using R = typename RealOf<V>::T;
   extern __shared__ __align__(16) unsigned char smraw_fib[];
   V* sm = (V*)smraw_fib;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* a = sm + 2 * N;
   V* b = a + (size_t)TF * N;
   const long long nfib = outer * inner;
@@ -215,7 +210,7 @@ __global__ void __launch_bounds__(256, 3) fft_fibres_kernel(const V* in, V* out,
     }
   }
   __syncthreads();
-  V* res = stockham_rows<SIGN>(a, b, nf, N, pl, (const V*)W);
+  V* res = stockham_rows<SIGN>(a, b, nf, N, pl, W);
   if (across) {
     const int step = blockDim.x / nf;
     const int f = threadIdx.x % nf, n0 = threadIdx.x / nf;
@@ -395,30 +390,29 @@ static bool fft2_try(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N,
   }
 }
 
-// FP64 operations of a radix-p butterfly with its twiddles
+// instructions of a radix-p butterfly in fixed point with its twiddles
 static double butterfly_ops(int p) {
   switch (p) {
-    case 3: return 20.0;
-    case 5: return 52.0;
-    case 7: return 90.0;
-    case 9: return 120.0;
-    default: return (double)(p - 1) * (p - 1) + 14.0 * p;
+    case 3: return 150.0;
+    case 5: return 400.0;
+    case 7: return 750.0;
+    case 9: return 800.0;
+    default: return 20.0 * (double)(p - 1) * (p - 1) + 60.0 * p;
   }
 }
 
-// Cycles of one transform of tf rows in each of `blocks` blocks on the SM with the most of them.  An SM has four FP64
-// units, a warp issues one FP64 instruction per 64 cycles on its unit (about 70 when all four are busy) however many of
-// its lanes work, so a pass takes the instructions of the warps on one unit, plus a barrier and a trip through shared
-// memory.
+// Cycles of one transform of tf rows in each of `blocks` blocks on the SM with the most of them: a pass takes the
+// instructions of the warps on the busiest of the SM's four schedulers, or those of one warp at its latency where there
+// are few, and a barrier; the conversions count as another pass.
 double fft_cycles(lrfg_ctx* ctx, const FftPlan& pl, long long tf, long long blocks) {
   const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
   const long long per_sm = (blocks + nsm - 1) / nsm;
-  double c = 0.0;
-  for (int s = 0; s < pl.nst; ++s) {
-    const int p = pl.radix[s];
-    const long long warps = per_sm * ((tf * (pl.N / p) + 31) / 32);
-    c += (double)((warps + 3) / 4) * butterfly_ops(p) * 70.0 + 400.0;
-  }
+  auto pass = [&](long long threads, double ops) {
+    const long long warps = per_sm * ((threads + 31) / 32);
+    return std::max((double)((warps + 3) / 4) * ops * 1.5, (double)(((threads + 255) / 256)) * ops * 3.0) + 200.0;
+  };
+  double c = pass(tf * pl.N, 120.0);
+  for (int s = 0; s < pl.nst; ++s) c += pass(tf * (pl.N / pl.radix[s]), butterfly_ops(pl.radix[s]));
   return c;
 }
 
@@ -429,12 +423,11 @@ static FftChoice& fft_choice(lrfg_ctx* ctx, int N, int kind, long long nrows, in
   return m[std::make_tuple(N, kind, nrows, extra)];
 }
 
-// Plan and tile for nrows FP64 rows, at most tf_max rows a tile: the cheapest by fft_cycles over the tiles and over
-// radix-9 passes or radix-3 ones (a few percent more operations in pieces a sixth as long: the shorter chain where a
-// launch has fewer butterflies than units), the larger tile on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid
-// in 32-row tiles ran on one or two SMs: 46 us per fibre pass and 88 us per fused row pass under event timing; 63^3 with
-// its Ga double grid 125^3 gained 19% from even tiles.  From six full tiles per SM on the rounding up costs less than the
-// shorter memory segments of a smaller tile, and tf_max stays.
+// Plan and tile for nrows rows, at most tf_max rows a tile: the cheapest by fft_cycles over the tiles and, for FP64 rows,
+// over radix-9 passes or radix-3 ones (more instructions in shorter chains, for launches with few butterflies), the
+// larger tile on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid in 32-row tiles ran on one or two SMs: 46 us
+// per fibre pass and 88 us per fused row pass under event timing (9 and 17 us with even tiles and fixed point).  From six
+// full tiles per SM on the rounding up costs less than the shorter memory segments of a smaller tile, and tf_max stays.
 FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf) {
   const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
   FftPlan best = make_plan(N, fp64 ? plan_radix<double2>() : plan_radix<float2>());
@@ -484,7 +477,7 @@ void fft_fibres(lrfg_ctx* ctx, const V* in, V* out, long long outer, int N, long
   LRFG_REQUIRE(N >= 1 && (N % 2 == 1), "fft length must be odd (got %d)", N);
   LRFG_REQUIRE(outer >= 0 && inner >= 0, "negative batch");
   if (outer == 0 || inner == 0) return;
-  const V* W = twiddle_table<R>(ctx, N);
+  const auto* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
   long long nfib = outer * inner;
@@ -528,7 +521,7 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename 
   LRFG_REQUIRE(fm.mode == 1 || in != out, "the accumulator cannot hold the input");
   LRFG_REQUIRE(!(fm.mode == 2 && fm.precond) || fm.inv_kk, "reciprocal table missing");
   if (inner == 0) return;
-  const V* W = twiddle_table<R>(ctx, N);
+  const auto* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
   const FftPlan pl = tile_complex(ctx, N, sizeof(V), outer * inner, &TF, &smem);
@@ -577,7 +570,7 @@ void fft_fibres_pad(lrfg_ctx* ctx, const double2* in, double2* out, long long ou
                     int sign) {
   LRFG_REQUIRE(L > n && L % 2 == 1 && n % 2 == 1 && in != out, "padded transform %d -> %d", n, L);
   if (outer == 0 || inner == 0) return;
-  const double2* W = twiddle_table<double>(ctx, L);
+  const auto* W = twiddle_table<double>(ctx, L);
   size_t smem;
   int TF;
   const FftPlan pl = tile_complex(ctx, L, sizeof(double2), outer * inner, &TF, &smem);
@@ -616,12 +609,12 @@ __device__ __forceinline__ double2 multiplier(int kind, int k, double param) {
 template <typename V>
 __global__ void __launch_bounds__(256) fibre_op_kernel(const double* in, double* out, long long outer,
                                                        int N, long long inner, int TF, FftPlan pl,
-                                                       const V* __restrict__ Wg, int kind, double param,
+                                                       const typename TwOf<V>::T* __restrict__ Wg, int kind, double param,
                                                        double scale) {
   using R = typename RealOf<V>::T;
   extern __shared__ __align__(16) unsigned char smraw_op[];
   V* sm = (V*)smraw_op;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* M = sm + N;
   V* a = sm + 2 * N;
   V* b = a + (size_t)TF * N;
@@ -670,7 +663,7 @@ __global__ void __launch_bounds__(256) fibre_op_kernel(const double* in, double*
 template <typename V>
 static void fibre_operator_t(lrfg_ctx* ctx, const double* in, double* out, long long outer, int N, long long inner,
                              int kind, double param, double scale) {
-  const V* W = twiddle_table<typename RealOf<V>::T>(ctx, N);
+  const auto* W = twiddle_table<typename RealOf<V>::T>(ctx, N);
   const long long nfib = outer * inner;
   int TF;  // a row carries two real fibres
   const FftPlan pl = choose_plan(ctx, N, sizeof(V) == sizeof(double2), (nfib + 1) / 2, tile_fibres(ctx, N, sizeof(V), 1, 2),
@@ -710,13 +703,13 @@ template <typename V>
 __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __restrict__ in, double* out,
                                                                 long long out_stride, long long outer, int N,
                                                                 long long inner, int TF, FftPlan pl,
-                                                                const V* __restrict__ Wg,
+                                                                const typename TwOf<V>::T* __restrict__ Wg,
                                                                 const __grid_constant__ GaussTerms terms, int nm,
                                                                 int mper) {
   using R = typename RealOf<V>::T;
   extern __shared__ __align__(16) unsigned char smraw_gm[];
   V* sm = (V*)smraw_gm;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* spec = sm + N;              // TF rows: the shared forward spectrum
   V* a = spec + (size_t)TF * N;  // TF rows
   V* b = a + (size_t)TF * N;     // TF rows
@@ -776,7 +769,7 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
 template <typename V>
 static void fibre_gauss_multi_t(lrfg_ctx* ctx, const double* in, double* out, long long out_stride, long long outer,
                                 int N, long long inner, const double* t, const double* scale, int nm) {
-  const V* Wt = twiddle_table<typename RealOf<V>::T>(ctx, N);
+  const auto* Wt = twiddle_table<typename RealOf<V>::T>(ctx, N);
   // few fibres (low-rank carriages): small tiles, and the terms split over grid.y (each block redoes the shared forward
   // transform of its tile), so that the launch covers the SMs: the cheapest of the splits by the inverse transforms a
   // block runs plus its forward one

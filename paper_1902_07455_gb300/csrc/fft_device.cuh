@@ -1,4 +1,5 @@
-// Batched odd-length complex FFTs of fibres staged in shared memory (FP64 double2 or FP32 float2).
+// Batched odd-length complex FFTs of fibres staged in shared memory (FP64 double2 data in fixed point, see fft_fixed.cuh,
+// or FP32 float2).
 //
 // Mixed-radix Stockham autosort, decimation in time.  After the stages with radices p_0..p_{s-1}
 // (L = p_0...p_{s-1}), row entry c*L + f holds the length-L DFT (frequency f) of the subsequence
@@ -16,6 +17,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -27,8 +29,17 @@ constexpr int kMaxGenericRadix = 31;
 
 // roots of unity exp(-2 pi i j / p) of the register radices, concatenated (filled once per device)
 constexpr int kRootOff3 = 0, kRootOff5 = 3, kRootOff7 = 8, kRootOff9 = 15, kRootOff27 = 24, kRootCount = 51;
-__constant__ double2 c_roots_d[kRootCount];
 __constant__ float2 c_roots_f[kRootCount];
+__constant__ int4 c_roots_x[kRootCount];  // fixed point (fft_fixed.cuh)
+
+// exp(-2 pi i j / p) in fixed point: upper and lower parts of cos 2^62 and -sin 2^62 (1 as 1 - 2^-62)
+static inline int4 fixed_root(int j, int p) {
+  const long double ang = 6.283185307179586476925286766559005768L * (long double)j / (long double)p;
+  const long long one = (1LL << 62) - 1;
+  const long long x = std::min(one, (long long)llroundl(cosl(ang) * 0x1p62L));
+  const long long y = std::min(one, (long long)llroundl(-sinl(ang) * 0x1p62L));
+  return make_int4((int)(x >> 31), (int)(x & 0x7fffffff), (int)(y >> 31), (int)(y & 0x7fffffff));
+}
 
 // Fills this translation unit's root tables on the current device (once per device); returns the CUDA
 // status of the copies.
@@ -37,18 +48,18 @@ static inline cudaError_t ensure_roots(int device) {
   static unsigned long long done = 0;  // one bit per device
   std::lock_guard<std::mutex> lock(mu);
   if (device >= 0 && device < 64 && (done >> device & 1ULL)) return cudaSuccess;
-  double2 hd[kRootCount];
   float2 hf[kRootCount];
+  int4 hx[kRootCount];
   const int radix[5] = {3, 5, 7, 9, 27}, off[5] = {kRootOff3, kRootOff5, kRootOff7, kRootOff9, kRootOff27};
   const double two_pi = 6.283185307179586476925286766559;
   for (int q = 0; q < 5; ++q)
     for (int j = 0; j < radix[q]; ++j) {
       const double ang = two_pi * (double)j / (double)radix[q];
-      hd[off[q] + j] = make_double2(std::cos(ang), -std::sin(ang));
       hf[off[q] + j] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
+      hx[off[q] + j] = fixed_root(j, radix[q]);
     }
-  cudaError_t e = cudaMemcpyToSymbol(c_roots_d, hd, sizeof(hd));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_roots_f, hf, sizeof(hf));
+  cudaError_t e = cudaMemcpyToSymbol(c_roots_f, hf, sizeof(hf));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_roots_x, hx, sizeof(hx));
   // complete before kernels on any stream (non-blocking ones included) read the tables
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e == cudaSuccess && device >= 0 && device < 64) done |= 1ULL << device;
@@ -62,6 +73,9 @@ template <> struct CplxOf<float> { using T = float2; };
 template <typename V> struct RealOf;
 template <> struct RealOf<double2> { using T = double; };
 template <> struct RealOf<float2> { using T = float; };
+// entries of a twiddle table: fixed point for FP64 data
+template <typename V> struct TwOf { using T = V; };
+template <> struct TwOf<double2> { using T = int4; };
 
 template <typename V>
 __device__ __forceinline__ V mkc(typename RealOf<V>::T x, typename RealOf<V>::T y) {
@@ -144,16 +158,8 @@ template <> struct RootOff<27> { static constexpr int v = kRootOff27; };
 // w_P^j (forward: exp(-2 pi i j / P), inverse: its conjugate); j a compile-time constant after unrolling
 template <int P, int SIGN, typename V>
 __device__ __forceinline__ V root(int j) {
-  V w;
-  if constexpr (sizeof(V) == sizeof(double2)) {
-    const double2 t = c_roots_d[RootOff<P>::v + j % P];
-    w.x = t.x;
-    w.y = t.y;
-  } else {
-    const float2 t = c_roots_f[RootOff<P>::v + j % P];
-    w.x = t.x;
-    w.y = t.y;
-  }
+  static_assert(sizeof(V) == sizeof(float2), "FP32");
+  V w = c_roots_f[RootOff<P>::v + j % P];
   if (SIGN > 0) w.y = -w.y;
   return w;
 }
@@ -161,7 +167,7 @@ __device__ __forceinline__ V root(int j) {
 template <int P, int SIGN, typename V>
 struct RegDFT;
 
-// Multiplications are written as multiply-adds with the additions that follow them (12 FP64 operations at p = 3).
+// Multiplications are written as multiply-adds with the additions that follow them (12 operations at p = 3).
 template <int SIGN, typename V>
 struct RegDFT<3, SIGN, V> {
   static __device__ __forceinline__ void run(V* x) {
@@ -198,7 +204,7 @@ struct RegDFT<5, SIGN, V> {
 // Prime radix by the symmetric halves of the inputs, s_r = x_r + x_{p-r} and d_r = x_r - x_{p-r}:
 //   X_q, X_{p-q} = x_0 + sum_r cos(2 pi q r / p) s_r  +-  i SIGN sum_r sin(2 pi q r / p) d_r,  r, q = 1..(p-1)/2,
 // real coefficients only: 36 multiply-adds and 24 additions at p = 7, against 36 complex products and as many complex
-// additions (216 operations) of the direct sum: fibre passes of 105 x 147 x 75 went from 99 to 49 us on average.
+// additions (216 operations) of the direct sum.
 template <int SIGN, typename V>
 struct RegDFT<7, SIGN, V> {
   static __device__ __forceinline__ void run(V* x) {
@@ -269,6 +275,12 @@ __device__ __forceinline__ int small_div(int x, int d, float inv) {
   return q;
 }
 
+}  // namespace lrfg
+
+#include "fft_fixed.cuh"
+
+namespace lrfg {
+
 // One Stockham pass of register radix P over nf rows (row stride ld) from a into b.
 template <int P, int SIGN, typename V>
 __device__ __forceinline__ void stockham_pass(const V* __restrict__ a, V* __restrict__ b, int nf, int ld, int N,
@@ -299,8 +311,12 @@ __device__ __forceinline__ void stockham_pass(const V* __restrict__ a, V* __rest
 
 // Transform `nf` rows of length pl.N (row stride ld) held in `a`, using `b` as scratch.  All threads
 // of the block take part; returns the buffer that holds the result (a or b).  Ends with a barrier.
+// (FP64 data: fft_fixed.cuh)
 template <int SIGN, typename V>
-__device__ V* stockham_rows(V* a, V* b, int nf, int ld, const FftPlan& pl, const V* W) {
+__device__ V* stockham_rows(V* a, V* b, int nf, int ld, const FftPlan& pl, const typename TwOf<V>::T* W) {
+  if constexpr (sizeof(V) == sizeof(double2)) {
+    return fix_rows<SIGN>(a, b, nf, ld, pl, W);
+  } else {
   const int N = pl.N;
   int L = 1;
   for (int s = 0; s < pl.nst; ++s) {
@@ -310,13 +326,7 @@ __device__ V* stockham_rows(V* a, V* b, int nf, int ld, const FftPlan& pl, const
       case 5: stockham_pass<5, SIGN>(a, b, nf, ld, N, L, W); break;
       case 7: stockham_pass<7, SIGN>(a, b, nf, ld, N, L, W); break;
       case 9: stockham_pass<9, SIGN>(a, b, nf, ld, N, L, W); break;
-      case 27:
-        // FP32 only (plan_radix): 27 FP64 complex values would cost too many registers
-        if constexpr (sizeof(V) == sizeof(float2)) {
-          stockham_pass<27, SIGN>(a, b, nf, ld, N, L, W);
-          break;
-        }
-        [[fallthrough]];
+      case 27: stockham_pass<27, SIGN>(a, b, nf, ld, N, L, W); break;
       default: {
         const int mp = N / (L * p);
         const int nb = N / p;
@@ -338,6 +348,7 @@ __device__ V* stockham_rows(V* a, V* b, int nf, int ld, const FftPlan& pl, const
     L *= p;
   }
   return a;
+  }
 }
 
 // Asynchronous global -> shared copies (cp.async, no register staging), so that a block keeps all of its

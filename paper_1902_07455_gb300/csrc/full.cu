@@ -37,12 +37,12 @@ template <typename R>
 __global__ void __launch_bounds__(256, 3) r2c_rows_kernel(const R* __restrict__ in, const R* __restrict__ coef, R scale,
                                                        typename CplxOf<R>::T* __restrict__ out, long long rows, int N,
                                                        int H, int TF, FftPlan pl,
-                                                       const typename CplxOf<R>::T* __restrict__ Wg) {
+                                                       const typename TwOf<typename CplxOf<R>::T>::T* __restrict__ Wg) {
   using V = typename CplxOf<R>::T;
   const float invN = 1.0f / (float)N, invH = 1.0f / (float)H;
   extern __shared__ __align__(16) unsigned char smraw_r2c[];
   V* sm = (V*)smraw_r2c;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* a = sm + 2 * N;
   V* b = a + (size_t)TF * N;
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256, 3) r2c_rows_kernel(const R* __restrict__ 
     }
   }
   __syncthreads();
-  V* Z = stockham_rows<-1>(a, b, nrow, N, pl, (const V*)W);
+  V* Z = stockham_rows<-1>(a, b, nrow, N, pl, W);
   // split: X[k] = (Z[k] + conj Z[N-k]) / 2,  Y[k] = (Z[k] - conj Z[N-k]) / (2i)
   for (int t = threadIdx.x; t < nr * H; t += blockDim.x) {
     const int f = small_div(t, H, invH), k = t - f * H;
@@ -96,12 +96,12 @@ template <typename R>
 __global__ void __launch_bounds__(256, 3) c2r_rows_kernel(const typename CplxOf<R>::T* __restrict__ in,
                                                        const R* __restrict__ coef, R scale, R* __restrict__ out,
                                                        long long rows, int N, int H, int TF, FftPlan pl,
-                                                       const typename CplxOf<R>::T* __restrict__ Wg) {
+                                                       const typename TwOf<typename CplxOf<R>::T>::T* __restrict__ Wg) {
   using V = typename CplxOf<R>::T;
   const float invN = 1.0f / (float)N;
   extern __shared__ __align__(16) unsigned char smraw_c2r[];
   V* sm = (V*)smraw_c2r;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* a = sm + 2 * N;
   V* b = a + (size_t)TF * N;
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(256, 3) c2r_rows_kernel(const typename CplxOf<
     }
   }
   __syncthreads();
-  V* Z = stockham_rows<1>(a, b, nrow, N, pl, (const V*)W);
+  V* Z = stockham_rows<1>(a, b, nrow, N, pl, W);
   for (int t = threadIdx.x; t < nr * N; t += blockDim.x) {
     const int f = small_div(t, N, invN), n = t - f * N;
     int row = f < TF ? f : f - TF;
@@ -165,12 +165,12 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
                                                                const R* __restrict__ coef, R scale,
                                                                typename CplxOf<R>::T* out, long long rows, int N,
                                                                int H, int TF, FftPlan pl,
-                                                               const typename CplxOf<R>::T* __restrict__ Wg) {
+                                                               const typename TwOf<typename CplxOf<R>::T>::T* __restrict__ Wg) {
   using V = typename CplxOf<R>::T;
   const float invN = 1.0f / (float)N, invH = 1.0f / (float)H;
   extern __shared__ __align__(16) unsigned char smraw_fused[];
   V* sm = (V*)smraw_fused;
-  V* W = sm;
+  auto* W = reinterpret_cast<typename TwOf<V>::T*>(sm);
   V* a = sm + 2 * N;
   V* b = a + (size_t)TF * N;
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
     }
   }
   __syncthreads();
-  V* Z = stockham_rows<1>(a, b, nrow, N, pl, (const V*)W);
+  V* Z = stockham_rows<1>(a, b, nrow, N, pl, W);
   // the product with the coefficient on both real rows of each complex row, in place
   {
     constexpr int kU = 4;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
     }
   }
   __syncthreads();
-  V* Z2 = stockham_rows<-1>(Z, Z == a ? b : a, nrow, N, pl, (const V*)W);
+  V* Z2 = stockham_rows<-1>(Z, Z == a ? b : a, nrow, N, pl, W);
   // split: X[k] = (Z[k] + conj Z[N-k]) / 2,  Y[k] = (Z[k] - conj Z[N-k]) / (2i)
   for (int t = threadIdx.x; t < nr * H; t += blockDim.x) {
     const int f = small_div(t, H, invH), k = t - f * H;
@@ -402,7 +402,7 @@ void full_forward(lrfg_ctx* ctx, const FullGrid& g, const R* real_in, const R* c
   using V = typename CplxOf<R>::T;
   const int N = g.N[g.d - 1];
   LRFG_CUDA(ensure_roots(ctx->device));
-  const V* W = twiddle_table<R>(ctx, N);
+  const auto* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
   const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
@@ -434,7 +434,7 @@ void full_inverse(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half_
   }
   const int N = g.N[g.d - 1];
   LRFG_CUDA(ensure_roots(ctx->device));
-  const V* W = twiddle_table<R>(ctx, N);
+  const auto* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
   const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
@@ -470,7 +470,7 @@ void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half
     if (N == 81) return rows2_launch<9, 9>(ctx, g, half_inout, coef, scale);
   }
   LRFG_CUDA(ensure_roots(ctx->device));
-  const V* W = twiddle_table<R>(ctx, N);
+  const auto* W = twiddle_table<R>(ctx, N);
   size_t smem;
   int TF;
   const FftPlan pl = row_tile<R>(ctx, N, g.rows, &TF, &smem);
@@ -484,7 +484,7 @@ void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half
 
 void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef) {
   LRFG_CUDA(ensure_roots(ctx->device));
-  const double2* W = twiddle_table<double>(ctx, N);
+  const auto* W = twiddle_table<double>(ctx, N);
   size_t smem;
   int TF;
   const FftPlan pl = row_tile<double>(ctx, N, rows, &TF, &smem);

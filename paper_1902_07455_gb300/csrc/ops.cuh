@@ -7,14 +7,14 @@
 namespace lrfg {
 
 // ---- fft.cu -------------------------------------------------------------------------------------
-// passes for length N with register radices up to max_radix (27 for FP32 data, 9 for FP64, whose
-// larger register footprint would limit occupancy)
+// passes for length N with register radices up to max_radix (27 for FP32 data, 9 for the fixed-point transforms of FP64
+// data, whose larger register footprint would limit occupancy)
 FftPlan make_plan(int N, int max_radix);
 template <typename V>
 constexpr int plan_radix() { return sizeof(V) == sizeof(float2) ? 27 : 9; }
-// device twiddle table W[j] = exp(-2 pi i j / N) in FP64 (double) or rounded to FP32 (float)
+// device twiddle table W[j] = exp(-2 pi i j / N) in fixed point (for FP64 data) or rounded to FP32 (float)
 template <typename R>
-const typename CplxOf<R>::T* twiddle_table(lrfg_ctx* ctx, int N);
+const typename TwOf<typename CplxOf<R>::T>::T* twiddle_table(lrfg_ctx* ctx, int N);
 // plan and rows of a tile (at most tf_max) for nrows rows
 FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf);
 // batched complex DFT along the middle axis of (outer, N, inner); sign -1 forward, +1 inverse
