@@ -31,11 +31,24 @@ constexpr int kFixMaxRows = 64;  // rows of a tile at most
 // 2^31 with the product of the lower parts, a quarter of a unit on average, left out; `mid` starts with its mean and the
 // half that rounds its shift.
 constexpr unsigned kFixHalf = 1u << 30, kFixLow = 1u << 29;
-__host__ __device__ __forceinline__ int fix_hi(long long a) { return (int)(a >> 31); }
-__host__ __device__ __forceinline__ int fix_lo(long long a) { return (int)(a & 0x7fffffffLL); }
+__device__ __forceinline__ int fix_hi(long long a) {
+  return (int)__funnelshift_r((unsigned)a, (unsigned)((unsigned long long)a >> 32), 31);
+}
+__device__ __forceinline__ int fix_lo(long long a) { return (int)((unsigned)a & 0x7fffffffu); }
+// a b + c as one instruction (the compiler takes (long long)a * b for a 64 x 64 product where a comes from a shift: three)
+__device__ __forceinline__ long long fix_mad(int a, int b, long long c) {
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ long long fix_mul(int a, int b) {
+  long long d;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(d) : "r"(a), "r"(b));
+  return d;
+}
 
-__host__ __device__ __forceinline__ Fix2 operator+(Fix2 a, Fix2 b) { return {a.x + b.x, a.y + b.y}; }
-__host__ __device__ __forceinline__ Fix2 operator-(Fix2 a, Fix2 b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ Fix2 operator+(Fix2 a, Fix2 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ Fix2 operator-(Fix2 a, Fix2 b) { return {a.x - b.x, a.y - b.y}; }
 
 // w = (x upper, x lower, y upper, y lower) of exp(-2 pi i j / N); SIGN > 0 multiplies by its conjugate.  The moduli of a and w
 // bound the sums of `mid`: sqrt 2 2^62 + 1.05 2^61 < 2^63.
@@ -44,21 +57,16 @@ __device__ __forceinline__ Fix2 fix_cmul(Fix2 a, int4 w) {
   const int ah = fix_hi(a.x), al = fix_lo(a.x), bh = fix_hi(a.y), bl = fix_lo(a.y);
   // re = a w_x - b w_y, im = b w_x + a w_y, or with the conjugate re = a w_x + b w_y, im = b w_x - a w_y
   constexpr long long cr = kFixHalf + (SIGN < 0 ? 0 : 2 * kFixLow), ci = kFixHalf + (SIGN < 0 ? 2 * kFixLow : 0);
-  const long long rr = (long long)ah * w.x, ii = (long long)bh * w.z;
-  const long long ri = (long long)ah * w.z, ir = (long long)bh * w.x;
-  const long long mrr = (long long)al * w.x + ((long long)ah * w.y + cr), mii = (long long)bl * w.z + (long long)bh * w.w;
-  const long long mri = (long long)al * w.z + (long long)ah * w.w, mir = (long long)bl * w.x + ((long long)bh * w.y + ci);
-  if (SIGN < 0) return {(rr - ii) + ((mrr - mii) >> 31), (ir + ri) + ((mir + mri) >> 31)};
-  return {(rr + ii) + ((mrr + mii) >> 31), (ir - ri) + ((mir - mri) >> 31)};
+  const int ch = SIGN < 0 ? -bh : bh, cl = SIGN < 0 ? -bl : bl, dh = SIGN < 0 ? ah : -ah, dl = SIGN < 0 ? al : -al;
+  const long long mr = fix_mad(cl, w.z, fix_mad(ch, w.w, fix_mad(al, w.x, fix_mad(ah, w.y, cr))));
+  const long long mi = fix_mad(dl, w.z, fix_mad(dh, w.w, fix_mad(bl, w.x, fix_mad(bh, w.y, ci))));
+  return {fix_mad(ch, w.z, fix_mad(ah, w.x, mr >> 31)), fix_mad(dh, w.z, fix_mad(bh, w.x, mi >> 31))};
 }
 
 // one component times a real factor (h, l)
 __device__ __forceinline__ long long fix_rmul(long long a, int h, int l) {
-  const int ah = fix_hi(a), al = fix_lo(a);
-  long long m = kFixHalf + kFixLow;
-  m += (long long)ah * l;
-  m += (long long)al * h;
-  return (m >> 31) + (long long)ah * h;
+  const int ah = fix_hi(a);
+  return fix_mad(ah, h, fix_mad(fix_lo(a), h, fix_mad(ah, l, kFixHalf + kFixLow)) >> 31);
 }
 
 // a / 2^s rounded to nearest, 0 <= s < 32, half = 2^s / 2
@@ -70,7 +78,7 @@ __device__ __forceinline__ long long fix_shift(long long a, int s, unsigned half
 
 // ---- conversions ------------------------------------------------------------------------------------------------
 // bits of a double to fixed point in a row's scale c: times 2^(1101 - c), rounded to nearest
-__host__ __device__ __forceinline__ long long fix_from_bits(unsigned long long u, int c) {
+__device__ __forceinline__ long long fix_from_bits(unsigned long long u, int c) {
   const int e = (int)((unsigned)(u >> 52) & 0x7ffu);
   unsigned long long m = u & 0xfffffffffffffULL;
   m |= (unsigned long long)(e ? 1u : 0u) << 52;
