@@ -796,6 +796,14 @@ void full_apply(lrfg_problem* P, const typename CplxOf<R>::T* v, typename CplxOf
     if (P->aniso) half_acc_aniso(ctx, g, v, out, P->B, precond);
     return;
   }
+  if constexpr (std::is_same<R, double>::value) {
+    if (g.d == 2 && fft_pair_2d_fits(ctx, g.N[0]) && ctx->pool->room(1, 2 * sizeof(V) * g.n_half)) {
+      DBuf<V> w1(ctx->pool, 2 * g.n_half);
+      full_operator_2d(ctx, g, v, out, w.a, inv, precond && !P->aniso, w1.get());
+      if (P->aniso) half_acc_aniso(ctx, g, v, out, P->B, precond);
+      return;
+    }
+  }
   for (int alpha = 0; alpha < g.d; ++alpha) {
     // grad^ (with 1/|N| of Phi^-1) and F^-1 on the complex axes, then on the rows fused with A~ and F there,
     // then F on the complex axes and grad^* (P~^-1 after the last component)

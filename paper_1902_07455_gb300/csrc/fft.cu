@@ -563,6 +563,81 @@ void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename 
   }
 }
 
+// The axis-0 passes of both components of a d = 2 half spectrum (N, H), FP64 (OP as in fft_fibres_kernel): rows f and nf + f
+// of a tile of nf fibres are the components 0 and 1 of fibre f.
+template <int OP>
+__global__ void __launch_bounds__(256, 3) fft_pair_2d_kernel(const double2* in, double2* out, int N, int H, int F, FftPlan pl,
+                                                             const int4* __restrict__ Wg, FibreMul<double> fm) {
+  extern __shared__ __align__(16) unsigned char smraw_2d[];
+  double2* sm = (double2*)smraw_2d;
+  int4* W = reinterpret_cast<int4*>(sm);
+  double2* a = sm + N;
+  double2* b = a + (size_t)2 * F * N;
+  const int i0 = blockIdx.x * F, nf = min(F, H - i0);
+  const size_t half = (size_t)N * H;
+  for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
+  // neighbouring threads take neighbouring fibres
+  const float inv_nf = 1.0f / (float)nf;
+  for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
+    const int n = small_div(t, nf, inv_nf), f = t - n * nf;
+    const double2* src = in + (size_t)n * H + i0 + f;
+    double2* p = a + (size_t)f * N + n;
+    if constexpr (OP == 1) {
+      const double2 v = *src;
+      p[0] = times_2pi_ik<double2>(v, fm.c2 * (double)freq_of(n, N));
+      p[(size_t)nf * N] = times_2pi_ik<double2>(v, fm.c2 * (double)(i0 + f));
+    } else {
+      p[0] = src[0];
+      p[(size_t)nf * N] = src[half];
+    }
+  }
+  __syncthreads();
+  const double2* res = stockham_rows<OP == 1 ? 1 : -1>(a, b, 2 * nf, N, pl, W);
+  for (int t = threadIdx.x; t < nf * N; t += blockDim.x) {
+    const int n = small_div(t, nf, inv_nf), f = t - n * nf;
+    double2* dst = out + (size_t)n * H + i0 + f;
+    const double2 x0 = res[(size_t)f * N + n], x1 = res[(size_t)(nf + f) * N + n];
+    if constexpr (OP == 1) {
+      dst[0] = x0;
+      dst[half] = x1;
+    } else {
+      const int k0 = freq_of(n, N), k1 = i0 + f;
+      const double2 r0 = times_2pi_ik<double2>(x0, -fm.c2 * (double)k0), r1 = times_2pi_ik<double2>(x1, -fm.c2 * (double)k1);
+      double2 r = make_double2(r0.x + r1.x, r0.y + r1.y);
+      if (fm.precond) {
+        const double s = fm.inv_kk[k0 * k0 + k1 * k1];
+        r.x *= s;
+        r.y *= s;
+      }
+      *dst = r;
+    }
+  }
+}
+
+bool fft_pair_2d_fits(lrfg_ctx* ctx, int N) {
+  return sizeof(double2) * 5 * (size_t)N <= (size_t)std::min(ctx->max_smem_optin, 200 * 1024);
+}
+
+template <int OP>
+static void fft_pair_2d(lrfg_ctx* ctx, const double2* in, double2* out, const FibreMul<double>& fm) {
+  LRFG_REQUIRE(fm.d == 2 && fm.axis == 0 && fm.L == 0 && in != out, "both components of a d = 2 half spectrum expected");
+  LRFG_REQUIRE(!(OP == 2 && fm.precond) || fm.inv_kk, "reciprocal table missing");
+  const int N = fm.N0, H = fm.H;
+  const auto* W = twiddle_table<double>(ctx, N);
+  size_t smem;
+  int TF;
+  const FftPlan pl = tile_complex(ctx, N, sizeof(double2), 2LL * H, &TF, &smem);
+  const int F = std::max(1, TF / 2);
+  smem = sizeof(double2) * (size_t)N * (1 + 4 * F);
+  const double n_el = (double)N * H;
+  LRFG_CUDA(raise_smem_limit((const void*)fft_pair_2d_kernel<OP>, smem));
+  LRFG_LAUNCH(ctx, KC_FFT_FIBRES, 2.0 * (5.0 * std::log2((double)N) + 2.0 * OP) * n_el, 3.0 * sizeof(double2) * n_el,
+              fft_pair_2d_kernel<OP><<<(unsigned)((H + F - 1) / F), 256, smem, ctx->stream>>>(in, out, N, H, F, pl, W, fm));
+}
+
+void fft_grad_2d(lrfg_ctx* ctx, const double2* v, double2* w, const FibreMul<double>& fm) { fft_pair_2d<1>(ctx, v, w, fm); }
+void fft_div_2d(lrfg_ctx* ctx, const double2* w, double2* out, const FibreMul<double>& fm) { fft_pair_2d<2>(ctx, w, out, fm); }
+
 // Plain transforms between n frequencies and the L > n points of the double grid along the middle axis: inverse
 // (outer, n, inner) -> (outer, L, inner) with zeros for the other frequencies, forward (outer, L, inner) -> (outer, n,
 // inner) keeping n of them.

@@ -159,13 +159,15 @@ __global__ void __launch_bounds__(256, 3) c2r_rows_kernel(const typename CplxOf<
 // directions pair rows f and f + TF in one complex FFT (real and imaginary parts), so after the inverse
 // transform the product acts on the two parts in place and the forward transform runs on the result as is.
 // `in` and `out` may alias (a block reads all of its rows before it writes them).  H: stored frequencies of a row, at
-// most (N + 1) / 2 (fewer on the double grid of the exact integration, where the others are zero and not wanted).
+// most (N + 1) / 2 (fewer on the double grid of the exact integration, where the others are zero and not wanted).  crows: rows
+// of the coefficient, rows beyond it (a second component) starting over.
 template <typename R>
 __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename CplxOf<R>::T* in,
                                                                const R* __restrict__ coef, R scale,
                                                                typename CplxOf<R>::T* out, long long rows, int N,
                                                                int H, int TF, FftPlan pl,
-                                                               const typename TwOf<typename CplxOf<R>::T>::T* __restrict__ Wg) {
+                                                               const typename TwOf<typename CplxOf<R>::T>::T* __restrict__ Wg,
+                                                               long long crows) {
   using V = typename CplxOf<R>::T;
   const float invN = 1.0f / (float)N, invH = 1.0f / (float)H;
   extern __shared__ __align__(16) unsigned char smraw_fused[];
@@ -215,7 +217,6 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
   {
     constexpr int kU = 4;
     const int total = nrow * N;
-    const R* c0 = coef + (size_t)r0 * N;
     for (int base = threadIdx.x; base < total; base += kU * blockDim.x) {
       R ca[kU], cb[kU];
 #pragma unroll
@@ -224,9 +225,10 @@ __global__ void __launch_bounds__(256, 3) c2r_mul_r2c_rows_kernel(const typename
         ca[u] = R(0);
         cb[u] = R(0);
         if (t < total) {
-          const int row = small_div(t, N, invN);
-          ca[u] = c0[t];
-          if (row + TF < nr) cb[u] = c0[t + (size_t)TF * N];
+          const int row = small_div(t, N, invN), k = t - row * N;
+          const long long ra = r0 + row, rb = ra + TF;
+          ca[u] = coef[(ra < crows ? ra : ra - crows) * N + k];
+          if (row + TF < nr) cb[u] = coef[(rb < crows ? rb : rb - crows) * N + k];
         }
       }
 #pragma unroll
@@ -479,10 +481,10 @@ void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half
   LRFG_LAUNCH(ctx, KC_ROWS_FUSED, 5.0 * N * std::log2((double)N) * (double)g.rows,
               (double)g.rows * (2.0 * g.H * sizeof(V) + N * sizeof(R)),
               c2r_mul_r2c_rows_kernel<R><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
-                  half_inout, coef, scale, half_inout, g.rows, N, g.H, TF, pl, W));
+                  half_inout, coef, scale, half_inout, g.rows, N, g.H, TF, pl, W, g.rows));
 }
 
-void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef) {
+void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef, long long crows) {
   LRFG_CUDA(ensure_roots(ctx->device));
   const auto* W = twiddle_table<double>(ctx, N);
   size_t smem;
@@ -494,7 +496,7 @@ void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_in
   LRFG_LAUNCH(ctx, KC_ROWS_FUSED, 5.0 * N * std::log2((double)N) * (double)rows,
               (double)rows * (2.0 * H * sizeof(double2) + N * sizeof(double)),
               c2r_mul_r2c_rows_kernel<double><<<(unsigned)blocks, 256, smem, ctx->stream>>>(
-                  half_inout, coef, 1.0, half_inout, rows, N, H, TF, pl, W));
+                  half_inout, coef, 1.0, half_inout, rows, N, H, TF, pl, W, crows));
 }
 
 template void full_rows_mul<double>(lrfg_ctx*, const FullGrid&, double2*, const double*, double);
@@ -748,6 +750,16 @@ void full_operator_3d(lrfg_ctx* ctx, const FullGrid& g, const typename CplxOf<R>
   fft_fibres_mul(ctx, (const V*)w2, out, fibre_mul<R>(g, 2, 0, -1, 1.0, 0, precond));
 }
 
+// Operator of a d = 2 grid in FP64, both components in each of three launches: the gradient's inverse axis-0 pass of both from
+// one read of v, the fused rows of both, the forward pass with the divergence summed in registers.  Small grids are bound
+// by the length of a launch's dependent passes and the gaps between launches (six of 8-17 us at 63 x 63).
+void full_operator_2d(lrfg_ctx* ctx, const FullGrid& g, const double2* v, double2* out, const double* coef, double scale,
+                      int precond, double2* w) {
+  fft_grad_2d(ctx, v, w, fibre_mul<double>(g, 1, 0, 0, scale, 0, 0));
+  half_rows_mul(ctx, 2 * g.rows, g.N[1], g.H, w, coef, g.rows);
+  fft_div_2d(ctx, w, out, fibre_mul<double>(g, 2, 0, 0, 1.0, 1, precond));
+}
+
 // The Ga operator (Eq. (ls_Ga_fourier)): as above with every transform between the grid's N frequencies and the double
 // grid's M points.  A zero-padded spectrum is padded axis by axis inside the passes, so the fibres of frequencies outside
 // the grid, zero before the inverse passes and dropped after the forward ones, are never transformed: axis 0 runs on a
@@ -765,7 +777,7 @@ void ga_operator(lrfg_ctx* ctx, const FullGrid& g, const FullGrid& gM, const dou
   if (g.d == 2) {
     for (int alpha = 0; alpha < 2; ++alpha) {
       fft_fibres_mul(ctx, v, w0, fm(1, 0, alpha, scale, 0, 0));
-      half_rows_mul(ctx, gM.N[0], last, g.H, w0, coef);
+      half_rows_mul(ctx, gM.N[0], last, g.H, w0, coef, gM.N[0]);
       fft_fibres_mul(ctx, (const double2*)w0, out, fm(2, 0, alpha, 1.0, alpha == 0, alpha == 1 && precond));
     }
     return;
@@ -774,13 +786,13 @@ void ga_operator(lrfg_ctx* ctx, const FullGrid& g, const FullGrid& gM, const dou
   const int n1 = g.N[1], m1 = gM.N[1];
   fft_fibres_mul(ctx, v, w1, fm(1, 0, 0, scale, 0, 0));
   fft_fibres_pad(ctx, w1, w0, gM.N[0], n1, m1, g.H, 1);
-  half_rows_mul(ctx, rows, last, g.H, w0, coef);
+  half_rows_mul(ctx, rows, last, g.H, w0, coef, rows);
   fft_fibres_pad(ctx, w0, w1, gM.N[0], n1, m1, g.H, -1);
   fft_fibres_mul(ctx, (const double2*)w1, out, fm(2, 0, 0, 1.0, 1, 0));
   fft_fibres_pad(ctx, v, w1, 1, g.N[0], gM.N[0], in0, 1);
   for (int alpha = 1; alpha <= 2; ++alpha) {
     fft_fibres_mul(ctx, (const double2*)w1, w0, fm(1, 1, alpha, scale, 0, 0));
-    half_rows_mul(ctx, rows, last, g.H, w0, coef);
+    half_rows_mul(ctx, rows, last, g.H, w0, coef, rows);
     fft_fibres_mul(ctx, (const double2*)w0, w2, fm(2, 1, alpha, 1.0, alpha == 1, 0));
   }
   fft_fibres_mul(ctx, (const double2*)w2, out, fm(2, 0, -1, 1.0, 0, precond));

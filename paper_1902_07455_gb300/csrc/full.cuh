@@ -39,8 +39,8 @@ void half_fibres_forward_div(lrfg_ctx* ctx, const FullGrid& g, V* half, V* acc, 
                              int precond);
 // the last-axis passes of full_inverse and full_forward fused around a product with the real coefficient:
 // half <- R2C(scale * coef (.) C2R(half)) along the rows (unnormalised transforms, in place)
-// (half_rows_mul: rows of N points with H stored frequencies, FP64)
-void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef);
+// (half_rows_mul: rows of N points with H stored frequencies, FP64; the crows rows of the coefficient repeat)
+void half_rows_mul(lrfg_ctx* ctx, long long rows, int N, int H, double2* half_inout, const double* coef, long long crows);
 template <typename R>
 void full_rows_mul(lrfg_ctx* ctx, const FullGrid& g, typename CplxOf<R>::T* half_inout, const R* coef, R scale);
 // out = (precond: P~^-1) grad^* F coef F^-1 grad^ v on a d = 3 grid (scale: 1/|N| of the unnormalised transforms);
@@ -49,6 +49,9 @@ template <typename R>
 void full_operator_3d(lrfg_ctx* ctx, const FullGrid& g, const typename CplxOf<R>::T* v, typename CplxOf<R>::T* out,
                       const R* coef, double scale, int precond, typename CplxOf<R>::T* w0, typename CplxOf<R>::T* w1,
                       typename CplxOf<R>::T* w2);
+// the same on a d = 2 grid in FP64; w: two half spectra, distinct from v and out
+void full_operator_2d(lrfg_ctx* ctx, const FullGrid& g, const double2* v, double2* out, const double* coef, double scale,
+                      int precond, double2* w);
 // the same for the exact integration on the double grid gM (d = 2 or 3, FP64), coef its modified coefficient; w0: gM.n_half,
 // w1, w2: gM.N[0] g.N[1] g.H elements (d = 3), distinct from v and out
 void ga_operator(lrfg_ctx* ctx, const FullGrid& g, const FullGrid& gM, const double2* v, double2* out, const double* coef,

@@ -38,6 +38,11 @@ struct FibreMul {
 };
 template <typename V>
 void fft_fibres_mul(lrfg_ctx* ctx, const V* in, V* out, const FibreMul<typename RealOf<V>::T>& fm);
+// both components of a d = 2 half spectrum (FP64): w_a = F_0^-1 (v 2 pi i k_a scale) for a = 0, 1, one after the other in w;
+// out = -2 pi i scale (k_0 F_0 w_0 + k_1 F_0 w_1) (precond: times 1/(k.k)); fm: modes 1 and 2 along axis 0
+void fft_grad_2d(lrfg_ctx* ctx, const double2* v, double2* w, const FibreMul<double>& fm);
+void fft_div_2d(lrfg_ctx* ctx, const double2* w, double2* out, const FibreMul<double>& fm);
+bool fft_pair_2d_fits(lrfg_ctx* ctx, int N);  // one fibre of both components fits in shared memory
 // plain transforms between n frequencies and L > n points (see fft.cu)
 void fft_fibres_pad(lrfg_ctx* ctx, const double2* in, double2* out, long long outer, int n, int L, long long inner,
                     int sign);
