@@ -12,7 +12,7 @@
 // The steps are chains of dependent FP64 operations, and on this part a warp issues one FP64 instruction per 64 cycles
 // whatever its instruction-level parallelism or active lanes (an SM has four such units): each kernel is laid out to put
 // few FP64 instructions on the longest of the four.  Three matrices of n = 30, k = 20 take 155 us (420 us with the same
-// algorithm laid out by arithmetic alone), one of n = 60, k = 20 402 us (744), n = 135, k = 10 2.0 ms (2.3).
+// algorithm laid out by arithmetic alone), one of n = 60, k = 20 402 us (744), n = 135, k = 10 1.45 ms (2.3).
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
@@ -419,7 +419,8 @@ __device__ __forceinline__ SyevxScratch syevx_scratch(double* scratch, int nl, i
   return g;
 }
 
-// K1.  nl, kl: the launch sizes (strides of the inputs and outputs).  nAg (optional): the active size of each item, the
+// K1 above n = 96 (n = 135: 1.60 -> 1.03 ms with the product dealt to all warps, one triangle and two multiply-adds an entry).
+// nl, kl: the launch sizes (strides of the inputs and outputs).  nAg (optional): the active size of each item, the
 // leading block of its matrix; the rest is zero.
 __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* __restrict__ Ag, int nl, int kl,
                                                                   double* wg, double* Vg, int ldv, double* scratch,
@@ -429,10 +430,11 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
   double* red = sm;            // 33 (32 partials + the result) + padding
   double* pv = red + 40;       // nl: p / w of the current reflector
   double* vv = pv + nl;        // nl: current reflector v
+  double* ps = vv + nl;        // kSyevxThreads: parts of the product A22 v
   const size_t nnl = (size_t)nl * nl;
   const SyevxScratch g = syevx_scratch(scratch, nl, kl, blockIdx.x);
   double *d = g.d, *e = g.e, *beta = g.beta;  // written once per step by thread 0
-  double* W = use_smem ? (vv + nl) : g.W;
+  double* W = use_smem ? (ps + kSyevxThreads) : g.W;
   const int tid = threadIdx.x, nthr = blockDim.x;
   double* wout = wg + (size_t)blockIdx.x * nl;
   double* Vout = Vg + (size_t)blockIdx.x * (size_t)nl * ldv;
@@ -451,30 +453,33 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     Vout[(size_t)i * ldv + t] = 0.0;
   }
   if (n == 0) return;
+  // in shared memory rows have an odd stride and only the lower triangle is kept up to date
+  const int ldw = use_smem ? (n | 1) : n;
   int top = 0;
   for (size_t t = tid; t < (size_t)n * n; t += nthr) {
-    const int i = (int)(t / n), j = (int)(t - (t / n) * n);
-    W[t] = A[(size_t)i * nl + j];
-    top = max(top, __double2hiint(W[t]) & 0x7fffffff);
+    const size_t i = t / n, j = t - i * n;
+    const double v = A[i * nl + j];
+    W[i * ldw + j] = v;
+    top = max(top, __double2hiint(v) & 0x7fffffff);
   }
   const double scale = range_scale(top, (int*)red);
-  for (size_t t = tid; t < (size_t)n * n; t += nthr) W[t] *= scale;
+  for (size_t t = tid; t < (size_t)n * n; t += nthr) W[t / n * ldw + t % n] *= scale;
   __syncthreads();
 
   // 1. tridiagonalisation
   for (int j = 0; j + 2 < n; ++j) {
     const int m = n - j - 1;
-    double x0 = W[(size_t)(j + 1) * n + j];
+    double x0 = W[(size_t)(j + 1) * ldw + j];
     double loc = 0.0;
     for (int i = tid; i < m; i += nthr) {
-      double xi = W[(size_t)(j + 1 + i) * n + j];
+      double xi = W[(size_t)(j + 1 + i) * ldw + j];
       vv[i] = xi;
       if (i > 0) loc += xi * xi;
     }
     const double tail2 = block_reduce_sum(loc, red, m);
     if (!(tail2 > kTailFloor)) {
       if (tid == 0) {
-        d[j] = W[(size_t)j * n + j];
+        d[j] = W[(size_t)j * ldw + j];
         e[j] = x0;
         beta[j] = 0.0;
       }
@@ -484,11 +489,12 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     // the reflector's scalars once (a square root and a division are long FP64 sequences: computed by
     // every thread they would occupy the FP64 pipe for thousands of cycles)
     if (tid == 0) {
-      const double alpha = -copysign(sqrt(x0 * x0 + tail2), x0);
+      const double s = fma(x0, x0, tail2), nrm = s * recip_sqrt(s);
+      const double alpha = -copysign(nrm, x0);
       const double v0 = x0 - alpha;
-      const double bb = 2.0 / (tail2 + v0 * v0);
+      const double bb = recip(fma(fabs(x0), nrm, s));  // 2 / (v^T v)
       vv[0] = v0;
-      d[j] = W[(size_t)j * n + j];
+      d[j] = W[(size_t)j * ldw + j];
       e[j] = alpha;
       beta[j] = bb;
       red[34] = bb;
@@ -496,45 +502,55 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     __syncthreads();
     const double b = red[34];
     // keep v in column j below the diagonal for the back-transformation
-    for (int i = tid; i < m; i += nthr) W[(size_t)(j + 1 + i) * n + j] = vv[i];
-    // p = b A22 v: thread i takes row i, reading column i of the symmetric trailing block so that
-    // neighbouring threads read neighbouring words (no warp reductions, which cost FP64 issue slots)
-    for (int i = tid; i < m; i += nthr) {
-      const double* col = W + (size_t)(j + 1) * n + (j + 1 + i);
-      // four independent accumulators: an FP64 FMA has a 64-cycle latency on this part
-      double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      int l = 0;
-      for (; l + 3 < m; l += 4) {
-        s0 = fma(col[(size_t)l * n], vv[l], s0);
-        s1 = fma(col[(size_t)(l + 1) * n], vv[l + 1], s1);
-        s2 = fma(col[(size_t)(l + 2) * n], vv[l + 2], s2);
-        s3 = fma(col[(size_t)(l + 3) * n], vv[l + 3], s3);
-      }
-      for (; l < m; ++l) s0 = fma(col[(size_t)l * n], vv[l], s0);
-      pv[i] = b * ((s0 + s1) + (s2 + s3));
-    }
+    for (int i = tid; i < m; i += nthr) W[(size_t)(j + 1 + i) * ldw + j] = vv[i];
+    // p = b A22 v, a row per lane; the columns of a row are dealt to all warps (a warp issues one FP64 instruction per 64
+    // cycles: the rows alone kept five warps busy at n = 135)
     const int warp = tid >> 5, lane = tid & 31, nw = nthr >> 5;
+    const int rw = (m + 31) >> 5, parts = max(1, nw / rw), chunk = (m + parts - 1) / parts;
+    for (int q = warp; q < rw * parts; q += nw) {
+      const int part = q / rw, i = (q - part * rw) * 32 + lane, l1 = min(m, (part + 1) * chunk);
+      if (i >= m) continue;
+      const double* row = W + (size_t)(j + 1 + i) * ldw + (j + 1);  // entries l <= i
+      const double* col = W + (size_t)(j + 1) * ldw + (j + 1 + i);  // the others, or all (neighbouring threads, neighbouring words)
+      const int mine = use_smem ? i : -1;
+      double s0 = 0.0, s1 = 0.0;
+      int l = part * chunk;
+      for (; l + 1 < l1; l += 2) {
+        s0 = fma(l <= mine ? row[l] : col[(size_t)l * ldw], vv[l], s0);
+        s1 = fma(l + 1 <= mine ? row[l + 1] : col[(size_t)(l + 1) * ldw], vv[l + 1], s1);
+      }
+      if (l < l1) s0 = fma(l <= mine ? row[l] : col[(size_t)l * ldw], vv[l], s0);
+      (parts > 1 ? ps + part * rw * 32 : pv)[i] = parts > 1 ? s0 + s1 : b * (s0 + s1);
+    }
     __syncthreads();
     double kl = 0.0;
-    for (int i = tid; i < m; i += nthr) kl += vv[i] * pv[i];
+    for (int i = tid; i < m; i += nthr) {
+      if (parts > 1) {
+        double p = ps[i];
+        for (int q = 1; q < parts; ++q) p += ps[q * rw * 32 + i];
+        pv[i] = b * p;
+      }
+      kl += vv[i] * pv[i];
+    }
     const double K = 0.5 * b * block_reduce_sum(kl, red, m);
     for (int i = tid; i < m; i += nthr) pv[i] -= K * vv[i];
     __syncthreads();
     // A22 -= v w^T + w v^T (one warp per row)
     for (int i = warp; i < m; i += nw) {
-      double* row = W + (size_t)(j + 1 + i) * n + (j + 1);
+      double* row = W + (size_t)(j + 1 + i) * ldw + (j + 1);
       const double vi = vv[i], wi = pv[i];
-      for (int l = lane; l < m; l += 32) row[l] -= vi * pv[l] + wi * vv[l];
+      const int end = use_smem ? i + 1 : m;
+      for (int l = lane; l < end; l += 32) row[l] = fma(-vi, pv[l], fma(-wi, vv[l], row[l]));
     }
     __syncthreads();
   }
   if (tid == 0) {
     if (n >= 2) {
-      d[n - 2] = W[(size_t)(n - 2) * n + (n - 2)];
-      e[n - 2] = W[(size_t)(n - 1) * n + (n - 2)];
+      d[n - 2] = W[(size_t)(n - 2) * ldw + (n - 2)];
+      e[n - 2] = W[(size_t)(n - 1) * ldw + (n - 2)];
       if (n >= 3) beta[n - 2] = 0.0;
     }
-    d[n - 1] = W[(size_t)(n - 1) * n + (n - 1)];
+    d[n - 1] = W[(size_t)(n - 1) * ldw + (n - 1)];
     e[n - 1] = 0.0;
     beta[n - 1] = 0.0;
   }
@@ -548,7 +564,7 @@ __global__ void __launch_bounds__(kSyevxThreads) syevx_tri_kernel(const double* 
     g.hdr[4] = 1.0 / scale;
   }
   if (use_smem)
-    for (size_t t = tid; t < (size_t)n * n; t += nthr) g.W[t] = W[t];
+    for (size_t t = tid; t < (size_t)n * n; t += nthr) g.W[t] = W[t / n * ldw + t % n];
 }
 
 // K1 for n <= 32 NR: the matrix in registers, row = lane (NR rows a lane), columns dealt to TW worker warps.  A warp issues
@@ -1155,9 +1171,9 @@ static void syevx_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, i
   } else if (n <= kSmallEig) {
     tri_small(syevx_tri_small_kernel<3, 6>, 224);
   } else {
-    const size_t wbytes = sizeof(double) * (size_t)n * n;
-    const size_t head1 = sizeof(double) * (40 + 2 * (size_t)n);
-    const int smem_w1 = head1 + wbytes <= lim ? 1 : 0;
+    const size_t wbytes = sizeof(double) * (size_t)n * (n | 1);
+    const size_t head1 = sizeof(double) * (40 + 2 * (size_t)n + kSyevxThreads);
+    const int smem_w1 = head1 + wbytes <= (size_t)std::min(ctx->max_smem_optin, 208 * 1024) ? 1 : 0;
     const size_t smem1 = head1 + (smem_w1 ? wbytes : 0);
     LRFG_CUDA(raise_smem_limit((const void*)syevx_tri_kernel, smem1));
     LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0,
