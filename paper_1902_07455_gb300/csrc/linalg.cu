@@ -305,17 +305,20 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // split further runs on a few SMs for that long; 16-tiles give four times the blocks at a quarter of the work
   if (tile == 32 && active_tiles(32) * std::max(1, K / GK) < nsm) tile = 16;
   const long long active = active_tiles(tile);
-  // Split long K so that the busiest SM has the fewest k-steps: a block of c k-steps, active * ceil(steps / c) blocks, and
-  // a round of blocks costs c steps plus about one for its first loads and its partial sums.  Rounding a target of two
-  // blocks per SM to whole k-steps left 228 blocks of two steps on 152 SMs (four steps on the busiest one) where 152
-  // blocks of three do: the 60 x 60 x 14580 Gram product took 140 us.  At most four blocks per SM (the partials' sum).
+  // Split long K for the shortest busiest SM.  With q blocks of c k-steps on it and `filled` of a tile's outputs on average:
+  // full tiles bound a lone block (q = 1), several even out to the average tile; a lone block's loads are not covered by
+  // another's arithmetic (about a third of a step each); a block costs about one step more for its first loads and its
+  // partial sums.  At most four blocks per SM.  One block per SM took 966 us for the 135 x 135 x 18225 Gram product of a
+  // compression (a third of whose tiles' outputs are padding), four take 404 us.
   const int steps = (K + GK - 1) / GK;
+  const double filled = dyn ? 1.0 : (sym ? 0.5 * M * (M + 1.0) : (double)M * N) * batch / ((double)tiles_of(tile) * tile * tile);
   int per = steps;
   if (active < 2LL * nsm) {
     double best = 0.0;
     for (int c = (int)std::max(1LL, std::min<long long>(steps, active * steps / (4LL * nsm))); c <= steps; ++c) {
       const long long blocks = active * ((steps + c - 1) / c);
-      const double cost = (double)((blocks + nsm - 1) / nsm) * (c + 1.0);
+      const double q = (double)((blocks + nsm - 1) / nsm);
+      const double cost = (filled * q + (1.0 - filled)) * c + (q < 2.0 ? 0.35 * c : 0.0) + q;
       if (best == 0.0 || cost < best) {
         best = cost;
         per = c;
