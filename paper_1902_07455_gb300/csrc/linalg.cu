@@ -273,7 +273,7 @@ void gemm(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alp
 template <typename T>
 static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const T* A, int lda,
                       long long sA, const T* B, int ldb, long long sB, double beta, T* C, int ldc, long long sC,
-                      int batch, const int* dynM, int mulM, const int* dynN, int mulN, bool sym = false) {
+                      int batch, const int* dynM, int mulM, const int* dynN, int mulN, bool sym = false, bool once = false) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   LRFG_REQUIRE(!sym || (M == N && transA != transB && beta == 0.0), "not a symmetric product");
   if (K <= 0) {
@@ -314,20 +314,26 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // split further runs on a few SMs for that long; 16-tiles give four times the blocks at a quarter of the work
   if (tile == 32 && active_tiles(32) * std::max(1, K / GK) < nsm) tile = 16;
   const long long active = active_tiles(tile);
-  // Split long K for the shortest busiest SM.  With q blocks of c k-steps on it and `filled` of a tile's outputs on average:
-  // full tiles bound a lone block (q = 1), several even out to the average tile; a lone block's loads are not covered by
-  // another's arithmetic (about a third of a step each); a block costs about one step more for its first loads and its
-  // partial sums.  At most four blocks per SM.  One block per SM took 966 us for the 135 x 135 x 18225 Gram product of a
-  // compression (a third of whose tiles' outputs are padding), four take 404 us.
+  // Split long K so that the busiest SM has the fewest k-steps: a block of c k-steps, active * ceil(steps / c) blocks, and
+  // a round of blocks costs c steps plus about one for its first loads and its partial sums.  At most four blocks per SM, two
+  // in a context whose pool has a budget (the partial sums' space).
+  // once: a product no lockstep batch repeats, so that its order of summation is free (a solve alone and in lockstep takes the
+  // same steps to 1e-9 only where both split alike).  Several blocks an SM even out to the average tile, `filled` of its
+  // outputs, and a lone block's loads are not covered by another's arithmetic (about a third of a step each): the 135 x 135 x
+  // 18225 Gram product of a compression, a third of whose tiles' outputs are padding, took 966 us in one block per SM and
+  // takes 404 us in four.
   const int steps = (K + GK - 1) / GK;
-  const double filled = dyn ? 1.0 : (sym ? 0.5 * M * (M + 1.0) : (double)M * N) * batch / ((double)tiles_of(tile) * tile * tile);
+  const double filled = dyn || !once ? 1.0 : (sym ? 0.5 * M * (M + 1.0) : (double)M * N) * batch / ((double)tiles_of(tile) * tile * tile);
   int per = steps;
   if (active < 2LL * nsm) {
     double best = 0.0;
-    for (int c = (int)std::max(1LL, std::min<long long>(steps, active * steps / (4LL * nsm))); c <= steps; ++c) {
+    const bool tight = ctx->pool->budget() != 0;
+    const long long most = (tight ? 2LL : 4LL) * nsm;
+    for (int c = (int)std::max(1LL, std::min<long long>(steps, active * steps / most)); c <= steps; ++c) {
       const long long blocks = active * ((steps + c - 1) / c);
+      if (tight && blocks > most) continue;
       const double q = (double)((blocks + nsm - 1) / nsm);
-      const double cost = (filled * q + (1.0 - filled)) * c + (q < 2.0 ? 0.35 * c : 0.0) + q;
+      const double cost = (filled * q + (1.0 - filled)) * c + (q < 2.0 && once ? 0.35 * c : 0.0) + q;
       if (best == 0.0 || cost < best) {
         best = cost;
         per = c;
@@ -374,8 +380,8 @@ void gemm_dyn(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double
 }
 
 void gemm_sym(lrfg_ctx* ctx, int trans, int M, int K, const double* A, int lda, long long sA, const double* B, int ldb,
-              long long sB, double* C, int ldc, long long sC, int batch, const int* dyn) {
-  gemm_impl<double>(ctx, trans, !trans, M, M, K, 1.0, A, lda, sA, B, ldb, sB, 0.0, C, ldc, sC, batch, dyn, 1, dyn, 1, true);
+              long long sB, double* C, int ldc, long long sC, int batch, const int* dyn, bool once) {
+  gemm_impl<double>(ctx, trans, !trans, M, M, K, 1.0, A, lda, sA, B, ldb, sB, 0.0, C, ldc, sC, batch, dyn, 1, dyn, 1, true, once);
 }
 
 void gemm_f32(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const float* A, int lda,

@@ -76,9 +76,11 @@ void gemm_dyn(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double
               long long sA, const double* B, int ldb, long long sB, double beta, double* C, int ldc, long long sC,
               int batch, const int* dynM, int mulM, const int* dynN, int mulN);
 // Symmetric products C[b] = A[b]^T B[b] (trans = 1; A, B: K x M) or A[b] B[b]^T (trans = 0; M x K): Gram matrices (A = B)
-// and F R F^T with a symmetric R (A = F R, B = F); half the work of gemm.  dyn: active size per item (may be null)
+// and F R F^T with a symmetric R (A = F R, B = F); half the work of gemm.  dyn: active size per item (may be null); once: a
+// product that no lockstep batch repeats (see gemm_impl's split of K)
 void gemm_sym(lrfg_ctx* ctx, int trans, int M, int K, const double* A, int lda, long long sA, const double* B, int ldb,
-              long long sB, double* C, int ldc, long long sC, int batch = 1, const int* dyn = nullptr);
+              long long sB, double* C, int ldc, long long sC, int batch = 1, const int* dyn = nullptr,
+              bool once = false);
 // FP32 product (same layout rules, FP32 operands and accumulation)
 void gemm_f32(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, double alpha, const float* A, int lda,
               long long sA, const float* B, int ldb, long long sB, double beta, float* C, int ldc, long long sC,

@@ -718,9 +718,9 @@ void tt_compress(lrfg_ctx* ctx, int d, const int* N, const double* values, int r
     const int m = use_rows ? rows : (int)cols;
     DBuf<double> G(ctx->pool, (size_t)m * m), lam(ctx->pool, m), V(ctx->pool, (size_t)m * m);
     if (use_rows)
-      gemm_sym(ctx, 0, m, (int)cols, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0);
+      gemm_sym(ctx, 0, m, (int)cols, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0, 1, nullptr, true);
     else
-      gemm_sym(ctx, 1, m, rows, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0);
+      gemm_sym(ctx, 1, m, rows, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0, 1, nullptr, true);
     // only the kept eigenpairs are decomposed (with a tolerance, every eigenvalue: the rule sums the tail): a cyclic
     // Jacobi of the whole m x m Gram matrix in one block took 46 ms per bond at m = 135, this 2.3 ms; a compression of
     // 135^3 values to rank 10 with its expansion went from 98.3 to 5.8 ms
