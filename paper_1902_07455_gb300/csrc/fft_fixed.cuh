@@ -12,10 +12,10 @@
 // sum, below FP64's rounding of the same transform: relative 2-norm errors against extended precision, random rows of 243,
 // 729 and 2187 entries: FP64 3.6e-16, 4.3e-16, 4.9e-16, this 7.9e-17, 8.9e-17, 1.5e-16.  Rows are scaled one by one, so
 // a small row keeps its own accuracy.
-// Measured: 243-point passes over 243^3 438 -> 200 us, fused row pass 1078 -> 496 us, FP64 application 9.55 -> 4.42 ms,
-// 105 x 147 x 75 anisotropic 0.93 -> 0.65 ms, Ga at 63^3 0.86 -> 0.56 ms.  The integer pipes bound it now (55% of their
-// rate, about 660 instructions a point); unrolling the conversions into the butterflies instead of their own loops took
-// 230 us a pass, waiting for instructions.
+// Measured: 243-point passes over 243^3 438 -> 175 us, fused row pass 1078 -> 412 us, FP64 application 9.55 -> 3.83 ms,
+// 105 x 147 x 75 anisotropic 0.93 -> 0.60 ms, Ga at 63^3 0.86 -> 0.50 ms.  The integer pipes bound it now (60% of their
+// rate, about 580 instructions a point, 24 warps an SM); with the conversions unrolled into the butterflies instead of in
+// loops of their own a pass took 30 us more, waiting for instructions.
 // A row with an entry that is not finite becomes NaN as a whole.
 #pragma once
 

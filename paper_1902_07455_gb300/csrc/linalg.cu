@@ -13,7 +13,7 @@ namespace lrfg {
 // the kernel is built to waste none of it: a block owns a 64 x 64 (small products: 32 x 32) output block
 // (clipped to the active sizes, which may be read from the device), each of its 256 threads owns up to 16
 // (4) outputs of that block exactly (no padded tile rows or columns are computed), operands are staged
-// through shared memory in k-steps of 32, and long K is split across blocks until about two blocks per SM are busy (split-K: each
+// through shared memory in k-steps of 32, and long K is split across blocks (see gemm_impl; split-K: each
 // split writes its partial block to a workspace; the last split of a tile to arrive, found by an arrival
 // counter, sums the partials in split order, so every product, and with it every solve, is bitwise
 // reproducible whatever else runs on the GPU, and no second launch is needed).  With many splits the sum is
