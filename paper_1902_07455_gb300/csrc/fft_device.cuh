@@ -32,13 +32,16 @@ constexpr int kRootOff3 = 0, kRootOff5 = 3, kRootOff7 = 8, kRootOff9 = 15, kRoot
 __constant__ float2 c_roots_f[kRootCount];
 __constant__ int4 c_roots_x[kRootCount];  // fixed point (fft_fixed.cuh)
 
-// exp(-2 pi i j / p) in fixed point: upper and lower parts of cos 2^62 and -sin 2^62 (1 as 1 - 2^-62)
+// exp(-2 pi i j / p) in fixed point: cos 2^62 and -sin 2^62 (1 as 1 - 2^-62), each as an upper part times 2^31 and a lower
+// one between -2^30 and 2^30 (2^31 - 1 for 1 itself, whose other component is 0): with both signs the lower parts leave
+// room for fix_cmul's sums.
 static inline int4 fixed_root(int j, int p) {
   const long double ang = 6.283185307179586476925286766559005768L * (long double)j / (long double)p;
   const long long one = (1LL << 62) - 1;
-  const long long x = std::min(one, (long long)llroundl(cosl(ang) * 0x1p62L));
-  const long long y = std::min(one, (long long)llroundl(-sinl(ang) * 0x1p62L));
-  return make_int4((int)(x >> 31), (int)(x & 0x7fffffff), (int)(y >> 31), (int)(y & 0x7fffffff));
+  auto upper = [](long long v) { return std::min(0x7fffffffLL, (v + (1LL << 30)) >> 31); };
+  const long long x = std::min(one, (long long)llroundl(cosl(ang) * 0x1p62L)), xh = upper(x);
+  const long long y = std::min(one, (long long)llroundl(-sinl(ang) * 0x1p62L)), yh = upper(y);
+  return make_int4((int)xh, (int)(x - xh * (1LL << 31)), (int)yh, (int)(y - yh * (1LL << 31)));
 }
 
 // Fills this translation unit's root tables on the current device (once per device); returns the CUDA

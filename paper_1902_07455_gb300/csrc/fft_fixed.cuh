@@ -5,12 +5,12 @@
 // two and transformed with integer additions and 32 x 32 -> 64-bit multiply-adds; the conversions are integer operations
 // on the bits of the doubles.
 //
-// Range: the scale brings the sum of the moduli of a row's components to at most 2^61 (1.05 times that with the parts the
+// Range: the scale brings the sum of the moduli of a row's components to at most 2^61 (1.06 times that with the parts the
 // estimate drops), which bounds every intermediate and final value of the transform, whatever the passes.  The first pass
 // is bounded by its own 2 p components, so its input has up to log2(N / p) more bits, dropped before the second (on long rows
 // pass by pass): rounding the input to 2^-53 of the largest component would be the largest error.  Errors of a row are then a few units of 2^-61 of that
 // sum, below FP64's rounding of the same transform: relative 2-norm errors against extended precision, random rows of 243,
-// 729 and 2187 entries: FP64 3.6e-16, 4.3e-16, 4.9e-16, this 7.9e-17, 8.9e-17, 1.5e-16.  Rows are scaled one by one, so
+// 729 and 2187 entries: FP64 3.6e-16, 4.3e-16, 4.9e-16, this 7.7e-17, 8.7e-17, 1.3e-16.  Rows are scaled one by one, so
 // a small row keeps its own accuracy.
 // Measured: 243-point passes over 243^3 438 -> 175 us, fused row pass 1078 -> 412 us, FP64 application 9.55 -> 3.83 ms,
 // 105 x 147 x 75 anisotropic 0.93 -> 0.60 ms, Ga at 63^3 0.86 -> 0.50 ms.  The integer pipes bound it now (60% of their
@@ -27,10 +27,10 @@ struct __align__(16) Fix2 {
 
 constexpr int kFixMaxRows = 64;  // rows of a tile at most
 
-// a * w with w = wh 2^31 + wl, 0 <= wl < 2^31, a factor times 2^62, a likewise split: a w / 2^62 = ah wh + (al wh + ah wl) /
-// 2^31 with the product of the lower parts, a quarter of a unit on average, left out; `mid` starts with its mean and the
-// half that rounds its shift.
-constexpr unsigned kFixHalf = 1u << 30, kFixLow = 1u << 29;
+// a * w with a = ah 2^31 + al, 0 <= al < 2^31, and w = wh 2^31 + wl, |wl| <= 2^30 (fixed_root), a factor times 2^62:
+// a w / 2^62 = ah wh + (al wh + ah wl) / 2^31, with the product of the lower parts left out, at most half a unit and on average
+// half of wl / 2^31; `mid` starts with the half that rounds its shift.
+constexpr unsigned kFixHalf = 1u << 30;
 __device__ __forceinline__ int fix_hi(long long a) {
   return (int)__funnelshift_r((unsigned)a, (unsigned)((unsigned long long)a >> 32), 31);
 }
@@ -50,23 +50,24 @@ __device__ __forceinline__ long long fix_mul(int a, int b) {
 __device__ __forceinline__ Fix2 operator+(Fix2 a, Fix2 b) { return {a.x + b.x, a.y + b.y}; }
 __device__ __forceinline__ Fix2 operator-(Fix2 a, Fix2 b) { return {a.x - b.x, a.y - b.y}; }
 
-// w = (x upper, x lower, y upper, y lower) of exp(-2 pi i j / N); SIGN > 0 multiplies by its conjugate.  The moduli of a and w
-// bound the sums of `mid`: sqrt 2 2^62 + 1.05 2^61 < 2^63.
+// w = (x upper, x lower, y upper, y lower) of exp(-2 pi i j / N); SIGN > 0 multiplies by its conjugate.  With |a| <= 1.06 2^61
+// and |w| <= 2^62 the sums of `mid` stay below 2^63: the two products of al and bl, each below 2^31, with w's upper parts are
+// together at most sqrt 2 2^31 2^31, those of ah and bh with its lower parts at most 1.06 2^30 sqrt 2 2^30, 1.79 2^62 in all
+// (2.16 2^62 with lower parts up to 2^31: one of some 10^4 rows with a single entry overflowed).
 template <int SIGN>
 __device__ __forceinline__ Fix2 fix_cmul(Fix2 a, int4 w) {
   const int ah = fix_hi(a.x), al = fix_lo(a.x), bh = fix_hi(a.y), bl = fix_lo(a.y);
   // re = a w_x - b w_y, im = b w_x + a w_y, or with the conjugate re = a w_x + b w_y, im = b w_x - a w_y
-  constexpr long long cr = kFixHalf + (SIGN < 0 ? 0 : 2 * kFixLow), ci = kFixHalf + (SIGN < 0 ? 2 * kFixLow : 0);
   const int ch = SIGN < 0 ? -bh : bh, cl = SIGN < 0 ? -bl : bl, dh = SIGN < 0 ? ah : -ah, dl = SIGN < 0 ? al : -al;
-  const long long mr = fix_mad(cl, w.z, fix_mad(ch, w.w, fix_mad(al, w.x, fix_mad(ah, w.y, cr))));
-  const long long mi = fix_mad(dl, w.z, fix_mad(dh, w.w, fix_mad(bl, w.x, fix_mad(bh, w.y, ci))));
+  const long long mr = fix_mad(cl, w.z, fix_mad(ch, w.w, fix_mad(al, w.x, fix_mad(ah, w.y, kFixHalf))));
+  const long long mi = fix_mad(dl, w.z, fix_mad(dh, w.w, fix_mad(bl, w.x, fix_mad(bh, w.y, kFixHalf))));
   return {fix_mad(ch, w.z, fix_mad(ah, w.x, mr >> 31)), fix_mad(dh, w.z, fix_mad(bh, w.x, mi >> 31))};
 }
 
 // one component times a real factor (h, l)
 __device__ __forceinline__ long long fix_rmul(long long a, int h, int l) {
   const int ah = fix_hi(a);
-  return fix_mad(ah, h, fix_mad(fix_lo(a), h, fix_mad(ah, l, kFixHalf + kFixLow)) >> 31);
+  return fix_mad(ah, h, fix_mad(fix_lo(a), h, fix_mad(ah, l, kFixHalf)) >> 31);
 }
 
 // a / 2^s rounded to nearest, 0 <= s < 32, half = 2^s / 2
