@@ -788,7 +788,8 @@ __global__ void __launch_bounds__(256) fibre_gauss_multi_kernel(const double* __
   V* spec = sm + N;              // TF rows: the shared forward spectrum
   V* a = spec + (size_t)TF * N;  // TF rows
   V* b = a + (size_t)TF * N;     // TF rows
-  __shared__ R mult[kMaxGaussHalf];  // exp(-t_m k^2), k = 0..(N-1)/2: an FP64 exponential takes tens of operations
+  R* mult = (R*)(b + (size_t)TF * N);  // exp(-t_m k^2), k = 0..(N-1)/2 < kMaxGaussHalf: an FP64 exponential takes tens of
+                                       // operations
   for (int j = threadIdx.x; j < N; j += blockDim.x) W[j] = Wg[j];
   const long long nfib = outer * inner;
   const long long g0 = (long long)blockIdx.x * (2LL * TF);
@@ -880,7 +881,8 @@ static void fibre_gauss_multi_t(lrfg_ctx* ctx, const double* in, double* out, lo
     }
   }
   known = {pl, tf, mper};
-  size_t smem = (size_t)(N * sizeof(V) + tf * per);
+  const int half = (N - 1) / 2;
+  size_t smem = (size_t)(N * sizeof(V) + tf * per) + (half < kMaxGaussHalf ? sizeof(V) / 2 * (half + 1) : 0);
   GaussTerms terms{};
   for (int m = 0; m < nm; ++m) {
     terms.t[m] = t[m];

@@ -27,6 +27,17 @@ struct __align__(16) Fix2 {
 
 constexpr int kFixMaxRows = 64;  // rows of a tile at most
 
+// what the transforms of a kernel keep beside its tiles: 192 bytes, which leave a row of 3627 points, the longest of prime
+// factors up to 31, its 64 bytes a point (static arrays of ints in each instantiation took up to 1.2 KB)
+struct FixShared {
+  unsigned short scale[kFixMaxRows];  // 16 top + room, see fix_rows
+  int2 part[8];
+};
+__device__ __forceinline__ FixShared& fix_shared() {
+  __shared__ FixShared s;
+  return s;
+}
+
 // a * w with a = ah 2^31 + al, 0 <= al < 2^31, and w = wh 2^31 + wl, |wl| <= 2^30 (fixed_root), a factor times 2^62:
 // a w / 2^62 = ah wh + (al wh + ah wl) / 2^31, with the product of the lower parts left out, at most half a unit and on average
 // half of wl / 2^31; `mid` starts with the half that rounds its shift.
@@ -173,11 +184,14 @@ struct FixDFT<9, SIGN> {  // 3 x 3, see reg_dft_split
 
 // A row's scale at a pass: the largest component's plus min(room, lg) bits, lg = log2 of the components a sum of the pass has,
 // rounded up, room that of the row's own sum.  A pass drops the bits between its and the one before's after its twiddles, so
-// that both round once (nothing to drop: room is null).
+// that both round once (nothing to drop: scale is null).
 struct FixDrop {
-  const int* room;
+  const unsigned short* scale;
   int before, now;
-  __device__ __forceinline__ int bits(int row) const { return min(room[row], now) - min(room[row], before); }
+  __device__ __forceinline__ int bits(int row) const {
+    const int room = scale[row] & 15;
+    return min(room, now) - min(room, before);
+  }
 };
 
 // One pass of radix P over nf rows from a into b.
@@ -202,7 +216,7 @@ __device__ __forceinline__ void fix_pass(const Fix2* __restrict__ a, Fix2* __res
 #pragma unroll
       for (int r = 1; r < P; ++r) x[r] = fix_cmul<SIGN>(x[r], W[f * r * mp]);
     }
-    if (drop.room) {
+    if (drop.scale) {
       const int s = drop.bits(row);
       const unsigned half = (1u << s) >> 1;
 #pragma unroll
@@ -227,7 +241,7 @@ __device__ __noinline__ void fix_pass_prime(int p, const Fix2* __restrict__ a, F
     const int f = bt - c * L;
     const Fix2* in = a + row * ld + c * L + f;
     Fix2* out = b + row * ld + c * L * p + f;
-    const int sh = drop.room ? drop.bits(row) : 0;
+    const int sh = drop.scale ? drop.bits(row) : 0;
     const unsigned half = (1u << sh) >> 1;
     auto load = [&](int r) {
       Fix2 v = in[r * mp * L];
@@ -292,8 +306,7 @@ __device__ __forceinline__ void fix_row(double2* row, int N, int first, int step
 // into the butterflies they made the kernels wait for instructions (the largest stall of a 243-point pass).
 template <int SIGN>
 __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPlan& pl, const int4* W) {
-  __shared__ int s_top[kFixMaxRows], s_room[kFixMaxRows];
-  __shared__ int2 s_part[8];
+  FixShared& sh = fix_shared();
   const int N = pl.N;
   if (N == 1 || nf <= 0) {
     __syncthreads();
@@ -309,18 +322,15 @@ __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPl
     double2* const p = a + row * ld;
     int2 m = fix_scan(p, N, part * 32 + lane, 32 * parts);
     if (parts > 1) {
-      if (lane == 0) s_part[warp] = m;
+      if (lane == 0) sh.part[warp] = m;
       asm volatile("bar.sync %0, %1;" ::"r"(1 + row), "r"(32 * parts) : "memory");
       const int q0 = warp - part;
-      for (int q = q0; q < q0 + parts; ++q) m.x = max(m.x, s_part[q].x);
+      for (int q = q0; q < q0 + parts; ++q) m.x = max(m.x, sh.part[q].x);
       m.y = 0;
-      for (int q = q0; q < q0 + parts; ++q) m.y += s_part[q].y >> min(m.x - s_part[q].x, 31);
+      for (int q = q0; q < q0 + parts; ++q) m.y += sh.part[q].y >> min(m.x - sh.part[q].x, 31);
     }
     const int room = fix_room(m);
-    if (lane == 0 && part == 0) {
-      s_top[row] = m.x + 18;
-      s_room[row] = room;
-    }
+    if (lane == 0 && part == 0) sh.scale[row] = (unsigned short)((m.x + 18) << 4 | room);  // room <= 14
     fix_row(p, N, part * 32 + lane, 32 * parts, m.x + 18 + min(room, lg));
   }
   __syncthreads();
@@ -331,7 +341,7 @@ __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPl
     FixDrop drop{nullptr, lg, lg};
     if (s > 0 && lg < all) {
       // rows of up to 600 entries gain little from a third scale
-      drop.room = s_room;
+      drop.scale = sh.scale;
       drop.now = (N <= 600 || s == pl.nst - 1) ? all : 32 - __clz(2 * L * p - 1);
       lg = drop.now;
     }
@@ -350,7 +360,7 @@ __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPl
   }
   double2* res = reinterpret_cast<double2*>(x);
   for (int row = warp / parts; row < nf; row += nw / parts) {
-    const int top = s_top[row], c = top + s_room[row] - 1101;
+    const int top = sh.scale[row] >> 4, c = top + (sh.scale[row] & 15) - 1101;
     for (int n = part * 32 + lane; n < N; n += 32 * parts) {
       const Fix2 v = x[row * ld + n];
       const double nan = __longlong_as_double(0x7ff8000000000000LL);
