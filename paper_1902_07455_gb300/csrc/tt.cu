@@ -465,8 +465,10 @@ void tt_round_batch(lrfg_ctx* ctx, const TTBatchView& x, int rmax, TTBatch& out,
       LRFG_LAUNCH(ctx, KC_TT_MISC, 2.0 * sbb * nb, 2.0 * sizeof(double) * sbb * nb,
                   balance_diag_kernel<<<nb, 1024, sizeof(double) * b, ctx->stream>>>(GA.get(), rd.get(), cb.get(), b));
     } else {
+      const size_t smem = 2 * sizeof(double) * b;  // above 48 KB from rank 3073 on
+      LRFG_CUDA(raise_smem_limit((const void*)balance_kernel, smem));
       LRFG_LAUNCH(ctx, KC_TT_MISC, 2.0 * sbb * nb, 4.0 * sizeof(double) * sbb * nb,
-                  balance_kernel<<<nb, 1024, 2 * sizeof(double) * b, ctx->stream>>>(GA.get(), R[j + 1].get(), cb.get(), b));
+                  balance_kernel<<<nb, 1024, smem, ctx->stream>>>(GA.get(), R[j + 1].get(), cb.get(), b));
     }
     // The unfolding X = M N (M: rows x b left part, N: b x cols right part) has the Gram matrices
     // GA = M^T M and R = N N^T.  Only the side whose numerical rank is smaller is factored (pivoted
