@@ -1251,6 +1251,17 @@ __host__ __device__ inline size_t chol_head_bytes(int b) {
   return (bytes + 255) / 256 * 256;
 }
 
+// Factors of a Gram matrix with a diagonal entry that is not finite (a NaN in the data, or squares past the FP64 range): NaN
+// as a whole, not the zeros of rank 0 that stopping at such a pivot would leave.  All threads of the block call it.
+__device__ void gram_not_finite(int b, double* RA, double* RAc, double* Pc, int* rhog) {
+  if (rhog && threadIdx.x == 0) rhog[blockIdx.x] = b;
+  for (size_t t = threadIdx.x; t < (size_t)b * b; t += blockDim.x) {
+    RA[t] = __longlong_as_double(0x7ff8000000000000LL);
+    if (RAc) RAc[t] = RA[t];
+    if (Pc) Pc[t] = RA[t];
+  }
+}
+
 // Left-looking form (Golub & Van Loan Sec. 4.2.8 ordering with diagonal pivoting): pivot k takes the
 // largest remaining diagonal of the Schur complement, kept as a vector, and only column k of L is formed,
 // L[i][k] = (G[i][p] - sum_{l<k} L[i][l] L[p][l]) / L[p][k], for the rows not yet pivots; b rho^2 / 2
@@ -1283,8 +1294,10 @@ __global__ void __launch_bounds__(kCholThreads) gram_factor_kernel(const double*
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
   for (size_t t = tid; t < bb; t += nthr) W[t] = G[t];
   double md = 0.0;
+  int inf_or_nan = 0;
   for (int i = tid; i < b; i += nthr) {
     const double gi = G[(size_t)i * b + i];
+    inf_or_nan |= !isfinite(gi);
     dv[i] = gi;
     done[i] = 0;
     pos[i] = b;
@@ -1293,7 +1306,7 @@ __global__ void __launch_bounds__(kCholThreads) gram_factor_kernel(const double*
   }
   for (int o = 16; o; o >>= 1) md = fmax(md, __shfl_xor_sync(0xffffffff, md, o));
   if (lane == 0) redv[warp] = md;
-  __syncthreads();
+  if (__syncthreads_or(inf_or_nan)) return gram_not_finite(b, RA, RAc, Pc, rhog);
   if (tid == 0) {
     double m = 0.0;
     for (int i = 0; i < nw; ++i) m = fmax(m, redv[i]);
@@ -1462,7 +1475,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
   }
   long long floor_bits = 0;
   int rho = b;
-  bool is_nan = false;  // the same in every thread
+  bool inf_or_nan = false;  // the same in every thread
   for (int k = 0; k < b; ++k) {
     // the largest remaining diagonal (ties: the smallest row)
     double best = dv[0];
@@ -1480,7 +1493,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     // (positive doubles compare as integers: no FP64 comparison in the loop)
     if (k == 0) floor_bits = piv > 0.0 ? __double_as_longlong(tau * piv) : 0;
     if (mh < 0 || __double_as_longlong(piv) <= floor_bits || mh >= 0x7ff00000) {
-      is_nan = mh >= 0x7ff00000 && isnan(piv);
+      inf_or_nan = mh >= 0x7ff00000;
       rho = k;
       break;
     }
@@ -1552,16 +1565,7 @@ __global__ void __launch_bounds__(32 * CW) gram_factor_small_kernel(const double
     }
   }
   __syncthreads();
-  if (is_nan) {
-    // a NaN on the diagonal stays one in every result instead of a factor of rank 0
-    if (rhog && tid == 0) rhog[blockIdx.x] = b;
-    for (int t = tid; t < b * b; t += 32 * CW) {
-      RA[t] = __longlong_as_double(0x7ff8000000000000LL);
-      if (RAc) RAc[t] = RA[t];
-      if (Pc) Pc[t] = RA[t];
-    }
-    return;
-  }
+  if (inf_or_nan) return gram_not_finite(b, RA, RAc, Pc, rhog);
   if (rhog && tid == 0) rhog[blockIdx.x] = rho;
   if (tid == 0) {
     // column q of L: (b - q - 1) rows of q multiply-adds; the triangular inverse (rho^3/6)
