@@ -35,56 +35,76 @@ void ttb_dot_device(lrfg_ctx* ctx, const TTBatchView& x, const TTBatchView& y, d
   }
 }
 
-void ttb_precond(lrfg_ctx* ctx, const TTBatchView& x, const std::vector<double>& t, const std::vector<double>& w,
+void ttb_precond(lrfg_ctx* ctx, const TTBatchView& x, const std::vector<double>& ts, const std::vector<double>& w,
                  int rmax, TTBatch& out, double tol, const TTView* omega, bool fp32, bool final) {
   const int d = x.d, nb = x.nb;
-  const int R = (int)t.size();
-  // the blocks G_m x_j of every item in one launch per carriage: terms[j][m][item] (a x N x b each)
+  const int R = (int)ts.size();
   std::vector<double> ones(R, 1.0);
-  SketchSource z;
-  z.kind = SketchSource::BLOCKS;
-  z.d = d;
-  z.nb = nb;
-  z.nblocks = R;
-  DBuf<double> terms[3];
-  for (int j = 0; j < d; ++j) {
-    z.N[j] = x.N[j];
+  int rk[4];
+  for (int j = 0; j <= d; ++j) rk[j] = (j == 0 || j == d) ? 1 : R * x.r[j];
+  // the blocks G_m x_j of items b0 .. b0 + g - 1 in one launch: [m][item] (a x N x b each)
+  auto blocks = [&](int j, int b0, int g) {
     const size_t e = x.elems(j);
-    terms[j] = DBuf<double>(ctx->pool, e * nb * R);
-    fibre_gauss_multi(ctx, x.core[j], terms[j].get(), (long long)(e * nb), (long long)x.r[j] * nb, x.N[j], x.r[j + 1],
-                      t.data(), (j == 0) ? w.data() : ones.data(), R, fp32);
-    z.blocks[j] = terms[j].get();
-    z.bstride[j] = (long long)(e * nb);
-  }
-  for (int j = 0; j <= d; ++j) {
-    z.s[j] = (j == 0 || j == d) ? 1 : R * x.r[j];
-    z.ry[j] = x.r[j];
-  }
+    DBuf<double> t(ctx->pool, e * g * R);
+    fibre_gauss_multi(ctx, x.core[j] + b0 * e, t.get(), (long long)(e * g), (long long)x.r[j] * g, x.N[j], x.r[j + 1],
+                      ts.data(), (j == 0) ? w.data() : ones.data(), R, fp32);
+    return t;
+  };
   if (omega) {
     // the blocks enter the sketch contractions as they are (never embedded in the block-diagonal carriage)
+    SketchSource z;
+    z.kind = SketchSource::BLOCKS;
+    z.d = d;
+    z.nb = nb;
+    z.nblocks = R;
+    DBuf<double> terms[3];
+    for (int j = 0; j < d; ++j) {
+      z.N[j] = x.N[j];
+      terms[j] = blocks(j, 0, nb);
+      z.blocks[j] = terms[j].get();
+      z.bstride[j] = (long long)(x.elems(j) * nb);
+    }
+    for (int j = 0; j <= d; ++j) {
+      z.s[j] = rk[j];
+      z.ry[j] = x.r[j];
+    }
     tt_round_sketch(ctx, z, *omega, rmax, out, tol, fp32, final);
     return;
   }
   // deterministic rounding: the carriages are block rows (first), block diagonal (middle) and block columns (last) over
   // m.  The items of a batch are rounded together (their eigenproblems and factors run on an SM each), in groups whose
-  // block-diagonal carriages stay below 1 GB; with a pool budget one at a time, the least memory the product takes.
+  // block-diagonal carriages stay below 1 GB; with a pool budget, or where the device has no room for a group, one at a time,
+  // with one carriage's blocks at a time: the least memory the product takes.
   long long item_elems = 0;
-  for (int j = 0; j < d; ++j) item_elems += (long long)z.s[j] * x.N[j] * z.s[j + 1];
-  const int group = ctx->pool->budget() ? 1 : (int)std::max(1LL, std::min<long long>(nb, (1LL << 27) / item_elems));
-  std::vector<TTBatch> parts;
-  for (int b0 = 0; b0 < nb; b0 += group) {
-    const int g = std::min(group, nb - b0);
-    TTBatch big, part;
-    ttb_alloc(ctx, big, d, x.N, z.s, g);
-    for (int j = 0; j < d; ++j)
-      stack_blocks(ctx, terms[j].get() + (size_t)b0 * x.elems(j), (long long)(x.elems(j) * nb), x.r[j], x.N[j], x.r[j + 1],
-                   R, j == 0 ? 0 : (j == d - 1 ? 2 : 1), g, big.core[j].get());
+  for (int j = 0; j < d; ++j) item_elems += (long long)rk[j] * x.N[j] * rk[j + 1];
+  int group = ctx->pool->budget() ? 1 : (int)std::max(1LL, std::min<long long>(nb, (1LL << 27) / item_elems));
+  auto round_items = [&](int b0, int g, TTBatch& part) {
+    TTBatch big;
+    ttb_alloc(ctx, big, d, x.N, rk, g);
+    for (int j = 0; j < d; ++j) {
+      const DBuf<double> t = blocks(j, b0, g);
+      stack_blocks(ctx, t.get(), (long long)(x.elems(j) * g), x.r[j], x.N[j], x.r[j + 1], R,
+                   j == 0 ? 0 : (j == d - 1 ? 2 : 1), g, big.core[j].get());
+    }
     tt_round_batch(ctx, batch_view(big), rmax, part, tol);
+  };
+  std::vector<TTBatch> parts;
+  for (int b0 = 0; b0 < nb;) {
+    const int g = std::min(group, nb - b0);
+    TTBatch part;
+    try {
+      round_items(b0, g, part);
+    } catch (const Error& err) {
+      if (err.status != LRFG_ENOMEM || g == 1) throw;
+      group = 1;
+      continue;
+    }
     if (g == nb) {
       out = std::move(part);
       return;
     }
     parts.push_back(std::move(part));
+    b0 += g;
   }
   LRFG_REQUIRE(tol == 0.0, "tolerance truncation of a batch in groups");
   ttb_alloc(ctx, out, d, x.N, parts[0].r, nb);
