@@ -315,8 +315,9 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   if (tile == 32 && active_tiles(32) * std::max(1, K / GK) < nsm) tile = 16;
   const long long active = active_tiles(tile);
   // Split long K so that the busiest SM has the fewest k-steps: a block of c k-steps, active * ceil(steps / c) blocks, and
-  // a round of blocks costs c steps plus about one for its first loads and its partial sums.  At most four blocks per SM, two
-  // in a context whose pool has a budget (the partial sums' space).
+  // a round of blocks costs c steps plus about one for its first loads and its partial sums.  At most four blocks per SM; in a
+  // context whose pool has a budget two, the tiles above the diagonal of a symmetric product counted as well (the partial
+  // sums have the space of all of them), and no split of less than a whole k-step.
   // once: a product no lockstep batch repeats, so that its order of summation is free (a solve alone and in lockstep takes the
   // same steps to 1e-9 only where both split alike).  Several blocks an SM even out to the average tile, `filled` of its
   // outputs, and a lone block's loads are not covered by another's arithmetic (about a third of a step each): the 135 x 135 x
@@ -329,9 +330,12 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
     double best = 0.0;
     const bool tight = ctx->pool->budget() != 0;
     const long long most = (tight ? 2LL : 4LL) * nsm;
-    for (int c = (int)std::max(1LL, std::min<long long>(steps, active * steps / most)); c <= steps; ++c) {
-      const long long blocks = active * ((steps + c - 1) / c);
-      if (tight && blocks > most) continue;
+    const long long all = (long long)((M + tile - 1) / tile) * ((N + tile - 1) / tile) * batch;
+    const long long stored = tight ? std::max(active, dyn ? all / 4 : all) : active;
+    for (int c = (int)std::max(1LL, std::min<long long>(steps, stored * steps / most)); c <= steps; ++c) {
+      const int parts = (steps + c - 1) / c;
+      const long long blocks = active * parts;
+      if (tight && (stored * parts > most || parts > std::max(1, K / GK))) continue;
       const double q = (double)((blocks + nsm - 1) / nsm);
       const double cost = (filled * q + (1.0 - filled)) * c + (q < 2.0 && once ? 0.35 * c : 0.0) + q;
       if (best == 0.0 || cost < best) {

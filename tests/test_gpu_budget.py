@@ -24,3 +24,23 @@ def _check(ctx, budget, call):
 def test_precond(ctx, shape, ranks, eps, rmax, budget):
     x = random_tt(shape, ranks, seed=1)
     _check(ctx, budget, lambda c: c.tt_precond(lrfg.TTensor.from_numpy(x), eps, rmax))
+
+
+def test_compress(ctx):
+    a = torch.as_tensor(lognormal_grf(3, 81, seed=5), device="cuda")
+    _check(ctx, 10_900_000, lambda c: c.tt_compress(a, 10))
+
+
+def test_solve(ctx):
+    cores = ctx.tt_compress(torch.as_tensor(lognormal_grf(3, 27, seed=5), device="cuda"), 4).cores
+
+    def solve(c):
+        P = c.problem(lrfg.TTensor([x.clone() for x in cores]), lrfg.TT, rank=5, tol=1e-12, maxit=2, stop_on_increase=False)
+        return P.solve([1.0, 0.0, 0.0], want_field=False)[0].Aeff
+
+    small = lrfg.Context(0, budget=2_530_000)
+    try:
+        got = solve(small)
+    finally:
+        small.close()
+    assert abs(got - solve(ctx)) <= 1e-9 * got
