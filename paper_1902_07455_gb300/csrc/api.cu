@@ -87,12 +87,8 @@ void* DevicePool::alloc(size_t bytes) {
   return p;
 }
 
-bool DevicePool::room(int count, size_t bytes) const {
-  if (!budget_) return true;
-  const size_t sz = rounded(bytes);
-  const auto it = sized_.find(sz);
-  const size_t have = it == sized_.end() ? 0 : it->second.size();
-  return have >= (size_t)count || reserved_ + ((size_t)count - have) * sz <= budget_;
+bool DevicePool::fits(int count, size_t bytes) const {
+  return !budget_ || in_use_ + (size_t)count * rounded(bytes) <= budget_;
 }
 
 void DevicePool::release(void* p) {
@@ -200,6 +196,7 @@ struct lrfg_problem {
   FullGrid g{};
   DBuf<double2> wc;          // FULL workspace: one half spectrum
   DBuf<double> wr;           // FULL workspace: one real grid
+  bool shared = false;       // FULL: the operator takes the passes its components share, see full_apply
   DBuf<double> inv64;        // FULL: reciprocal tables of k.k (the grid g points at them)
   DBuf<float> inv32;
   // LRFG_MIXED (FULL only): FP32 copies of the coefficient and FP32 workspaces
@@ -787,19 +784,23 @@ void full_apply(lrfg_problem* P, const typename CplxOf<R>::T* v, typename CplxOf
   const FullGrid& g = P->g;
   FullWork<R> w(P);
   const double inv = 1.0 / (double)g.n_real;
-  // the shared passes need two more half spectra; under a pool budget that has no room for them the components run one
-  // by one
+  // The shared passes need two more half spectra.  Whether a problem takes them is decided when it is made, from its grid,
+  // the pool's budget and the blocks then handed out, so that its applications round alike whatever else the pool has
+  // held; where the memory turns out to be missing, they run component by component from then on.
   using V = typename CplxOf<R>::T;
-  if (g.d == 3 && ctx->pool->room(2, sizeof(V) * g.n_half)) {
-    DBuf<V> w1(ctx->pool, g.n_half), w2(ctx->pool, g.n_half);
-    full_operator_3d<R>(ctx, g, v, out, w.a, inv, precond && !P->aniso, w.wc, w1.get(), w2.get());
-    if (P->aniso) half_acc_aniso(ctx, g, v, out, P->B, precond);
-    return;
-  }
-  if constexpr (std::is_same<R, double>::value) {
-    if (g.d == 2 && fft_pair_2d_fits(ctx, g.N[0]) && ctx->pool->room(1, 2 * sizeof(V) * g.n_half)) {
-      DBuf<V> w1(ctx->pool, 2 * g.n_half);
-      full_operator_2d(ctx, g, v, out, w.a, inv, precond && !P->aniso, w1.get());
+  if (P->shared) {
+    DBuf<V> w1, w2;
+    try {
+      w1 = DBuf<V>(ctx->pool, g.d == 3 ? g.n_half : 2 * g.n_half);
+      if (g.d == 3) w2 = DBuf<V>(ctx->pool, g.n_half);
+    } catch (const Error& e) {
+      if (e.status != LRFG_ENOMEM) throw;
+      P->shared = false;
+    }
+    if (P->shared) {
+      if (g.d == 3) full_operator_3d<R>(ctx, g, v, out, w.a, inv, precond && !P->aniso, w.wc, w1.get(), w2.get());
+      else if constexpr (std::is_same<R, double>::value)
+        full_operator_2d(ctx, g, v, out, w.a, inv, precond && !P->aniso, w1.get());
       if (P->aniso) half_acc_aniso(ctx, g, v, out, P->B, precond);
       return;
     }
@@ -1900,6 +1901,10 @@ lrfg_status lrfg_problem_create(lrfg_ctx* ctx, const lrfg_coeff* coeff, const lr
         P->wcf = DBuf<float2>(ctx->pool, P->g.n_half);
         P->wrf = DBuf<float>(ctx->pool, P->g.n_real);
       }
+      // the shared passes' two half spectra beside a solve's four vectors (d = 2: FP64, both components in a launch)
+      const bool mixed = P->opts.prec == LRFG_MIXED;
+      P->shared = !P->ga && (P->d == 3 || (!mixed && fft_pair_2d_fits(ctx, P->N[0]))) &&
+                  ctx->pool->fits(6, (mixed ? sizeof(float2) : sizeof(double2)) * P->g.n_half);
     } else {
       double xmax = 0.0;
       for (int j = 0; j < P->d; ++j) xmax += (double)((P->N[j] - 1) / 2) * ((P->N[j] - 1) / 2);

@@ -58,8 +58,8 @@ class DevicePool {
   void release(void* p);
   void trim();
   size_t budget() const { return budget_; }
-  // whether `count` blocks of `bytes` fit without passing the budget (or returning cached blocks to the driver)
-  bool room(int count, size_t bytes) const;
+  // whether `count` blocks of `bytes` fit the budget beside the blocks handed out (cached ones can go back to the driver)
+  bool fits(int count, size_t bytes) const;
   size_t in_use() const { return in_use_; }
   size_t reserved() const { return reserved_; }
   // high-water mark of in_use() since the last reset_peak()
