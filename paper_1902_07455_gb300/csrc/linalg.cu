@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
     acc[j] = (T)0;
   }
   // the next k-step's operands are on their way to registers while this one's are multiplied (135 x 135 x 18225 Gram product
-  // 404 -> 334 us, the small products of an application 5-15% shorter)
+  // 404 -> 334 us, the small products of an application 5-15% shorter).  The 64 x 64 FP64 kernels take 229-240 registers with
+  // them in four of their six forms, one block an SM; the 32 x 32 ones at most 112, two or more.
   constexpr int NL = TILE * GK / 256;
   T ra[NL], rb[NL];
   auto fetch = [&](int k0) {
@@ -319,10 +320,11 @@ static void gemm_impl(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K
   // context whose pool has a budget two, the tiles above the diagonal of a symmetric product counted as well (the partial
   // sums have the space of all of them), and no split of less than a whole k-step.
   // once: a product no lockstep batch repeats, so that its order of summation is free (a solve alone and in lockstep takes the
-  // same steps to 1e-9 only where both split alike).  Several blocks an SM even out to the average tile, `filled` of its
-  // outputs, and a lone block's loads are not covered by another's arithmetic (about a third of a step each): the 135 x 135 x
-  // 18225 Gram product of a compression, a third of whose tiles' outputs are padding, took 966 us in one block per SM and
-  // takes 404 us in four.
+  // same steps to 1e-9 only where both split alike).  Several blocks an SM, side by side or in turn, even out to the average
+  // tile, `filled` of its outputs, and a lone block's first loads and last sums are covered by nothing (about a third of a
+  // step each).  Limited to one / two / four blocks an SM, a compression of 135^3 values, whose 135 x 135 x 18225 Gram product is a
+  // third padding, takes 4.09 / 3.63 / 3.49 ms, the lockstep tensor at 81^3 28.4 / 27.2 / 27.1 ms, the other roundings the same
+  // within 1%.
   const int steps = (K + GK - 1) / GK;
   const double filled = dyn || !once ? 1.0 : (sym ? 0.5 * M * (M + 1.0) : (double)M * N) * batch / ((double)tiles_of(tile) * tile * tile);
   int per = steps;
