@@ -1,5 +1,5 @@
 // Dense FP64 building blocks for the rank truncation and the solvers: batched GEMM (Gram matrices and
-// core contractions) and reductions.
+// core contractions), a cyclic Jacobi eigensolver and reductions.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -425,6 +425,254 @@ void gemm_nosplit(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, do
   else
     launch_dgemm<64, double>(ctx, transA, transB, grid, flops, bytes, M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C,
                              ldc, sC, 1, kchunk, nullptr, 1, nullptr, 1, nullptr, nullptr);
+}
+
+// ------------------------------------------------------------------------------------------------
+// Symmetric eigensolver by cyclic two-sided Jacobi rotations with the round-robin (circle) ordering, so that each round applies
+// m'/2 disjoint rotations in parallel (Golub & Van Loan, "Matrix Computations", 4th ed., Sec. 8.5: the 2 x 2 symmetric Schur
+// step and parallel orderings).  One block per matrix, working matrices in shared memory when they fit, else in a global
+// scratch slice.  Its errors on small eigenvalues are a tenth of eps64 ||A||, the level of the rounding of a Gram matrix
+// itself, where the tridiagonal solver's are eps64 ||A||: compressions that reach that level take it (see tt_compress).
+// 46 ms for one matrix of 135 rows, against 1.45 ms for ten eigenpairs by the tridiagonal solver.
+// syevj_floor is launched behind the tridiagonal solver and reads its eigenvalues on the device: the host, which has the
+// compression's other launches to queue meanwhile, does not wait for them (80 us of a 3.5 ms compression).
+// ------------------------------------------------------------------------------------------------
+constexpr int kJacobiMaxSweeps = 30;
+constexpr int kJacobiThreads = 512;
+
+__device__ __forceinline__ void rr_pair(int round, int i, int mp, int* p, int* q) {
+  // circle method: player mp-1 fixed, the others rotate
+  const int n1 = mp - 1;
+  if (i == 0) { *p = round % n1; *q = n1; return; }
+  *p = (round + i) % n1;
+  *q = (round - i + n1) % n1;
+}
+
+__device__ __forceinline__ double block_total(double v, double* red) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffff, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0;
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
+  return s;
+}
+
+// power of two that brings the largest entry (bits of its upper word, over the block) near 1; red: 32 ints
+__device__ double pow2_near_one(int hi_abs, int* red) {
+  const int m = __reduce_max_sync(0xffffffff, hi_abs);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  int b = 0;
+  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) b = max(b, red[q]);
+  const int ex = b >> 20;
+  return ex == 0 || ex == 0x7ff ? 1.0 : __hiloint2double(min(2046, max(1, 2046 - ex)) << 20, 0);
+}
+
+// whether k eigenvalues w of a Gram matrix reach down to its rounding
+__device__ __forceinline__ bool at_floor(const double* w, int k) { return w[k - 1] < 64.0 * 2.220446049250313e-16 * w[0]; }
+
+// Four combinations of the columns (of_rows: C is m x n) or rows (n x m) of C with random signs: Y (m x 4); nothing unless the k
+// eigenvalues w reach the floor.  A warp per entry of m, or a thread.
+constexpr int kImages = 4;
+__global__ void __launch_bounds__(256) random_images_kernel(const double* __restrict__ C, int m, int n, int of_rows,
+                                                            const double* __restrict__ w, int k, double* __restrict__ Y) {
+  if (!at_floor(w, k)) return;
+  const int lane = threadIdx.x & 31, step = of_rows ? 32 : 1;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = of_rows ? t >> 5 : t;
+  if (i >= m) return;
+  double y[kImages] = {0.0, 0.0, 0.0, 0.0};
+  for (int j = of_rows ? lane : 0; j < n; j += step) {
+    const double v = of_rows ? C[(size_t)i * n + j] : C[(size_t)j * m + i];
+    const unsigned h = ((unsigned)j + 1u) * 2654435761u;
+    const unsigned bits = (h ^ (h >> 15)) * 2246822519u;
+#pragma unroll
+    for (int l = 0; l < kImages; ++l) y[l] += (bits >> (28 + l) & 1u) ? v : -v;
+  }
+#pragma unroll
+  for (int l = 0; l < kImages; ++l) {
+    if (of_rows)
+      for (int o = 16; o; o >>= 1) y[l] += __shfl_xor_sync(0xffffffff, y[l], o);
+    if (!of_rows || lane == 0) Y[(size_t)i * kImages + l] = y[l];
+  }
+}
+
+// k > 0: only where the first k of the eigenvalues w, known already, reach the floor, and the k vectors known (in Vout) leave more
+// than 1e-13 of the images Y
+__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double* __restrict__ Ag, double* w,
+                                                               double* Vout, int m, double* scratch, int use_smem,
+                                                               double eps, int k, const double* __restrict__ Y) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int mp = m + (m & 1);
+  const int npair = mp / 2;
+  double* cs = (double*)smraw;                         // 2 npair (c, s)
+  int* pq = (int*)(cs + 2 * npair);                    // 2 npair
+  double* red = (double*)(pq + 2 * npair);             // 32 partial sums
+  int* rank = (int*)(red + 32);                        // m (+1) ints
+  double* A;
+  double* V;
+  if (use_smem == 2) {         // A and V in shared memory
+    A = (double*)(rank + m + (m & 1));
+    V = A + (size_t)m * m;
+  } else if (use_smem == 1) {  // A in shared memory, V in a global scratch slice
+    A = (double*)(rank + m + (m & 1));
+    V = scratch + (size_t)blockIdx.x * m * m;
+  } else {
+    A = scratch + (size_t)blockIdx.x * 2 * m * m;
+    V = A + (size_t)m * m;
+  }
+  if (k > 0) {
+    if (!at_floor(w, k)) return;
+    double* T = A;  // k x 4
+    for (int q = threadIdx.x; q < k * kImages; q += blockDim.x) {
+      const int t = q % k, l = q / k;
+      double s = 0.0;
+      for (int i = 0; i < m; ++i) s = fma(Vout[(size_t)i * m + t], Y[(size_t)i * kImages + l], s);
+      T[q] = s;
+    }
+    __syncthreads();
+    double all = 0.0, left = 0.0;
+    for (int q = threadIdx.x; q < m * kImages; q += blockDim.x) {
+      const int i = q / kImages, l = q % kImages;
+      double r = Y[q];
+      all = fma(r, r, all);
+      for (int t = 0; t < k; ++t) r = fma(-Vout[(size_t)i * m + t], T[l * k + t], r);
+      left = fma(r, r, left);
+    }
+    all = block_total(all, red);
+    left = block_total(left, red);
+    if (left <= 1e-26 * all) return;
+    __syncthreads();
+  }
+  const double* Ain = Ag + (size_t)blockIdx.x * m * m;
+  // scaled by a power of two to entries near 1, so that the squares stay in range
+  int top = 0;
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    A[t] = Ain[t];
+    V[t] = ((t / m) == (t % m)) ? 1.0 : 0.0;
+    top = max(top, __double2hiint(A[t]) & 0x7fffffff);
+  }
+  const double scale = pow2_near_one(top, (int*)red);
+  double loc = 0.0;
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    A[t] *= scale;
+    loc += A[t] * A[t];
+  }
+  const double fro2 = block_total(loc, red);
+  const double tol2 = 16.0 * eps * eps * fro2;
+  double prev_off = fro2;
+  if (m > 1 && fro2 > 0.0) {
+    for (int sweep = 0; sweep < kJacobiMaxSweeps; ++sweep) {
+      for (int round = 0; round < mp - 1; ++round) {
+        for (int i = threadIdx.x; i < npair; i += blockDim.x) {
+          int p, q;
+          rr_pair(round, i, mp, &p, &q);
+          if (p > q) { int t = p; p = q; q = t; }
+          double c = 1, s = 0;
+          if (q < m) {
+            double apq = A[(size_t)p * m + q];
+            double app = A[(size_t)p * m + p], aqq = A[(size_t)q * m + q];
+            if (apq != 0.0 && fabs(apq) > 0.01 * eps * sqrt(fabs(app * aqq))) {
+              double tau = (aqq - app) / (2.0 * apq);
+              double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+              c = 1.0 / sqrt(1.0 + t * t);
+              s = t * c;
+            }
+          } else {
+            q = -1;
+          }
+          cs[2 * i] = c;
+          cs[2 * i + 1] = s;
+          pq[2 * i] = p;
+          pq[2 * i + 1] = (s == 0.0) ? -1 : q;
+        }
+        __syncthreads();
+        // rows: A <- J^T A
+        for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {
+          int i = t / m, j = t - (t / m) * m;
+          int q = pq[2 * i + 1];
+          if (q < 0) continue;
+          int p = pq[2 * i];
+          double c = cs[2 * i], s = cs[2 * i + 1];
+          double ap = A[(size_t)p * m + j], aq = A[(size_t)q * m + j];
+          A[(size_t)p * m + j] = c * ap - s * aq;
+          A[(size_t)q * m + j] = s * ap + c * aq;
+        }
+        __syncthreads();
+        // columns: A <- A J, V <- V J
+        for (int t = threadIdx.x; t < npair * m; t += blockDim.x) {
+          int i = t / m, j = t - (t / m) * m;
+          int q = pq[2 * i + 1];
+          if (q < 0) continue;
+          int p = pq[2 * i];
+          double c = cs[2 * i], s = cs[2 * i + 1];
+          double ap = A[(size_t)j * m + p], aq = A[(size_t)j * m + q];
+          A[(size_t)j * m + p] = c * ap - s * aq;
+          A[(size_t)j * m + q] = s * ap + c * aq;
+          double vp = V[(size_t)j * m + p], vq = V[(size_t)j * m + q];
+          V[(size_t)j * m + p] = c * vp - s * vq;
+          V[(size_t)j * m + q] = s * vp + c * vq;
+        }
+        __syncthreads();
+      }
+      double off = 0;
+      for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+        int i = t / m, j = t - (t / m) * m;
+        if (i != j) off += A[t] * A[t];
+      }
+      off = block_total(off, red);
+      // converged, or rounding has stopped the decrease (off-diagonal mass at the precision floor)
+      if (off <= tol2 || (off > 0.25 * prev_off && off <= 4096.0 * eps * eps * fro2)) break;
+      prev_off = off;
+    }
+  }
+  // sort descending: rank[j] = position of eigenvalue j (ties by index)
+  for (int j = threadIdx.x; j < m; j += blockDim.x) {
+    double lj = A[(size_t)j * m + j];
+    int pos = 0;
+    for (int i = 0; i < m; ++i) {
+      double li = A[(size_t)i * m + i];
+      if (li > lj || (li == lj && i < j)) ++pos;
+    }
+    rank[j] = pos;
+  }
+  __syncthreads();
+  double* wb = w + (size_t)blockIdx.x * m;
+  double* Vb = Vout + (size_t)blockIdx.x * m * m;
+  for (int j = threadIdx.x; j < m; j += blockDim.x) wb[rank[j]] = A[(size_t)j * m + j] / scale;
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    int i = t / m, j = t - (t / m) * m;
+    Vb[(size_t)i * m + rank[j]] = V[t];
+  }
+}
+
+static void jacobi_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch, int k, const double* Y) {
+  const int npair = (m + 1) / 2;
+  size_t head = sizeof(double) * 2 * npair + sizeof(int) * 2 * npair + sizeof(double) * 32 + sizeof(int) * (m + (m & 1));
+  head = (head + 15) / 16 * 16;
+  const size_t limit = (size_t)std::min(ctx->max_smem_optin, 220 * 1024);
+  const size_t one = head + sizeof(double) * (size_t)m * std::max(m, kImages), two = one + sizeof(double) * (size_t)m * m;
+  const int use_smem = two <= limit ? 2 : (one <= limit ? 1 : 0);
+  const size_t smem = use_smem == 2 ? two : (use_smem == 1 ? one : head);
+  DBuf<double> scratch;
+  if (use_smem < 2) scratch = DBuf<double>(ctx->pool, (size_t)(2 - use_smem) * m * m * batch);
+  LRFG_CUDA(raise_smem_limit((const void*)jacobi_kernel, smem));
+  // one sweep of the two-sided cyclic Jacobi costs about 9 m^3 flops (rows, columns and V)
+  LRFG_LAUNCH(ctx, KC_EIGEN, k > 0 ? 0.0 : 9.0 * (double)m * m * m * batch, k > 0 ? 0.0 : 3.0 * sizeof(double) * (double)m * m * batch,
+              jacobi_kernel<<<batch, kJacobiThreads, smem, ctx->stream>>>(A, w, V, m, scratch.get(), use_smem,
+                                                                         2.220446049250313e-16, k, Y));
+}
+
+void syevj(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch) {
+  if (m <= 0 || batch <= 0) return;
+  jacobi_launch(ctx, A, w, V, m, batch, 0, nullptr);
+}
+
+void syevj_floor(lrfg_ctx* ctx, const double* G, double* w, double* V, int m, int k, const double* C, int n, bool of_rows) {
+  DBuf<double> Y(ctx->pool, (size_t)m * kImages);
+  const int blocks = of_rows ? (m + 7) / 8 : (m + 255) / 256;
+  LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0, random_images_kernel<<<blocks, 256, 0, ctx->stream>>>(C, m, n, of_rows, w, k, Y.get()));
+  jacobi_launch(ctx, G, w, V, m, 1, k, Y.get());
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -94,7 +94,13 @@ void gemm_nosplit(lrfg_ctx* ctx, int transA, int transB, int M, int N, int K, do
 // FP64 k largest eigenpairs by tridiagonalisation, bisection and inverse iteration: w[0..k) descending,
 // eigenvectors in the first k columns of V (n x n row-major per batch item).  A is left unchanged.
 void syevx(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int batch = 1);
-// the same with kv >= k eigenvalues in w
+// symmetric eigen-decomposition of `batch` m x m matrices (row-major, stride m*m) by Jacobi rotations: all eigenvalues in
+// descending order into w (stride m), eigenvectors as the columns of V.  A is left unchanged.
+void syevj(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch = 1);
+// The same over the k eigenpairs (w, V) that syevx found of the Gram matrix G (m x m) of C (m x n, or of_rows false: n x m), where
+// their eigenvalues reach the rounding of G and the vectors do not span C to rounding; else nothing.  Decided on the device.
+void syevj_floor(lrfg_ctx* ctx, const double* G, double* w, double* V, int m, int k, const double* C, int n, bool of_rows);
+// syevx with kv >= k eigenvalues in w
 void syevx_values(lrfg_ctx* ctx, const double* A, double* w, double* V, int n, int k, int kv, int batch);
 // The same on the leading n_eff[b] x n_eff[b] block of A (the rest of A is zero); the eigenvector
 // rows beyond n_eff and the columns beyond min(k, n_eff) are zero.

@@ -723,12 +723,22 @@ void tt_compress(lrfg_ctx* ctx, int d, const int* N, const double* values, int r
       gemm_sym(ctx, 0, m, (int)cols, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0, 1, nullptr, true);
     else
       gemm_sym(ctx, 1, m, rows, C.get(), (int)cols, 0, C.get(), (int)cols, 0, G.get(), m, 0, 1, nullptr, true);
-    // only the kept eigenpairs are decomposed (with a tolerance, every eigenvalue: the rule sums the tail): a cyclic
-    // Jacobi of the whole m x m Gram matrix in one block took 46 ms per bond at m = 135, this 2.3 ms; a compression of
-    // 135^3 values to rank 10 with its expansion went from 98.3 to 5.8 ms
+    // Only the kept eigenpairs are decomposed (with a tolerance, every eigenvalue: the rule sums the tail): a cyclic
+    // Jacobi of the whole m x m Gram matrix in one block takes 46 ms per bond at m = 135, this 1.45 ms; a compression of
+    // 135^3 values to rank 10 with its expansion went from 98.3 to 3.5 ms.  Its eigenvalues are good to eps ||G||, Jacobi's to
+    // the rounding of G, a tenth of that: ranks or tolerances that reach so far down (errors of the values below some
+    // 1e-7 of their norm) are left to Jacobi, unless the kept vectors hold the values to rounding already.
     const int kmax = std::min(rmax, m), kv = tol_j > 0.0 ? m : kmax;
-    syevx_values(ctx, G.get(), lam.get(), V.get(), m, kmax, kv, 1);
+    const double eps = 2.220446049250313e-16;
     int k = kmax;
+    // (the tail's eigenvalues carry some eps ||G|| / 4 each)
+    if (tol_j > 0.0 && tol_j * tol_j < 8.0 * m * eps) {
+      syevj(ctx, G.get(), lam.get(), V.get(), m);
+    } else {
+      syevx_values(ctx, G.get(), lam.get(), V.get(), m, kmax, kv, 1);
+      if (tol_j == 0.0 && k < m)
+        syevj_floor(ctx, G.get(), lam.get(), V.get(), m, k, C.get(), use_rows ? (int)cols : rows, use_rows);
+    }
     if (tol_j > 0.0) {
       std::vector<double> hl(m);
       LRFG_CUDA(cudaMemcpyAsync(hl.data(), lam.get(), sizeof(double) * m, cudaMemcpyDeviceToHost, ctx->stream));
