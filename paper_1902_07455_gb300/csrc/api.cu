@@ -943,7 +943,7 @@ void solve_full(lrfg_problem* P, const double* E, lrfg_result* res, lrfg_field**
   half_precond(ctx, g, (const V*)r.get(), p.get());
   half_dot(ctx, g, (const V*)r.get(), (const V*)p.get(), d_rz);
   half_dot(ctx, g, (const V*)p.get(), (const V*)p.get(), d_zz);
-  double* zz = ctx->host_scalars;
+  double* zz = ctx->host_scalar;
   auto read_zz = [&]() { LRFG_CUDA(cudaMemcpyAsync(zz, d_zz, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream)); };
   read_zz();
   LRFG_CUDA(cudaStreamSynchronize(ctx->stream));
@@ -957,7 +957,7 @@ void solve_full(lrfg_problem* P, const double* E, lrfg_result* res, lrfg_field**
   const bool ahead = n < (1LL << 20);
   auto step_product = [&]() {
     full_apply<R>(P, p.get(), q.get(), 0);
-    half_dot(ctx, g, (const V*)p.get(), (const V*)q.get(), d_pq, d_rz, d_alpha, 1);  // alpha = rz / pq
+    half_dot(ctx, g, (const V*)p.get(), (const V*)q.get(), d_pq, d_rz, d_alpha);  // alpha = rz / pq
   };
   if (nb > 0.0 && P->opts.maxit > 0) step_product();
   while (nb > 0.0 && it < P->opts.maxit) {
@@ -1483,7 +1483,7 @@ lrfg_status lrfg_create(lrfg_ctx** out, int device, void* stream, size_t budget)
     LRFG_CUDA(cudaMalloc(&ctx->work_dev, sizeof(double) * 2 * KC_COUNT));
     LRFG_CUDA(cudaMemsetAsync(ctx->work_dev, 0, sizeof(double) * 2 * KC_COUNT, ctx->stream));
     const size_t ncnt = (size_t)kSplitKCounters * (1 + kSplitKGroups);
-    LRFG_CUDA(cudaMallocHost(&ctx->host_scalars, sizeof(double) * kHostScalars));
+    LRFG_CUDA(cudaMallocHost(&ctx->host_scalar, sizeof(double)));
     LRFG_CUDA(cudaEventCreateWithFlags(&ctx->host_ready, cudaEventDisableTiming));
     LRFG_CUDA(cudaMalloc(&ctx->splitk_cnt, sizeof(unsigned int) * ncnt));
     LRFG_CUDA(cudaMemsetAsync(ctx->splitk_cnt, 0, sizeof(unsigned int) * ncnt, ctx->stream));
@@ -1508,7 +1508,7 @@ lrfg_status lrfg_destroy(lrfg_ctx* ctx) {
   delete ctx->pool;
   if (ctx->work_dev) cudaFree(ctx->work_dev);
   if (ctx->splitk_cnt) cudaFree(ctx->splitk_cnt);
-  if (ctx->host_scalars) cudaFreeHost(ctx->host_scalars);
+  if (ctx->host_scalar) cudaFreeHost(ctx->host_scalar);
   if (ctx->host_ready) cudaEventDestroy(ctx->host_ready);
   for (auto& kv : ctx->twiddles) {
     cudaFree(kv.second.W);

@@ -182,8 +182,8 @@ struct lrfg_ctx {
   double* work_dev = nullptr;
   // split-K arrival counters, one per output tile of a split product (all zero between launches)
   unsigned int* splitk_cnt = nullptr;
-  // page-locked scalars the solvers read back, and the event that says they have arrived
-  double* host_scalars = nullptr;
+  // the page-locked scalar that the full-format solver reads back, and the event that says it has arrived
+  double* host_scalar = nullptr;
   cudaEvent_t host_ready = nullptr;
 };
 
@@ -222,7 +222,6 @@ class KTimer {
   cudaEvent_t start_ = nullptr;
 };
 
-constexpr int kHostScalars = 64;
 // capacity of the split-K arrival counters (a split product has fewer than 4 x 2 x 152 output tiles), and
 // of the group counters of the two-level reduction (at most kSplitKGroups groups per tile), stored after them
 constexpr int kSplitKCounters = 4096;

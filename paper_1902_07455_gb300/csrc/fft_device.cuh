@@ -30,7 +30,7 @@ constexpr int kMaxGenericRadix = 31;
 // roots of unity exp(-2 pi i j / p) of the register radices, concatenated (filled once per device)
 constexpr int kRootOff3 = 0, kRootOff5 = 3, kRootOff7 = 8, kRootOff9 = 15, kRootOff27 = 24, kRootCount = 51;
 __constant__ float2 c_roots_f[kRootCount];
-__constant__ int4 c_roots_x[kRootCount];  // fixed point (fft_fixed.cuh)
+__constant__ int4 c_roots_x[kRootOff27];  // fixed point (fft_fixed.cuh), radices up to 9
 
 // exp(-2 pi i j / p) in fixed point: cos 2^62 and -sin 2^62 (1 as 1 - 2^-62), each as an upper part times 2^31 and a lower
 // one between -2^30 and 2^30 (2^31 - 1 for 1 itself, whose other component is 0): with both signs the lower parts leave
@@ -52,14 +52,14 @@ static inline cudaError_t ensure_roots(int device) {
   std::lock_guard<std::mutex> lock(mu);
   if (device >= 0 && device < 64 && (done >> device & 1ULL)) return cudaSuccess;
   float2 hf[kRootCount];
-  int4 hx[kRootCount];
+  int4 hx[kRootOff27];
   const int radix[5] = {3, 5, 7, 9, 27}, off[5] = {kRootOff3, kRootOff5, kRootOff7, kRootOff9, kRootOff27};
   const double two_pi = 6.283185307179586476925286766559;
   for (int q = 0; q < 5; ++q)
     for (int j = 0; j < radix[q]; ++j) {
       const double ang = two_pi * (double)j / (double)radix[q];
       hf[off[q] + j] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
-      hx[off[q] + j] = fixed_root(j, radix[q]);
+      if (radix[q] <= 9) hx[off[q] + j] = fixed_root(j, radix[q]);
     }
   cudaError_t e = cudaMemcpyToSymbol(c_roots_f, hf, sizeof(hf));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_roots_x, hx, sizeof(hx));

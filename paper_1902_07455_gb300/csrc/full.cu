@@ -999,12 +999,12 @@ __device__ bool last_block_sum(const double* mine, double* partial, unsigned int
   return true;
 }
 
-// *out = <x, y>; then, if ratio: mode 1 -> *ratio = *aux / *out, mode 2 -> *out / *aux (0 when the divisor is 0): the
-// PCG step lengths, formed once on the device
+// *out = <x, y>; then, if ratio, *ratio = *aux / *out (0 when the divisor is 0): the PCG step length, formed once on the
+// device
 template <typename V>
 __global__ void __launch_bounds__(256) half_dot_kernel(const V* __restrict__ x, const V* __restrict__ y, long long n,
                                                        int H, double* partial, unsigned int* counter, double* out,
-                                                       const double* aux, double* ratio, int mode) {
+                                                       const double* aux, double* ratio) {
   __shared__ double red[8];
   constexpr int kU = 4;  // elements' loads in flight before any is used
   DotAcc<V> acc;
@@ -1031,10 +1031,7 @@ __global__ void __launch_bounds__(256) half_dot_kernel(const V* __restrict__ x, 
   if (!last_block_sum<1>(mine, partial, counter, red, total)) return;
   if (threadIdx.x == 0) {
     *out = total[0];
-    if (ratio) {
-      const double num = mode == 1 ? *aux : total[0], den = mode == 1 ? total[0] : *aux;
-      *ratio = den != 0.0 ? num / den : 0.0;
-    }
+    if (ratio) *ratio = total[0] != 0.0 ? *aux / total[0] : 0.0;
   }
 }
 
@@ -1104,12 +1101,12 @@ static int red_blocks(long long n) { return (int)std::max(1LL, std::min<long lon
 
 template <typename V>
 void half_dot(lrfg_ctx* ctx, const FullGrid& g, const V* x, const V* y, double* out_dev, const double* aux,
-              double* ratio, int mode) {
+              double* ratio) {
   const int blocks = red_blocks(g.n_half);
   DBuf<double> partial(ctx->pool, kRedBlocks);
   LRFG_LAUNCH(ctx, KC_REDUCE, 4.0 * g.n_half, 2.0 * sizeof(V) * g.n_half,
               half_dot_kernel<V><<<blocks, 256, 0, ctx->stream>>>(x, y, g.n_half, g.H, partial.get(), ctx->splitk_cnt,
-                                                                 out_dev, aux, ratio, mode));
+                                                                 out_dev, aux, ratio));
 }
 
 void aniso_energy_sum(lrfg_ctx* ctx, const FullGrid& g, const double2* v, const double* B, double* out_dev,
@@ -1305,7 +1302,7 @@ void convert(lrfg_ctx* ctx, const A* in, B* out, long long n) {
   template void half_acc_div<V>(lrfg_ctx*, const FullGrid&, const V*, V*, int, double, int, int);         \
   template void half_precond<V>(lrfg_ctx*, const FullGrid&, const V*, V*);                                \
   template void half_acc_aniso<V>(lrfg_ctx*, const FullGrid&, const V*, V*, const double*, int);          \
-  template void half_dot<V>(lrfg_ctx*, const FullGrid&, const V*, const V*, double*, const double*, double*, int); \
+  template void half_dot<V>(lrfg_ctx*, const FullGrid&, const V*, const V*, double*, const double*, double*); \
   template void energy_sum<R>(lrfg_ctx*, const FullGrid&, const R*, const R*, double, double*, int);      \
   template void pcg_residual<V>(lrfg_ctx*, const FullGrid&, V*, const V*, const double*, double*, double*, double*); \
   template void pcg_direction<V>(lrfg_ctx*, const FullGrid&, V*, V*, const V*, const double*, const double*, bool);

@@ -72,10 +72,10 @@ void half_acc_aniso(lrfg_ctx* ctx, const FullGrid& g, const V* in, V* acc, const
 void aniso_energy_sum(lrfg_ctx* ctx, const FullGrid& g, const double2* v, const double* B, double* out_dev,
                       int accumulate);
 // Hermitian-weighted real inner product over the full spectrum (FP64 accumulation) into a device scalar
-// optional: *ratio = *aux / result (mode 1) or result / *aux (mode 2), 0 for a zero divisor
+// optional: *ratio = *aux / result, 0 for a zero divisor
 template <typename V>
 void half_dot(lrfg_ctx* ctx, const FullGrid& g, const V* x, const V* y, double* out_dev, const double* aux = nullptr,
-              double* ratio = nullptr, int mode = 0);
+              double* ratio = nullptr);
 // out_dev (+)= sum_k a_k (E + e_k)^2 (FP64 accumulation)
 template <typename R>
 void energy_sum(lrfg_ctx* ctx, const FullGrid& g, const R* e, const R* a, double E, double* out_dev, int accumulate);
