@@ -110,15 +110,18 @@ struct BlockSum {
   double* out[3];
 };
 
-// blockIdx.y: carriage, blockIdx.z: item
+// blockIdx.y: carriage, blockIdx.z: item.  A thread's indices advance without divisions (with 64-bit divisions for each element
+// the sum of two trains of ranks 200 and 100 at 729^3, 820 MB, took 466 us, now 380)
 __global__ void block_sum_kernel(const __grid_constant__ BlockSum t) {
   const int j = blockIdx.y, item = blockIdx.z, n = t.N[j];
   const int A = j == 0 ? 1 : t.off[j][t.m], B = j == t.d - 1 ? 1 : t.off[j + 1][t.m];
   const long long total = (long long)A * n * B;
   double* out = t.out[j] + item * total;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-    const long long rest = e / B;
-    const int ib = (int)(e - rest * B), ia = (int)(rest / n), nn = (int)(rest - (long long)ia * n);
+  long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x, row = e / B;
+  const long long step = (long long)gridDim.x * blockDim.x, step_rows = step / B;
+  int ib = (int)(e - row * B), ia = (int)(row / n), nn = (int)(row - (long long)ia * n);
+  const int db = (int)(step - step_rows * B), da = (int)(step_rows / n), dn = (int)(step_rows - (long long)da * n);
+  for (; e < total; e += step) {
     int ta = 0, tb = 0;
     if (j > 0)
       while (ia >= t.off[j][ta + 1]) ++ta;
@@ -134,6 +137,11 @@ __global__ void block_sum_kernel(const __grid_constant__ BlockSum t) {
       if (j == 0) v *= t.sd[ta] ? t.s[ta] * t.sd[ta][item] : t.s[ta];
     }
     out[e] = v;
+    ib += db;
+    nn += dn;
+    ia += da;
+    if (ib >= B) { ib -= B; ++nn; }
+    if (nn >= n) { nn -= n; ++ia; }
   }
 }
 
