@@ -30,6 +30,7 @@ constexpr int kMaxGenericRadix = 31;
 // roots of unity exp(-2 pi i j / p) of the register radices, concatenated (filled once per device)
 constexpr int kRootOff3 = 0, kRootOff5 = 3, kRootOff7 = 8, kRootOff9 = 15, kRootOff27 = 24, kRootCount = 51;
 __constant__ float2 c_roots_f[kRootCount];
+__constant__ double2 c_roots_d[kRootOff27];  // radices up to 9 (rows of one butterfly)
 __constant__ int4 c_roots_x[kRootOff27];  // fixed point (fft_fixed.cuh), radices up to 9
 
 // exp(-2 pi i j / p) in fixed point: cos 2^62 and -sin 2^62 (1 as 1 - 2^-62), each as an upper part times 2^31 and a lower
@@ -52,6 +53,7 @@ static inline cudaError_t ensure_roots(int device) {
   std::lock_guard<std::mutex> lock(mu);
   if (device >= 0 && device < 64 && (done >> device & 1ULL)) return cudaSuccess;
   float2 hf[kRootCount];
+  double2 hd[kRootOff27];
   int4 hx[kRootOff27];
   const int radix[5] = {3, 5, 7, 9, 27}, off[5] = {kRootOff3, kRootOff5, kRootOff7, kRootOff9, kRootOff27};
   const double two_pi = 6.283185307179586476925286766559;
@@ -59,9 +61,12 @@ static inline cudaError_t ensure_roots(int device) {
     for (int j = 0; j < radix[q]; ++j) {
       const double ang = two_pi * (double)j / (double)radix[q];
       hf[off[q] + j] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
-      if (radix[q] <= 9) hx[off[q] + j] = fixed_root(j, radix[q]);
+      if (radix[q] > 9) continue;
+      hd[off[q] + j] = make_double2(std::cos(ang), -std::sin(ang));
+      hx[off[q] + j] = fixed_root(j, radix[q]);
     }
   cudaError_t e = cudaMemcpyToSymbol(c_roots_f, hf, sizeof(hf));
+  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_roots_d, hd, sizeof(hd));
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_roots_x, hx, sizeof(hx));
   // complete before kernels on any stream (non-blocking ones included) read the tables
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -161,8 +166,9 @@ template <> struct RootOff<27> { static constexpr int v = kRootOff27; };
 // w_P^j (forward: exp(-2 pi i j / P), inverse: its conjugate); j a compile-time constant after unrolling
 template <int P, int SIGN, typename V>
 __device__ __forceinline__ V root(int j) {
-  static_assert(sizeof(V) == sizeof(float2), "FP32");
-  V w = c_roots_f[RootOff<P>::v + j % P];
+  V w;
+  if constexpr (sizeof(V) == sizeof(double2)) w = c_roots_d[RootOff<P>::v + j % P];
+  else w = c_roots_f[RootOff<P>::v + j % P];
   if (SIGN > 0) w.y = -w.y;
   return w;
 }

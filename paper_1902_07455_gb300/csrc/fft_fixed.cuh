@@ -16,7 +16,7 @@
 // 105 x 147 x 75 anisotropic 0.93 -> 0.60 ms, Ga at 63^3 0.86 -> 0.50 ms.  The integer pipes bound it now (60% of their
 // rate, about 580 instructions a point, 24 warps an SM); with the conversions unrolled into the butterflies instead of in
 // loops of their own a pass took 30 us more, waiting for instructions.
-// A row with an entry that is not finite becomes NaN as a whole.
+// A row with an entry that is not finite becomes NaN as a whole.  Rows of up to 9 points stay in FP64 (fp64_rows).
 #pragma once
 
 namespace lrfg {
@@ -302,6 +302,20 @@ __device__ __forceinline__ void fix_row(double2* row, int N, int first, int step
   }
 }
 
+// Rows of one butterfly in FP64, a row a thread: converting them would take longer than the transform
+// (90,000 rows of 3 points under a multiplier 35 us, in fixed point 84; of 9 points 53 and 96).
+template <int P, int SIGN>
+__device__ __noinline__ void fp64_rows(const double2* __restrict__ a, double2* __restrict__ b, int nf, int ld) {
+  for (int row = threadIdx.x; row < nf; row += blockDim.x) {
+    double2 x[P];
+#pragma unroll
+    for (int r = 0; r < P; ++r) x[r] = a[row * ld + r];
+    RegDFT<P, SIGN, double2>::run(x);
+#pragma unroll
+    for (int r = 0; r < P; ++r) b[row * ld + r] = x[r];
+  }
+}
+
 // The transform of nf rows (double2 in, double2 out): see stockham_rows.  The conversions are loops of their own: unrolled
 // into the butterflies they made the kernels wait for instructions (the largest stall of a 243-point pass).
 template <int SIGN>
@@ -311,6 +325,16 @@ __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPl
   if (N == 1 || nf <= 0) {
     __syncthreads();
     return a;
+  }
+  if (N <= 9) {
+    switch (N) {
+      case 3: fp64_rows<3, SIGN>(a, b, nf, ld); break;
+      case 5: fp64_rows<5, SIGN>(a, b, nf, ld); break;
+      case 7: fp64_rows<7, SIGN>(a, b, nf, ld); break;
+      default: fp64_rows<9, SIGN>(a, b, nf, ld);
+    }
+    __syncthreads();
+    return b;
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int all = 31;  // above every room
