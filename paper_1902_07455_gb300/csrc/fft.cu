@@ -428,12 +428,17 @@ static FftChoice& fft_choice(lrfg_ctx* ctx, int N, int kind, long long nrows, in
 // larger tile on a tie (fewer blocks restage fewer tables).  A 63 x 63 grid in 32-row tiles ran on one or two SMs: 46 us
 // per fibre pass and 88 us per fused row pass under event timing (9 and 17 us with even tiles and fixed point).  From six
 // full tiles per SM on the rounding up costs less than the shorter memory segments of a smaller tile, and tf_max stays.
-FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf) {
+// segments: long FP32 rows strided in memory, where a pass is bound by the accesses and not by its instructions.  A smaller tile
+// then keeps whole 32-byte sectors (four rows, unless there are fewer than two for an SM), has to leave fewer rows to the busiest SM, all of whose blocks fit its shared
+// memory, and is tried only where the largest gives an SM fewer than two blocks (down to half of it where it gives one): by
+// the instructions alone 8000 rows of 625 points took 135 us in tiles of 1 (54 in tiles of 16), 1000 of 3125 points 75 us (62).
+FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf, bool segments) {
   const long long nsm = ctx->num_sms > 0 ? ctx->num_sms : 152;
   FftPlan best = make_plan(N, fp64 ? plan_radix<double2>() : plan_radix<float2>());
   *tf = tf_max;
-  if ((nrows + tf_max - 1) / tf_max >= 6 * nsm) return best;
-  FftChoice& known = fft_choice(ctx, N, fp64 ? 1 : 0, nrows, tf_max);
+  const long long full = (nrows + tf_max - 1) / tf_max, full_rows = (full + nsm - 1) / nsm * tf_max;
+  if (full >= (segments ? 2 : 6) * nsm) return best;
+  FftChoice& known = fft_choice(ctx, N, segments ? 4 : (fp64 ? 1 : 0), nrows, tf_max);
   if (known.tf) {
     *tf = known.tf;
     return known.plan;
@@ -443,7 +448,12 @@ FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max
   for (int q = 0; q < (fp64 ? 2 : 1); ++q) {
     const FftPlan pl = q ? small : best;
     for (int t = tf_max; t >= 1; --t) {
-      const double c = fft_cycles(ctx, pl, t, (nrows + t - 1) / t);
+      const long long blocks = (nrows + t - 1) / t, per_sm = (blocks + nsm - 1) / nsm;
+      if (segments && t < tf_max &&
+          ((nrows > 2 * nsm && t % 4) || per_sm * t >= full_rows || (full >= nsm && 2 * t < tf_max) ||
+           (per_sm > 1 && per_sm * (2LL + 2 * t) * N * (long long)sizeof(float2) > ctx->max_smem_optin)))
+        continue;
+      const double c = fft_cycles(ctx, pl, t, blocks);
       if (cost == 0.0 || c < 0.97 * cost) {
         cost = c;
         best = pl;
@@ -466,7 +476,8 @@ static FftPlan tile_complex(lrfg_ctx* ctx, int N, size_t elem, long long nfib, i
   long long tf = (limit - 2 * row) / (2 * row);
   tf = std::max<long long>(1, std::min<long long>(tf, 32));
   if (tf > tf_min) tf = (tf / tf_min) * tf_min;
-  const FftPlan pl = choose_plan(ctx, N, elem == sizeof(double2), nfib, (int)tf, tf_out);
+  const bool fp64 = elem == sizeof(double2);
+  const FftPlan pl = choose_plan(ctx, N, fp64, nfib, (int)tf, tf_out, !fp64 && limit > 72 * 1024);
   *smem_out = (size_t)(2 * row + 2 * *tf_out * row);
   return pl;
 }

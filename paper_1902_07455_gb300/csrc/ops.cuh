@@ -15,8 +15,8 @@ constexpr int plan_radix() { return sizeof(V) == sizeof(float2) ? 27 : 9; }
 // device twiddle table W[j] = exp(-2 pi i j / N) in fixed point (for FP64 data) or rounded to FP32 (float)
 template <typename R>
 const typename TwOf<typename CplxOf<R>::T>::T* twiddle_table(lrfg_ctx* ctx, int N);
-// plan and rows of a tile (at most tf_max) for nrows rows
-FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf);
+// plan and rows of a tile (at most tf_max) for nrows rows (segments: see fft.cu)
+FftPlan choose_plan(lrfg_ctx* ctx, int N, bool fp64, long long nrows, int tf_max, int* tf, bool segments = false);
 // batched complex DFT along the middle axis of (outer, N, inner); sign -1 forward, +1 inverse
 // (V = double2 or float2)
 template <typename V>
