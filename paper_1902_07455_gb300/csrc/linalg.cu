@@ -472,36 +472,16 @@ __device__ double pow2_near_one(int hi_abs, int* red) {
 // whether k eigenvalues w of a Gram matrix reach down to its rounding
 __device__ __forceinline__ bool at_floor(const double* w, int k) { return w[k - 1] < 64.0 * 2.220446049250313e-16 * w[0]; }
 
-// Four combinations of the columns (of_rows: C is m x n) or rows (n x m) of C with random signs: Y (m x 4); nothing unless the k
-// eigenvalues w reach the floor.  A warp per entry of m, or a thread.
+// combinations of the columns or rows of C that judge what the known vectors leave of it
 constexpr int kImages = 4;
-__global__ void __launch_bounds__(256) random_images_kernel(const double* __restrict__ C, int m, int n, int of_rows,
-                                                            const double* __restrict__ w, int k, double* __restrict__ Y) {
-  if (!at_floor(w, k)) return;
-  const int lane = threadIdx.x & 31, step = of_rows ? 32 : 1;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = of_rows ? t >> 5 : t;
-  if (i >= m) return;
-  double y[kImages] = {0.0, 0.0, 0.0, 0.0};
-  for (int j = of_rows ? lane : 0; j < n; j += step) {
-    const double v = of_rows ? C[(size_t)i * n + j] : C[(size_t)j * m + i];
-    const unsigned h = ((unsigned)j + 1u) * 2654435761u;
-    const unsigned bits = (h ^ (h >> 15)) * 2246822519u;
-#pragma unroll
-    for (int l = 0; l < kImages; ++l) y[l] += (bits >> (28 + l) & 1u) ? v : -v;
-  }
-#pragma unroll
-  for (int l = 0; l < kImages; ++l) {
-    if (of_rows)
-      for (int o = 16; o; o >>= 1) y[l] += __shfl_xor_sync(0xffffffff, y[l], o);
-    if (!of_rows || lane == 0) Y[(size_t)i * kImages + l] = y[l];
-  }
-}
 
 // k > 0: only where the first k of the eigenvalues w, known already, reach the floor, and the k vectors known (in Vout) leave more
-// than 1e-13 of the images Y
+// than 1e-13 of C (m x n, or of_rows 0: n x m, whose Gram matrix is given): of four combinations of its columns (rows)
+// with random signs
 __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double* __restrict__ Ag, double* w,
                                                                double* Vout, int m, double* scratch, int use_smem,
-                                                               double eps, int k, const double* __restrict__ Y) {
+                                                               double eps, int k, const double* __restrict__ C, int n,
+                                                               int of_rows) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int mp = m + (m & 1);
   const int npair = mp / 2;
@@ -523,11 +503,28 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double* __
   }
   if (k > 0) {
     if (!at_floor(w, k)) return;
-    double* T = A;  // k x 4
+    double *Y = A, *T = A + m * kImages;  // m x 4, k x 4
+    const int lane = threadIdx.x & 31, part = of_rows ? lane : 0, step = of_rows ? 32 : 1;
+    for (int i = of_rows ? threadIdx.x >> 5 : threadIdx.x; i < m; i += of_rows ? blockDim.x >> 5 : blockDim.x) {
+      double y[kImages] = {0.0, 0.0, 0.0, 0.0};
+      for (int j = part; j < n; j += step) {
+        const double v = of_rows ? C[(size_t)i * n + j] : C[(size_t)j * m + i];
+        const unsigned h = ((unsigned)j + 1u) * 2654435761u, bits = (h ^ (h >> 15)) * 2246822519u;
+#pragma unroll
+        for (int l = 0; l < kImages; ++l) y[l] += (bits >> (28 + l) & 1u) ? v : -v;
+      }
+#pragma unroll
+      for (int l = 0; l < kImages; ++l) {
+        if (of_rows)
+          for (int o = 16; o; o >>= 1) y[l] += __shfl_xor_sync(0xffffffff, y[l], o);
+        if (part == 0) Y[i * kImages + l] = y[l];
+      }
+    }
+    __syncthreads();
     for (int q = threadIdx.x; q < k * kImages; q += blockDim.x) {
       const int t = q % k, l = q / k;
       double s = 0.0;
-      for (int i = 0; i < m; ++i) s = fma(Vout[(size_t)i * m + t], Y[(size_t)i * kImages + l], s);
+      for (int i = 0; i < m; ++i) s = fma(Vout[(size_t)i * m + t], Y[i * kImages + l], s);
       T[q] = s;
     }
     __syncthreads();
@@ -646,12 +643,13 @@ __global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(const double* __
   }
 }
 
-static void jacobi_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch, int k, const double* Y) {
+static void jacobi_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch, int k,
+                          const double* C, int n, bool of_rows) {
   const int npair = (m + 1) / 2;
   size_t head = sizeof(double) * 2 * npair + sizeof(int) * 2 * npair + sizeof(double) * 32 + sizeof(int) * (m + (m & 1));
   head = (head + 15) / 16 * 16;
   const size_t limit = (size_t)std::min(ctx->max_smem_optin, 220 * 1024);
-  const size_t one = head + sizeof(double) * (size_t)m * std::max(m, kImages), two = one + sizeof(double) * (size_t)m * m;
+  const size_t one = head + sizeof(double) * (size_t)m * std::max(m, 2 * kImages), two = one + sizeof(double) * (size_t)m * m;
   const int use_smem = two <= limit ? 2 : (one <= limit ? 1 : 0);
   const size_t smem = use_smem == 2 ? two : (use_smem == 1 ? one : head);
   DBuf<double> scratch;
@@ -660,19 +658,16 @@ static void jacobi_launch(lrfg_ctx* ctx, const double* A, double* w, double* V, 
   // one sweep of the two-sided cyclic Jacobi costs about 9 m^3 flops (rows, columns and V)
   LRFG_LAUNCH(ctx, KC_EIGEN, k > 0 ? 0.0 : 9.0 * (double)m * m * m * batch, k > 0 ? 0.0 : 3.0 * sizeof(double) * (double)m * m * batch,
               jacobi_kernel<<<batch, kJacobiThreads, smem, ctx->stream>>>(A, w, V, m, scratch.get(), use_smem,
-                                                                         2.220446049250313e-16, k, Y));
+                                                                         2.220446049250313e-16, k, C, n, of_rows));
 }
 
 void syevj(lrfg_ctx* ctx, const double* A, double* w, double* V, int m, int batch) {
   if (m <= 0 || batch <= 0) return;
-  jacobi_launch(ctx, A, w, V, m, batch, 0, nullptr);
+  jacobi_launch(ctx, A, w, V, m, batch, 0, nullptr, 0, false);
 }
 
 void syevj_floor(lrfg_ctx* ctx, const double* G, double* w, double* V, int m, int k, const double* C, int n, bool of_rows) {
-  DBuf<double> Y(ctx->pool, (size_t)m * kImages);
-  const int blocks = of_rows ? (m + 7) / 8 : (m + 255) / 256;
-  LRFG_LAUNCH(ctx, KC_EIGEN, 0.0, 0.0, random_images_kernel<<<blocks, 256, 0, ctx->stream>>>(C, m, n, of_rows, w, k, Y.get()));
-  jacobi_launch(ctx, G, w, V, m, 1, k, Y.get());
+  jacobi_launch(ctx, G, w, V, m, 1, k, C, n, of_rows);
 }
 
 // ------------------------------------------------------------------------------------------------
