@@ -305,7 +305,7 @@ __device__ __forceinline__ void fix_row(double2* row, int N, int first, int step
 // Rows of one butterfly in FP64, a row a thread: converting them would take longer than the transform
 // (90,000 rows of 3 points under a multiplier 35 us, in fixed point 84; of 9 points 53 and 96).
 template <int P, int SIGN>
-__device__ __noinline__ void fp64_rows(const double2* __restrict__ a, double2* __restrict__ b, int nf, int ld) {
+__device__ __forceinline__ void fp64_butterflies(const double2* __restrict__ a, double2* __restrict__ b, int nf, int ld) {
   for (int row = threadIdx.x; row < nf; row += blockDim.x) {
     double2 x[P];
 #pragma unroll
@@ -313,6 +313,15 @@ __device__ __noinline__ void fp64_rows(const double2* __restrict__ a, double2* _
     RegDFT<P, SIGN, double2>::run(x);
 #pragma unroll
     for (int r = 0; r < P; ++r) b[row * ld + r] = x[r];
+  }
+}
+template <int SIGN>
+__device__ __noinline__ void fp64_rows(int N, const double2* a, double2* b, int nf, int ld) {
+  switch (N) {
+    case 3: fp64_butterflies<3, SIGN>(a, b, nf, ld); break;
+    case 5: fp64_butterflies<5, SIGN>(a, b, nf, ld); break;
+    case 7: fp64_butterflies<7, SIGN>(a, b, nf, ld); break;
+    default: fp64_butterflies<9, SIGN>(a, b, nf, ld);
   }
 }
 
@@ -327,12 +336,7 @@ __device__ double2* fix_rows(double2* a, double2* b, int nf, int ld, const FftPl
     return a;
   }
   if (N <= 9) {
-    switch (N) {
-      case 3: fp64_rows<3, SIGN>(a, b, nf, ld); break;
-      case 5: fp64_rows<5, SIGN>(a, b, nf, ld); break;
-      case 7: fp64_rows<7, SIGN>(a, b, nf, ld); break;
-      default: fp64_rows<9, SIGN>(a, b, nf, ld);
-    }
+    fp64_rows<SIGN>(N, a, b, nf, ld);
     __syncthreads();
     return b;
   }
